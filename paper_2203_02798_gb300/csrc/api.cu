@@ -121,6 +121,7 @@ int lsk_destroy(lsk_ctx* ctx) {
     if (ctx->flag) cudaFree(ctx->flag);
     if (ctx->prof) lsk_prof_delete(ctx->prof);
     lsk_batch_free(ctx);
+    lsq_host_free(ctx);
     free(ctx);
     return LSK_OK;
 }
@@ -845,7 +846,7 @@ int lsk_sketch_precondition_lsq(lsk_ctx* ctx, const lsk_mat* A, const double* b,
     if (rc) return rc;
     if (opts->max_iter < 1 || opts->max_refine < 0 || !(opts->tol > 0.0))
         return fail(ctx, LSK_ERR_INVALID_ARG, "bad LSQ options");
-    rc = ws_ensure(ctx, sketch_bytes(A, opts->r, opts->k, prec, ctx->sm_count, lsq_workspace_bytes(A)));
+    rc = ws_ensure(ctx, sketch_bytes(A, opts->r, opts->k, prec, ctx->sm_count, lsq_workspace_bytes(A, ctx->sm_count)));
     if (rc) return rc;
     const SketchBufs bufs = carve(ctx->ws, A, opts->r, opts->k);
     cudaError_t e = sketch_and_factor(ctx, A, opts->r, opts->k, opts->seed, prec, bufs, nullptr);
@@ -860,7 +861,7 @@ int lsk_sketch_precondition_lsq(lsk_ctx* ctx, const lsk_mat* A, const double* b,
         return flag_to_status(ctx, f);
     }
     lsk_lsq_info tmp;
-    rc = lsq_run(ctx, A, b, x, opts, bufs.Rinv64, bufs.Rinv32, bufs.scratch, info ? info : &tmp);
+    rc = lsq_run(ctx, A, b, x, opts, bufs.Rinv64, bufs.scratch, info ? info : &tmp);
     if (rc == LSK_ERR_CUDA) return fail(ctx, rc, "lsk_sketch_precondition_lsq: CUDA error %s",
                                         cudaGetErrorString(cudaGetLastError()));
     if (rc == LSK_ERR_NOT_CONVERGED) return fail(ctx, rc, "least squares did not reach tol");

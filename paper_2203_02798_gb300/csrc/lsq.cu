@@ -20,27 +20,583 @@
 // device; the host reads them back every few iterations for the stop test.
 #include "lsk_internal.cuh"
 
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
+#include <new>
 #include <string.h>
+
+namespace cg = cooperative_groups;
 
 namespace {
 
-struct LsqrState {
-    double alpha, beta, rhobar, phibar, anorm2, atb_norm, eta, bnorm;
-    double arnorm, rnorm;
+struct CgState {
+    double atb_norm, eta;
+    double rho, rho0;   // ||s||^2 now and at the start of the inner solve
     int done, it;
-    double rho, rho0;   // CG on the normal equations: ||s||^2 now and at the start
 };
 
 constexpr int kPassThreads = 256;
 
-// ---- FP64 residual + A^T r, dense: warp per row ---------------------------
+// Programmatic dependent launch: the passes and the vector step of the inner
+// solve alternate some 130 times, so each lets the next one's blocks start
+// (and load what no kernel of the solve writes) while it finishes; everything
+// the previous kernel writes is read after pdl_wait, with __ldcg (a load the
+// compiler may not take for one of constant memory and move ahead of the wait).  Every kernel launched
+// this way waits before it returns, so completion stays in launch order.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class F, class... Args>
+cudaError_t launch_pdl(F* kernel, int blocks, int threads, size_t smem, int cluster, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// ---- FP32 pairs: x = h + l carries ~48 bits at the FP32 rate (FP64 runs at
+// 1/64 of it here).  Products by FMA, sums by Knuth's TwoSum; a dot product
+// kept this way is the "Dot2" of Ogita, Rump & Oishi (SIAM J. Sci. Comput. 26,
+// 2005): as accurate as one computed in twice the working precision.
+__device__ __forceinline__ float2 to_pair(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+// (h, l) += a * (xh + xl)
+__device__ __forceinline__ void pair_fma(float& h, float& l, float a, float xh, float xl) {
+    const float p = a * xh;
+    const float e = fmaf(a, xl, fmaf(a, xh, -p));
+    const float s = h + p;
+    const float t = s - h;
+    l += ((h - (s - t)) + (p - t)) + e;
+    h = s;
+}
+// (h, l) += (h2, l2)
+__device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2) {
+    const float s = h + h2;
+    const float t = s - h;
+    l += ((h - (s - t)) + (h2 - t)) + l2;
+    h = s;
+}
+
+// Sum each of RB per-lane values over groups of L lanes: at every step a lane
+// keeps half of its values and hands over the other half, so the RB sums cost
+// about RB + 3 exchanges instead of 5 RB.  On return the sum of value r is in
+// the lanes of the group whose bit log2(L) - 1 - b is bit b of r (sum_lane,
+// sum_index).
+template <int RB, int L>
+__device__ __forceinline__ int sum_lane(int r) {
+    int l = 0;
+#pragma unroll
+    for (int b = 0; (1 << b) < RB; ++b) l |= ((r >> b) & 1) * (L >> (b + 1));
+    return l;
+}
+template <int RB, int L>
+__device__ __forceinline__ int sum_index(int lane) {
+    int r = 0;
+#pragma unroll
+    for (int b = 0; (1 << b) < RB; ++b) r |= (lane & (L >> (b + 1))) ? 1 << b : 0;
+    return r;
+}
+template <int RB, int L>
+__device__ __forceinline__ float warp_sum_rows(float (&v)[RB], int lane) {
+    int o = L / 2;
+#pragma unroll
+    for (int m = RB; m > 1; m >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int r = 0; r < m / 2; ++r) {   // even values stay in the lower lanes
+            const float keep = up ? v[2 * r + 1] : v[2 * r];
+            const float give = up ? v[2 * r] : v[2 * r + 1];
+            v[r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    float t = v[0];
+    for (; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+template <int RB, int L>
+__device__ __forceinline__ float2 warp_sum_rows(float (&h)[RB], float (&l)[RB], int lane) {
+    int o = L / 2;
+#pragma unroll
+    for (int m = RB; m > 1; m >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int r = 0; r < m / 2; ++r) {
+            float kh = up ? h[2 * r + 1] : h[2 * r], kl = up ? l[2 * r + 1] : l[2 * r];
+            const float gh = up ? h[2 * r] : h[2 * r + 1], gl = up ? l[2 * r] : l[2 * r + 1];
+            pair_add(kh, kl, __shfl_xor_sync(0xffffffffu, gh, o), __shfl_xor_sync(0xffffffffu, gl, o));
+            h[r] = kh;
+            l[r] = kl;
+        }
+    }
+    for (; o; o >>= 1) pair_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], o), __shfl_xor_sync(0xffffffffu, l[0], o));
+    return make_float2(h[0], l[0]);
+}
+
+// ---- dense passes, d <= 256 --------------------------------------------------
+// A warp takes RB x (32 / L) rows at a time: L lanes own a row, each E entries
+// of it -- kVec: E / 4 runs of four columns (16-byte loads; d, lda multiples
+// of 4, A 16-byte aligned), else columns L apart -- and the next rows' loads
+// are in flight while it computes.
+template <int L, int E, int RB, bool kVec>
+struct DenseRows {
+    static constexpr int kRpl = 32 / L;            // rows a load instruction covers
+    static constexpr int kRows = RB * kRpl;        // rows a warp takes at a time
+    float a[RB][E];
+    static __device__ __forceinline__ int col(int li, int e) { return kVec ? 4 * (li + L * (e / 4)) + e % 4 : li + L * e; }
+    __device__ __forceinline__ void load(const float* __restrict__ A, int64_t lda, int64_t n, int d, int64_t i0, int lane) {
+        const int sub = lane / L, li = lane % L;
+        const float* row = A + (i0 + sub) * lda;
+        const int64_t rs = (int64_t)kRpl * lda;
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const bool in = i0 + r * kRpl + sub < n;
+            if constexpr (kVec) {
+#pragma unroll
+                for (int v = 0; v < E / 4; ++v) {
+                    const int c = 4 * (li + L * v);
+                    const float4 t = (in && c < d) ? __ldg(reinterpret_cast<const float4*>(row + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    a[r][4 * v] = t.x;
+                    a[r][4 * v + 1] = t.y;
+                    a[r][4 * v + 2] = t.z;
+                    a[r][4 * v + 3] = t.w;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int c = li + L * e;
+                    a[r][e] = (in && c < d) ? __ldg(row + c) : 0.f;
+                }
+            }
+            row += rs;
+        }
+    }
+    __device__ __forceinline__ void take(const DenseRows& o) {
+#pragma unroll
+        for (int r = 0; r < RB; ++r)
+#pragma unroll
+            for (int e = 0; e < E; ++e) a[r][e] = o.a[r][e];
+    }
+};
+
+// r = b - A x and partial sums of A^T r in one read of A.  The dots and the
+// sums over rows are FP32 pairs, r itself FP64; FP64 arithmetic throughout (two
+// FMAs, two conversions an entry at 1/64 rate) took 471 us at 316,227 x 128,
+// where reading A takes 24; this takes 57.
+template <int L, int E, int RB, bool kVec>
+__global__ void __launch_bounds__(kPassThreads, 2) resid_dense_rows_kernel(
+    const float* __restrict__ A, int64_t lda, int64_t n, int d, const double* __restrict__ b,
+    const double* __restrict__ x, double* __restrict__ qpart) {
+    using Rows = DenseRows<L, E, RB, kVec>;
+    __shared__ double qs[(kPassThreads / 32) * Rows::kRpl][L * E];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane / L, li = lane % L;
+    float xh[E], xl[E], qh[E], ql[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int j = Rows::col(li, e);
+        const float2 v = to_pair(j < d ? x[j] : 0.0);
+        xh[e] = v.x;
+        xl[e] = v.y;
+        qh[e] = ql[e] = 0.f;
+    }
+    const int mine = sum_index<RB, L>(lane) * Rows::kRpl + sub;   // the row whose sum this lane receives
+    const int64_t step = (int64_t)gridDim.x * (kPassThreads / 32) * Rows::kRows;
+    int64_t i0 = ((int64_t)blockIdx.x * (kPassThreads / 32) + w) * Rows::kRows;
+    Rows cur, nxt;
+    double bn = 0.0;
+    if (i0 < n) {
+        cur.load(A, lda, n, d, i0, lane);
+        if (i0 + mine < n) bn = b[i0 + mine];
+    }
+    for (; i0 < n; i0 += step) {
+        const double bi = bn;
+        if (i0 + step < n) {
+            nxt.load(A, lda, n, d, i0 + step, lane);
+            bn = i0 + step + mine < n ? b[i0 + step + mine] : 0.0;
+        }
+        float h[RB], l[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            h[r] = l[r] = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) pair_fma(h[r], l[r], cur.a[r][e], xh[e], xl[e]);
+        }
+        const float2 dot = warp_sum_rows<RB, L>(h, l, lane);
+        const float2 ri = to_pair(i0 + mine < n ? (bi - (double)dot.x) - (double)dot.y : 0.0);
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const int src = sub * L + sum_lane<RB, L>(r);
+            const float rh = __shfl_sync(0xffffffffu, ri.x, src);
+            const float rl = __shfl_sync(0xffffffffu, ri.y, src);
+#pragma unroll
+            for (int e = 0; e < E; ++e) pair_fma(qh[e], ql[e], cur.a[r][e], rh, rl);
+        }
+        cur.take(nxt);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) qs[w * Rows::kRpl + sub][Rows::col(li, e)] = (double)qh[e] + (double)ql[e];
+    __syncthreads();
+    for (int j = threadIdx.x; j < d; j += blockDim.x) {
+        double t = 0.0;
+        for (int z = 0; z < (kPassThreads / 32) * Rows::kRpl; ++z) t += qs[z][j];
+        qpart[(int64_t)blockIdx.x * d + j] = t;
+    }
+}
+
+// u = A p: partial sums of u^2 (pairs) and of A^T u; u is used while its rows
+// are in registers and not kept.  Passes alternate their direction (rev): where
+// A is larger than L2, the rows one pass reads last are still there for the
+// next (119 us a pass against 153 at 900,000 x 256, 25 against 30 at 316,227 x
+// 128; 40 us there with one row group in flight and u read and written).
+template <int L, int E, int RB, bool kVec>
+__global__ void __launch_bounds__(kPassThreads, 2) cg_pass_dense_rows_kernel(
+    const float* __restrict__ A, int64_t lda, int64_t n, int d, const float* __restrict__ p,
+    const CgState* __restrict__ st, int rev, float* __restrict__ qpart, double* __restrict__ sspart) {
+    using Rows = DenseRows<L, E, RB, kVec>;
+    __shared__ float qs[(kPassThreads / 32) * Rows::kRpl][L * E];
+    __shared__ double ssw[kPassThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane / L, li = lane % L;
+    const int64_t groups = (n + Rows::kRows - 1) / Rows::kRows, step = (int64_t)gridDim.x * (kPassThreads / 32);
+    int64_t g = (int64_t)blockIdx.x * (kPassThreads / 32) + w;
+    Rows cur, nxt;
+    if (g < groups) cur.load(A, lda, n, d, (rev ? groups - 1 - g : g) * Rows::kRows, lane);
+    pdl_wait();
+    pdl_launch_next();
+    if (__ldcg(&st->done)) return;
+    float pr[E], q[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int j = Rows::col(li, e);
+        pr[e] = j < d ? __ldcg(p + j) : 0.f;
+        q[e] = 0.f;
+    }
+    float sh = 0.f, sl = 0.f;
+    for (; g < groups; g += step) {
+        const int64_t gn = g + step;
+        if (gn < groups) nxt.load(A, lda, n, d, (rev ? groups - 1 - gn : gn) * Rows::kRows, lane);
+        float dot[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            dot[r] = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) dot[r] = fmaf(cur.a[r][e], pr[e], dot[r]);
+        }
+        const float u = warp_sum_rows<RB, L>(dot, lane);   // rows past n are zero
+        pair_fma(sh, sl, u, u, 0.f);
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const float ui = __shfl_sync(0xffffffffu, u, sub * L + sum_lane<RB, L>(r));
+#pragma unroll
+            for (int e = 0; e < E; ++e) q[e] = fmaf(cur.a[r][e], ui, q[e]);
+        }
+        cur.take(nxt);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) qs[w * Rows::kRpl + sub][Rows::col(li, e)] = q[e];
+    // each row's u is in L / RB lanes: one of them counts
+    const double ss = warp_sum((lane & (L / RB - 1)) == 0 ? (double)sh + (double)sl : 0.0);
+    if (lane == 0) ssw[w] = ss;
+    __syncthreads();
+    for (int j = threadIdx.x; j < d; j += blockDim.x) {
+        float t = 0.f;
+        for (int z = 0; z < (kPassThreads / 32) * Rows::kRpl; ++z) t += qs[z][j];
+        qpart[(int64_t)blockIdx.x * d + j] = t;
+    }
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int z = 0; z < kPassThreads / 32; ++z) t += ssw[z];
+        sspart[blockIdx.x] = t;
+    }
+}
+
+// ---- CSR: both products of a pass without atomics ---------------------------
+// A solve makes some 60 passes over the same matrix, so its rows are cut into
+// tiles of `rows_per` rows once and each tile's entries also stored sorted by
+// column (local row, value).  A pass then forms u = A p on a tile from the CSR
+// entries (segments: rows) and A^T u from the sorted ones (segments:
+// columns; the CSR arrays were checked by the sketch): in both, the block multiplies a coalesced run of entries by the
+// vector's values in shared memory and sums the segments from there.  With
+// one thread per row and shared-memory float atomics (compare-and-swap loops)
+// for A^T u, a pass took 35 us at 500,000 x 256 and 2.6 M entries; this takes 15,
+// and building the tiles 45 once.
+constexpr int kTileRowsMax = 4096;
+constexpr int kTilesPerSm = 3;
+// Entries are taken six quads a thread at a time (16-byte loads, all in flight
+// before any product): 6,144 to a run, so that a tile of 500,000 sparse rows is
+// one run; 80 registers a thread, three blocks an SM, one wave of tiles.
+constexpr int kQuads = 6;
+constexpr int kTileEntries = kQuads * 4 * kPassThreads;
+
+struct CsrTiles {
+    int64_t n, d, ntiles;
+    int rows_per;
+    const float* V;
+    const int32_t* J;
+    const int64_t* I;
+    int32_t* cptr;     // ntiles x (d + 1): column offsets inside each tile
+    float* tval;       // nnz
+    uint16_t* trow;    // nnz
+};
+
+__global__ void __launch_bounds__(kPassThreads) csr_tiles_kernel(CsrTiles t, int64_t nnz) {
+    extern __shared__ int cnt[];                     // d
+    __shared__ uint16_t rid[kTileEntries];           // row of each entry of the run in hand
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * t.rows_per;
+    const int rows = (int)min((int64_t)t.rows_per, t.n - r0);
+    const int d = (int)t.d;
+    for (int j = threadIdx.x; j < d; j += blockDim.x) cnt[j] = 0;
+    __syncthreads();
+    const int64_t base = t.I[r0], end = min(t.I[r0 + rows], nnz);
+#pragma unroll 8
+    for (int64_t e = base + threadIdx.x; e < end; e += kPassThreads)
+        atomicAdd(&cnt[min((uint32_t)__ldg(t.J + e), (uint32_t)(d - 1))], 1);
+    __syncthreads();
+    if (w == 0) {   // exclusive scan
+        int32_t* out = t.cptr + (int64_t)blockIdx.x * (d + 1);
+        int run = 0;
+        for (int j0 = 0; j0 < d; j0 += 32) {
+            const int j = j0 + lane;
+            const int v = j < d ? cnt[j] : 0;
+            int s = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, s, o);
+                if (lane >= o) s += up;
+            }
+            if (j < d) {
+                cnt[j] = run + s - v;
+                out[j] = run + s - v;
+            }
+            run += __shfl_sync(0xffffffffu, s, 31);
+        }
+        if (lane == 0) out[d] = run;
+    }
+    for (int64_t c0 = base; c0 < end; c0 += kTileEntries) {
+        const int m = (int)min((int64_t)kTileEntries, end - c0);
+        __syncthreads();
+        for (int r = threadIdx.x; r < rows; r += kPassThreads) {
+            const int k0 = (int)max(t.I[r0 + r] - c0, (int64_t)0), k1 = (int)min(t.I[r0 + r + 1] - c0, (int64_t)m);
+            for (int k = k0; k < k1; ++k) rid[k] = (uint16_t)r;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = threadIdx.x; k < m; k += kPassThreads) {
+            const float v = __ldg(t.V + c0 + k);
+            const int pos = atomicAdd(&cnt[min((uint32_t)__ldg(t.J + c0 + k), (uint32_t)(d - 1))], 1);
+            t.tval[base + pos] = v;
+            t.trow[base + pos] = rid[k];
+        }
+    }
+}
+
+// out[s] += sum over the entries e of segment s of val[e] vec[idx[e]], for the
+// segments [ptr[s], ptr[s + 1]) of a run of entries.  The run starts at a
+// multiple of four (`shift` entries before the first segment); 2^lg lanes a
+// segment.  Values are float, or pairs (float2) for the residual pass.
+__device__ __forceinline__ float seg_mul(float v, float x) { return v * x; }
+__device__ __forceinline__ float2 seg_mul(float v, float2 x) {
+    const float p = v * x.x;
+    return make_float2(p, fmaf(v, x.y, fmaf(v, x.x, -p)));
+}
+__device__ __forceinline__ void seg_add(float& s, float v) { s += v; }
+__device__ __forceinline__ void seg_add(float2& s, float2 v) { pair_add(s.x, s.y, v.x, v.y); }
+__device__ __forceinline__ float seg_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float2 seg_shfl(float2 v, int o) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ float seg_zero(float) { return 0.f; }
+__device__ __forceinline__ float2 seg_zero(float2) { return make_float2(0.f, 0.f); }
+
+__device__ __forceinline__ int4 idx_quad(const int32_t* p) { return __ldg(reinterpret_cast<const int4*>(p)); }
+__device__ __forceinline__ int4 idx_quad(const uint16_t* p) {
+    const ushort4 t = __ldg(reinterpret_cast<const ushort4*>(p));
+    return make_int4(t.x, t.y, t.z, t.w);
+}
+
+struct EntryQuads {
+    float4 v[kQuads];
+    int4 j[kQuads];
+};
+
+// Entries [e0, e0 + 6144) of the run, e0 a multiple of four, up to `end` of
+// the arrays (vec4: both are 16-byte aligned; the last quad may be ragged).
+template <class Idx>
+__device__ __forceinline__ void load_quads(EntryQuads& r, const float* __restrict__ val, const Idx* __restrict__ idx,
+                                           int64_t e0, int64_t end, bool vec4) {
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) {
+        const int64_t e = e0 + 4 * (threadIdx.x + q * kPassThreads);
+        r.v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        r.j[q] = make_int4(0, 0, 0, 0);
+        if (vec4 && e + 4 <= end) {
+            r.v[q] = __ldg(reinterpret_cast<const float4*>(val + e));
+            r.j[q] = idx_quad(idx + e);
+        } else if (e < end) {
+            r.v[q].x = val[e];
+            r.j[q].x = idx[e];
+            if (e + 1 < end) r.v[q].y = val[e + 1], r.j[q].y = idx[e + 1];
+            if (e + 2 < end) r.v[q].z = val[e + 2], r.j[q].z = idx[e + 2];
+            if (e + 3 < end) r.v[q].w = val[e + 3], r.j[q].w = idx[e + 3];
+        }
+    }
+}
+
+template <class T>
+__device__ __forceinline__ void mul_quads(const EntryQuads& r, const T* vec, int nvec, T* prod, int m) {
+    const uint32_t top = (uint32_t)(nvec - 1);
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) {
+        const int e = 4 * (threadIdx.x + q * kPassThreads);
+        if (e >= m) continue;
+        const T a = seg_mul(r.v[q].x, vec[min((uint32_t)r.j[q].x, top)]), b = seg_mul(r.v[q].y, vec[min((uint32_t)r.j[q].y, top)]);
+        const T c = seg_mul(r.v[q].z, vec[min((uint32_t)r.j[q].z, top)]), f = seg_mul(r.v[q].w, vec[min((uint32_t)r.j[q].w, top)]);
+        if constexpr (sizeof(T) == sizeof(float)) {
+            *reinterpret_cast<float4*>(prod + e) = make_float4(a, b, c, f);
+        } else {
+            *reinterpret_cast<float4*>(prod + e) = make_float4(a.x, a.y, b.x, b.y);
+            *reinterpret_cast<float4*>(prod + e + 2) = make_float4(c.x, c.y, f.x, f.y);
+        }
+    }
+}
+
+template <class T>
+__device__ __forceinline__ void sum_segments(const T* prod, int c0, int m, int shift, const int32_t* ptr, int nseg,
+                                             int lg, T* out) {
+    const int G = 1 << lg, sub = threadIdx.x & (G - 1);
+    for (int s0 = 0; s0 < nseg; s0 += kPassThreads >> lg) {
+        const int s = s0 + (threadIdx.x >> lg);
+        T t = seg_zero(T{});
+        int k0 = 0, k1 = 0;
+        if (s < nseg) {
+            k0 = max(ptr[s] + shift, c0);
+            k1 = min(ptr[s + 1] + shift, c0 + m);
+            for (int k = k0 + sub; k < k1; k += G) seg_add(t, prod[k - c0]);
+        }
+        for (int o = G >> 1; o; o >>= 1) seg_add(t, seg_shfl(t, o));
+        if (k1 > k0 && sub == 0) seg_add(out[s], t);
+    }
+}
+
+__device__ __forceinline__ int seg_lanes(int nseg) {   // log2 of the lanes a segment
+    int lg = 0;
+    while (lg < 5 && (nseg << (lg + 1)) <= kPassThreads) ++lg;
+    return lg;
+}
+
+// T = float: u = A p and partial sums of A^T u, ||u||^2.
+// T = float2: r = b - A x and partial sums of A^T r (FP64 partials).
+template <class T>
+__global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(CsrTiles t, const float* __restrict__ p,
+                                                                 const double* __restrict__ x,
+                                                                 const double* __restrict__ b,
+                                                                 const CgState* __restrict__ st,
+                                                                 void* __restrict__ qpart, double* __restrict__ sspart) {
+    constexpr bool kResid = sizeof(T) == sizeof(float2);
+    extern __shared__ __align__(16) unsigned char tile_sh[];
+    __shared__ double ssw[kPassThreads / 32];
+    const int d = (int)t.d;
+    T* prod = reinterpret_cast<T*>(tile_sh);
+    T* vec = prod + kTileEntries;            // p or x
+    T* q = vec + d;
+    T* u = q + d;
+    int32_t* rptr = reinterpret_cast<int32_t*>(u + t.rows_per);   // rows_per + 1
+    int32_t* cptr = rptr + t.rows_per + 1;                        // d + 1
+    // the first run's entries do not depend on the previous kernel
+    const bool vec4 = ((reinterpret_cast<uintptr_t>(t.V) | reinterpret_cast<uintptr_t>(t.J)) & 15) == 0;
+    EntryQuads r;
+    int64_t base = 0, base4 = 0, end = 0;
+    if (blockIdx.x < t.ntiles) {
+        const int64_t r0 = (int64_t)blockIdx.x * t.rows_per;
+        base = t.I[r0];
+        end = t.I[min(r0 + t.rows_per, t.n)];
+        base4 = base & ~(int64_t)3;
+        load_quads(r, t.V, t.J, base4, end, vec4);
+    }
+    pdl_wait();
+    pdl_launch_next();
+    if (!kResid && __ldcg(&st->done)) return;
+    for (int j = threadIdx.x; j < d; j += kPassThreads) {
+        if constexpr (kResid) vec[j] = to_pair(x[j]);
+        else vec[j] = __ldcg(p + j);
+        q[j] = seg_zero(T{});
+    }
+    float sh = 0.f, sl = 0.f;
+    for (int64_t tile = blockIdx.x; tile < t.ntiles; tile += gridDim.x) {
+        const int64_t r0 = tile * t.rows_per;
+        const int rows = (int)min((int64_t)t.rows_per, t.n - r0);
+        if (tile != blockIdx.x) {
+            base = t.I[r0];
+            end = t.I[r0 + rows];
+            base4 = base & ~(int64_t)3;
+            load_quads(r, t.V, t.J, base4, end, vec4);
+        }
+        const int count = (int)(end - base4), shift = (int)(base - base4);
+        __syncthreads();   // the last tile's readers of rptr, cptr, u
+        for (int i = threadIdx.x; i <= rows; i += kPassThreads) {
+            rptr[i] = (int32_t)(t.I[r0 + i] - base);
+            if (i < rows) u[i] = seg_zero(T{});
+        }
+        for (int j = threadIdx.x; j <= d; j += kPassThreads) cptr[j] = t.cptr[tile * (d + 1) + j];
+        __syncthreads();
+        const int lgr = seg_lanes(rows), lgd = seg_lanes(d);
+        for (int c0 = 0; c0 < count; c0 += kTileEntries) {
+            const int m = min(kTileEntries, count - c0);
+            if (c0) load_quads(r, t.V, t.J, base4 + c0, end, vec4);
+            mul_quads(r, vec, d, prod, m);
+            if (c0 + kTileEntries >= count) load_quads(r, t.tval, t.trow, base4, end, true);   // for the next product
+            __syncthreads();
+            sum_segments(prod, c0, m, shift, rptr, rows, lgr, u);
+            __syncthreads();
+        }
+        for (int i = threadIdx.x; i < rows; i += kPassThreads) {
+            if constexpr (kResid) u[i] = to_pair((b[r0 + i] - (double)u[i].x) - (double)u[i].y);
+            else pair_fma(sh, sl, u[i], u[i], 0.f);
+        }
+        __syncthreads();
+        for (int c0 = 0; c0 < count; c0 += kTileEntries) {
+            const int m = min(kTileEntries, count - c0);
+            if (c0) load_quads(r, t.tval, t.trow, base4 + c0, end, true);
+            mul_quads(r, u, rows, prod, m);
+            __syncthreads();
+            sum_segments(prod, c0, m, shift, cptr, d, lgd, q);
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < d; j += kPassThreads) {
+        if constexpr (kResid) reinterpret_cast<double*>(qpart)[(int64_t)blockIdx.x * d + j] = (double)q[j].x + (double)q[j].y;
+        else reinterpret_cast<float*>(qpart)[(int64_t)blockIdx.x * d + j] = q[j];
+    }
+    if constexpr (!kResid) {
+        const double ss = warp_sum((double)sh + (double)sl);
+        if ((threadIdx.x & 31) == 0) ssw[threadIdx.x >> 5] = ss;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int z = 0; z < kPassThreads / 32; ++z) s += ssw[z];
+            sspart[blockIdx.x] = s;
+        }
+    }
+}
+
+// ---- FP64 residual + A^T r, dense, d > 256: warp per row -------------------
 __global__ void __launch_bounds__(kPassThreads) resid64_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const double* __restrict__ b,
-    const double* __restrict__ x, float* __restrict__ u32, double* __restrict__ qpart,
-    double* __restrict__ sspart) {
+    const double* __restrict__ x, double* __restrict__ qpart) {
     extern __shared__ double sh[];   // x (d) then per-warp q (8 * d)
     double* xs = sh;
     double* qs = sh + d;
@@ -49,7 +605,6 @@ __global__ void __launch_bounds__(kPassThreads) resid64_dense_kernel(
     for (int64_t j = threadIdx.x; j < 8 * d; j += blockDim.x) qs[j] = 0.0;
     __syncthreads();
     double* qw = qs + w * d;
-    double ss = 0.0;
     const int64_t wid = (int64_t)blockIdx.x * 8 + w, nw = (int64_t)gridDim.x * 8;
     for (int64_t i = wid; i < n; i += nw) {
         const float* row = A + i * lda;
@@ -57,8 +612,6 @@ __global__ void __launch_bounds__(kPassThreads) resid64_dense_kernel(
         for (int64_t j = lane; j < d; j += 32) dot = fma((double)row[j], xs[j], dot);
         dot = warp_sum(dot);
         const double ri = b[i] - dot;
-        if (lane == 0) u32[i] = (float)ri;
-        ss = fma(ri, ri, ss);
         for (int64_t j = lane; j < d; j += 32) qw[j] = fma((double)row[j], ri, qw[j]);
     }
     __syncthreads();
@@ -67,22 +620,13 @@ __global__ void __launch_bounds__(kPassThreads) resid64_dense_kernel(
         for (int t = 0; t < 8; ++t) s += qs[t * d + j];
         qpart[(int64_t)blockIdx.x * d + j] = s;
     }
-    // each warp's ss is replicated across lanes (ri is uniform): lane 0 adds
-    __shared__ double ssw[8];
-    if (lane == 0) ssw[w] = ss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < 8; ++t) s += ssw[t];
-        sspart[blockIdx.x] = s;
-    }
 }
 
 // ---- FP64 residual + A^T r, CSR: thread per row ----------------------------
 __global__ void __launch_bounds__(kPassThreads) resid64_csr_kernel(
     const float* __restrict__ V, const int32_t* __restrict__ J, const int64_t* __restrict__ I,
     int64_t n, int64_t nnz, int64_t d, const double* __restrict__ b, const double* __restrict__ x,
-    float* __restrict__ u32, double* __restrict__ qpart, double* __restrict__ sspart, int* flag) {
+    double* __restrict__ qpart, int* flag) {
     extern __shared__ double sh[];
     double* xs = sh;
     double* qs = sh + d;
@@ -91,7 +635,6 @@ __global__ void __launch_bounds__(kPassThreads) resid64_csr_kernel(
         qs[j] = 0.0;
     }
     __syncthreads();
-    double ss = 0.0;
     bool bad = false;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -106,8 +649,6 @@ __global__ void __launch_bounds__(kPassThreads) resid64_csr_kernel(
                 else bad = true;
             }
         const double ri = b[i] - dot;
-        u32[i] = (float)ri;
-        ss = fma(ri, ri, ss);
         if (ok)
             for (int64_t p = k0; p < k1; ++p) {
                 const int32_t j = J[p];
@@ -115,135 +656,24 @@ __global__ void __launch_bounds__(kPassThreads) resid64_csr_kernel(
             }
     }
     if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
-    ss = warp_sum(ss);
-    __shared__ double ssw[kPassThreads / 32];
-    if ((threadIdx.x & 31) == 0) ssw[threadIdx.x >> 5] = ss;
     __syncthreads();
     for (int64_t j = threadIdx.x; j < d; j += blockDim.x) qpart[(int64_t)blockIdx.x * d + j] = qs[j];
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < kPassThreads / 32; ++t) s += ssw[t];
-        sspart[blockIdx.x] = s;
-    }
 }
 
-// out[j] = sum_z part[z][j] in z order groups: with blockDim >= 4d the
-// partials are split four ways (z mod 4) and the four sums added in order.
-__device__ __forceinline__ void reduce_partials(const float* __restrict__ part, int nblocks, int64_t d,
-                                                float* __restrict__ out) {
-    __shared__ float red4[4][256];
-    if (d <= 256 && blockDim.x >= 4 * d) {
-        const int j = threadIdx.x % d, g = threadIdx.x / d;
-        if (g < 4) {
-            float s = 0.f;
-            for (int z = g; z < nblocks; z += 4) s += part[(int64_t)z * d + j];
-            red4[g][j] = s;
-        }
-        __syncthreads();
-        if (threadIdx.x < d) out[threadIdx.x] = (red4[0][threadIdx.x] + red4[1][threadIdx.x]) +
-                                                (red4[2][threadIdx.x] + red4[3][threadIdx.x]);
-    } else {
-        for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-            float s = 0.f;
-            for (int z = 0; z < nblocks; ++z) s += part[(int64_t)z * d + j];
-            out[j] = s;
-        }
-    }
-}
-
-// u <- A p - (alpha/beta) u; partial sums of u^2 and of A^T u.  Dense,
-// d <= 256: a warp takes RB rows at a time (all RB rows' loads in flight
-// before any arithmetic), lane l owns columns l, l + 32, ... (CPL of them),
-// so p and the warp's share of A^T u stay in registers.
-template <int CPL, int RB>
-__global__ void __launch_bounds__(kPassThreads, 2) lsqr_pass_dense_rows_kernel(
+// u = A p: partial sums of u^2 and of A^T u.  Dense, any d: warp per row.
+__global__ void __launch_bounds__(kPassThreads) cg_pass_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ p,
-    const LsqrState* __restrict__ st, float* __restrict__ u, float* __restrict__ qpart,
-    double* __restrict__ sspart) {
-    __shared__ float qs[kPassThreads / 32][CPL * 32];
-    __shared__ double ssw[kPassThreads / 32];
-    if (st->done) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float pr[CPL], q[CPL];
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-        const int j = lane + 32 * c;
-        pr[c] = j < d ? p[j] : 0.f;
-        q[c] = 0.f;
-    }
-    const float ab = (st->beta > 0.0) ? (float)(st->alpha / st->beta) : 0.f;
-    double ss = 0.0;
-    const int64_t nw = (int64_t)gridDim.x * (kPassThreads / 32);
-    for (int64_t i0 = ((int64_t)blockIdx.x * (kPassThreads / 32) + w) * RB; i0 < n; i0 += nw * RB) {
-        float a[RB][CPL];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            const int64_t row = i0 + r;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                const int j = lane + 32 * c;
-                a[r][c] = (row < n && j < d) ? __ldg(A + row * lda + j) : 0.f;
-            }
-        }
-        const float uold = (lane < RB && i0 + lane < n) ? u[i0 + lane] : 0.f;
-        float dot[RB];
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            float t = 0.f;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) t = fmaf(a[r][c], pr[c], t);
-            dot[r] = t;
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1)
-#pragma unroll
-            for (int r = 0; r < RB; ++r) dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], o);
-        float unew = 0.f;
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            const float ui = (i0 + r < n) ? dot[r] - ab * __shfl_sync(0xffffffffu, uold, r) : 0.f;
-            if (lane == r) unew = ui;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) q[c] = fmaf(a[r][c], ui, q[c]);
-        }
-        if (lane < RB && i0 + lane < n) {
-            u[i0 + lane] = unew;
-            ss = fma((double)unew, (double)unew, ss);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) qs[w][lane + 32 * c] = q[c];
-    ss = warp_sum(ss);
-    if (lane == 0) ssw[w] = ss;
-    __syncthreads();
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        float t = 0.f;
-#pragma unroll
-        for (int z = 0; z < kPassThreads / 32; ++z) t += qs[z][j];
-        qpart[(int64_t)blockIdx.x * d + j] = t;
-    }
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int z = 0; z < kPassThreads / 32; ++z) t += ssw[z];
-        sspart[blockIdx.x] = t;
-    }
-}
-
-// u <- A p - (alpha/beta) u; partial sums of u^2 and of A^T u.  Dense, any d:
-// warp per row.
-__global__ void __launch_bounds__(kPassThreads) lsqr_pass_dense_kernel(
-    const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ p,
-    const LsqrState* __restrict__ st, float* __restrict__ u, float* __restrict__ qpart,
-    double* __restrict__ sspart) {
+    const CgState* __restrict__ st, float* __restrict__ qpart, double* __restrict__ sspart) {
     extern __shared__ float shf[];   // p (d) then per-warp q (8 * d)
-    if (st->done) return;
+    pdl_wait();
+    pdl_launch_next();
+    if (__ldcg(&st->done)) return;
     float* ps = shf;
     float* qs = shf + d;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) ps[j] = p[j];
+    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) ps[j] = __ldcg(p + j);
     for (int64_t j = threadIdx.x; j < 8 * d; j += blockDim.x) qs[j] = 0.f;
     __syncthreads();
-    const float ab = (st->beta > 0.0) ? (float)(st->alpha / st->beta) : 0.f;
     float* qw = qs + w * d;
     double ss = 0.0;
     const int64_t wid = (int64_t)blockIdx.x * 8 + w, nw = (int64_t)gridDim.x * 8;
@@ -252,9 +682,7 @@ __global__ void __launch_bounds__(kPassThreads) lsqr_pass_dense_kernel(
         float dot = 0.f;
         for (int64_t j = lane; j < d; j += 32) dot = fmaf(row[j], ps[j], dot);
         dot = warp_sum(dot);
-        const float ui = dot - ab * u[i];
-        __syncwarp();
-        if (lane == 0) u[i] = ui;
+        const float ui = dot;
         ss = fma((double)ui, (double)ui, ss);
         for (int64_t j = lane; j < d; j += 32) qw[j] = fmaf(row[j], ui, qw[j]);
     }
@@ -274,239 +702,347 @@ __global__ void __launch_bounds__(kPassThreads) lsqr_pass_dense_kernel(
     }
 }
 
-__global__ void __launch_bounds__(kPassThreads) lsqr_pass_csr_kernel(
-    const float* __restrict__ V, const int32_t* __restrict__ J, const int64_t* __restrict__ I,
-    int64_t n, int64_t nnz, int64_t d, const float* __restrict__ p, const LsqrState* __restrict__ st,
-    float* __restrict__ u, float* __restrict__ qpart, double* __restrict__ sspart) {
-    extern __shared__ float shf[];
-    if (st->done) return;
-    float* ps = shf;
-    float* qs = shf + d;
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        ps[j] = p[j];
-        qs[j] = 0.f;
-    }
-    __syncthreads();
-    const float ab = (st->beta > 0.0) ? (float)(st->alpha / st->beta) : 0.f;
-    double ss = 0.0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int64_t k0 = I[i], k1 = I[i + 1];
-        const bool ok = !(k0 < 0 || k1 < k0 || k1 > nnz);
-        float dot = 0.f;
-        if (ok)
-            for (int64_t q = k0; q < k1; ++q) {
-                const int32_t j = J[q];
-                if (j >= 0 && j < d) dot = fmaf(V[q], ps[j], dot);
-            }
-        const float ui = dot - ab * u[i];
-        u[i] = ui;
-        ss = fma((double)ui, (double)ui, ss);
-        if (ok)
-            for (int64_t q = k0; q < k1; ++q) {
-                const int32_t j = J[q];
-                if (j >= 0 && j < d) atomicAdd(&qs[j], V[q] * ui);
-            }
-    }
-    ss = warp_sum(ss);
-    __shared__ double ssw[kPassThreads / 32];
-    if ((threadIdx.x & 31) == 0) ssw[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) qpart[(int64_t)blockIdx.x * d + j] = qs[j];
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < kPassThreads / 32; ++t) s += ssw[t];
-        sspart[blockIdx.x] = s;
-    }
-}
-
 // ---- inner solve: CG on the preconditioned normal equations ----------------
 // N^T A^T A N z = g with g = N^T A^T r formed in FP64 by the residual pass.
-// The pass kernels run with alpha = 0 (u = A p): u = A N p_cg, A^T u and
-// ||u||^2 in FP32 / FP64; the d-vectors (z, s, p_cg) stay in FP64.  Unlike
-// LSQR on min ||A N y - r||, whose FP32 n-vectors carry r itself (mostly
-// orthogonal to range(A) when the residual is large), every FP32 quantity
-// here is relative to the correction being sought, so each refinement step
-// gains ~inner_tol whatever the size of the residual.
+// The pass kernels form u = A N p_cg, A^T u and ||u||^2 in FP32 / pairs; the
+// d-vectors (z, s, p_cg) stay in FP64.  Unlike LSQR on min ||A N y - r||,
+// whose FP32 n-vectors carry r itself (mostly orthogonal to range(A) when the
+// residual is large), every FP32 quantity here is relative to the correction
+// being sought, so each refinement step gains ~inner_tol whatever the size of
+// the residual.
+//
+// The work between two passes -- sum the blocks' partials, w = N^T (A^T u),
+// z += a p_cg, s -= a w, p_cg = s + b p_cg, p = N p_cg -- is a chain of two
+// d x d products and two dot products.  One block took 84 us for it at d = 128
+// (FP64 issues at 2 lanes a cycle per SM, and its reads of N were serial),
+// twice the pass itself.  Here a cluster of 16 CTAs runs it in one launch:
+// for d <= 256 every warp owns one row of N^T and one of N, as FP32 pairs
+// in registers before anything is waited for (with FP64 products each of the
+// two took 4,800 of the step's 25,000 cycles at d = 256), one more warp a CTA
+// does the scalars, and the two vectors that each step needs whole are
+// exchanged through distributed shared memory: 9 us a step.  d > 256 reads N
+// from L2 in FP64.
+// kStart: the residual pass's FP64 partials, eta and the start of a solve.
+constexpr int kVecCtas = 16, kVecThreads = 512, kVecWarps = kVecCtas * kVecThreads / 32;
+constexpr int kVecBlock = kVecThreads + 32;   // one more warp for the scalars
 
-// p = N v for an FP64 d-vector staged in shared memory (N upper triangular):
-// one warp per row of N, so consecutive lanes read consecutive entries
-__device__ __forceinline__ void apply_n(const double* __restrict__ N64, int64_t d, const double* vs, float* p) {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int64_t i = threadIdx.x >> 5; i < d; i += nw) {
-        double t = 0.0;
-        for (int64_t j = i + lane; j < d; j += 32) t = fma(N64[i * d + j], vs[j], t);
-        t = warp_sum(t);
+// the lane's eight entries of a row of N (or N^T) times v, summed over the warp
+__device__ __forceinline__ double row_dot(const float2 (&n)[8], const float2* v, int d, int lane, int c_lo, int c_hi) {
+    float h = 0.f, l = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        if (c >= c_lo && c <= c_hi) {
+            const float2 x = v[min(lane + 32 * c, d - 1)];
+            l = fmaf(n[c].y, x.x, l);
+            pair_fma(h, l, n[c].x, x.x, x.y);
+        }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) pair_add(h, l, __shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+    return (double)h + (double)l;
+}
+
+template <bool kStart>
+__global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __restrict__ part_, const double* __restrict__ sspart,
+                                                           int nblocks, int d, const double* __restrict__ N,
+                                                           const double* __restrict__ Nt, const float2* __restrict__ N2,
+                                                           const float2* __restrict__ Nt2, int first, double inner_tol,
+                                                           CgState* st, double* __restrict__ s, double* __restrict__ pc,
+                                                           double* __restrict__ z, float* __restrict__ p) {
+    using T = typename std::conditional<kStart, double, float>::type;
+    const T* part = reinterpret_cast<const T*>(part_);
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double qv[1024], sv[1024], pv[1024];
+    __shared__ float2 v2[256];      // the vector being multiplied, as pairs (d <= 256)
+    __shared__ T red[kVecThreads];
+    __shared__ double gv[kVecCtas]; // the CTAs' shares of ||u||^2
+    __shared__ double sc[4];        // step length, ||s||^2, beta
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, cta = (int)cl.block_rank();
+    const bool scalar_warp = tid >= kVecThreads, small = d <= kVecWarps;
+    const int gw = scalar_warp ? d : w * kVecCtas + cta;   // rows gw, gw + 256, ... of N^T and N
+    float2 nt[8], nn[8];
+    if (small && gw < d) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int i = lane + 32 * c;
+            nt[c] = i <= gw ? __ldg(Nt2 + gw * d + i) : make_float2(0.f, 0.f);
+            nn[c] = (i >= gw && i < d) ? __ldg(N2 + gw * d + i) : make_float2(0.f, 0.f);
+        }
+    }
+    pdl_wait();
+    pdl_launch_next();
+    // everything the pass and the previous step left is loaded at once
+    const int done = kStart ? 0 : __ldcg(&st->done);
+    const double rho = kStart ? 0.0 : __ldcg(&st->rho);
+    // the partials of this CTA's columns: ng threads a column, then a tree
+    const int cpc = (d + kVecCtas - 1) / kVecCtas, j0 = cta * cpc, nc = max(0, min(cpc, d - j0));
+    int ng = 1;
+    while (2 * ng * cpc <= kVecThreads) ng *= 2;
+    const int col = tid % cpc, grp = tid / cpc;
+    T acc = 0;
+    double zj = 0.0, sj = 0.0, pj = 0.0;   // d <= 256: this warp's entry
+    double g = 0.0;
+    if (!scalar_warp) {
+        if (grp < ng && col < nc) {
+            const T* src = part + j0 + col;
+            for (int q = grp; q < nblocks; q += 10 * ng) {   // ten loads in flight
+                T v[10];
+#pragma unroll
+                for (int k = 0; k < 10; ++k) v[k] = q + k * ng < nblocks ? __ldcg(src + (int64_t)(q + k * ng) * d) : (T)0;
+#pragma unroll
+                for (int k = 0; k < 10; ++k) acc += v[k];
+            }
+        }
+        if (!kStart) {
+            for (int j = tid; j < d; j += kVecThreads) pv[j] = __ldcg(pc + j);
+            if (small && gw < d) {
+                zj = __ldcg(z + gw);
+                sj = __ldcg(s + gw);
+                pj = __ldcg(pc + gw);
+            }
+        }
+        red[tid] = acc;
+    } else if (!kStart) {
+        for (int q = cta + kVecCtas * lane; q < nblocks; q += kVecCtas * 32) g += __ldcg(sspart + q);
+        g = warp_sum(g);
+        if (lane < kVecCtas) cl.map_shared_rank(gv, lane)[cta] = g;
+    }
+    __syncthreads();
+    for (int m = ng >> 1; m; m >>= 1) {
+        if (grp < m) red[tid] += red[tid + m * cpc];
+        __syncthreads();
+    }
+    for (int e = tid; e < nc * kVecCtas; e += kVecBlock)
+        cl.map_shared_rank(qv, e / nc)[j0 + e % nc] = (double)red[e % nc];
+    cl.sync();   // qv = A^T u (or A^T r) and gv in every CTA
+    if (done) return;   // the same in every CTA: written only after the second cluster barrier
+    if (small) {
+        if (tid < d) v2[tid] = to_pair(qv[tid]);
+        __syncthreads();
+    }
+    double t = 0.0;
+    if (scalar_warp) {
+        if (!kStart) {
+            double G = lane < kVecCtas ? gv[lane] : 0.0;
+            G = warp_sum(G);
+            if (lane == 0) sc[0] = G > 0.0 ? rho / G : 0.0;
+        } else if (cta == 0) {   // eta = ||A^T r|| / ||A^T b||
+            double a2 = 0.0;
+            for (int j = lane; j < d; j += 32) a2 = fma(qv[j], qv[j], a2);
+            a2 = warp_sum(a2);
+            if (lane == 0) {
+                const double atrn = sqrt(a2), atb = first ? atrn : st->atb_norm;
+                st->atb_norm = atb;
+                st->eta = atb > 0.0 ? atrn / atb : 0.0;
+            }
+        }
+    } else if (small && gw < d) {
+        t = row_dot(nt, v2, d, lane, 0, gw >> 5);   // (N^T q)_gw
+    }
+    __syncthreads();
+    const double a = kStart ? 0.0 : sc[0];
+    if (!scalar_warp)
+        for (int j = gw; j < d; j += kVecWarps) {
+            if (!small) {
+                t = 0.0;
+                for (int i = lane; i <= j; i += 32) t = fma(Nt[(int64_t)j * d + i], qv[i], t);
+                t = warp_sum(t);
+                if (!kStart) {
+                    zj = __ldcg(z + j);
+                    sj = __ldcg(s + j);
+                    pj = pv[j];
+                }
+            }
+            const double snew = kStart ? t : fma(-a, t, sj);
+            if (lane == 0) {
+                s[j] = snew;
+                z[j] = kStart ? 0.0 : fma(a, pj, zj);
+            }
+            if (lane < kVecCtas) cl.map_shared_rank(sv, lane)[j] = snew;
+        }
+    cl.sync();   // sv = the new s in every CTA
+    if (scalar_warp) {
+        double r2 = 0.0;
+        for (int j = lane; j < d; j += 32) r2 = fma(sv[j], sv[j], r2);
+        r2 = warp_sum(r2);
+        if (lane == 0) {
+            sc[2] = (!kStart && rho > 0.0) ? r2 / rho : 0.0;
+            if (cta == 0) {
+                st->rho = r2;
+                if (kStart) {
+                    st->rho0 = r2;
+                    st->it = 0;
+                    st->done = r2 == 0.0 ? 1 : 0;
+                } else {
+                    st->it += 1;
+                    if (a == 0.0 || r2 <= inner_tol * inner_tol * st->rho0) st->done = 1;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const double bta = sc[2];
+    for (int j = tid; j < d; j += kVecBlock) {
+        const double v = kStart ? sv[j] : fma(bta, pv[j], sv[j]);
+        pv[j] = v;
+        if (small) v2[j] = to_pair(v);
+        if (cta == 0) pc[j] = v;
+    }
+    __syncthreads();
+    if (scalar_warp) return;
+    for (int i = gw; i < d; i += kVecWarps) {   // p = N p_cg
+        if (small) {
+            t = row_dot(nn, v2, d, lane, gw >> 5, (d - 1) >> 5);
+        } else {
+            t = 0.0;
+            for (int j = i + lane; j < d; j += 32) t = fma(N[(int64_t)i * d + j], pv[j], t);
+            t = warp_sum(t);
+        }
         if (lane == 0) p[i] = (float)t;
     }
 }
 
-// Start of an inner solve after the residual pass: A^T r, eta,
-// g = N^T A^T r, s = p_cg = g, z = 0, p = N p_cg.  One block.
-__global__ void cg_start_kernel(const double* __restrict__ qpart, int nblocks, int64_t d,
-                                const double* __restrict__ N64, int first, LsqrState* st,
-                                double* __restrict__ s, double* __restrict__ pc, double* __restrict__ z,
-                                double* __restrict__ atr, float* __restrict__ p) {
-    __shared__ double red[32];
-    __shared__ double pcs[1024];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        double t = 0.0;
-        for (int q = 0; q < nblocks; ++q) t += qpart[(int64_t)q * d + j];
-        atr[j] = t;
-    }
-    __syncthreads();
-    double a2 = 0.0, g2 = 0.0;
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        a2 = fma(atr[j], atr[j], a2);
-        double t = 0.0;
-        for (int64_t i = 0; i <= j; ++i) t = fma(N64[i * d + j], atr[i], t);   // (N^T A^T r)_j
-        s[j] = t;
-        pc[j] = t;
-        pcs[j] = t;
-        z[j] = 0.0;
-        g2 = fma(t, t, g2);
-    }
-    a2 = warp_sum(a2);
-    g2 = warp_sum(g2);
-    if (lane == 0) {
-        red[wid] = a2;
-        red[16 + wid] = g2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double A2 = 0.0, G2 = 0.0;
-        for (int t = 0; t < nw; ++t) {
-            A2 += red[t];
-            G2 += red[16 + t];
+// N^T, and both as pairs for d <= 256 (converting them in every step would
+// cost more FP64-pipe cycles than the products)
+__global__ void __launch_bounds__(256) factor_forms_kernel(const double* __restrict__ N, int d, double* __restrict__ Nt,
+                                                           float2* __restrict__ N2, float2* __restrict__ Nt2) {
+    __shared__ double tile[32][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5, i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+    for (int k = y; k < 32; k += 8)
+        if (i0 + k < d && j0 + x < d) {
+            const double v = N[(int64_t)(i0 + k) * d + j0 + x];
+            tile[k][x] = v;
+            if (N2) N2[(i0 + k) * d + j0 + x] = to_pair(v);
         }
-        const double atrn = sqrt(A2);
-        if (first) st->atb_norm = atrn;
-        st->eta = (st->atb_norm > 0.0) ? atrn / st->atb_norm : 0.0;
-        st->alpha = 0.0;           // the pass forms u = A p
-        st->beta = 1.0;
-        st->rho = G2;
-        st->rho0 = G2;
-        st->it = 0;
-        st->done = (G2 == 0.0) ? 1 : 0;
-    }
     __syncthreads();
-    apply_n(N64, d, pcs, p);
+    for (int k = y; k < 32; k += 8)
+        if (j0 + k < d && i0 + x < d) {
+            const double v = tile[x][k];
+            if (Nt2) Nt2[(j0 + k) * d + i0 + x] = to_pair(v);
+            else Nt[(int64_t)(j0 + k) * d + i0 + x] = v;
+        }
 }
 
-// One CG step after the pass: gamma = ||A N p_cg||^2, w = N^T (A^T u),
-// z += a p_cg, s -= a w, p_cg = s + b p_cg, p = N p_cg.  One block.
-__global__ void cg_step_kernel(const float* __restrict__ qpart, const double* __restrict__ sspart, int nblocks,
-                               int64_t d, const double* __restrict__ N64, LsqrState* st, double* __restrict__ s,
-                               double* __restrict__ pc, double* __restrict__ z, float* __restrict__ qtmp,
-                               double inner_tol, float* __restrict__ p) {
-    __shared__ double red[32];
-    __shared__ double sc[2];
-    __shared__ double pcs[1024];
-    if (st->done) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double g2 = 0.0;
-    for (int q = threadIdx.x; q < nblocks; q += blockDim.x) g2 += sspart[q];
-    g2 = warp_sum(g2);
-    if (lane == 0) red[wid] = g2;
-    reduce_partials(qpart, nblocks, d, qtmp);   // A^T u
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double G = 0.0;
-        for (int t = 0; t < nw; ++t) G += red[t];
-        sc[0] = (G > 0.0) ? st->rho / G : 0.0;   // step length
-    }
-    __syncthreads();
-    const double a = sc[0];
-    double r2 = 0.0;
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        double w = 0.0;
-        for (int64_t i = 0; i <= j; ++i) w = fma(N64[i * d + j], (double)qtmp[i], w);   // (N^T A^T u)_j
-        z[j] = fma(a, pc[j], z[j]);
-        const double sj = fma(-a, w, s[j]);
-        s[j] = sj;
-        r2 = fma(sj, sj, r2);
-    }
-    r2 = warp_sum(r2);
-    __syncthreads();
-    if (lane == 0) red[wid] = r2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double R2 = 0.0;
-        for (int t = 0; t < nw; ++t) R2 += red[t];
-        sc[1] = (st->rho > 0.0) ? R2 / st->rho : 0.0;
-        st->rho = R2;
-        st->it += 1;
-        if (a == 0.0 || R2 <= inner_tol * inner_tol * st->rho0) st->done = 1;
-    }
-    __syncthreads();
-    if (st->done) return;
-    const double bta = sc[1];
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) {
-        const double v = fma(bta, pc[j], s[j]);
-        pc[j] = v;
-        pcs[j] = v;
-    }
-    __syncthreads();
-    apply_n(N64, d, pcs, p);
+// x <- x + N y (FP64), one warp a row.
+__global__ void __launch_bounds__(256) update_x_kernel(const double* __restrict__ N64, int64_t d,
+                                                       const double* __restrict__ y, double* __restrict__ x) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= d) return;
+    double s = 0.0;
+    for (int64_t j = i + lane; j < d; j += 32) s = fma(N64[i * d + j], y[j], s);
+    s = warp_sum(s);
+    if (lane == 0) x[i] += s;
 }
 
-// x <- x + N y (FP64).  One block.
-__global__ void update_x_kernel(const double* __restrict__ N64, int64_t d, const double* __restrict__ y,
-                                double* __restrict__ x) {
-    __shared__ double ys[1024];
-    for (int64_t j = threadIdx.x; j < d; j += blockDim.x) ys[j] = y[j];
-    __syncthreads();
-    for (int64_t i = threadIdx.x; i < d; i += blockDim.x) {
-        double s = 0.0;
-        for (int64_t j = i; j < d; ++j) s = fma(N64[i * d + j], ys[j], s);
-        x[i] += s;
-    }
+template <bool kStart>
+cudaError_t launch_vec(const void* part, const double* sspart, int nblocks, int64_t d, const double* N, const double* Nt,
+                       const float2* N2, const float2* Nt2, int first, double inner_tol, CgState* S, double* s, double* pc, double* z, float* p,
+                       cudaStream_t st) {
+    // 16 CTAs a cluster is above the portable 8: opt in (idempotent, the same value always)
+    cudaError_t e = cudaFuncSetAttribute(cg_vec_kernel<kStart>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    LSK_PROF("lsq_small", st) e = launch_pdl(cg_vec_kernel<kStart>, kVecCtas, kVecBlock, 0, kVecCtas, st, part, sspart,
+                                             nblocks, (int)d, N, Nt, N2, Nt2, first, inner_tol, S, s, pc, z, p);
+    return e;
 }
 
 constexpr int kMaxPassBlocks = 2432;   // >= 8 x the SM count of any sm_103 part
 
-// Blocks of a pass over A: enough to keep every SM streaming, few enough
-// that each block covers several row groups (fewer partials to reduce).
+// Blocks of a pass over A: two per SM of the d <= 256 kernels are resident, and
+// fewer blocks leave fewer partials to sum; each covers two row groups or more.
 int pass_grid(const lsk_mat* A, int sm_count) {
     const int64_t n = A->n;
     const bool rows_kernel = A->kind == LSK_DENSE && A->d <= 256;
-    const int64_t per_block = rows_kernel ? (kPassThreads / 32) * (A->d <= 64 ? 16 : 8) * 2 : kPassThreads * 2;
+    const int64_t per_block = rows_kernel ? (kPassThreads / 32) * (A->d <= 32 ? 32 : A->d <= 64 ? 16 : 8) * 2 : kPassThreads * 2;
     int64_t g = (n + per_block - 1) / per_block;
-    const int64_t cap = std::min<int64_t>(rows_kernel ? 4 * sm_count : 8 * sm_count, kMaxPassBlocks);
+    const int64_t cap = std::min<int64_t>(rows_kernel ? 2 * sm_count : 8 * sm_count, kMaxPassBlocks);
     if (g > cap) g = cap;
     if (g < 1) g = 1;
     return (int)g;
 }
 
-template <int CPL, int RB>
-void launch_rows_pass(const lsk_mat* A, int nb, const float* p, const LsqrState* S, float* u, float* qpart,
+template <int L, int E, int RB, bool kVec>
+void launch_rows_pass(const lsk_mat* A, int nb, const float* p, const CgState* S, int rev, float* qpart,
                       double* sspart, cudaStream_t st) {
-    LSK_PROF("lsq_pass", st) lsqr_pass_dense_rows_kernel<CPL, RB><<<nb, kPassThreads, 0, st>>>(
-        (const float*)A->values, A->ld, A->n, A->d, p, S, u, qpart, sspart);
+    LSK_PROF("lsq_pass", st) launch_pdl(cg_pass_dense_rows_kernel<L, E, RB, kVec>, nb, kPassThreads, 0, 1, st,
+                                        (const float*)A->values, A->ld, A->n, (int)A->d, p, S, rev, qpart, sspart);
 }
 
-void lsqr_pass(const lsk_mat* A, int nb, size_t sh32, const float* p, const LsqrState* S, float* u,
-               float* qpart, double* sspart, cudaStream_t st) {
-    const int64_t n = A->n, d = A->d;
-    if (A->kind == LSK_DENSE && d <= 256) {
-        switch ((d + 31) / 32) {
-            case 1: launch_rows_pass<1, 16>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 2: launch_rows_pass<2, 16>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 3: launch_rows_pass<3, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 4: launch_rows_pass<4, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 5: launch_rows_pass<5, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 6: launch_rows_pass<6, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-            case 7: launch_rows_pass<7, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-            default: launch_rows_pass<8, 8>(A, nb, p, S, u, qpart, sspart, st); break;
-        }
-    } else if (A->kind == LSK_DENSE) {
-        LSK_PROF("lsq_pass", st) lsqr_pass_dense_kernel<<<nb, kPassThreads, sh32, st>>>(
-            (const float*)A->values, A->ld, n, d, p, S, u, qpart, sspart);
+// 16-byte loads of whole rows: d and ld multiples of 4, values 16-byte aligned
+bool rows_vec4(const lsk_mat* A) {
+    return A->d % 4 == 0 && A->ld % 4 == 0 && (reinterpret_cast<uintptr_t>(A->values) & 15) == 0;
+}
+
+void cg_pass_dense(const lsk_mat* A, int nb, const float* p, const CgState* S, int rev, float* qpart, double* sspart,
+                   cudaStream_t st) {
+    const int64_t d = A->d;
+    if (d > 256)
+        LSK_PROF("lsq_pass", st) launch_pdl(cg_pass_dense_kernel, nb, kPassThreads, (size_t)9 * d * 4, 1, st,
+                                            (const float*)A->values, A->ld, A->n, d, p, S, qpart, sspart);
+    else if (rows_vec4(A)) {
+        if (d <= 32) launch_rows_pass<8, 4, 8, true>(A, nb, p, S, rev, qpart, sspart, st);
+        else if (d <= 64) launch_rows_pass<16, 4, 8, true>(A, nb, p, S, rev, qpart, sspart, st);
+        else if (d <= 128) launch_rows_pass<32, 4, 8, true>(A, nb, p, S, rev, qpart, sspart, st);
+        else launch_rows_pass<32, 8, 4, true>(A, nb, p, S, rev, qpart, sspart, st);
     } else {
-        LSK_PROF("lsq_pass", st) lsqr_pass_csr_kernel<<<nb, kPassThreads, sh32, st>>>(
-            (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, p, S, u, qpart, sspart);
+        if (d <= 32) launch_rows_pass<32, 1, 16, false>(A, nb, p, S, rev, qpart, sspart, st);
+        else if (d <= 64) launch_rows_pass<32, 2, 16, false>(A, nb, p, S, rev, qpart, sspart, st);
+        else if (d <= 128) launch_rows_pass<32, 4, 8, false>(A, nb, p, S, rev, qpart, sspart, st);
+        else launch_rows_pass<32, 8, 4, false>(A, nb, p, S, rev, qpart, sspart, st);
     }
+}
+
+template <int L, int E, int RB, bool kVec>
+void launch_resid(const lsk_mat* A, int nb, const double* b, const double* x, double* qpart, cudaStream_t st) {
+    LSK_PROF("lsq_resid64", st) resid_dense_rows_kernel<L, E, RB, kVec><<<nb, kPassThreads, 0, st>>>(
+        (const float*)A->values, A->ld, A->n, (int)A->d, b, x, qpart);
+}
+
+// dense b - A x and the blocks' partial sums of A^T (b - A x)
+cudaError_t resid_dense(const lsk_mat* A, int nb, const double* b, const double* x, double* qpart, cudaStream_t st) {
+    const int64_t d = A->d;
+    if (d > 256) {
+        const size_t sh = (size_t)9 * d * 8;
+        if (sh > 48 * 1024) {
+            const cudaError_t e = allow_dynamic_smem(resid64_dense_kernel);
+            if (e != cudaSuccess) return e;
+        }
+        LSK_PROF("lsq_resid64", st) resid64_dense_kernel<<<nb, kPassThreads, sh, st>>>((const float*)A->values, A->ld,
+                                                                                       A->n, d, b, x, qpart);
+    } else if (rows_vec4(A)) {
+        if (d <= 32) launch_resid<8, 4, 4, true>(A, nb, b, x, qpart, st);
+        else if (d <= 64) launch_resid<16, 4, 4, true>(A, nb, b, x, qpart, st);
+        else if (d <= 128) launch_resid<32, 4, 8, true>(A, nb, b, x, qpart, st);
+        else launch_resid<32, 8, 4, true>(A, nb, b, x, qpart, st);
+    } else {
+        if (d <= 32) launch_resid<32, 1, 8, false>(A, nb, b, x, qpart, st);
+        else if (d <= 64) launch_resid<32, 2, 8, false>(A, nb, b, x, qpart, st);
+        else if (d <= 128) launch_resid<32, 4, 4, false>(A, nb, b, x, qpart, st);
+        else launch_resid<32, 8, 4, false>(A, nb, b, x, qpart, st);
+    }
+    return cudaGetLastError();
+}
+
+// ---- CSR tiles: plan, workspace ----------------------------------------------
+CsrTiles tiles_plan(const lsk_mat* A, int sm_count) {
+    CsrTiles t{};
+    t.n = A->n;
+    t.d = A->d;
+    int64_t rp = (A->n + kTilesPerSm * (int64_t)sm_count - 1) / (kTilesPerSm * (int64_t)sm_count);
+    rp = std::max<int64_t>(32, std::min<int64_t>(rp, kTileRowsMax));
+    t.rows_per = (int)rp;
+    t.ntiles = (A->n + rp - 1) / rp;
+    t.V = (const float*)A->values;
+    t.J = A->colidx;
+    t.I = A->rowptr;
+    return t;
+}
+size_t tiles_smem(const CsrTiles& t, size_t elem) {
+    return (kTileEntries + 2 * (size_t)t.d + t.rows_per) * elem + (t.rows_per + t.d + 2) * 4 + 16;
+}
+size_t tiles_bytes(const lsk_mat* A, int sm_count) {
+    const CsrTiles t = tiles_plan(A, sm_count);
+    return ws_round((size_t)t.ntiles * (t.d + 1) * 4) + ws_round((size_t)A->nnz * 4) + ws_round((size_t)A->nnz * 2);
 }
 
 }  // namespace
@@ -525,8 +1061,7 @@ __global__ void sum_qpart_kernel(const double* __restrict__ qpart, int nblocks, 
 
 size_t atr64_workspace_bytes(const lsk_mat* A) {
     const int nb = kMaxPassBlocks;
-    return ws_round((size_t)(A->n > 0 ? A->n : 1) * 4) + ws_round((size_t)nb * A->d * 8) + ws_round((size_t)nb * 8) +
-           ws_round((size_t)A->d * 8) + 1024;
+    return ws_round((size_t)nb * A->d * 8) + ws_round((size_t)A->d * 8) + 1024;
 }
 
 cudaError_t atr64_launch(const lsk_mat* A, const double* b, const double* x, double* atr, void* ws, int* flag,
@@ -534,116 +1069,167 @@ cudaError_t atr64_launch(const lsk_mat* A, const double* b, const double* x, dou
     const int64_t n = A->n, d = A->d;
     const int nb = pass_grid(A, sm_count);
     WsCarver wc{(char*)ws, 0};
-    float* u = wc.take<float>(n > 0 ? n : 1);
     double* qpart = wc.take<double>((size_t)nb * d);
-    double* sspart = wc.take<double>(nb);
     double* zero = wc.take<double>(d);
     cudaError_t e = cudaSuccess;
     if (!x) {
         if ((e = cudaMemsetAsync(zero, 0, (size_t)d * 8, st)) != cudaSuccess) return e;
         x = zero;
     }
-    const bool dense = A->kind == LSK_DENSE;
-    const size_t sh64 = dense ? (size_t)9 * d * 8 : (size_t)2 * d * 8;
-    if (sh64 > 48 * 1024) {
-        if ((e = allow_dynamic_smem(resid64_dense_kernel)) != cudaSuccess) return e;
-        if ((e = allow_dynamic_smem(resid64_csr_kernel)) != cudaSuccess) return e;
+    if (A->kind == LSK_DENSE) {
+        if ((e = resid_dense(A, nb, b, x, qpart, st)) != cudaSuccess) return e;
+    } else {
+        const size_t sh = (size_t)2 * d * 8;
+        if (sh > 48 * 1024 && (e = allow_dynamic_smem(resid64_csr_kernel)) != cudaSuccess) return e;
+        LSK_PROF("lsq_resid64", st) resid64_csr_kernel<<<nb, kPassThreads, sh, st>>>(
+            (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, b, x, qpart, flag);
     }
-    if (dense)
-        LSK_PROF("lsq_resid64", st) resid64_dense_kernel<<<nb, kPassThreads, sh64, st>>>((const float*)A->values, A->ld, n, d, b, x,
-                                                                                          u, qpart, sspart);
-    else
-        LSK_PROF("lsq_resid64", st) resid64_csr_kernel<<<nb, kPassThreads, sh64, st>>>((const float*)A->values, A->colidx, A->rowptr,
-                                                                                        n, A->nnz, d, b, x, u, qpart, sspart, flag);
     LSK_PROF("lsq_small", st) sum_qpart_kernel<<<(unsigned)((d + 255) / 256), 256, 0, st>>>(qpart, nb, d, atr);
     return cudaGetLastError();
 }
 
-size_t lsq_workspace_bytes(const lsk_mat* A) {
-    const int64_t n = A->n, d = A->d;
+// Pinned copies of the solver's state for the lagged stopping test.
+struct LsqHost {
+    CgState* state;       // two, pinned
+    cudaEvent_t ev[2];
+    cudaError_t read(int slot, const CgState* S, cudaStream_t st) {
+        const cudaError_t e = cudaMemcpyAsync(state + slot, S, sizeof(CgState), cudaMemcpyDeviceToHost, st);
+        return e != cudaSuccess ? e : cudaEventRecord(ev[slot], st);
+    }
+    cudaError_t wait(int slot) { return cudaEventSynchronize(ev[slot]); }
+};
+
+void lsq_host_free(lsk_ctx* ctx) {
+    LsqHost* h = ctx->lsq_host;
+    if (!h) return;
+    for (cudaEvent_t ev : h->ev)
+        if (ev) cudaEventDestroy(ev);
+    if (h->state) cudaFreeHost(h->state);
+    delete h;
+    ctx->lsq_host = nullptr;
+}
+
+namespace {
+LsqHost* lsq_host(lsk_ctx* ctx) {
+    if (ctx->lsq_host) return ctx->lsq_host;
+    ctx->lsq_host = new (std::nothrow) LsqHost();
+    LsqHost* h = ctx->lsq_host;
+    if (!h) return nullptr;
+    if (cudaMallocHost(&h->state, 2 * sizeof(CgState)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&h->ev[1], cudaEventDisableTiming) != cudaSuccess) {
+        lsq_host_free(ctx);
+        return nullptr;
+    }
+    return h;
+}
+}  // namespace
+
+size_t lsq_workspace_bytes(const lsk_mat* A, int sm_count) {
+    const int64_t d = A->d;
     const int nb = kMaxPassBlocks;
-    return ws_round(sizeof(LsqrState)) + ws_round((size_t)n * 4) + 6 * ws_round((size_t)d * 8) +
-           ws_round((size_t)nb * d * 8) + ws_round((size_t)nb * 8) + 3 * ws_round((size_t)d * 4) +
-           ws_round((size_t)2 * d * 4) + 4096;
+    return ws_round(sizeof(CgState)) + 4 * ws_round((size_t)d * 8) + 2 * ws_round((size_t)d * d * 8) +
+           ws_round((size_t)nb * d * 8) + ws_round((size_t)nb * 8) + ws_round((size_t)d * 4) +
+           (A->kind == LSK_CSR ? tiles_bytes(A, sm_count) : 0) + 4096;
 }
 
 int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const lsk_lsq_opts* o,
-            const double* Rinv64, const float* /* FP32 factor: not used, the inner solve runs on Rinv64 */,
-            void* ws, lsk_lsq_info* info) {
+            const double* Rinv64, void* ws, lsk_lsq_info* info) {
     cudaStream_t st = ctx->stream;
-    const int64_t n = A->n, d = A->d;
-    const int nb = pass_grid(A, ctx->sm_count);
+    const int64_t d = A->d;
+    const bool dense = A->kind == LSK_DENSE;
     WsCarver wc{(char*)ws, 0};
-    LsqrState* S = wc.take<LsqrState>(1);
-    float* u = wc.take<float>(n > 0 ? n : 1);
+    CgState* S = wc.take<CgState>(1);
     double* y = wc.take<double>(d);
-    double* atr = wc.take<double>(d);
-    double* qpart64 = wc.take<double>((size_t)nb * d);
-    double* sspart = wc.take<double>(nb);
-    float* p = wc.take<float>(d);
-    float* qtmp = wc.take<float>(2 * d);
     double* cg_s = wc.take<double>(d);
     double* cg_p = wc.take<double>(d);
+    double* Nt = wc.take<double>((size_t)d * d);
+    float2 *N2 = nullptr, *Nt2 = nullptr;
+    if (d <= kVecWarps) {
+        N2 = wc.take<float2>((size_t)d * d);
+        Nt2 = reinterpret_cast<float2*>(Nt);
+    }
+    double* qpart64 = wc.take<double>((size_t)kMaxPassBlocks * d);
+    double* sspart = wc.take<double>(kMaxPassBlocks);
+    float* p = wc.take<float>(d);
     float* qpart32 = reinterpret_cast<float*>(qpart64);   // reused by the FP32 pass
 
-    LsqrState h{};
+    CgState h{};
+    LsqHost* host = lsq_host(ctx);
+    if (!host) return LSK_ERR_CUDA;
     cudaError_t e = cudaMemsetAsync(x, 0, (size_t)d * 8, st);
     if (e != cudaSuccess) return LSK_ERR_CUDA;
-    const bool dense = A->kind == LSK_DENSE;
-    const size_t sh64 = dense ? (size_t)9 * d * 8 : (size_t)2 * d * 8;
-    const size_t sh32 = dense ? (size_t)9 * d * 4 : (size_t)2 * d * 4;
-    if (sh64 > 48 * 1024) {
-        if (allow_dynamic_smem(resid64_dense_kernel) != cudaSuccess ||
-            allow_dynamic_smem(resid64_csr_kernel) != cudaSuccess)
+    const dim3 tg((unsigned)((d + 31) / 32), (unsigned)((d + 31) / 32));
+    LSK_PROF("lsq_small", st) factor_forms_kernel<<<tg, 256, 0, st>>>(Rinv64, (int)d, Nt, N2, Nt2);
+    int nb = pass_grid(A, ctx->sm_count);
+    CsrTiles t{};
+    size_t sh32 = 0, sh64 = 0;
+    if (!dense) {
+        t = tiles_plan(A, ctx->sm_count);
+        t.cptr = wc.take<int32_t>((size_t)t.ntiles * (d + 1));
+        t.tval = wc.take<float>((size_t)A->nnz);
+        t.trow = wc.take<uint16_t>((size_t)A->nnz);
+        sh32 = tiles_smem(t, sizeof(float));
+        sh64 = tiles_smem(t, sizeof(float2));
+        if (allow_dynamic_smem(tile_pass_kernel<float>) != cudaSuccess ||
+            allow_dynamic_smem(tile_pass_kernel<float2>) != cudaSuccess)
             return LSK_ERR_CUDA;
-    }
-    if (sh32 > 48 * 1024) {
-        if (allow_dynamic_smem(lsqr_pass_dense_kernel) != cudaSuccess ||
-            allow_dynamic_smem(lsqr_pass_csr_kernel) != cudaSuccess)
-            return LSK_ERR_CUDA;
+        nb = (int)std::max<int64_t>(1, std::min<int64_t>(t.ntiles, kTilesPerSm * (int64_t)ctx->sm_count));
+        if (t.ntiles > 0)
+            LSK_PROF("lsq_tiles", st) csr_tiles_kernel<<<(unsigned)t.ntiles, kPassThreads, (size_t)d * 4, st>>>(t, A->nnz);
     }
     int total_it = 0, refinements = 0, status = LSK_ERR_NOT_CONVERGED;
     double eta = INFINITY;
-    for (int t = 0; t <= o->max_refine; ++t) {
-        if (dense)
-            LSK_PROF("lsq_resid64", st) resid64_dense_kernel<<<nb, kPassThreads, sh64, st>>>((const float*)A->values, A->ld, n, d, b, x, u,
-                                                                 qpart64, sspart);
-        else
-            LSK_PROF("lsq_resid64", st) resid64_csr_kernel<<<nb, kPassThreads, sh64, st>>>((const float*)A->values, A->colidx, A->rowptr, n,
-                                                               A->nnz, d, b, x, u, qpart64, sspart, ctx->flag);
-        LSK_PROF("lsq_small", st) cg_start_kernel<<<1, 256, 0, st>>>(qpart64, nb, d, Rinv64, t == 0 ? 1 : 0, S, cg_s, cg_p, y, atr, p);
+    for (int step = 0; step <= o->max_refine; ++step) {
+        if (dense) {
+            if (resid_dense(A, nb, b, x, qpart64, st) != cudaSuccess) return LSK_ERR_CUDA;
+        } else {
+            LSK_PROF("lsq_resid64", st) tile_pass_kernel<float2><<<nb, kPassThreads, sh64, st>>>(t, nullptr, x, b, S, qpart64, sspart);
+        }
+        if (launch_vec<true>(qpart64, sspart, nb, d, Rinv64, Nt, N2, Nt2, step == 0 ? 1 : 0, 0.0, S, cg_s, cg_p, y, p, st) != cudaSuccess)
+            return LSK_ERR_CUDA;
         e = cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return LSK_ERR_CUDA;
         eta = h.eta;
-        refinements = t;
+        refinements = step;
         if (!(eta > o->tol)) {
             status = LSK_OK;
             break;
         }
-        if (t == o->max_refine) break;
+        if (step == o->max_refine) break;
         // the inner solve need only reduce its residual by the factor left to
-        // reach tol (with a margin of 10), and never by less than inner_tol
-        double stop_rel = 0.1 * o->tol / eta;
+        // reach tol (with a margin of 20), and never by less than inner_tol
+        double stop_rel = 0.05 * o->tol / eta;
         if (stop_rel < o->inner_tol) stop_rel = o->inner_tol;
         if (stop_rel > 0.5) stop_rel = 0.5;
-        int it = 0;
-        while (!h.done && it < o->max_iter) {
-            lsqr_pass(A, nb, sh32, p, S, u, qpart32, sspart, st);
-            LSK_PROF("lsq_small", st) cg_step_kernel<<<1, 1024, 0, st>>>(qpart32, sspart, nb, d, Rinv64, S, cg_s, cg_p, y, qtmp,
-                                               stop_rel, p);
-            ++it;
-            if ((it & 3) == 0 || it >= o->max_iter) {   // stopping test every 4 iterations
-                e = cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-                if (e != cudaSuccess) return LSK_ERR_CUDA;
+        // The stopping test lags: iterations are queued four at a time with a
+        // copy of the state behind each four, and the host waits for the copy
+        // two batches back, so the GPU always has work queued (kernels queued
+        // past the end return at once).
+        int queued = 0;
+        for (int batch = 0; queued < o->max_iter; ++batch) {
+            if (batch >= 2) {
+                if ((e = host->wait(batch & 1)) != cudaSuccess) return LSK_ERR_CUDA;
+                if (host->state[batch & 1].done) break;
             }
+            for (int k = 0; k < 4 && queued < o->max_iter; ++k, ++queued) {
+                if (dense)
+                    cg_pass_dense(A, nb, p, S, queued & 1, qpart32, sspart, st);
+                else
+                    LSK_PROF("lsq_pass", st) launch_pdl(tile_pass_kernel<float>, nb, kPassThreads, sh32, 1, st, t, (const float*)p,
+                                                        (const double*)nullptr, (const double*)nullptr, (const CgState*)S,
+                                                        (void*)qpart32, sspart);
+                if (launch_vec<false>(qpart32, sspart, nb, d, Rinv64, Nt, N2, Nt2, 0, stop_rel, S, cg_s, cg_p, y, p, st) != cudaSuccess)
+                    return LSK_ERR_CUDA;
+            }
+            if ((e = host->read(batch & 1, S, st)) != cudaSuccess) return LSK_ERR_CUDA;
         }
         e = cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return LSK_ERR_CUDA;
         total_it += h.it;
-        LSK_PROF("lsq_small", st) update_x_kernel<<<1, 256, 0, st>>>(Rinv64, d, y, x);
+        LSK_PROF("lsq_small", st) update_x_kernel<<<(unsigned)((d + 7) / 8), 256, 0, st>>>(Rinv64, d, y, x);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return LSK_ERR_CUDA;
