@@ -33,7 +33,8 @@ __device__ __forceinline__ void tile_of(int t, int nt, int& ta, int& tb) {
 
 __global__ void __launch_bounds__(256) gram_dense_kernel(const float* __restrict__ A, int64_t lda,
                                                          int64_t n, int64_t d, int64_t rows_per,
-                                                         double* __restrict__ part) {
+                                                         double* __restrict__ part, const int* __restrict__ only_if) {
+    if (only_if && !*only_if) return;
     __shared__ __align__(16) float As[GK][GT];
     __shared__ __align__(16) float Bs[GK][GT];
     const int nt = (int)((d + GT - 1) / GT);
@@ -101,8 +102,10 @@ __global__ void __launch_bounds__(256) gram_dense_kernel(const float* __restrict
 template <typename OutT>
 __global__ void __launch_bounds__(256) gram_dense_reduce_kernel(const double* __restrict__ part, int64_t nchunks,
                                                                  int64_t d, double alpha, double beta,
-                                                                 OutT* __restrict__ C) {
+                                                                 OutT* __restrict__ C,
+                                                                 const int* __restrict__ only_if) {
     __shared__ double acc[8][33];
+    if (only_if && !*only_if) return;
     const int nt = (int)((d + GT - 1) / GT);
     const int ntiles = nt * (nt + 1) / 2;
     const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -268,7 +271,8 @@ CsrPlan csr_plan(int64_t n, int64_t d, int sm_count) {
 size_t gram_workspace_bytes(const lsk_mat* A, int sm_count) {
     if (A->kind == LSK_DENSE) {
         const DensePlan p = dense_plan(A->n, A->d, sm_count);
-        return ws_round((size_t)p.nchunks * p.ntiles * GT * GT * 8);
+        return ws_round((size_t)p.nchunks * p.ntiles * GT * GT * 8) +
+               (gram_tc3_supported(A) ? gram_tc3_workspace_bytes(A, sm_count) : 0);
     }
     const CsrPlan p = csr_plan(A->n, A->d, sm_count);
     return ws_round((size_t)p.nblocks * A->d * A->d * 4);
@@ -282,10 +286,16 @@ cudaError_t gram_launch_t(const lsk_mat* A, double alpha, double beta, OutT* C, 
     if (A->kind == LSK_DENSE) {
         const DensePlan p = dense_plan(n, d, sm_count);
         double* part = (double*)ws;
+        const int* redo = nullptr;
+        if (gram_tc3_supported(A)) {   // the kernels below then run only where it could not
+            cudaError_t e = gram_tc3_launch<OutT>(A, alpha, beta, C, (char*)ws + ws_round((size_t)p.nchunks * p.ntiles * GT * GT * 8),
+                                                  flag, sm_count, st, &redo);
+            if (e != cudaSuccess) return e;
+        }
         dim3 grid((unsigned)p.ntiles, (unsigned)p.nchunks);
-        LSK_PROF("gram_dense", st) gram_dense_kernel<<<grid, 256, 0, st>>>((const float*)A->values, A->ld, n, d, p.rows_per, part);
+        LSK_PROF("gram_dense", st) gram_dense_kernel<<<grid, 256, 0, st>>>((const float*)A->values, A->ld, n, d, p.rows_per, part, redo);
         LSK_PROF("gram_reduce", st) gram_dense_reduce_kernel<OutT>
-            <<<(unsigned)((len + 31) / 32), 256, 0, st>>>(part, p.nchunks, d, alpha, beta, C);
+            <<<(unsigned)((len + 31) / 32), 256, 0, st>>>(part, p.nchunks, d, alpha, beta, C, redo);
     } else {
         const CsrPlan p = csr_plan(n, d, sm_count);
         if (p.smem > 48 * 1024) {

@@ -34,6 +34,8 @@
 // are bounded; a timeout sets the TIMEOUT flag.
 #include "tc_common.cuh"
 
+#include <algorithm>
+
 namespace {
 
 constexpr int kKC = 32;            // rows of A per chunk (the K of the MMAs)
@@ -80,32 +82,59 @@ __host__ __device__ constexpr int stages_of(int npad) {
 // Rows row0 .. row0 + 7 of A (zeros at and past r_end or d), lane t: float4
 // number t + 32 h of each row (columns 4 t + 128 h .. + 3): 512 contiguous
 // bytes a row per warp instruction.
-template <int NPAD, int PR>
-__device__ __forceinline__ void load_piece(const GrParams& p, int64_t row0, int64_t r_end, int lane,
-                                           float4 (&v)[PR][(NPAD + kMT - 1) / kMT]) {
+template <int NPAD>
+__device__ __forceinline__ void load_row(const GrParams& p, int64_t row, int64_t r_end, int lane,
+                                         float4 (&v)[(NPAD + kMT - 1) / kMT]) {
     constexpr int H = (NPAD + kMT - 1) / kMT;
+    const float* src = p.A + row * p.lda;
 #pragma unroll
-    for (int r = 0; r < PR; ++r) {
-        const int64_t row = row0 + r;
-        const float* src = p.A + row * p.lda;
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-            const int c = 4 * lane + kMT * h;
-            v[r][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < r_end && c < p.d) {
-                if (p.vec && c + 3 < p.d) {
-                    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
-                                 : "=f"(v[r][h].x), "=f"(v[r][h].y), "=f"(v[r][h].z), "=f"(v[r][h].w)
-                                 : "l"(src + c));
-                } else {
-                    v[r][h].x = __ldg(src + c);
-                    v[r][h].y = c + 1 < p.d ? __ldg(src + c + 1) : 0.f;
-                    v[r][h].z = c + 2 < p.d ? __ldg(src + c + 2) : 0.f;
-                    v[r][h].w = c + 3 < p.d ? __ldg(src + c + 3) : 0.f;
-                }
+    for (int h = 0; h < H; ++h) {
+        const int c = 4 * lane + kMT * h;
+        v[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < r_end && c < p.d) {
+            if (p.vec && c + 3 < p.d) {
+                asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                             : "=f"(v[h].x), "=f"(v[h].y), "=f"(v[h].z), "=f"(v[h].w)
+                             : "l"(src + c));
+            } else {
+                v[h].x = __ldg(src + c);
+                v[h].y = c + 1 < p.d ? __ldg(src + c + 1) : 0.f;
+                v[h].z = c + 2 < p.d ? __ldg(src + c + 2) : 0.f;
+                v[h].w = c + 3 < p.d ? __ldg(src + c + 3) : 0.f;
             }
         }
     }
+}
+// The eight rows from row0 on; rows of whole 16-byte quads that are all in
+// range go without per-row checks (the registers of lanes past d, zero before,
+// are left as they are).
+template <int NPAD>
+__device__ __forceinline__ void load_piece_quads(const GrParams& p, int64_t row0, int64_t r_end, int lane,
+                                                 float4 (&v)[8][(NPAD + kMT - 1) / kMT]) {
+    constexpr int H = (NPAD + kMT - 1) / kMT;
+    if (p.vec && (p.d & 3) == 0 && row0 + 8 <= r_end) {
+        const char* src = reinterpret_cast<const char*>(p.A + row0 * p.lda + 4 * lane);
+        const int64_t step = p.lda * 4;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                if (4 * lane + kMT * h < p.d)
+                    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                                 : "=f"(v[r][h].x), "=f"(v[r][h].y), "=f"(v[r][h].z), "=f"(v[r][h].w)
+                                 : "l"(src + 4 * kMT * h));
+            src += step;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) load_row<NPAD>(p, row0 + r, r_end, lane, v[r]);
+    }
+}
+template <int NPAD, int PR>
+__device__ __forceinline__ void load_piece(const GrParams& p, int64_t row0, int64_t r_end, int lane,
+                                           float4 (&v)[PR][(NPAD + kMT - 1) / kMT]) {
+#pragma unroll
+    for (int r = 0; r < PR; ++r) load_row<NPAD>(p, row0 + r, r_end, lane, v[r]);
 }
 
 // Split the piece into bf16 hi / lo and store it as rows PR part .. PR part +
@@ -435,3 +464,521 @@ cudaError_t gram_tc_launch(const lsk_mat* A, double alpha, double beta, float* C
     LSK_PROF("gram_reduce", st) gram_tc_reduce_kernel<<<(unsigned)rg, 256, 0, st>>>(p.part, grid, p.d, p.npad, alpha, beta, C);
     return cudaGetLastError();
 }
+
+namespace {
+
+// ---- the FP32 form -------------------------------------------------------------
+// C to FP32 accuracy from bf16 products.  Every entry is split as
+//     x = hi + mid + lo,   hi = x rounded to a multiple of the column's unit,
+//                          mid, lo = bf16 roundings of what is left,
+// where the unit is a power of two a fixed number of bits below the column's
+// largest recent entry.  hi then has at most eight significant bits and the
+// sums of hi hi over a segment of rows are whole numbers of units^2 up to 2^24:
+// exact in the FP32 accumulator, so the tensor pipe's accumulation, which rounds
+// toward zero, has nothing to round there.  This is the error-free splitting of
+// Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59, 2012) with the first slice
+// on a fixed grid.  The other products but lo lo (hi mid, hi lo, mid lo, both
+// ways round, and mid mid) go to a second accumulator, a small part of the
+// first, where that rounding no longer matters.  The unit is only a choice of
+// rounding: an entry above the maximum seen (the first rows of the CTA, then a
+// quarter of each segment and of the one before) costs exactness in its
+// segment, no more.  The CTAs' partials keep the two accumulators apart and are
+// summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
+// (2.9e-8 for the CUDA-core kernel; storing C in FP32 alone costs 1.85e-8),
+// 4.5e-8 against 2.5e-7 with five rows scaled x100.  A column below 2^-48 (its
+// small products would leave FP32's range) or a diagonal that is not finite
+// sets *redo, and the CUDA-core kernel forms C.
+//
+// Work: a job is a 128-column panel of C's rows against the columns from the
+// panel's first on (d > 128: two jobs, N = npad and npad - 128; the SMs are
+// shared out by N), so each CTA's two accumulators (2 N <= 512 columns) fill
+// its TMEM.  Each CTA takes a contiguous range of rows.  At 1M x 256
+// the eight products over the block triangle are 0.41 ms of the tensor pipe's
+// measured rate; this takes 0.55 ms (CUDA cores: 4.20), bound by shared-memory
+// bandwidth (the MMAs' operands and the workers' stores keep its data pipe
+// full).  What it took: MMAs issued by an elected lane of a warp that runs
+// along, so that the descriptors stay in uniform registers (else issue takes 120
+// cycles an MMA), few flushes, and partials stored by columns.
+
+// Unit and segment.  Segments of seg_chunks 32-row chunks are summed in TMEM,
+// then added to the CTA's partial in FP32.  With the column's maximum at
+// 128 .. 256 units a segment of 256 rows stays exact, with 64 .. 128 units one of
+// 1,024.  Up to 1,024 rows a CTA take the finer unit (few rows to average the
+// roundings of lo over); more rows the longer segments, since every flush of
+// the accumulators costs L2 reductions (1.5 GB of them at 1M x 256 with 256-row
+// segments: 0.13 ms).
+struct Gr3Params {
+    GrParams a;          // A, lda, n, d, vec, part, flag
+    int chunks;          // 32-row chunks of A
+    int ctas[2];         // CTAs of the two jobs (ctas[1] = 0 for d <= 128)
+    int seg_chunks;
+    uint32_t magic_add;  // exponent of 1.5 * 2^23 units above the column maximum's, and the 1.5
+    int* redo;
+};
+
+__host__ __device__ constexpr uint32_t stage3_bytes(int npad) { return 3 * half_bytes(npad); }
+__host__ __device__ constexpr int stages3_of(int npad) {
+    return (int)((232448 - 6144) / stage3_bytes(npad)) < kMaxStages ? (int)((232448 - 6144) / stage3_bytes(npad)) : kMaxStages;
+}
+__host__ __device__ constexpr uint32_t tmem3_cols(int npad) { return npad <= 32 ? 64u : npad <= 64 ? 128u : npad <= 128 ? 256u : 512u; }
+// FP32 words of one CTA's partial: two planes of 128 x N
+__host__ __device__ constexpr size_t part3_floats(int npad) { return 2u * kMT * (size_t)npad; }
+
+// two FP32 additions in one instruction (the low word is the first of the pair)
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ uint32_t to_bf16x2(float2 v) {   // v.x in the low half
+    uint32_t h;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(v.y), "f"(v.x));
+    return h;
+}
+__device__ __forceinline__ float2 neg_bf16x2(uint32_t h) {
+    return make_float2(-__uint_as_float(h << 16), -__uint_as_float(h & 0xFFFF0000u));
+}
+
+// The three bf16 terms of the pair v; m: 1.5 * 2^23 units of its columns
+// (x + m has x's nearest multiple of the unit in its low bits).
+__device__ __forceinline__ void split3_grid(float2 v, float2 m, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    hi = to_bf16x2(add2(add2(v, m), make_float2(-m.x, -m.y)));
+    const float2 r = add2(v, neg_bf16x2(hi));
+    mid = to_bf16x2(r);
+    lo = to_bf16x2(add2(r, neg_bf16x2(mid)));
+}
+
+// 1.5 * 2^23 units for a column whose largest |entry| has these bits (add: magic_add)
+__device__ __forceinline__ float unit_magic(uint32_t max_bits, uint32_t add) {
+    return __uint_as_float((max_bits & 0x7F800000u) + add);
+}
+__device__ __forceinline__ uint4 ld_shared4(const uint32_t* p) {
+    uint4 v;
+    asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(tc::smem_u32(p)));
+    return v;
+}
+__device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t h) {   // per half: max(m, |h|), m >= 0
+    const __nv_bfloat162 r = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&m), __habs2(*reinterpret_cast<__nv_bfloat162*>(&h)));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// Split a piece and store it as row group `part` of the stage's three tiles;
+// mx[h]: the largest |hi| of the lane's columns (bf16 pairs) in its first two rows.
+template <int NPAD>
+__device__ __forceinline__ void store_piece3(uint8_t* tile, int part, int lane, const float4 (&v)[8][(NPAD + kMT - 1) / kMT],
+                                             const float4 (&mg)[(NPAD + kMT - 1) / kMT], uint2 (&mx)[(NPAD + kMT - 1) / kMT]) {
+    constexpr int H = (NPAD + kMT - 1) / kMT;
+    const uint32_t c0 = 4u * (uint32_t)lane;
+    uint8_t* const b = tile + (uint32_t)part * kSbo(NPAD);
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const uint32_t c = c0 + kMT * h;
+            const uint32_t off = (c >> 6) * 1024u + r * 128u + (((((c & 63u) >> 3) ^ (uint32_t)r) & 7u) << 4) + (c & 7u) * 2u;
+            uint2 hi, mid, lo;
+            split3_grid(make_float2(v[r][h].x, v[r][h].y), make_float2(mg[h].x, mg[h].y), hi.x, mid.x, lo.x);
+            split3_grid(make_float2(v[r][h].z, v[r][h].w), make_float2(mg[h].z, mg[h].w), hi.y, mid.y, lo.y);
+            if (r < 2) {
+                mx[h].x = max_abs_bf16x2(r ? mx[h].x : 0u, hi.x);
+                mx[h].y = max_abs_bf16x2(r ? mx[h].y : 0u, hi.y);
+            }
+            *reinterpret_cast<uint2*>(b + off) = hi;
+            *reinterpret_cast<uint2*>(b + half_bytes(NPAD) + off) = mid;
+            *reinterpret_cast<uint2*>(b + 2 * half_bytes(NPAD) + off) = lo;
+        }
+}
+
+// One CTA of a job: the panel of p's first 128 columns against all of p's
+// columns (NPAD of them, padded), 32-row chunks [g0, g1), partial into `part`.
+template <int NPAD, class SH>
+__device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params& q, int g0, int g1, float* part, uint8_t* smem) {
+    constexpr int kWorkers = SH::kWorkers, kMmaWarp = SH::kMmaWarp;
+    constexpr int H = (NPAD + kMT - 1) / kMT;
+    constexpr int kStages = stages3_of(NPAD);
+    constexpr uint32_t sbytes = stage3_bytes(NPAD);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * sbytes);
+    uint64_t* full = bars;                 // [kStages] (4 arrivals: the pieces of a chunk)
+    uint64_t* empty = bars + kStages;      // [kStages] (MMA commit)
+    uint64_t* done = bars + 2 * kStages;   // segment accumulated     (MMA commit)
+    uint64_t* drained = done + 1;          // accumulators read       (4 epilogue warps)
+    uint64_t* fin = done + 2;              // every MMA complete      (MMA commit)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    uint32_t* cmax = reinterpret_cast<uint32_t*>(smem + kStages * sbytes + 1024);   // largest |entry| of the columns, as bits:
+                                                                                    // [2] segments (even, odd), [1] earlier ones
+    static_assert(2 * kMaxStages * 8 + 64 <= 1024, "the barriers fit before the maxima");
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nchunks = g1 - g0, nseg = (nchunks + q.seg_chunks - 1) / q.seg_chunks;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            tc::mbar_init(full + s, 4);
+            tc::mbar_init(empty + s, 1);
+        }
+        tc::mbar_init(done, 1);
+        tc::mbar_init(drained, 4);
+        tc::mbar_init(fin, 1);
+        *abort = 0;
+        tc::fence_mbar_init();
+    }
+    constexpr int kCols = kMT * H;
+    for (int j = threadIdx.x; j < 3 * kCols; j += SH::kThreads) cmax[j] = 0u;
+    if (warp == kMmaWarp) {
+        tc::tmem_alloc(tmem_slot, tmem3_cols(NPAD));
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+
+    // Worker w owns rows 8 (w % 4) .. of the chunks w / 4, w / 4 + 4, ...: a piece
+    // in registers (two where they fit), the next one's loads in flight.
+    constexpr int NB = H == 1 ? 2 : 1;
+    float4 v[NB][8][H];
+    const int grp = warp & 3, c0 = warp >> 2;
+    const int64_t row_base = (int64_t)g0 * kKC + grp * 8, r_end = min(p.n, (int64_t)g1 * kKC);
+    if (warp < kWorkers) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int h = 0; h < H; ++h) v[b][r][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+            load_piece_quads<NPAD>(p, row_base + (int64_t)(c0 + 4 * b) * kKC, r_end, lane, v[b]);
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {   // the first rows give the columns' units
+            float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 t = v[0][i][h];
+                m.x = fmaxf(m.x, fabsf(t.x));
+                m.y = fmaxf(m.y, fabsf(t.y));
+                m.z = fmaxf(m.z, fabsf(t.z));
+                m.w = fmaxf(m.w, fabsf(t.w));
+            }
+            uint32_t* c = cmax + 4 * lane + kMT * h;
+            atomicMax(c, __float_as_uint(m.x));
+            atomicMax(c + 1, __float_as_uint(m.y));
+            atomicMax(c + 2, __float_as_uint(m.z));
+            atomicMax(c + 3, __float_as_uint(m.w));
+        }
+    }
+    __syncthreads();
+
+    if (warp < kWorkers) {
+        uint32_t* const cm = cmax + 4 * lane;
+        // split row group `grp` of chunk c into its stage
+        const auto put = [&](int c, const float4 (&t)[8][H]) -> bool {
+            const int z = c / q.seg_chunks;   // the unit: the largest entry of this segment so far and of the last
+            uint32_t* const cur = cm + (z & 1) * kCols;
+            uint32_t* const last = cm + (~z & 1) * kCols;
+            if (z > 0 && c % q.seg_chunks == 0 && grp == 0)
+#pragma unroll
+                for (int i = 0; i < H; ++i)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) atomicMax(cm + 2 * kCols + kMT * i + k, atomicExch(cur + kMT * i + k, 0u));
+            float4 mg[H];
+            uint2 mx[H];
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                const uint4 b = ld_shared4(cur + kMT * i), d = ld_shared4(last + kMT * i);   // other warps may be raising these
+                mg[i] = make_float4(unit_magic(max(b.x, d.x), q.magic_add), unit_magic(max(b.y, d.y), q.magic_add),
+                                    unit_magic(max(b.z, d.z), q.magic_add), unit_magic(max(b.w, d.w), q.magic_add));
+            }
+            const int s = c % kStages;
+            int okl = 1;
+            if (lane == 0) okl = tc::mbar_wait(empty + s, ((uint32_t)(c / kStages) & 1u) ^ 1u, abort) ? 1 : 0;
+            if (!__shfl_sync(0xffffffffu, okl, 0)) return false;
+            store_piece3<NPAD>(smem + (size_t)s * sbytes, grp, lane, t, mg, mx);
+            tc::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(full + s);
+#pragma unroll
+            for (int i = 0; i < H; ++i) {   // tell the other warps (a quarter of the rows look)
+                const uint4 b = ld_shared4(cur + kMT * i);
+                const uint32_t m[4] = {mx[i].x << 16, mx[i].x & 0xFFFF0000u, mx[i].y << 16, mx[i].y & 0xFFFF0000u};
+                const uint32_t o[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (m[k] > o[k]) atomicMax(cur + kMT * i + k, m[k]);
+            }
+            return true;
+        };
+        for (int c = c0; c < nchunks; c += 4 * NB) {
+            if (!put(c, v[0])) break;
+            load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 4 * NB) * kKC, r_end, lane, v[0]);
+            if constexpr (NB == 2) {
+                if (c + 4 >= nchunks || !put(c + 4, v[1])) break;
+                load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 12) * kKC, r_end, lane, v[1]);
+            }
+        }
+    } else {
+        // Accumulator warps: TMEM lane quarter warp % 4 (rows of the panel);
+        // lane 0 of the first also issues the MMAs (the accumulators fill TMEM,
+        // so a segment's MMAs start when the last one's sums are read out).
+        const uint32_t base = tc::smem_u32(smem);
+        constexpr uint32_t idesc = tc::idesc_bf16_f32_mn(128, (uint32_t)NPAD);
+        const uint32_t acc0 = tmem, acc1 = tmem + (uint32_t)NPAD;
+        const int quarter = warp & 3, row = quarter * 32 + lane;
+        bool okm = true;
+        int s = 0;
+        uint32_t ph = 0;
+        // the descriptors of stage 0, first 16 rows; the others differ in the
+        // start address alone (16-byte units, bits 0 .. 13)
+        const uint64_t d0 = tc::desc_sw128_mnmajor(base, 1024u, kSbo(NPAD));
+        for (int z = 0; z < nseg; ++z) {
+            if (warp == kMmaWarp) {   // the whole warp goes along, so descriptors stay in uniform registers
+                if (z > 0) okm = tc::mbar_wait(drained, (uint32_t)(z - 1) & 1u, abort);
+                tc::fence_after_sync();
+                const int ng = min(q.seg_chunks, nchunks - z * q.seg_chunks);
+                for (int g = 0; g < ng && okm; ++g) {
+                    okm = __all_sync(0xffffffffu, tc::mbar_wait(full + s, ph, abort));
+                    if (!okm) break;
+                    tc::fence_after_sync();
+                    if (tc::elect_one()) {
+#pragma unroll
+                        for (int kk = 0; kk < kKC / 16; ++kk) {
+                            // 16 rows = two 8-row groups
+                            const uint64_t dh = d0 + (((uint32_t)s * sbytes + 2u * kSbo(NPAD) * kk) >> 4);
+                            const uint64_t dm = dh + (half_bytes(NPAD) >> 4), dl = dm + (half_bytes(NPAD) >> 4);
+                            tc::mma_bf16(acc0, dh, dh, idesc, (g | kk) != 0);
+                            tc::mma_bf16(acc1, dh, dm, idesc, (g | kk) != 0);
+                            tc::mma_bf16(acc1, dm, dh, idesc, 1);
+                            tc::mma_bf16(acc1, dh, dl, idesc, 1);
+                            tc::mma_bf16(acc1, dl, dh, idesc, 1);
+                            tc::mma_bf16(acc1, dm, dm, idesc, 1);
+                            tc::mma_bf16(acc1, dm, dl, idesc, 1);
+                            tc::mma_bf16(acc1, dl, dm, idesc, 1);
+                        }
+                        tc::mma_commit(empty + s);
+                        if (g + 1 == ng) tc::mma_commit(done);
+                    }
+                    __syncwarp();
+                    if (++s == kStages) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            int okw = okm;
+            if (lane == 0 && okm) okw = tc::mbar_wait(done, (uint32_t)z & 1u, abort) ? 1 : 0;
+            if (!__shfl_sync(0xffffffffu, okw, 0)) break;
+            tc::fence_after_sync();
+            for (int col = 0; col < NPAD; col += 32) {
+                uint32_t va[32], vb[32];
+                const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col;
+                tc::tmem_ld_32x32b_x32(ta, va);
+                tc::tmem_ld_32x32b_x32(ta + (uint32_t)NPAD, vb);
+                tc::tmem_ld_wait();
+                if (col == quarter * 32) {   // the diagonal: an entry outside FP32's range shows here first
+                    float dg = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (i == lane) dg = __uint_as_float(va[i]) + __uint_as_float(vb[i]);
+                    if (!(fabsf(dg) <= 3.402823466e38f)) atomicOr(q.redo, 1);
+                }
+                if (col + 32 >= NPAD) {
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(drained);
+                }
+                // the partial is stored by columns: a warp's 32 rows are one
+                // 128-byte line (row-major v4 reductions, a line a lane, took
+                // 7,700 cycles a flush at N = 128)
+                float* dst = part + (size_t)col * kMT + row;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (z == 0) {   // (one thread an address: the first segment stores, later ones add)
+                        dst[i * kMT] = __uint_as_float(va[i]);
+                        dst[(NPAD + i) * kMT] = __uint_as_float(vb[i]);
+                    } else {
+                        asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + i * kMT), "f"(__uint_as_float(va[i])) : "memory");
+                        asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + (NPAD + i) * kMT), "f"(__uint_as_float(vb[i])) : "memory");
+                    }
+                }
+            }
+        }
+        if (warp == kMmaWarp) {   // also when a wait gave up: every MMA issued is complete before TMEM goes
+            if (tc::elect_one()) tc::mma_commit(fin);
+            __syncwarp();
+            volatile int never = 0;
+            tc::mbar_wait(fin, 0, &never);
+        }
+        __syncwarp();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tmem, tmem3_cols(NPAD));
+    }
+    for (int j = threadIdx.x; j < kCols; j += SH::kThreads) {
+        const uint32_t m = max(max(cmax[j], cmax[kCols + j]), cmax[2 * kCols + j]);
+        if (m != 0u && m < 0x27800000u) atomicOr(q.redo, 1);   // below 2^-48
+    }
+    if (threadIdx.x == 0 && *abort) set_flag(p.flag, LSK_FLAG_TIMEOUT);
+}
+
+using Shape3 = GramShape<16, 3>;   // 16 workers, 4 accumulator warps
+
+template <int NPAD>
+__global__ void __launch_bounds__(Shape3::kThreads, 1) gram_tc3_kernel(const Gr3Params p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int job = (int)blockIdx.x >= p.ctas[0];
+    const int64_t c = (int)blockIdx.x - (job ? p.ctas[0] : 0), nc = job ? p.ctas[1] : p.ctas[0];
+    const int g0 = (int)(p.chunks * c / nc), g1 = (int)(p.chunks * (c + 1) / nc);
+    float* part = p.a.part + (job ? p.ctas[0] * part3_floats(NPAD) + c * part3_floats(NPAD - kMT) : c * part3_floats(NPAD));
+    if constexpr (NPAD > kMT) {
+        if (job) {
+            GrParams b = p.a;
+            b.A += kMT;
+            b.d -= kMT;
+            gram_tc3_body<NPAD - kMT, Shape3>(b, p, g0, g1, part, smem);
+            return;
+        }
+    }
+    gram_tc3_body<NPAD, Shape3>(p.a, p, g0, g1, part, smem);
+}
+
+// C[a][b] = C[b][a] = alpha sum + beta C for a <= b: a block takes 32
+// consecutive entries; thread (g, x) adds both planes of the partials g, g + 8,
+// ... of entry x as FP32 pairs, then the 8 group sums are added in order.
+template <typename OutT>
+__global__ void __launch_bounds__(256) gram_tc3_reduce_kernel(const float* __restrict__ part, int ctas0, int ctas1, int d,
+                                                              int npad, const int* __restrict__ redo, double alpha,
+                                                              double beta, OutT* __restrict__ C) {
+    __shared__ double acc[8][33];
+    if (*redo) return;
+    const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int e = (int)blockIdx.x * 32 + x;
+    const int b = e / d, a = e % d;
+    const bool upper = e < d * d && a <= b;
+    float s = 0.f, c = 0.f;
+    if (upper) {
+        const int job = a >= kMT, w = job ? npad - kMT : npad, n = job ? ctas1 : ctas0;
+        const size_t one = part3_floats(w), plane = (size_t)kMT * w;
+        const float* src = part + (job ? ctas0 * part3_floats(npad) : 0) + (size_t)(b - job * kMT) * kMT + (a - job * kMT);
+        const auto add = [&](float v) {
+            const float t = s + v, u = t - s;
+            c += (s - (t - u)) + (v - u);
+            s = t;
+        };
+        for (int z = g; z < n; z += 32) {   // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool in = z + 8 * k < n;
+                v[2 * k] = in ? src[(z + 8 * k) * one] : 0.f;
+                v[2 * k + 1] = in ? src[(z + 8 * k) * one + plane] : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) add(v[k]);
+        }
+    }
+    acc[g][x] = (double)s + (double)c;
+    __syncthreads();
+    if (g == 0 && upper) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += acc[k][x];
+        const double ab = alpha * t;
+        C[(size_t)a * d + b] = (OutT)(beta != 0.0 ? ab + beta * (double)C[(size_t)a * d + b] : ab);
+        if (a != b) C[(size_t)b * d + a] = (OutT)(beta != 0.0 ? ab + beta * (double)C[(size_t)b * d + a] : ab);
+    }
+}
+
+struct Gr3Plan {
+    int npad, chunks, ctas[2];
+    size_t part_bytes;
+};
+// The SMs are shared out between the two jobs by a chunk's cost: 6 N cycles of
+// products, or the split of a 128-column panel (some 450) where N is small.
+Gr3Plan gram_tc3_plan(const lsk_mat* A, int sm_count) {
+    Gr3Plan q{};
+    q.npad = (int)((A->d + 31) / 32) * 32;
+    q.chunks = (int)((A->n + kKC - 1) / kKC);
+    if (q.npad > kMT) {
+        const int w0 = 6 * q.npad, w1 = std::max(6 * (q.npad - kMT), 450);
+        q.ctas[1] = std::max(1, (sm_count * w1 + (w0 + w1) / 2) / (w0 + w1));
+        q.ctas[0] = std::max(1, sm_count - q.ctas[1]);
+    } else {
+        q.ctas[0] = sm_count;
+    }
+    for (int j = 0; j < 2; ++j) q.ctas[j] = std::min(q.ctas[j], q.chunks);
+    q.part_bytes = q.ctas[0] * part3_floats(q.npad) * 4 + (q.npad > kMT ? q.ctas[1] * part3_floats(q.npad - kMT) * 4 : 0);
+    return q;
+}
+
+template <int NPAD>
+cudaError_t launch_tc3(const Gr3Params& p, cudaStream_t st) {
+    size_t smem = stages3_of(NPAD) * (size_t)stage3_bytes(NPAD);
+    if constexpr (NPAD > kMT) smem = std::max(smem, stages3_of(NPAD - kMT) * (size_t)stage3_bytes(NPAD - kMT));
+    smem += 6144;
+    cudaError_t e = allow_dynamic_smem(gram_tc3_kernel<NPAD>);
+    if (e != cudaSuccess) return e;
+    LSK_PROF("gram_tc3", st) gram_tc3_kernel<NPAD><<<p.ctas[0] + p.ctas[1], Shape3::kThreads, smem, st>>>(p);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Dense A with d <= 256 and at least 2^19 entries: the CUDA-core kernel's two
+// launches are the shorter chain below (21 against 29 us at 2,048 x 32, 29
+// against 28 at 10,000 x 50, 65 against 42 at 10,000 x 256).
+bool gram_tc3_supported(const lsk_mat* A) {
+    return A->kind == LSK_DENSE && A->d >= 1 && A->d <= 256 && A->n * A->d >= (int64_t)1 << 19;
+}
+
+size_t gram_tc3_workspace_bytes(const lsk_mat* A, int sm_count) {
+    return ws_round(gram_tc3_plan(A, sm_count).part_bytes) + ws_round(sizeof(int));
+}
+
+// alpha A^T A + beta C, or nothing with **redo != 0 where a column is out of
+// the splitting's range (the caller then runs the CUDA-core kernels, which return
+// at once when *redo is 0)
+template <typename OutT>
+cudaError_t gram_tc3_launch(const lsk_mat* A, double alpha, double beta, OutT* C, void* ws, int* flag, int sm_count,
+                            cudaStream_t st, const int** redo) {
+    const Gr3Plan q = gram_tc3_plan(A, sm_count);
+    WsCarver wc{(char*)ws, 0};
+    Gr3Params p{};
+    p.a.A = (const float*)A->values;
+    p.a.lda = A->ld;
+    p.a.n = A->n;
+    p.a.d = (int)A->d;
+    p.a.npad = q.npad;
+    p.a.vec = (A->ld % 4 == 0) && (((uintptr_t)A->values & 15) == 0);
+    p.a.part = wc.take<float>(q.part_bytes / 4);
+    p.a.flag = flag;
+    p.redo = wc.take<int>(1);
+    *redo = p.redo;
+    p.chunks = q.chunks;
+    p.ctas[0] = q.ctas[0];
+    p.ctas[1] = q.ctas[1];
+    const bool few = q.chunks <= 32 * q.ctas[0];   // at most 1,024 rows a CTA
+    p.seg_chunks = few ? 8 : 32;
+    p.magic_add = ((few ? 16u : 17u) << 23) + 0x400000u;
+    cudaError_t e = cudaMemsetAsync(p.redo, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    switch (q.npad) {
+        case 32: e = launch_tc3<32>(p, st); break;
+        case 64: e = launch_tc3<64>(p, st); break;
+        case 96: e = launch_tc3<96>(p, st); break;
+        case 128: e = launch_tc3<128>(p, st); break;
+        case 160: e = launch_tc3<160>(p, st); break;
+        case 192: e = launch_tc3<192>(p, st); break;
+        case 224: e = launch_tc3<224>(p, st); break;
+        default: e = launch_tc3<256>(p, st); break;
+    }
+    if (e != cudaSuccess) return e;
+    LSK_PROF("gram_reduce", st) gram_tc3_reduce_kernel<OutT><<<(unsigned)((A->d * A->d + 31) / 32), 256, 0, st>>>(
+        p.a.part, q.ctas[0], q.ctas[1], (int)A->d, q.npad, p.redo, alpha, beta, C);
+    return cudaGetLastError();
+}
+template cudaError_t gram_tc3_launch<float>(const lsk_mat*, double, double, float*, void*, int*, int, cudaStream_t, const int**);
+template cudaError_t gram_tc3_launch<double>(const lsk_mat*, double, double, double*, void*, int*, int, cudaStream_t, const int**);
