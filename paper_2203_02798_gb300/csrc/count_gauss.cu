@@ -193,9 +193,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Shape<NG, kRing>::kT
                     const int64_t jq = (int64_t)(gq >> 5) * kSetRows + (int64_t)rank * kHalfRows + 4 * (gq & 31);
                     const int64_t c = c0 + 2 * cp;
                     float4 z0 = make_float4(0.f, 0.f, 0.f, 0.f), z1 = z0;
-                    if (jq < p.k) {
-                        if (c < c_end) z0 = gauss4((uint64_t)c, (uint32_t)(jq >> 2), p.k0, p.k1);
-                        if (c + 1 < c_end) z1 = gauss4((uint64_t)(c + 1), (uint32_t)(jq >> 2), p.k0, p.k1);
+                    if (jq < p.k) {   // columns past the slice meet zero rows of the operand
+                        z0 = gauss4((uint64_t)c, (uint32_t)(jq >> 2), p.k0, p.k1);
+                        z1 = gauss4((uint64_t)(c + 1), (uint32_t)(jq >> 2), p.k0, p.k1);
                     }
                     const float a0[4] = {z0.x, z0.y, z0.z, z0.w}, a1[4] = {z1.x, z1.y, z1.z, z1.w};
 #pragma unroll
@@ -228,9 +228,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Shape<NG, kRing>::kT
                     tc::tmem_ld_32x32b_x32(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(set * p.npad + col), v);
                     tc::tmem_ld_wait();
                     if (j < p.k) {
+                        if ((p.d & 3) == 0) {   // a lane's row is contiguous: 16-byte stores
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (col + e < p.d) dst[col + e] = __uint_as_float(v[e]);
+                            for (int e = 0; e < 32; e += 4)
+                                if (col + e < p.d)
+                                    *reinterpret_cast<uint4*>(dst + col + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (col + e < p.d) dst[col + e] = __uint_as_float(v[e]);
+                        }
                     }
                 }
             }
@@ -391,33 +398,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Shape<NG, kRing>::kT
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else {
         // ------------------------------------------------------------ MMA issue (even CTA)
-        if (lane == 0 && rank == 0) {
+        // (the whole warp goes along, one elected lane issues: uniform descriptors)
+        if (rank == 0) {
             const uint32_t base = tc::smem_u32(stages);
             const uint32_t idesc = tc::idesc_bf16_f32(kSetRows, (uint32_t)p.npad);
+            const uint64_t da0 = tc::desc_sw64_kmajor(base), db0 = tc::desc_sw64_kmajor(base + a_bytes());
             bool okm = true;
+            int s = 0;
+            uint32_t ph = 0;
             for (int g = 0; g < nchunks; ++g) {
-                const int s = g % kStages;
-                if (!tc::mbar_wait_cluster(fullS + s, (uint32_t)(g / kStages) & 1u, abort)) {
-                    okm = false;
-                    break;
-                }
+                okm = __all_sync(0xffffffffu, tc::mbar_wait_cluster(fullS + s, ph, abort));
+                if (!okm) break;
                 tc::fence_after_sync();
-                const uint32_t a = base + s * sbytes, bh = a + a_bytes(), bl = bh + bbytes;
+                if (tc::elect_one()) {
+                    const uint64_t a = da0 + ((uint32_t)s * sbytes >> 4), bh = db0 + ((uint32_t)s * sbytes >> 4);
+                    const uint64_t bl = bh + (bbytes >> 4);
 #pragma unroll
-                for (int kk = 0; kk < kKC / 16; ++kk) {
-                    const uint32_t ko = 32u * kk;
-                    for (int set = 0; set < p.nsets; ++set) {
-                        const uint32_t at = a + (uint32_t)set * (kHalfRows * kKC * 2) + ko;
-                        const uint32_t dt = tmem + (uint32_t)(set * p.npad);
-                        tc::mma_bf16_pair(dt, tc::desc_sw64_kmajor(at), tc::desc_sw64_kmajor(bh + ko), idesc,
-                                          (g | kk) != 0);
-                        tc::mma_bf16_pair(dt, tc::desc_sw64_kmajor(at), tc::desc_sw64_kmajor(bl + ko), idesc, 1);
+                    for (int kk = 0; kk < kKC / 16; ++kk) {
+                        const uint32_t ko = 32u * kk >> 4;
+                        for (int set = 0; set < p.nsets; ++set) {
+                            const uint64_t at = a + ((uint32_t)set * (kHalfRows * kKC * 2) >> 4) + ko;
+                            const uint32_t dt = tmem + (uint32_t)(set * p.npad);
+                            tc::mma_bf16_pair(dt, at, bh + ko, idesc, (g | kk) != 0);
+                            tc::mma_bf16_pair(dt, at, bl + ko, idesc, 1);
+                        }
                     }
+                    tc::mma_commit_pair(emptyS + s);
                 }
-                tc::mma_commit_pair(emptyS + s);
+                __syncwarp();
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            if (okm && nchunks > 0) tc::mma_commit_pair(done);
-            tc::mma_commit_pair(fin);
+            if (tc::elect_one()) {
+                if (okm && nchunks > 0) tc::mma_commit_pair(done);
+                tc::mma_commit_pair(fin);
+            }
+            __syncwarp();
         }
         if (lane == 0) {
             // both CTAs: the last multicast commit has landed here

@@ -185,19 +185,20 @@ __device__ __forceinline__ void gauss_tc_body(const GtParams& p, const int blk) 
                 const int64_t jq = j0 + 4 * gq;
                 const int64_t c = c0 + 2 * cp;
                 float4 z0 = make_float4(0.f, 0.f, 0.f, 0.f), z1 = z0;
-                if (jq < p.k) {
+                // a warp's two row quads: both past k, or drawn without a branch
+                // (columns past the slice are drawn and dropped below)
+                if (j0 + 4 * ((warp * 32 + kWorkerThreads * i) >> 4) < p.k) {
+                    const int64_t ca = min(c, c_end - 1), cb = min(c + 1, c_end - 1);
                     // column of G = the row's bucket
-                    if (c < c_end)
-                        z0 = gauss4((uint64_t)(p.idx ? __ldg(p.idx + c) : c), (uint32_t)(jq >> 2), p.k0, p.k1);
-                    if (c + 1 < c_end)
-                        z1 = gauss4((uint64_t)(p.idx ? __ldg(p.idx + c + 1) : c + 1), (uint32_t)(jq >> 2), p.k0,
-                                    p.k1);
+                    z0 = gauss4((uint64_t)(p.idx ? __ldg(p.idx + ca) : ca), (uint32_t)(jq >> 2), p.k0, p.k1);
+                    z1 = gauss4((uint64_t)(p.idx ? __ldg(p.idx + cb) : cb), (uint32_t)(jq >> 2), p.k0, p.k1);
                 }
                 const float a0[4] = {z0.x, z0.y, z0.z, z0.w}, a1[4] = {z1.x, z1.y, z1.z, z1.w};
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const bool rowok = jq + t < p.k;
-                    const float g0 = rowok ? a0[t] * p.scale : 0.f, g1 = rowok ? a1[t] * p.scale : 0.f;
+                    const float g0 = rowok && c < c_end ? a0[t] * p.scale : 0.f;
+                    const float g1 = rowok && c + 1 < c_end ? a1[t] * p.scale : 0.f;
                     if constexpr (kA == 1) {
                         const __nv_bfloat162 h = __floats2bfloat162_rn(g0, g1);
                         gw[i][t][0] = *reinterpret_cast<const uint32_t*>(&h);
@@ -286,52 +287,69 @@ __device__ __forceinline__ void gauss_tc_body(const GtParams& p, const int blk) 
                     tc::tmem_ld_32x32b_x32(tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(tile * p.npad + col), v);
                     tc::tmem_ld_wait();
                     if (j < p.k) {
+                        if ((p.d & 3) == 0) {   // a lane's row is contiguous: 16-byte stores
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (col + e < p.d) dst[col + e] = __uint_as_float(v[e]);
+                            for (int e = 0; e < 32; e += 4)
+                                if (col + e < p.d)
+                                    *reinterpret_cast<uint4*>(dst + col + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 32; ++e)
+                                if (col + e < p.d) dst[col + e] = __uint_as_float(v[e]);
+                        }
                     }
                 }
             }
         }
     } else if (warp == kMmaWarp) {
-        if (lane == 0) {
-            const uint32_t base = tc::smem_u32(stages);
-            // A (G) K-major, B (SA) MN-major
-            const uint32_t idesc = tc::idesc_bf16_f32(128, (uint32_t)p.npad) | (1u << 16);
-            bool okm = true;
-            for (int g = 0; g < nchunks; ++g) {
-                const int s = g % kStages;
-                if (!tc::mbar_wait(full + s, (uint32_t)(g / kStages) & 1u, abort)) {
-                    okm = false;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t a = base + s * sbytes, b = a + kA * a_bytes();
-                // (A term, SA term) of each product: BF16 mode G (SA_hi + SA_lo);
-                // FP32 mode the six products of order down to 2^-16
-                constexpr int kPA[6] = {0, 0, 1, 0, 1, 2}, kPB[6] = {0, 1, 0, 2, 1, 0};
+        // The whole warp goes along and one elected lane issues, so that the
+        // descriptors stay in uniform registers (a lane's own branch moves every
+        // operand there, some 120 cycles an MMA).  A descriptor differs from its
+        // tile's first one in the start address alone (16-byte units).
+        const uint32_t base = tc::smem_u32(stages);
+        // A (G) K-major, B (SA) MN-major
+        const uint32_t idesc = tc::idesc_bf16_f32(128, (uint32_t)p.npad) | (1u << 16);
+        const uint64_t da0 = tc::desc_sw64_kmajor(base);
+        const uint64_t db0 = tc::desc_sw128_mnmajor(base + kA * a_bytes(), 1024u, b_sbo(p.npad));
+        bool okm = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int g = 0; g < nchunks; ++g) {
+            okm = __all_sync(0xffffffffu, tc::mbar_wait(full + s, ph, abort));
+            if (!okm) break;
+            tc::fence_after_sync();
+            // (A term, SA term) of each product: BF16 mode G (SA_hi + SA_lo);
+            // FP32 mode the six products of order down to 2^-16
+            constexpr int kPA[6] = {0, 0, 1, 0, 1, 2}, kPB[6] = {0, 1, 0, 2, 1, 0};
+            if (tc::elect_one()) {
+                const uint64_t das = da0 + ((uint32_t)s * sbytes >> 4), dbs = db0 + ((uint32_t)s * sbytes >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kKC / 16; ++kk) {
-                    const uint32_t ko = 32u * kk;
 #pragma unroll
                     for (int t = 0; t < kM / kMT; ++t) {
                         const uint32_t dt = tmem + (uint32_t)(t * p.npad);
 #pragma unroll
-                        for (int q = 0; q < Terms<T>::kProducts; ++q) {
-                            const uint32_t at = a + (uint32_t)kPA[q] * a_bytes() + (uint32_t)t * (kMT * kKC * 2) + ko;
-                            const uint32_t bt = b + (uint32_t)kPB[q] * b_bytes(p.npad) + 2u * b_sbo(p.npad) * kk;
-                            tc::mma_bf16(dt, tc::desc_sw64_kmajor(at), tc::desc_sw128_mnmajor(bt, 1024u, b_sbo(p.npad)),
-                                         idesc, (g | kk | q) != 0);
-                        }
+                        for (int q = 0; q < Terms<T>::kProducts; ++q)
+                            tc::mma_bf16(dt, das + ((kPA[q] * a_bytes() + t * (kMT * kKC * 2) + 32u * kk) >> 4),
+                                         dbs + ((kPB[q] * b_bytes(p.npad) + 2u * b_sbo(p.npad) * kk) >> 4), idesc,
+                                         (g | kk | q) != 0);
                     }
                 }
                 tc::mma_commit(empty + s);
             }
+            __syncwarp();
+            if (++s == kStages) {
+                s = 0;
+                ph ^= 1u;
+            }
+        }
+        if (tc::elect_one()) {
             if (okm && nchunks > 0) tc::mma_commit(done);
             tc::mma_commit(fin);
-            volatile int never = 0;
-            tc::mbar_wait(fin, 0, &never);
         }
+        __syncwarp();
+        volatile int never = 0;
+        tc::mbar_wait(fin, 0, &never);
         __syncwarp();
     }
     tc::fence_before_sync();
