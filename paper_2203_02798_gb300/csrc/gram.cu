@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(1024) gram_csr_kernel(const float* __restrict_
 
 // C[a][b] = C[b][a] = alpha sum_z part[z][a][b] + beta C (a <= b): a block
 // takes 32 consecutive entries; thread (g, x) adds the partials z = g, g + 8,
-// ... of entry x in FP64, then the 8 group sums are added in order
+// ... of entry x with compensation, then the 8 group sums are added in order
 // (deterministic).
 template <typename OutT>
 __global__ void __launch_bounds__(256) gram_csr_reduce_kernel(const float* __restrict__ part, int64_t nblocks,
@@ -202,20 +202,16 @@ __global__ void __launch_bounds__(256) gram_csr_reduce_kernel(const float* __res
     const int64_t e = (int64_t)blockIdx.x * 32 + x;
     const int64_t a = e / d, b = e % d;
     const bool upper = e < len && a <= b;
-    double s = 0.0;
-    if (upper) {
-        int64_t z = g;
-        for (; z + 24 < nblocks; z += 32) {   // four loads in flight
-            const float x0 = part[z * len + e], x1 = part[(z + 8) * len + e];
-            const float x2 = part[(z + 16) * len + e], x3 = part[(z + 24) * len + e];
-            s += (double)x0;
-            s += (double)x1;
-            s += (double)x2;
-            s += (double)x3;
+    float s = 0.f, c = 0.f;
+    if (upper)
+        for (int64_t z = g; z < nblocks; z += 64) {   // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = z + 8 * i < nblocks ? part[(z + 8 * i) * len + e] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) comp_add(s, c, v[i]);
         }
-        for (; z < nblocks; z += 8) s += (double)part[z * len + e];
-    }
-    acc[g][x] = s;
+    acc[g][x] = (double)s + (double)c;
     __syncthreads();
     if (g == 0 && upper) {
         double t = 0.0;

@@ -864,11 +864,6 @@ __global__ void __launch_bounds__(256) gram_tc3_reduce_kernel(const float* __res
         const int job = a >= kMT, w = job ? npad - kMT : npad, n = job ? ctas1 : ctas0;
         const size_t one = part3_floats(w), plane = (size_t)kMT * w;
         const float* src = part + (job ? ctas0 * part3_floats(npad) : 0) + (size_t)(b - job * kMT) * kMT + (a - job * kMT);
-        const auto add = [&](float v) {
-            const float t = s + v, u = t - s;
-            c += (s - (t - u)) + (v - u);
-            s = t;
-        };
         for (int z = g; z < n; z += 32) {   // eight loads in flight
             float v[8];
 #pragma unroll
@@ -878,7 +873,7 @@ __global__ void __launch_bounds__(256) gram_tc3_reduce_kernel(const float* __res
                 v[2 * k + 1] = in ? src[(z + 8 * k) * one + plane] : 0.f;
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) add(v[k]);
+            for (int k = 0; k < 8; ++k) comp_add(s, c, v[k]);
         }
     }
     acc[g][x] = (double)s + (double)c;
