@@ -12,6 +12,8 @@
 //   sum_{p,q in row} v_p v_q Btilde[J_p, J_q] using the symmetry of Btilde.
 #include "lsk_internal.cuh"
 
+#include <algorithm>
+
 namespace {
 
 constexpr int RM = 128;   // rows of A per block
@@ -19,74 +21,84 @@ constexpr int RN = 64;    // columns of B per tile
 constexpr int RK = 16;    // reduction step
 constexpr int RMP = RM + 4;
 
-// thread (ty, tx) = (tid / 16, tid % 16): rows 8*ty..8*ty+7, cols 4*tx..4*tx+3
+// thread (ty, tx) = (tid / 16, tid % 16): rows 8*ty..8*ty+7, cols 4*tx..4*tx+3.
+// kList: the rows list[0 .. *count) of A and x only, a persistent grid.
+template <bool kList>
 __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ B,
-    int64_t c, int upper_tri, float alpha, float beta, float* __restrict__ x) {
+    int64_t c, int upper_tri, float alpha, float beta, float* __restrict__ x, const int* __restrict__ list,
+    const int* __restrict__ count) {
     __shared__ __align__(16) float As[RK][RMP];
     __shared__ __align__(16) float Bs[RK][RN];
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const int64_t i0 = (int64_t)blockIdx.x * RM;
-    float rowsum[8];
+    const int64_t rows = kList ? (int64_t)*count : n;
+    const auto row_of = [&](int64_t i) { return kList ? (int64_t)__ldg(list + i) : i; };
+    for (int64_t i0 = (int64_t)blockIdx.x * RM; i0 < rows; i0 += (int64_t)gridDim.x * RM) {
+        float rowsum[8];
 #pragma unroll
-    for (int a = 0; a < 8; ++a) rowsum[a] = 0.f;
+        for (int a = 0; a < 8; ++a) rowsum[a] = 0.f;
 
-    for (int64_t c0 = 0; c0 < c; c0 += RN) {
-        const int64_t kmax = upper_tri ? min(d, c0 + RN) : d;
-        float acc[8][4];
+        for (int64_t c0 = 0; c0 < c; c0 += RN) {
+            const int64_t kmax = upper_tri ? min(d, c0 + RN) : d;
+            float acc[8][4];
 #pragma unroll
-        for (int a = 0; a < 8; ++a)
+            for (int a = 0; a < 8; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-        for (int64_t k0 = 0; k0 < kmax; k0 += RK) {
+                for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+            for (int64_t k0 = 0; k0 < kmax; k0 += RK) {
 #pragma unroll
-            for (int t = 0; t < (RM * RK) / 256; ++t) {
-                const int idx = tid + 256 * t;
-                const int row = idx / RK, kk = idx % RK;
-                const int64_t i = i0 + row, kx = k0 + kk;
-                As[kk][row] = (i < n && kx < kmax) ? __ldg(A + i * lda + kx) : 0.f;
+                for (int t = 0; t < (RM * RK) / 256; ++t) {
+                    const int idx = tid + 256 * t;
+                    const int row = idx / RK, kk = idx % RK;
+                    const int64_t i = i0 + row, kx = k0 + kk;
+                    As[kk][row] = (i < rows && kx < kmax) ? __ldg(A + row_of(i) * lda + kx) : 0.f;
+                }
+#pragma unroll
+                for (int t = 0; t < (RK * RN) / 256; ++t) {
+                    const int idx = tid + 256 * t;
+                    const int kk = idx / RN, cc = idx % RN;
+                    const int64_t kx = k0 + kk, cx = c0 + cc;
+                    Bs[kk][cc] = (kx < kmax && cx < c) ? __ldg(B + kx * c + cx) : 0.f;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int kk = 0; kk < RK; ++kk) {
+                    const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][8 * ty]);
+                    const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][8 * ty + 4]);
+                    const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][4 * tx]);
+                    const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                    const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+                    for (int a = 0; a < 8; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bb[b], acc[a][b]);
+                }
+                __syncthreads();
             }
 #pragma unroll
-            for (int t = 0; t < (RK * RN) / 256; ++t) {
-                const int idx = tid + 256 * t;
-                const int kk = idx / RN, cc = idx % RN;
-                const int64_t kx = k0 + kk, cx = c0 + cc;
-                Bs[kk][cc] = (kx < kmax && cx < c) ? __ldg(B + kx * c + cx) : 0.f;
-            }
-            __syncthreads();
+            for (int a = 0; a < 8; ++a)
 #pragma unroll
-            for (int kk = 0; kk < RK; ++kk) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][8 * ty]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][8 * ty + 4]);
-                const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][4 * tx]);
-                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-                for (int a = 0; a < 8; ++a)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bb[b], acc[a][b]);
-            }
-            __syncthreads();
+                for (int b = 0; b < 4; ++b) rowsum[a] = fmaf(acc[a][b], acc[a][b], rowsum[a]);
         }
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) rowsum[a] = fmaf(acc[a][b], acc[a][b], rowsum[a]);
-    }
-    // the 16 threads of a half-warp share rows: reduce across tx
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        float v = rowsum[a];
-#pragma unroll
-        for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        rowsum[a] = v;
-    }
-    if (tx == 0) {
+        // the 16 threads of a half-warp share rows: reduce across tx
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
-            const int64_t i = i0 + 8 * ty + a;
-            if (i < n) x[i] = (beta != 0.f) ? fmaf(alpha, rowsum[a], beta * x[i]) : alpha * rowsum[a];
+            float v = rowsum[a];
+#pragma unroll
+            for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            rowsum[a] = v;
         }
+        if (tx == 0) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const int64_t i = i0 + 8 * ty + a;
+                if (i < rows) {
+                    float* const xi = x + row_of(i);
+                    *xi = (beta != 0.f) ? fmaf(alpha, rowsum[a], beta * *xi) : alpha * rowsum[a];
+                }
+            }
+        }
+        if (!kList) return;   // one tile a block
     }
 }
 
@@ -167,7 +179,7 @@ size_t rownorms_workspace_bytes(const lsk_mat* A, int64_t c, int upper_tri, int3
         if ((prec == LSK_PREC_BF16 || prec == LSK_PREC_TF32) &&
             (rownorms_tc_supported(A, c, upper_tri) || rownorms_tc_supported(A, c, upper_tri, true)))
             return rownorms_tc_workspace_bytes(A, c, upper_tri);
-        return 0;
+        return rownorms_tc3_workspace_bytes(A, c, upper_tri);
     }
     return ws_round((size_t)A->d * A->d * 4);
 }
@@ -188,9 +200,22 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         return rownorms_tc_launch(A, B, c, (float)alpha, (float)beta, upper_tri, x, ws, flag, sm_count, st,
                                   min_tiles, (const uint8_t*)prepared);
     if (A->kind == LSK_DENSE) {
-        const unsigned grid = (unsigned)((n + RM - 1) / RM);
-        LSK_PROF("rownorm_dense_simt", st) rownorm_dense_kernel<<<grid, 256, 0, st>>>((const float*)A->values, A->ld, n, d, B, c,
-                                                   upper_tri ? 1 : 0, (float)alpha, (float)beta, x);
+        // the tensor-core kernel where A is large enough (then this one does the
+        // rows it leaves), else CUDA cores for all
+        const int *list = nullptr, *count = nullptr;
+        cudaError_t e = cudaSuccess;
+        const bool tc3 = rownorms_tc3_launch(A, B, c, (float)alpha, (float)beta, upper_tri ? 1 : 0, x, ws, flag, st,
+                                             &list, &count, &e);
+        if (e != cudaSuccess) return e;
+        const unsigned tiles = (unsigned)((n + RM - 1) / RM);
+        if (tc3) {
+            const unsigned grid = std::min(tiles, 4u * (unsigned)sm_count);
+            LSK_PROF("rownorm_dense_simt", st) rownorm_dense_kernel<true><<<grid, 256, 0, st>>>(
+                (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, list, count);
+        } else {
+            LSK_PROF("rownorm_dense_simt", st) rownorm_dense_kernel<false><<<tiles, 256, 0, st>>>(
+                (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, nullptr, nullptr);
+        }
     } else {
         float* M = prepared ? (float*)prepared : (float*)ws;   // prepared: built by bbt_group_launch
         const dim3 bg((unsigned)((d + 15) / 16), (unsigned)((d + 15) / 16));

@@ -1,0 +1,554 @@
+// rownorms_tc3.cu -- row norms x_i = alpha ||A_i B||^2 + beta x_i to FP32
+// accuracy on tcgen05 (dense A, d <= 256).
+//
+// A and B are scaled by powers of two, columns of A by s_j and columns of B
+// by 1 / t_l with the rows of B taking 1 / s_j, so that a typical entry of A
+// is about 2^10 and the largest of each column of B 128 .. 256.  Each scaled
+// entry is then split into three bf16 terms,
+//     y = hi + mid + lo,   hi = the bf16 rounding of the nearest integer,
+// so that the products hi hi are whole numbers: their sum over K <= 256 is
+// exact in the FP32 accumulator while it stays below 2^24, which the tensor
+// pipe (it rounds toward zero) would otherwise spoil by some 2^-19.  The
+// products hi mid, mid hi, hi lo, lo hi and mid mid, 2^-8 of the first or less,
+// go to a second accumulator; (acc0 + acc1) t_l is squared and summed in the
+// epilogue.  (Ozaki, Ogita, Oishi & Rump, Numer. Algorithms 59, 2012, with the
+// first slice on a fixed grid.)
+//
+// That holds for rows within a factor of about 30 of the typical row: a row whose
+// acc1 is not small against acc0, whose acc0 reaches 2^24 or whose sum is not
+// finite is put on a list, and the CUDA-core kernel does the listed rows.
+//
+// One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
+// half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
+// 24 KB stages (128 rows x 32 K, three slices).  Warps: 0-7 epilogue (two per
+// TMEM lane quarter), 8 MMA issue (even CTA), 9-19 converters (64-row pieces:
+// 16-byte loads, scale, split, 64-byte-swizzled stores).  Up to 128 columns
+// the accumulators are double-buffered.  750,001 x 200 times 200 x 200:
+// 0.41 ms against 1.98 on CUDA cores; errors 4.5e-8 (root mean square, relative)
+// against 6.8e-8, 2e-7 at most against 3.5e-7.
+#include "tc_common.cuh"
+
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
+
+namespace {
+
+constexpr int kRows = 128, kKC = 32, kMaxQ = 8;
+constexpr int kEpiWarps = 8, kMmaWarp = 8, kConv0 = 9, kConvWarps = 11;
+constexpr int kThreads = (kConv0 + kConvWarps) * 32;
+constexpr uint32_t kSlice = kRows * kKC * 2;          // one bf16 tile of a stage: 8 KB
+constexpr uint32_t kStage = 3 * kSlice;
+constexpr int kMaxStages = 8, kMinStages = 3;
+constexpr size_t kSmemLimit = 232448;
+constexpr uint32_t kTail = 1024;                      // barriers
+constexpr uint32_t kXchg = 4 * kRows * 4;             // the epilogue halves' exchange
+constexpr size_t kExtra = 1024 + kTail + 2 * 256 * 4 + kXchg;
+constexpr int kSampleGroups = 64, kSampleRows = 8;
+
+struct Rn3Params {
+    const float* A;
+    int64_t lda, n;
+    float* x;
+    float alpha, beta;
+    int d, c, nq, npad, ntiles, stages, nbuf;
+    uint32_t n0[kMaxQ], nn[kMaxQ], hoff[kMaxQ];
+    uint32_t hb;              // bytes of one slice of a CTA's half of B
+    const uint8_t* img;       // [half][slice][hb]
+    const float *s, *t;       // column scales of A, result scales of B's columns
+    int *list, *count;        // rows left to the CUDA-core kernel
+    int* flag;
+};
+
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(min(max(e, -126), 127) + 127) << 23); }
+__device__ __forceinline__ int exponent(float v) { return (int)(__float_as_uint(v) >> 23) - 127; }   // v > 0
+
+// s_j: 2^10 over the power of two below the median, over 64 groups of 8
+// consecutive rows spread over A, of the largest |a_ij| (a few outlying rows
+// do not move it; a column that is mostly zero takes its largest).
+__global__ void __launch_bounds__(256) rn3_units_kernel(const float* __restrict__ A, int64_t lda, int64_t n, int d,
+                                                        float* __restrict__ s, int* __restrict__ count) {
+    __shared__ float gm[kSampleGroups][33];
+    __shared__ float med[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = (int)blockIdx.x * 32 + lane;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
+    for (int g = w; g < kSampleGroups; g += 8) {
+        const int64_t r0 = (n - kSampleRows) * g / (kSampleGroups - 1);
+        float v[kSampleRows], m = 0.f;
+#pragma unroll
+        for (int i = 0; i < kSampleRows; ++i) v[i] = j < d ? __ldg(A + (r0 + i) * lda + j) : 0.f;
+#pragma unroll
+        for (int i = 0; i < kSampleRows; ++i) m = fmaxf(m, fabsf(v[i]));
+        gm[g][lane] = m;
+    }
+    __syncthreads();
+    float mx = 0.f;
+    for (int g = 0; g < kSampleGroups; ++g) mx = fmaxf(mx, gm[g][lane]);
+    for (int g = w; g < kSampleGroups; g += 8) {
+        const float v = gm[g][lane];
+        int rank = 0;
+        for (int h = 0; h < kSampleGroups; ++h) rank += gm[h][lane] < v || (gm[h][lane] == v && h < g);
+        if (rank == kSampleGroups / 2) med[lane] = v;
+    }
+    __syncthreads();
+    if (w == 0 && j < 256) {
+        const float m = med[lane] > 0.f ? med[lane] : mx;
+        s[j] = (m > 0.f && m <= 3.402823466e38f) ? pow2f(10 - exponent(m)) : 1.f;
+    }
+}
+
+// scaled value y (an integer part below 2^24) as hi + mid + lo
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ uint32_t to_bf16x2(float2 v) {   // v.x in the low half
+    uint32_t h;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(v.y), "f"(v.x));
+    return h;
+}
+__device__ __forceinline__ float2 neg_bf16x2(uint32_t h) {
+    return make_float2(-__uint_as_float(h << 16), -__uint_as_float(h & 0xFFFF0000u));
+}
+__device__ __forceinline__ void split3(float2 y, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    constexpr float kMagic = 12582912.f;   // 1.5 * 2^23: y + magic has the nearest integer in its low bits
+    hi = to_bf16x2(add2(add2(y, make_float2(kMagic, kMagic)), make_float2(-kMagic, -kMagic)));
+    const float2 r = add2(y, neg_bf16x2(hi));
+    mid = to_bf16x2(r);
+    lo = to_bf16x2(add2(r, neg_bf16x2(mid)));
+}
+
+// The image of B: 8 columns a block.  Column l (0-based in this pass, column
+// c0 + l of B) is scaled so that its largest |b_jl| / s_j is in [128, 256).
+__global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict__ B, int ldb, int c0, const Rn3Params p,
+                                                        uint8_t* __restrict__ img, float* __restrict__ t) {
+    __shared__ float red[32][9];
+    const int col = threadIdx.x & 7, part = threadIdx.x >> 3, l = (int)blockIdx.x * 8 + col;
+    float m = 0.f;
+    if (l < p.c)
+        for (int j = part; j < p.d; j += 32) m = fmaxf(m, fabsf(__ldg(B + (int64_t)j * ldb + c0 + l)) / p.s[j]);
+    red[part][col] = m;
+    __syncthreads();
+    for (int k = 0; k < 32; ++k) m = fmaxf(m, red[k][col]);
+    const int e = (m > 0.f && m <= 3.402823466e38f) ? exponent(m) : 0;
+    const float f = pow2f(7 - e);
+    if (part == 0) t[l] = pow2f(e - 7);
+    for (int i = part; i < p.nq * (kKC / 2); i += 32) {
+        const int q = i / (kKC / 2), kl = (i % (kKC / 2)) * 2, r = l - (int)p.n0[q];
+        if (r < 0) continue;
+        const int k = kKC * q + kl;
+        const float b0 = (k < p.d && l < p.c) ? __ldg(B + (int64_t)k * ldb + c0 + l) / p.s[k] * f : 0.f;
+        const float b1 = (k + 1 < p.d && l < p.c) ? __ldg(B + (int64_t)(k + 1) * ldb + c0 + l) / p.s[k + 1] * f : 0.f;
+        uint32_t w[3];
+        split3(make_float2(b0, b1), w[0], w[1], w[2]);
+        const int hn = (int)p.nn[q] / 2, h = r / hn;
+        const uint32_t off = (uint32_t)h * 3 * p.hb + p.hoff[q] + tc::sw64_offset((uint32_t)(r - h * hn), (uint32_t)kl);
+#pragma unroll
+        for (int z = 0; z < 3; ++z) *reinterpret_cast<uint32_t*>(img + off + (uint32_t)z * p.hb) = w[z];
+    }
+}
+
+// Lane l: float4 number l + 32 i of a 64-row x 32-column piece (row l / 8 + 4 i,
+// columns 4 (l % 8) ..).
+template <bool VEC>
+__device__ __forceinline__ void load_piece(const Rn3Params& p, int64_t row0, int q, int lane, float4 (&v)[16]) {
+    const int k = kKC * q + 4 * (lane & 7);
+    const int64_t r0 = row0 + (lane >> 3);
+    if (VEC && row0 + 64 <= p.n && kKC * q + kKC <= p.d) {
+        const float* src = p.A + r0 * p.lda + k;
+        const int64_t step = 4 * p.lda;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+                         : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w) : "l"(src));
+            src += step;
+        }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t row = r0 + 4 * i;
+        if (row >= p.n || k >= p.d) continue;
+        const float* src = p.A + row * p.lda + k;
+        if (VEC) {   // d a multiple of 4: the quad is whole
+            v[i] = __ldg(reinterpret_cast<const float4*>(src));
+        } else {
+            v[i].x = __ldg(src);
+            if (k + 1 < p.d) v[i].y = __ldg(src + 1);
+            if (k + 2 < p.d) v[i].z = __ldg(src + 2);
+            if (k + 3 < p.d) v[i].w = __ldg(src + 3);
+        }
+    }
+}
+
+// Scale, split and store the piece: rows 64 half + l / 8 + 4 i of the stage's
+// K-major 64-byte-swizzled tiles (two base offsets a lane, as the swizzle phase
+// of a row depends on i's parity alone).
+__device__ __forceinline__ void store_piece(uint8_t* stage, int half, int lane, float4 s, const float4 (&v)[16]) {
+    const uint32_t l8 = (uint32_t)lane >> 3, c4 = (uint32_t)lane & 7u;
+    const uint32_t lane_part = (uint32_t)half * 4096u + l8 * 64u + (c4 & 1u) * 8u;
+    uint8_t* const even = stage + lane_part + ((((c4 >> 1) ^ (l8 >> 1)) & 3u) << 4);
+    uint8_t* const odd = stage + lane_part + 256u + ((((c4 >> 1) ^ (2u + (l8 >> 1))) & 3u) << 4);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        uint2 hi, mid, lo;
+        split3(mul2(make_float2(v[i].x, v[i].y), make_float2(s.x, s.y)), hi.x, mid.x, lo.x);
+        split3(mul2(make_float2(v[i].z, v[i].w), make_float2(s.z, s.w)), hi.y, mid.y, lo.y);
+        uint8_t* const dst = ((i & 1) ? odd : even) + (i >> 1) * 512;
+        *reinterpret_cast<uint2*>(dst) = hi;
+        *reinterpret_cast<uint2*>(dst + kSlice) = mid;
+        *reinterpret_cast<uint2*>(dst + 2 * kSlice) = lo;
+    }
+}
+
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    int ok = 0;
+    if ((threadIdx.x & 31) == 0) ok = tc::mbar_wait(bar, parity, abort) ? 1 : 0;
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+template <bool VEC>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm_tc3_kernel(const Rn3Params p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int S = p.stages;
+    const uint32_t rank = tc::cluster_ctarank();
+    const int cid = (int)tc::cluster_id_x(), ncl = (int)tc::nclusters_x();
+    uint8_t* sB = smem + S * kStage;                       // this CTA's half of B: three slices
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + 3 * p.hb);
+    uint64_t* full = bars;                       // [S] even CTA: stage filled in both CTAs (4 arrivals)
+    uint64_t* empty = bars + kMaxStages;         // [S] stage consumed (multicast commit)
+    uint64_t* tfull = bars + 2 * kMaxStages;     // [2] accumulators done (multicast commit)
+    uint64_t* tempty = tfull + 2;                // [2] even CTA: accumulators read in both (16 arrivals)
+    uint64_t* fin = tfull + 4;                   // all MMAs complete (multicast commit)
+    uint64_t* xfull = fin + 1;                   // [4 quarters][4] second half's sums written (1 arrival)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xfull + 16);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int* stored = const_cast<int*>(abort) + 1;   // [S] pieces stored per stage (in use order)
+    float* ss = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTail);   // [256] column scales of A
+    float* ts = ss + 256;                                                              // [256] result scales
+    float* xchg = ts + 256;                                                            // [4][128]
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            tc::mbar_init(full + s, 4);
+            tc::mbar_init(empty + s, 1);
+            stored[s] = 0;
+        }
+        for (int a = 0; a < 2; ++a) {
+            tc::mbar_init(tfull + a, 1);
+            tc::mbar_init(tempty + a, 2 * kEpiWarps);
+        }
+        tc::mbar_init(fin, 1);
+        for (int k = 0; k < 16; ++k) tc::mbar_init(xfull + k, 1);
+        *abort = 0;
+        tc::fence_mbar_init();
+    }
+    for (int j = threadIdx.x; j < 256; j += kThreads) {
+        ss[j] = p.s[j];
+        ts[j] = j < p.npad ? p.t[j] : 0.f;
+    }
+    if (warp == kMmaWarp) {
+        tc::tmem_alloc_pair(tmem_slot, 512u);
+        tc::tmem_relinquish_pair();
+    }
+    {   // this CTA's half of B
+        const uint4* src = reinterpret_cast<const uint4*>(p.img + (size_t)rank * 3 * p.hb);
+        uint4* dst = reinterpret_cast<uint4*>(sB);
+        const uint32_t n16 = (3 * p.hb) >> 4;
+        for (uint32_t i = threadIdx.x; i < n16; i += kThreads) dst[i] = __ldg(src + i);
+    }
+    tc::fence_proxy_async_smem();
+    tc::fence_before_sync();
+    tc::cluster_sync();   // barriers of both CTAs initialised, B halves in place
+    tc::fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+    const int my_tiles = (cid < p.ntiles) ? (p.ntiles - 1 - cid) / ncl + 1 : 0;
+    const uint32_t acc1 = p.nbuf == 2 ? 128u : 256u;   // the second accumulator's column
+
+    if (warp < kEpiWarps) {
+        // ------------------------------------------------------------ epilogue
+        // quarter warp % 4 of the rows; half warp / 4: column blocks of 32 of its parity
+        const int quarter = warp & 3, half = warp >> 2, lr = quarter * 32 + lane;
+        for (int i = 0; i < my_tiles; ++i) {
+            const int b = p.nbuf == 2 ? i & 1 : 0;
+            const uint32_t par = (uint32_t)(p.nbuf == 2 ? i >> 1 : i) & 1u;
+            if (!warp_wait(tfull + b, par, abort)) break;
+            tc::fence_after_sync();
+            const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + 256u * (uint32_t)b;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s0 = 0.f, s1 = 0.f, mx = 0.f;
+            for (int col = 32 * half; col < p.npad; col += 64) {
+                uint32_t v0[32], v1[32];
+                tc::tmem_ld_32x32b_x32(taddr + (uint32_t)col, v0);
+                tc::tmem_ld_32x32b_x32(taddr + acc1 + (uint32_t)col, v1);
+                tc::tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    const float a0 = __uint_as_float(v0[e]), a1 = __uint_as_float(v1[e]);
+                    const float y = (a0 + a1) * ts[col + e];
+                    sum[e & 3] = fmaf(y, y, sum[e & 3]);
+                    mx = fmaxf(mx, fabsf(a0));
+                    if (e & 1) {
+                        s0 = fmaf(a0, a0, s0);
+                        s1 = fmaf(a1, a1, s1);
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) {
+                if (rank == 0) tc::mbar_arrive(tempty + b);
+                else tc::mbar_arrive_cluster(tempty + b, 0);
+            }
+            float tot = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            // outside the split's range: NaN, which no sum within it is
+            if (!(s1 <= 9.765625e-4f * s0 && mx < 16777216.f)) tot = __uint_as_float(0x7FC00000u);
+            // The second half's sum goes to the first through shared memory.
+            // Four cells a row: the second half is at most two tiles ahead (the
+            // MMAs of a tile wait for both halves of the one two before).
+            float* const cell = xchg + (i & 3) * kRows + lr;
+            uint64_t* const xbar = xfull + 4 * quarter + (i & 3);
+            if (half == 1) {
+                *cell = tot;
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(xbar);
+            } else {
+                if (!warp_wait(xbar, (uint32_t)(i >> 2) & 1u, abort)) break;
+                tot += *cell;
+                const int64_t row = ((int64_t)cid + (int64_t)i * ncl) * (2 * kRows) + rank * kRows + lr;
+                if (row < p.n) {
+                    if (tot <= 3.402823466e38f) p.x[row] = (p.beta != 0.f) ? fmaf(p.alpha, tot, p.beta * p.x[row]) : p.alpha * tot;
+                    else p.list[atomicAdd(p.count, 1)] = (int)row;
+                }
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        // ------------------------------------------------------------ MMA issue (even CTA)
+        // the whole warp goes along, one elected lane issues (uniform descriptors)
+        if (rank == 0) {
+            const uint64_t da0 = tc::desc_sw64_kmajor(tc::smem_u32(smem)), db0 = tc::desc_sw64_kmajor(tc::smem_u32(sB));
+            bool ok = true;
+            int s = 0;
+            uint32_t ph = 0;
+            for (int i = 0; i < my_tiles && ok; ++i) {
+                const int b = p.nbuf == 2 ? i & 1 : 0;
+                const uint32_t par = (uint32_t)(p.nbuf == 2 ? i >> 1 : i) & 1u;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait_cluster(tempty + b, par ^ 1u, abort));
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t d0 = tmem + 256u * (uint32_t)b;
+#pragma unroll
+                for (int q = 0; q < kMaxQ; ++q) {
+                    if (q >= p.nq) break;
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait_cluster(full + s, ph, abort));
+                    if (!ok) break;
+                    tc::fence_after_sync();
+                    if (tc::elect_one()) {
+                        const uint32_t idesc = tc::idesc_bf16_f32(2 * kRows, p.nn[q]);
+                        const uint32_t t0 = d0 + p.n0[q], t1 = t0 + acc1;
+                        const uint64_t as = da0 + ((uint32_t)s * kStage >> 4), bs = db0 + (p.hoff[q] >> 4);
+                        constexpr int kPA[6] = {0, 0, 1, 0, 2, 1}, kPB[6] = {0, 1, 0, 2, 0, 1};
+#pragma unroll
+                        for (int kk = 0; kk < kKC / 16; ++kk)
+#pragma unroll
+                            for (int z = 0; z < 6; ++z)
+                                tc::mma_bf16_pair(z ? t1 : t0, as + ((kPA[z] * kSlice + 32u * kk) >> 4),
+                                                  bs + ((kPB[z] * p.hb + 32u * kk) >> 4), idesc,
+                                                  z < 2 ? (q | kk) != 0 : 1);
+                        tc::mma_commit_pair(empty + s);
+                        if (q + 1 == p.nq) tc::mma_commit_pair(tfull + b);
+                    }
+                    __syncwarp();
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            if (tc::elect_one()) tc::mma_commit_pair(fin);
+            __syncwarp();
+        }
+        if (lane == 0) {
+            // both CTAs: the last multicast commit has landed here, so no
+            // arrival is still on its way when the CTA leaves
+            volatile int never = 0;
+            tc::mbar_wait(fin, 0, &never);
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------------ converters
+        // piece pc: half pc % 2 of chunk g = pc / 2 = (tile g / nq, K-chunk g % nq);
+        // the uses of each stage are claimed in piece order (stored[s])
+        const int G = my_tiles * p.nq;
+        float4 v[16];
+        for (int pc = warp - kConv0; pc < 2 * G; pc += kConvWarps) {
+            const int g = pc >> 1, half = pc & 1, t = g / p.nq, q = g - t * p.nq, u = g / S, s = g - u * S;
+            load_piece<VEC>(p, ((int64_t)cid + (int64_t)t * ncl) * (2 * kRows) + rank * kRows + half * 64, q, lane, v);
+            const float4 sc = *reinterpret_cast<const float4*>(ss + kKC * q + 4 * (lane & 7));
+            int ok = 1;
+            if (lane == 0)
+                ok = tc::counter_wait(reinterpret_cast<volatile int*>(stored + s), 2 * u, abort) &&
+                     tc::mbar_wait(empty + s, ((uint32_t)u & 1u) ^ 1u, abort);
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            store_piece(smem + (size_t)s * kStage, half, lane, sc, v);
+            tc::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                if (rank == 0) tc::mbar_arrive(full + s);
+                else tc::mbar_arrive_cluster(full + s, 0);
+                atomicAdd(stored + s, 1);
+            }
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::cluster_sync();   // no CTA leaves while its peer may still arrive on its barriers
+    if (warp == kMmaWarp) {
+        tc::fence_after_sync();
+        tc::tmem_dealloc_pair(tmem, 512u);
+    }
+    if (threadIdx.x == 0 && *abort) set_flag(p.flag, LSK_FLAG_TIMEOUT);
+}
+
+// Columns c0 .. c0 + c of B in one pass; false if B's image leaves no ring.
+bool pass_plan(int64_t d, int64_t c, int upper_tri, Rn3Params& p) {
+    p.d = (int)d;
+    p.c = (int)c;
+    p.nq = (int)((d + kKC - 1) / kKC);
+    p.npad = (int)((c + 31) / 32) * 32;
+    p.nbuf = p.npad <= 128 ? 2 : 1;
+    uint32_t off = 0;
+    for (int q = 0; q < kMaxQ; ++q) {
+        p.n0[q] = (upper_tri && q < p.nq) ? (uint32_t)(kKC * q) : 0u;
+        p.nn[q] = q < p.nq ? (uint32_t)p.npad - p.n0[q] : 0u;
+        p.hoff[q] = off;
+        off += (p.nn[q] / 2) * (kKC * 2);
+    }
+    p.hb = off;
+    const int64_t room = (int64_t)kSmemLimit - (int64_t)kExtra - 3 * (int64_t)p.hb;
+    p.stages = (int)std::min<int64_t>(kMaxStages, room / (int64_t)kStage);
+    return p.stages >= kMinStages;
+}
+size_t smem_of(const Rn3Params& p) { return (size_t)p.stages * kStage + 3 * (size_t)p.hb + kExtra; }
+
+// passes over A (0: not this kernel) and the columns of each
+int passes_of(const lsk_mat* A, int64_t c, int upper_tri, double beta, int64_t* per) {
+    if (A->kind != LSK_DENSE || A->d < 1 || A->d > 256 || c < 1 || c > 256) return 0;
+    // below this the CUDA-core kernel's one launch is shorter than the scales,
+    // the image and the ring's set-up (at 2^30: 40 against 50 us at 65,537 x 128 x
+    // 128 triangular, 50 against 62 at 262,145 x 64 x 64, 60 against 77 at 17,000 x
+    // 256 x 256)
+    if (A->n * A->d * c < (int64_t)1 << 30) return 0;
+    Rn3Params p{};
+    *per = c;
+    if (pass_plan(A->d, c, upper_tri, p)) return 1;
+    // a wide general B goes in two halves; the second adds to x, which a listed
+    // row's recomputation could not take back
+    if (upper_tri || beta != 0.0) return 0;
+    *per = (c / 2 + 31) / 32 * 32;
+    return pass_plan(A->d, *per, 0, p) ? 2 : 0;
+}
+
+size_t image_bytes(const lsk_mat* A, int64_t c, int upper_tri) {
+    Rn3Params p{};
+    pass_plan(A->d, c, upper_tri, p);
+    return ws_round(6 * (size_t)p.hb);
+}
+
+// clusters that fit on the device at once (cached per device, kernel and size)
+int pair_clusters(bool vec, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, bool, size_t>, int> cache;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_tuple(dev, vec, smem);
+    const auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    const void* fn = vec ? (const void*)rownorm_tc3_kernel<true> : (const void*)rownorm_tc3_kernel<false>;
+    int n = 0;
+    if (allow_dynamic_smem(fn) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2, 1, 1);
+        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) n = 0;
+    }
+    cudaGetLastError();
+    cache[key] = n;
+    return n;
+}
+
+}  // namespace
+
+size_t rownorms_tc3_workspace_bytes(const lsk_mat* A, int64_t c, int upper_tri) {
+    int64_t per = 0;
+    const int np = passes_of(A, c, upper_tri, 0.0, &per);
+    if (!np) return 0;
+    return image_bytes(A, per, upper_tri) + 2 * ws_round(256 * 4) + ws_round((size_t)np * A->n * 4) + ws_round(4);
+}
+
+// False: not this kernel's shape.  True: launched (*e its status); rows
+// list[0 .. *count) of x are then left to the caller.
+bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alpha, float beta, int upper_tri, float* x,
+                         void* ws, int* flag, cudaStream_t st, const int** list, const int** count, cudaError_t* e) {
+    int64_t per = 0;
+    const int np = passes_of(A, c, upper_tri, beta, &per);
+    if (!np) return false;
+    const bool vec = (A->d % 4 == 0) && (A->ld % 4 == 0) && (((uintptr_t)A->values & 15) == 0);
+    WsCarver wc{(char*)ws, 0};
+    uint8_t* img = wc.take<uint8_t>(image_bytes(A, per, upper_tri));
+    float* s = wc.take<float>(256);
+    float* t = wc.take<float>(256);
+    int* rows = wc.take<int>((size_t)np * A->n);
+    int* cnt = wc.take<int>(1);
+    LSK_PROF("rownorm_tc_prep", st) rn3_units_kernel<<<8, 256, 0, st>>>((const float*)A->values, A->ld, A->n, (int)A->d, s, cnt);
+    for (int k = 0; k < np; ++k) {
+        Rn3Params p{};
+        const int64_t c0 = k * per, ck = std::min<int64_t>(per, c - c0);
+        if (!pass_plan(A->d, ck, upper_tri, p)) {
+            *e = cudaErrorNotSupported;
+            return true;
+        }
+        p.A = (const float*)A->values;
+        p.lda = A->ld;
+        p.n = A->n;
+        p.x = x;
+        p.alpha = alpha;
+        p.beta = k ? 1.f : beta;
+        p.ntiles = (int)((A->n + 2 * kRows - 1) / (2 * kRows));
+        p.img = img;
+        p.s = s;
+        p.t = t;
+        p.list = rows;
+        p.count = cnt;
+        p.flag = flag;
+        const size_t smem = smem_of(p);
+        const int ncl = std::min(p.ntiles, pair_clusters(vec, smem));
+        if (ncl <= 0) {
+            if (k == 0) return false;
+            *e = cudaErrorNotSupported;
+            return true;
+        }
+        LSK_PROF("rownorm_tc_prep", st) rn3_image_kernel<<<p.npad / 8, 256, 0, st>>>(B, (int)c, (int)c0, p, img, t);
+        if (vec)
+            LSK_PROF("rownorm_dense_tc3", st) rownorm_tc3_kernel<true><<<2 * ncl, kThreads, smem, st>>>(p);
+        else
+            LSK_PROF("rownorm_dense_tc3", st) rownorm_tc3_kernel<false><<<2 * ncl, kThreads, smem, st>>>(p);
+    }
+    *list = rows;
+    *count = cnt;
+    *e = cudaGetLastError();
+    return true;
+}
