@@ -264,51 +264,52 @@ __global__ void __launch_bounds__(SH::kThreads, 1) gram_tc_kernel(const GrParams
             if (!put(pc, v)) break;
         }
     } else if (warp == kMmaWarp) {
-        if (lane == 0) {
-            const uint32_t base = tc::smem_u32(stages);
-            bool okm = true;
-            int s = 0;
-            uint32_t ph = 0;
-            for (int z = 0; z < my_slices && okm; ++z) {
-                const int64_t r_begin = ((int64_t)blockIdx.x + (int64_t)z * gridDim.x) * kSliceRows;
-                const int64_t r_end = min(p.n, r_begin + kSliceRows);
-                const int nchunks = (int)((r_end - r_begin + kKC - 1) / kKC);
-                // the previous slice's accumulator has been read out
-                if (z > 0 && !tc::mbar_wait(drained, (uint32_t)(z - 1) & 1u, abort)) break;
+        // the whole warp goes along and an elected lane issues, so that the
+        // descriptors stay in uniform registers
+        const uint64_t d0 = tc::desc_sw128_mnmajor(tc::smem_u32(stages), 1024u, kSbo(NPAD));
+        bool okm = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int z = 0; z < my_slices && okm; ++z) {
+            const int64_t r_begin = ((int64_t)blockIdx.x + (int64_t)z * gridDim.x) * kSliceRows;
+            const int64_t r_end = min(p.n, r_begin + kSliceRows);
+            const int nchunks = (int)((r_end - r_begin + kKC - 1) / kKC);
+            // the previous slice's accumulator has been read out
+            if (z > 0) okm = __all_sync(0xffffffffu, tc::mbar_wait(drained, (uint32_t)(z - 1) & 1u, abort));
+            tc::fence_after_sync();
+            for (int g = 0; g < nchunks && okm; ++g) {
+                okm = __all_sync(0xffffffffu, tc::mbar_wait(full + s, ph, abort));
+                if (!okm) break;
                 tc::fence_after_sync();
-                for (int g = 0; g < nchunks; ++g) {
-                    if (!tc::mbar_wait(full + s, ph, abort)) {
-                        okm = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t hi = base + (uint32_t)s * sbytes, lo = hi + half_bytes(NPAD);
+                if (tc::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < kKC / 16; ++kk) {
-                        const uint32_t ko = 2u * kSbo(NPAD) * kk;   // 16 rows = two 8-row groups
+                        // 16 rows = two 8-row groups
+                        const uint64_t dk = d0 + (((uint32_t)s * sbytes + 2u * kSbo(NPAD) * kk) >> 4);
+#pragma unroll
                         for (int t = 0; t < ntiles; ++t) {
-                            const uint32_t off = (uint32_t)t * 2048u + ko;   // columns from 128 t
                             const uint32_t idesc = tc::idesc_bf16_f32_mn(128, (uint32_t)(NPAD - t * kMT));
                             const uint32_t dt = tmem + 256u * t;
-                            const uint64_t dh = tc::desc_sw128_mnmajor(hi + off, 1024u, kSbo(NPAD));
-                            const uint64_t dl = tc::desc_sw128_mnmajor(lo + off, 1024u, kSbo(NPAD));
+                            const uint64_t dh = dk + (t * 2048u >> 4), dl = dh + (half_bytes(NPAD) >> 4);   // columns from 128 t
                             tc::mma_bf16(dt, dh, dh, idesc, (g | kk) != 0);
                             tc::mma_bf16(dt, dh, dl, idesc, 1);
                             tc::mma_bf16(dt, dl, dh, idesc, 1);
                         }
                     }
                     tc::mma_commit(empty + s);
-                    if (++s == kStages) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                    if (g + 1 == nchunks) tc::mma_commit(done);
                 }
-                if (okm) tc::mma_commit(done);
+                __syncwarp();
+                if (++s == kStages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            tc::mma_commit(fin);
-            volatile int never = 0;
-            tc::mbar_wait(fin, 0, &never);
         }
+        if (tc::elect_one()) tc::mma_commit(fin);
+        __syncwarp();
+        volatile int never = 0;
+        tc::mbar_wait(fin, 0, &never);
         __syncwarp();
     } else if (warp - kEpi0 < nepi) {
         // epilogue warp e: TMEM lane quarter q = warp % 4, accumulators
@@ -325,7 +326,8 @@ __global__ void __launch_bounds__(SH::kThreads, 1) gram_tc_kernel(const GrParams
             for (int t = e >> 2; t < ntiles; t += nepi >> 2) {
                 const int row = t * kMT + q * 32 + lane;   // column a of A
                 const int ncols = NPAD - t * kMT;        // columns b = t*128 .. npad-1
-                float* dst = p.part + ((int64_t)blockIdx.x * NPAD + row) * NPAD + t * kMT;
+                // by columns: a warp's 32 rows are one 128-byte line
+                float* dst = p.part + ((int64_t)blockIdx.x * NPAD + t * kMT) * NPAD + row;
                 // 64 columns per TMEM round trip (ncols is a multiple of 32)
                 for (int col = 0; col < ncols; col += 64) {
                     uint32_t va[32], vb[32];
@@ -341,14 +343,10 @@ __global__ void __launch_bounds__(SH::kThreads, 1) gram_tc_kernel(const GrParams
                     }
                     if (row < p.d) {
 #pragma unroll
-                        for (int k = 0; k < 64; k += 4) {
-                            const uint32_t* w = k < 32 ? va + k : vb + (k - 32);
+                        for (int k = 0; k < 64; ++k)
                             if (k < 32 || two)
-                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + col + k),
-                                             "f"(__uint_as_float(w[0])), "f"(__uint_as_float(w[1])),
-                                             "f"(__uint_as_float(w[2])), "f"(__uint_as_float(w[3]))
-                                             : "memory");
-                        }
+                                asm volatile("red.global.add.f32 [%0], %1;" ::"l"(dst + (int64_t)(col + k) * NPAD),
+                                             "f"(__uint_as_float(k < 32 ? va[k] : vb[k - 32])) : "memory");
                     }
                 }
             }
@@ -370,13 +368,13 @@ __global__ void gram_tc_reduce_kernel(const float* __restrict__ part, int slices
     const int64_t len = (int64_t)d * d, plen = (int64_t)npad * npad;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
-        int a = (int)(e / d), b = (int)(e % d);
+        int b = (int)(e / d), a = (int)(e % d);   // C[b][a] (symmetric)
         if (a > b) {
             const int t = a;
             a = b;
             b = t;
         }
-        const int64_t idx = (int64_t)a * npad + b;
+        const int64_t idx = (int64_t)b * npad + a;   // the partial's columns, a <= b
         float s = 0.f, c = 0.f;
         for (int z = 0; z < slices; ++z) {
             const float x = part[(int64_t)z * plen + idx];

@@ -314,53 +314,54 @@ __global__ void __launch_bounds__(kThreads, 1) rownorm_tc_kernel(const RnParams 
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------ MMA issue
-        if (lane == 0) {
-            // One thread issues everything, so its per-chunk instruction chain
-            // is on the critical path: stage and phase advance incrementally
-            // (no division), and the K-chunk loop is unrolled so the per-chunk
-            // constants of p are read with static indices (no local copy).
-            const uint32_t sA_u32 = tc::smem_u32(sA), sB_u32 = tc::smem_u32(sB);
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
-            for (int i = 0; i < my_tiles && ok; ++i) {
-                const int acc = i & 1;
-                if (!tc::mbar_wait(tempty + acc, ((uint32_t)(i >> 1) & 1u) ^ 1u, abort)) break;
-                tc::fence_after_sync();
-                const uint32_t d_base = tmem + (uint32_t)acc * kAccCols;
+        // One thread issues everything, so its per-chunk instruction chain is on
+        // the critical path: the whole warp goes along and an elected lane
+        // issues (the descriptors then stay in uniform registers), stage and
+        // phase advance incrementally, and the K-chunk loop is unrolled so the
+        // per-chunk constants of p are read with static indices.
+        const uint64_t da0 = tc::desc_sw64_kmajor(tc::smem_u32(sA)), db0 = tc::desc_sw64_kmajor(tc::smem_u32(sB));
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < my_tiles && ok; ++i) {
+            const int acc = i & 1;
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(tempty + acc, ((uint32_t)(i >> 1) & 1u) ^ 1u, abort));
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint32_t d_base = tmem + (uint32_t)acc * kAccCols;
 #pragma unroll
-                for (int q = 0; q < kMaxQ; ++q) {
-                    if (q >= p.nq) break;
-                    if (!tc::mbar_wait(full + s, ph, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t a_hi = sA_u32 + (uint32_t)s * kStageBytes, a_lo = a_hi + kHalfStage;
-                    const uint32_t b_hi = sB_u32 + p.boff[q], b_lo = b_hi + p.b_bytes;
+            for (int q = 0; q < kMaxQ; ++q) {
+                if (q >= p.nq) break;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(full + s, ph, abort));
+                if (!ok) break;
+                tc::fence_after_sync();
+                if (tc::elect_one()) {
+                    const uint64_t a_hi = da0 + ((uint32_t)s * kStageBytes >> 4), a_lo = a_hi + (kHalfStage >> 4);
+                    const uint64_t b_hi = db0 + (p.boff[q] >> 4), b_lo = b_hi + (p.b_bytes >> 4);
                     const uint32_t idesc = tc::idesc_bf16_f32(128, p.nn[q]);
                     const uint32_t d_tmem = d_base + p.n0[q];
 #pragma unroll
                     for (int kk = 0; kk < kKC / 16; ++kk) {
-                        const uint32_t ko = 32u * kk;   // 16 bf16 = 32 bytes along the swizzled row
-                        tc::mma_bf16(d_tmem, tc::desc_sw64_kmajor(a_hi + ko), tc::desc_sw64_kmajor(b_hi + ko), idesc,
-                                     (q | kk) != 0);
-                        tc::mma_bf16(d_tmem, tc::desc_sw64_kmajor(a_hi + ko), tc::desc_sw64_kmajor(b_lo + ko), idesc, 1);
-                        tc::mma_bf16(d_tmem, tc::desc_sw64_kmajor(a_lo + ko), tc::desc_sw64_kmajor(b_hi + ko), idesc, 1);
+                        const uint32_t ko = 2u * kk;   // 16 bf16 = 32 bytes along the swizzled row
+                        tc::mma_bf16(d_tmem, a_hi + ko, b_hi + ko, idesc, (q | kk) != 0);
+                        tc::mma_bf16(d_tmem, a_hi + ko, b_lo + ko, idesc, 1);
+                        tc::mma_bf16(d_tmem, a_lo + ko, b_hi + ko, idesc, 1);
                     }
                     tc::mma_commit(empty + s);
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                    if (q + 1 == p.nq) tc::mma_commit(tfull + acc);
                 }
-                if (ok) tc::mma_commit(tfull + acc);
+                __syncwarp();
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            // every MMA issued must be complete before TMEM is released
-            tc::mma_commit(fin);
-            volatile int never = 0;
-            tc::mbar_wait(fin, 0, &never);
         }
+        // every MMA issued must be complete before TMEM is released
+        if (tc::elect_one()) tc::mma_commit(fin);
+        __syncwarp();
+        volatile int never = 0;
+        tc::mbar_wait(fin, 0, &never);
         __syncwarp();
     } else {
         // ------------------------------------------------------------ converters
@@ -498,47 +499,48 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------ MMA issue (even CTA)
-        if (lane == 0 && rank == 0) {
-            const uint32_t sA_u32 = tc::smem_u32(sA), sB_u32 = tc::smem_u32(sB);
+        // (the whole warp goes along, an elected lane issues: uniform descriptors)
+        if (rank == 0) {
+            const uint64_t da0 = tc::desc_sw64_kmajor(tc::smem_u32(sA)), db0 = tc::desc_sw64_kmajor(tc::smem_u32(sB));
             bool ok = true;
             int s = 0;
             uint32_t ph = 0;
             for (int i = 0; i < my_tiles && ok; ++i) {
                 const int acc = i & 1;
-                if (!tc::mbar_wait_cluster(tempty + acc, ((uint32_t)(i >> 1) & 1u) ^ 1u, abort)) break;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait_cluster(tempty + acc, ((uint32_t)(i >> 1) & 1u) ^ 1u, abort));
+                if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t d_base = tmem + (uint32_t)acc * kAccCols;
 #pragma unroll
                 for (int q = 0; q < kMaxQ; ++q) {
                     if (q >= p.nq) break;
-                    if (!tc::mbar_wait_cluster(full + s, ph, abort)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait_cluster(full + s, ph, abort));
+                    if (!ok) break;
                     tc::fence_after_sync();
-                    const uint32_t a_hi = sA_u32 + (uint32_t)s * kStageBytes, a_lo = a_hi + kHalfStage;
-                    const uint32_t b_hi = sB_u32 + p.hoff[q], b_lo = b_hi + p.hb_bytes;
-                    const uint32_t idesc = tc::idesc_bf16_f32(2 * kRows, p.nn[q]);
-                    const uint32_t d_tmem = d_base + p.n0[q];
+                    if (tc::elect_one()) {
+                        const uint64_t a_hi = da0 + ((uint32_t)s * kStageBytes >> 4), a_lo = a_hi + (kHalfStage >> 4);
+                        const uint64_t b_hi = db0 + (p.hoff[q] >> 4), b_lo = b_hi + (p.hb_bytes >> 4);
+                        const uint32_t idesc = tc::idesc_bf16_f32(2 * kRows, p.nn[q]);
+                        const uint32_t d_tmem = d_base + p.n0[q];
 #pragma unroll
-                    for (int kk = 0; kk < kKC / 16; ++kk) {
-                        const uint32_t ko = 32u * kk;
-                        tc::mma_bf16_pair(d_tmem, tc::desc_sw64_kmajor(a_hi + ko), tc::desc_sw64_kmajor(b_hi + ko),
-                                          idesc, (q | kk) != 0);
-                        tc::mma_bf16_pair(d_tmem, tc::desc_sw64_kmajor(a_hi + ko), tc::desc_sw64_kmajor(b_lo + ko),
-                                          idesc, 1);
-                        tc::mma_bf16_pair(d_tmem, tc::desc_sw64_kmajor(a_lo + ko), tc::desc_sw64_kmajor(b_hi + ko),
-                                          idesc, 1);
+                        for (int kk = 0; kk < kKC / 16; ++kk) {
+                            const uint32_t ko = 2u * kk;
+                            tc::mma_bf16_pair(d_tmem, a_hi + ko, b_hi + ko, idesc, (q | kk) != 0);
+                            tc::mma_bf16_pair(d_tmem, a_hi + ko, b_lo + ko, idesc, 1);
+                            tc::mma_bf16_pair(d_tmem, a_lo + ko, b_hi + ko, idesc, 1);
+                        }
+                        tc::mma_commit_pair(empty + s);
+                        if (q + 1 == p.nq) tc::mma_commit_pair(tfull + acc);
                     }
-                    tc::mma_commit_pair(empty + s);
+                    __syncwarp();
                     if (++s == S) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
-                if (ok) tc::mma_commit_pair(tfull + acc);
             }
-            tc::mma_commit_pair(fin);
+            if (tc::elect_one()) tc::mma_commit_pair(fin);
+            __syncwarp();
         }
         if (lane == 0) {
             // both CTAs: the last multicast commit has landed here, so no
