@@ -32,39 +32,62 @@ constexpr int TT = 16;   // tile edge of the triangular pair products (16 x 16 o
 // FP32 Cholesky pieces: 32 x 32 tiles (CB) of the lower triangle.
 constexpr int CB = 32;
 
-// Unblocked Cholesky of one 32 x 32 tile by one warp, row `lane` in a[]:
-// compile-time recursion over (j, k) keeps every index static, so a[] stays
-// in registers (a nested #pragma unroll of this size is not fully unrolled).
-template <int J, int K>
-struct DiagUpdate {
-    static __device__ __forceinline__ void run(float (&a)[CB], float lij, int lane) {
-        const float lkj = __shfl_sync(0xffffffffu, lij, K);   // L[K][J] from lane K
-        if (K <= lane) a[K] -= lij * lkj;
-        DiagUpdate<J, K + 1>::run(a, lij, lane);
+// Cholesky of one 32 x 32 tile by one warp, row `lane` in a[], four pivots at a
+// time (compile-time recursion over the blocks keeps every index static, so
+// a[] stays in registers): the ten entries of a 4 x 4 pivot block are fetched
+// with independent shuffles and factored by every lane for itself, each lane
+// solves its row's four entries, and the rows meet through shared memory (one
+// 16-byte store, one broadcast load a row) for the rank-four update of the
+// columns behind.  One pivot at a time, with a shuffle for every update, the
+// tile took 6,500 cycles, on the critical path of every step.
+template <int J>
+struct DiagBlock {
+    // 1 / sqrt of a pivot (1 where it is not positive and finite, noted in bad);
+    // the pair correction absorbs the approximation's rounding
+    static __device__ __forceinline__ float pivot(float piv, bool& bad) {
+        const bool ok = piv > 0.f && piv <= 3.402823466e38f;
+        bad |= !ok;
+        float r;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(ok ? piv : 1.f));
+        return r;
     }
-};
-template <int J>
-struct DiagUpdate<J, CB> {
-    static __device__ __forceinline__ void run(float (&)[CB], float, int) {}
-};
-template <int J>
-struct DiagStep {
-    static __device__ __forceinline__ void run(float (&a)[CB], int lane, int* flag) {
-        float piv = __shfl_sync(0xffffffffu, a[J], J);
-        if (!(piv > 0.f) || !isfinite(piv)) {
-            if (lane == 0) set_flag(flag, LSK_FLAG_RANK_DEFICIENT);
-            piv = 1.f;
+    static __device__ __forceinline__ void run(float (&a)[CB], int lane, float4* rows, bool& bad) {
+        const unsigned m = 0xffffffffu;
+        const float p00 = __shfl_sync(m, a[J], J);
+        const float p10 = __shfl_sync(m, a[J], J + 1), p11 = __shfl_sync(m, a[J + 1], J + 1);
+        const float p20 = __shfl_sync(m, a[J], J + 2), p21 = __shfl_sync(m, a[J + 1], J + 2), p22 = __shfl_sync(m, a[J + 2], J + 2);
+        const float p30 = __shfl_sync(m, a[J], J + 3), p31 = __shfl_sync(m, a[J + 1], J + 3), p32 = __shfl_sync(m, a[J + 2], J + 3),
+                    p33 = __shfl_sync(m, a[J + 3], J + 3);
+        const float r0 = pivot(p00, bad);
+        const float l10 = p10 * r0, l20 = p20 * r0, l30 = p30 * r0;
+        const float r1 = pivot(fmaf(-l10, l10, p11), bad);
+        const float l21 = fmaf(-l20, l10, p21) * r1, l31 = fmaf(-l30, l10, p31) * r1;
+        const float r2 = pivot(fmaf(-l21, l21, fmaf(-l20, l20, p22)), bad);
+        const float l32 = fmaf(-l31, l21, fmaf(-l30, l20, p32)) * r2;
+        const float r3 = pivot(fmaf(-l32, l32, fmaf(-l31, l31, fmaf(-l30, l30, p33))), bad);
+        // the lane's row of the four columns (rows above the block are not read again)
+        const float x0 = a[J] * r0;
+        const float x1 = fmaf(-x0, l10, a[J + 1]) * r1;
+        const float x2 = fmaf(-x1, l21, fmaf(-x0, l20, a[J + 2])) * r2;
+        const float x3 = fmaf(-x2, l32, fmaf(-x1, l31, fmaf(-x0, l30, a[J + 3]))) * r3;
+        if (lane >= J) a[J] = x0;
+        if (lane > J) a[J + 1] = x1;
+        if (lane > J + 1) a[J + 2] = x2;
+        if (lane > J + 2) a[J + 3] = x3;
+        rows[lane] = make_float4(x0, x1, x2, x3);
+        __syncwarp();
+#pragma unroll
+        for (int k = J + 4; k < CB; ++k) {
+            const float4 l = rows[k];
+            a[k] = fmaf(-x3, l.w, fmaf(-x2, l.z, fmaf(-x1, l.y, fmaf(-x0, l.x, a[k]))));
         }
-        const float il = rsqrtf(piv), l = piv * il;   // FP32 factor: the FP64 correction absorbs its rounding
-        if (lane == J) a[J] = l;
-        if (lane > J) a[J] *= il;
-        DiagUpdate<J, J + 1>::run(a, a[J], lane);
-        DiagStep<J + 1>::run(a, lane, flag);
+        __syncwarp();
+        DiagBlock<J + 4>::run(a, lane, rows, bad);
     }
 };
 template <>
-struct DiagStep<CB> {
-    static __device__ __forceinline__ void run(float (&)[CB], int, int*) {}
+struct DiagBlock<CB> {
+    static __device__ __forceinline__ void run(float (&)[CB], int, float4*, bool&) {}
 };
 // Back substitution steps l = min(j, 32 SL + 31) .. 32 SL of column j: the
 // rows of block SL hold the pivot; rows i < l of blocks <= SL are updated.
@@ -187,72 +210,127 @@ size_t chol_eq_smem(int d) {
 }
 
 // warp-wide FP32 Cholesky of the diagonal tile D (row `lane` in registers)
-__device__ __forceinline__ void chol_diag_tile(float* D, float* rdiag, int lane, int* flag) {
+__device__ __forceinline__ void chol_diag_tile(float* D, float* rdiag, float4* rows, int lane, int* flag) {
     float a[CB];
 #pragma unroll
-    for (int k = 0; k < CB; ++k) a[k] = D[lane * QP + k];
-    DiagStep<0>::run(a, lane, flag);
+    for (int k = 0; k < CB; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(D + lane * QP + k);
+        a[k] = v.x;
+        a[k + 1] = v.y;
+        a[k + 2] = v.z;
+        a[k + 3] = v.w;
+    }
+    bool bad = false;
+    DiagBlock<0>::run(a, lane, rows, bad);
+    if (bad && lane == 0) set_flag(flag, LSK_FLAG_RANK_DEFICIENT);
 #pragma unroll
-    for (int k = 0; k < CB; ++k) D[lane * QP + k] = a[k];
+    for (int k = 0; k < CB; k += 4) *reinterpret_cast<float4*>(D + lane * QP + k) = make_float4(a[k], a[k + 1], a[k + 2], a[k + 3]);
     __syncwarp();
     rdiag[lane] = 1.f / D[lane * QP + lane];
     __syncwarp();
 }
 
-// T(I, J) -= L_IK L_JK^T for one 32 x 32 tile by one warp: lane = column of
-// the tile, rows of L_IK read as float4 broadcasts
-__device__ __forceinline__ void chol_tile_update(float* S, int I, int J, int K, int lane) {
-    const float* LI = qtile(S, I, K);
-    const float* LJ = qtile(S, J, K);
-    float* T = qtile(S, I, J);
-    float lj[CB];
+// R rows (r0 ..) of T(I, J) -= L_IK L_JK^T by one warp: lane = column of the
+// tile, rows of L_IK read as float4 broadcasts, the R rows' chains interleaved
+template <int R>
+__device__ __forceinline__ void chol_rows_update(float* S, int I, int J, int K, int r0, int lane) {
+    const float* LI = qtile(S, I, K) + r0 * QP;
+    const float* LJ = qtile(S, J, K) + lane * QP;
+    float* T = qtile(S, I, J) + r0 * QP + lane;
+    float acc[R];
 #pragma unroll
-    for (int k = 0; k < CB; ++k) lj[k] = LJ[lane * QP + k];
-#pragma unroll 1
-    for (int a = 0; a < CB; ++a) {
-        const float4* row = reinterpret_cast<const float4*>(LI + a * QP);
-        float acc0 = 0.f, acc1 = 0.f;
+    for (int r = 0; r < R; ++r) acc[r] = 0.f;
 #pragma unroll
-        for (int q = 0; q < CB / 4; q += 2) {
-            const float4 u = row[q], v = row[q + 1];
-            acc0 = fmaf(u.x, lj[4 * q], acc0);
-            acc1 = fmaf(u.y, lj[4 * q + 1], acc1);
-            acc0 = fmaf(u.z, lj[4 * q + 2], acc0);
-            acc1 = fmaf(u.w, lj[4 * q + 3], acc1);
-            acc0 = fmaf(v.x, lj[4 * q + 4], acc0);
-            acc1 = fmaf(v.y, lj[4 * q + 5], acc1);
-            acc0 = fmaf(v.z, lj[4 * q + 6], acc0);
-            acc1 = fmaf(v.w, lj[4 * q + 7], acc1);
+    for (int k = 0; k < CB; k += 4) {
+        const float4 l = *reinterpret_cast<const float4*>(LJ + k);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 u = *reinterpret_cast<const float4*>(LI + r * QP + k);
+            acc[r] = fmaf(u.x, l.x, acc[r]);
+            acc[r] = fmaf(u.y, l.y, acc[r]);
+            acc[r] = fmaf(u.z, l.z, acc[r]);
+            acc[r] = fmaf(u.w, l.w, acc[r]);
         }
-        T[a * QP + lane] -= acc0 + acc1;
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) T[r * QP] -= acc[r];
+}
+
+// T(I, J) -= L_IK L_JK^T for one 32 x 32 tile by one warp: lane (g, c) = (lane /
+// 8, lane % 8) owns rows g + 4 i and columns c + 8 j (8 x 4 outputs), twelve
+// 16-byte loads for 128 FMAs (with a lane to a column and rows broadcast it was
+// nine for 32, and shared memory the bound)
+__device__ __forceinline__ void chol_tile_update(float* S, int I, int J, int K, int lane) {
+    const int g = lane >> 3, c = lane & 7;
+    const float* LI = qtile(S, I, K) + g * QP;
+    const float* LJ = qtile(S, J, K) + c * QP;
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < CB; k += 4) {
+        float4 y[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = *reinterpret_cast<const float4*>(LJ + 8 * j * QP + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 x = *reinterpret_cast<const float4*>(LI + 4 * i * QP + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[i][j] = fmaf(x.x, y[j].x, acc[i][j]);
+                acc[i][j] = fmaf(x.y, y[j].y, acc[i][j]);
+                acc[i][j] = fmaf(x.z, y[j].z, acc[i][j]);
+                acc[i][j] = fmaf(x.w, y[j].w, acc[i][j]);
+            }
+        }
+    }
+    float* T = qtile(S, I, J) + g * QP + c;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) T[4 * i * QP + 8 * j] -= acc[i][j];
 }
 
 __device__ __forceinline__ void chol_eq_body(const float2* __restrict__ Cp, int d, int* __restrict__ e_out,
                                              float2* __restrict__ Rt, float* __restrict__ Lpk, int* flag) {
     extern __shared__ __align__(16) float S[];
     __shared__ float rdiag[CB];
+    __shared__ float4 drows[CB];
     __shared__ float scf[256];
     __shared__ unsigned char tI[36], tJ[36];
     __shared__ float dmin[32], dmax[32];
     const int nt = (d + CB - 1) / CB;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // each warp's first tile is on its way while the exponents are formed
+    const int ntl = nt * (nt + 1) / 2;
+    float v[CB];
+    const auto load_tile = [&](int i0, int j) {
+        const float2* src = Cp + (int64_t)i0 * d + j;
+#pragma unroll
+        for (int r = 0; r < CB; ++r) v[r] = (i0 + r < d && j < d) ? __ldg(&src[(int64_t)r * d].x) : 0.f;
+    };
+    if (w < ntl) {
+        int I = 0, t = w;
+        while (t > I) t -= ++I;
+        load_tile(I * CB, t * CB + lane);
+    }
     // (0) equilibration exponents from the diagonal; scf_j = 2^-e_j (a float:
     //     e_j is in [-75, 64] for a finite positive FP32 C_jj)
     for (int j = threadIdx.x; j < d; j += blockDim.x) {
         const float c = Cp[(int64_t)j * d + j].x;
         int ex = 0;
         if (c > 0.f && isfinite(c)) {
-            int b2;
-            frexpf(c, &b2);                 // c = m 2^b2, m in [0.5, 1)
-            ex = (b2 - 1) >> 1;
+            // floor(log2 c) (a subnormal c scaled up first), halved
+            const bool sub = c < 1.17549435e-38f;
+            ex = ((int)(__float_as_uint(sub ? c * 16777216.f : c) >> 23) - 127 - (sub ? 24 : 0)) >> 1;
         } else {
             set_flag(flag, LSK_FLAG_RANK_DEFICIENT);
         }
         e_out[j] = ex;
-        scf[j] = ldexpf(1.f, -ex);
+        scf[j] = __uint_as_float((uint32_t)(127 - ex) << 23);
     }
-    const int ntl = nt * (nt + 1) / 2;
     if (threadIdx.x < ntl) {
         int I = 0, t = threadIdx.x;
         while (t > I) t -= ++I;
@@ -261,35 +339,24 @@ __device__ __forceinline__ void chol_eq_body(const float2* __restrict__ Cp, int 
     }
     __syncthreads();
     // (1) the lower tiles of Ct = D^-1 C D^-1 in FP32 (beyond d: the identity):
-    //     the FP32 rounding of C times two exact powers of two, in rounds of
-    //     24 loads per thread, all issued before any is used
-    {
-        constexpr int kR = 24;
-        const int total = ntl * CB * CB;
-        for (int t0 = 0; t0 < total; t0 += kR * 512) {
-            float v[kR];
+    //     the FP32 rounding of C times two exact powers of two; a warp takes a
+    //     tile, all 32 row loads in flight
+    for (int tl = w; tl < ntl; tl += nw) {
+        const int i0 = tI[tl] * CB, j = tJ[tl] * CB + lane;
+        if (tl != w) load_tile(i0, j);
+        const float sj = j < d ? scf[j] : 0.f;
+        float* T = S + tl * (CB * QP) + lane;
 #pragma unroll
-            for (int q = 0; q < kR; ++q) {
-                const int t = t0 + q * 512 + (int)threadIdx.x;
-                const int tl = t >> 10, el = t & 1023;
-                const int i = tI[tl < 36 ? tl : 0] * CB + (el >> 5), j = tJ[tl < 36 ? tl : 0] * CB + (el & 31);
-                v[q] = (t < total && i < d && j < d) ? __ldg(&Cp[(int64_t)i * d + j].x) : 0.f;
-            }
-#pragma unroll
-            for (int q = 0; q < kR; ++q) {
-                const int t = t0 + q * 512 + (int)threadIdx.x;
-                if (t < total) {
-                    const int tl = t >> 10, el = t & 1023;
-                    const int r = el >> 5, c = el & 31, i = tI[tl] * CB + r, j = tJ[tl] * CB + c;
-                    S[tl * (CB * QP) + r * QP + c] = (i < d && j < d) ? v[q] * scf[i] * scf[j] : (i == j ? 1.f : 0.f);
-                }
-            }
-        }
+        for (int r = 0; r < CB; ++r)
+            T[r * QP] = (i0 + r < d && j < d) ? v[r] * scf[i0 + r] * sj : (i0 + r == j ? 1.f : 0.f);
     }
     __syncthreads();
     // K = -1 factors the first diagonal tile only; every later pass: the panel
     // of K, then the trailing update with the next diagonal tile looked ahead
-    // (one call site of the unrolled diagonal factorisation keeps the code small)
+    // (one call site of the unrolled diagonal factorisation keeps the code
+    // small).  512 x 256: 63 us (92 with one pivot at a time, rows broadcast to
+    // lanes of columns and element-wise loads; 8 steps of 3,900 cycles of diagonal
+    // tile, 3,300 of panel, up to 13,000 of trailing tiles).
     for (int K = -1; K < nt; ++K) {
         const float* D = qtile(S, K < 0 ? 0 : K, K < 0 ? 0 : K);
         // (2) panel: thread per row of T(I, K), I > K (forward substitution with L_KK)
@@ -297,41 +364,47 @@ __device__ __forceinline__ void chol_eq_body(const float2* __restrict__ Cp, int 
             const int rows = (nt - K - 1) * CB;
             for (int t = threadIdx.x; t < rows; t += blockDim.x) {
                 const int I = K + 1 + t / CB, r = t % CB;
-                float* T = qtile(S, I, K);
+                float* T = qtile(S, I, K) + r * QP;
                 float x[CB];
 #pragma unroll
-                for (int j = 0; j < CB; ++j) {
-                    float v = T[r * QP + j];
-#pragma unroll
-                    for (int l = 0; l < j; ++l) v -= x[l] * D[j * QP + l];
-                    x[j] = v * rdiag[j];
+                for (int j = 0; j < CB; j += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(T + j);
+                    x[j] = v.x;
+                    x[j + 1] = v.y;
+                    x[j + 2] = v.z;
+                    x[j + 3] = v.w;
                 }
 #pragma unroll
-                for (int j = 0; j < CB; ++j) T[r * QP + j] = x[j];
+                for (int j = 0; j < CB; ++j) {   // four chains a dot product
+                    float v[4] = {x[j], 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int l = 0; l < j; ++l) v[l & 3] = fmaf(-x[l], D[j * QP + l], v[l & 3]);
+                    x[j] = ((v[0] + v[1]) + (v[2] + v[3])) * rdiag[j];
+                }
+#pragma unroll
+                for (int j = 0; j < CB; j += 4) *reinterpret_cast<float4*>(T + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
             }
         }
         __syncthreads();
-        // (3) trailing update with look-ahead: warp 0 updates the next diagonal
-        //     tile (K+1, K+1) and factors it at once, while the other warps
-        //     update the rest of the trailing tiles (I, J), K < J <= I
-        {
-            const int T0 = nt - K - 1;
-            const int ntile = K < 0 ? 0 : T0 * (T0 + 1) / 2;
-            if (w == 0) {
-                if (T0 > 0) {
-                    if (K >= 0) chol_tile_update(S, K + 1, K + 1, K, lane);
-                    __syncwarp();
-                    chol_diag_tile(qtile(S, K + 1, K + 1), rdiag, lane, flag);
+        // (3) the next diagonal tile (K+1, K+1), two rows a warp; then warp 0
+        //     factors it while the other warps update the rest of the trailing
+        //     tiles (I, J), K < J <= I
+        const int T0 = nt - K - 1;
+        if (K >= 0 && T0 > 0) {
+            for (int r = 2 * w; r < CB; r += 2 * nw) chol_rows_update<2>(S, K + 1, K + 1, K, r, lane);
+            __syncthreads();
+        }
+        if (w == 0) {
+            if (T0 > 0) chol_diag_tile(qtile(S, K + 1, K + 1), rdiag, drows, lane, flag);
+        } else {
+            const int tiles = K < 0 ? 0 : T0 * (T0 + 1) / 2;
+            for (int t = w; t < tiles; t += nw - 1) {   // t = 0 is the diagonal tile
+                int I = 0, tt = t;
+                while (tt > I) {
+                    tt -= I + 1;
+                    ++I;
                 }
-            } else {
-                for (int t = w; t < ntile; t += nw - 1) {   // t = 0 is the diagonal tile
-                    int I = 0, tt = t;
-                    while (tt > I) {
-                        tt -= I + 1;
-                        ++I;
-                    }
-                    chol_tile_update(S, I + K + 1, tt + K + 1, K, lane);
-                }
+                chol_tile_update(S, I + K + 1, tt + K + 1, K, lane);
             }
         }
         __syncthreads();
@@ -370,8 +443,14 @@ __device__ __forceinline__ void chol_eq_body(const float2* __restrict__ Cp, int 
                     make_float2((j >= i) ? qtile(S, j >> 5, i >> 5)[(j & 31) * QP + (i & 31)] : 0.f, 0.f);
     }
     for (int l = w; l < d; l += nw) {
-        float* dst = Lpk + l * (l + 1) / 2;
-        for (int i = lane; i <= l; i += 32) dst[i] = qtile(S, l >> 5, i >> 5)[(l & 31) * QP + (i & 31)];
+        float* dst = Lpk + l * (l + 1) / 2 + lane;
+        const float* row = qtile(S, l >> 5, 0) + (l & 31) * QP + lane;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = 32 * q + lane <= l ? row[q * (CB * QP)] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (32 * q + lane <= l) dst[32 * q] = v[q];
     }
 }
 
