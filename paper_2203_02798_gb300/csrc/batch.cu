@@ -42,8 +42,9 @@
 //   W      most waves the grouped problems are dealt into (phase 2 of a wave
 //          overlaps phases 1 / 3 of its neighbours; more waves shorten the
 //          head and the tail of that pipeline, fewer make larger grouped grids);
-//   slice  chunks of 32 columns of r per block of the grouped Gaussian stage
-//          (longer slices: fewer partials to add, fewer blocks);
+//   slice  chunks of 32 columns of r, at most, per block of the grouped Gaussian
+//          stage (longer slices: fewer partials to add, fewer blocks; a wave
+//          that would not fill the SMs takes shorter ones, group_slice());
 //   tiles  128-row tiles per CTA, at least, of the dense row norms (more: fewer
 //          CTAs per problem, so problems on other streams share the SMs).
 struct BatchTune {
@@ -217,7 +218,7 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
     if (W > 0) {
         if ((e = cudaStreamWaitEvent(b->pstream, b->fork, 0)) != cudaSuccess) return e;
         for (int w = 0; w < W; ++w) {
-            if ((e = cs_group_launch(b->cg[w], b->table, ctx->sm_count, b->pstream)) != cudaSuccess) return e;
+            if ((e = cs_group_launch(b->cg[w], b->table, ctx->flag, b->pstream)) != cudaSuccess) return e;
             if ((e = cudaEventRecord(ev_prep(w), b->pstream)) != cudaSuccess) return e;
         }
     }
@@ -302,6 +303,20 @@ bool groupable(const lsk_batch_item& it, int32_t prec) {
            qr_group_supported(it.k, it.A.d);
 }
 
+// Chunks per block of one wave's Gaussian stage.  A block draws 256 x 32 entries
+// a chunk, 3.5 us, and has an SM to itself: blocks of 128 chunks left most SMs
+// without one when the wave holds a few dozen problems (24 problems, 52 blocks:
+// 457 us).  A wave is cut into kGaussBlocksPerSm blocks an SM, down to 8 chunks
+// (below, writing the k x d partials costs more than it shares out), unless
+// the schedule's longer slices give that many already: 196 us.  Of 2, 4 and 8
+// blocks an SM the whole call takes 1071, 1078 and 1093 us with 24 problems,
+// 4.37, 4.53 and 4.83 ms with 64, 7.22, 7.25 and 7.55 ms with 160 small ones.
+constexpr int64_t kGaussBlocksPerSm = 2, kGaussMinSlice = 8;
+int group_slice(int64_t chunks, int slice, int sm_count) {
+    const int64_t want = (chunks + kGaussBlocksPerSm * sm_count - 1) / (kGaussBlocksPerSm * sm_count);
+    return (int)std::min<int64_t>(slice, std::max(want, kGaussMinSlice));
+}
+
 // Arena layout of the grouped problems, their launch tables, and the upload
 // of the tables (only when they changed; the previous batch on the context
 // stream is finished first, since it may still read the old table).
@@ -326,11 +341,16 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
     for (int q = 0; q < ng; ++q) b->wave[order[q]] = q % std::max(b->waves, 1);
     std::vector<int64_t> wrows(b->waves, 0), wcnt(b->waves, 0);
     size_t bytes = 0;
+    std::vector<int64_t> wchunks(b->waves, 0);   // (256-row tile, 32-column chunk) pairs of G
+    for (int i = 0; i < count; ++i)
+        if (b->grouped[i]) wchunks[b->wave[i]] += ((items[i].k + 255) / 256) * ((sketch_rows(items[i]) + 31) / 32);
+    std::vector<int> wslice(b->waves);
+    for (int w = 0; w < b->waves; ++w) wslice[w] = group_slice(wchunks[w], tune.slice, ctx->sm_count);
     for (int i = 0; i < count; ++i) {
         if (!b->grouped[i]) continue;
         const int64_t rs = sketch_rows(items[i]), k = items[i].k, d = items[i].A.d;
         bytes += ws_round((size_t)rs * d * 4) + ws_round((size_t)k * d * 4) +
-                 gauss_group_part_bytes(rs, d, k, tune.slice) + ws_round(qr_workspace_bytes(k, d)) +
+                 gauss_group_part_bytes(rs, d, k, wslice[b->wave[i]]) + ws_round(qr_workspace_bytes(k, d)) +
                  ws_round((size_t)d * d * 4) + (compacts(items[i]) ? ws_round((size_t)(rs + 1) * 4) : 0) +
                  ws_round(prepared_bytes(items[i], prec));
         wrows[b->wave[i]] += items[i].A.n;
@@ -361,7 +381,7 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
         const int64_t rs = sketch_rows(items[i]), k = items[i].k, d = items[i].A.d;
         float* SA = wc.take<float>((size_t)rs * d);
         float* GSA = wc.take<float>((size_t)k * d);
-        float* part = (float*)wc.take<char>(gauss_group_part_bytes(rs, d, k, tune.slice));
+        float* part = (float*)wc.take<char>(gauss_group_part_bytes(rs, d, k, wslice[b->wave[i]]));
         void* qws = wc.take<char>(qr_workspace_bytes(k, d));
         float* Ri32 = wc.take<float>((size_t)d * d);
         uint32_t* cidx = compacts(items[i]) ? wc.take<uint32_t>((size_t)rs + 1) : nullptr;
@@ -375,7 +395,7 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
         b->SA[i] = SA;
         b->Rinv32[i] = Ri32;
         b->cidx[i] = cidx;
-        GaussJob gjob{SA, rs, d, k, items[i].seed, GSA, part, tune.slice};
+        GaussJob gjob{SA, rs, d, k, items[i].seed, GSA, part, wslice[b->wave[i]]};
         if (cidx) {
             gjob.idx = cidx;
             gjob.rcount = cidx + rs;

@@ -75,86 +75,6 @@ __global__ void cs_place_kernel(int64_t n, uint64_t row0, uint32_t r, uint32_t k
     }
 }
 
-// Block-local exclusive scan of kScanTile entries; writes the tile total.
-__global__ void scan_tiles_kernel(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
-                                  uint32_t* __restrict__ tile_sums, int64_t len) {
-    __shared__ uint32_t warp_tot[kScanBlock / 32];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    uint32_t v[kScanItems];
-    uint32_t run = 0;
-#pragma unroll
-    for (int t = 0; t < kScanItems; ++t) {
-        const int64_t i = base + t;
-        v[t] = (i < len) ? in[i] : 0u;
-        const uint32_t x = v[t];
-        v[t] = run;
-        run += x;
-    }
-    // exclusive scan of the per-thread totals across the block
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_tot[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        uint32_t w = (lane < kScanBlock / 32) ? warp_tot[lane] : 0u;
-        uint32_t wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        if (lane < kScanBlock / 32) warp_tot[lane] = wi - w;
-        if (lane == kScanBlock / 32 - 1) tile_sums[blockIdx.x] = wi;
-    }
-    __syncthreads();
-    const uint32_t excl = warp_tot[wid] + incl - run;
-#pragma unroll
-    for (int t = 0; t < kScanItems; ++t) {
-        const int64_t i = base + t;
-        if (i < len) out[i] = v[t] + excl;
-    }
-}
-
-__global__ void scan_add_kernel(uint32_t* __restrict__ out, const uint32_t* __restrict__ tile_off,
-                                int64_t len) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < len) out[i] += tile_off[i / kScanTile];
-}
-
-// Exclusive scan of `len` uint32 into `out` (may alias nothing); `tmp` must
-// hold scan_tmp_words(len) words.
-size_t scan_tmp_words(int64_t len) {
-    size_t words = 0;
-    int64_t l = len;
-    while (true) {
-        const int64_t tiles = (l + kScanTile - 1) / kScanTile;
-        words += 2 * (size_t)tiles + 64;
-        if (tiles <= 1) break;
-        l = tiles;
-    }
-    return words;
-}
-
-cudaError_t exclusive_scan(const uint32_t* in, uint32_t* out, int64_t len, uint32_t* tmp,
-                           cudaStream_t st) {
-    if (len <= 0) return cudaSuccess;
-    const int64_t tiles = (len + kScanTile - 1) / kScanTile;
-    uint32_t* sums = tmp;
-    LSK_PROF("cs_scan", st) scan_tiles_kernel<<<(unsigned)tiles, kScanBlock, 0, st>>>(in, out, sums, len);
-    if (tiles > 1) {
-        uint32_t* sums_off = tmp + tiles + 32;
-        cudaError_t e = exclusive_scan(sums, sums_off, tiles, sums_off + tiles + 32, st);
-        if (e != cudaSuccess) return e;
-        LSK_PROF("cs_scan", st) scan_add_kernel<<<(unsigned)((len + 255) / 256), 256, 0, st>>>(out, sums_off, len);
-    }
-    return cudaGetLastError();
-}
-
 // Single-pass exclusive scan of the counters (decoupled look-back): block b
 // takes tile t (the t-th ticket, kScanTile counts), scans it, publishes its
 // aggregate, then adds the published values of the tiles before it, nearest
@@ -645,52 +565,59 @@ __global__ void cs_hash_debug_kernel(int64_t n, uint32_t r, uint32_t k0, uint32_
 // Compaction of the sketch's rows to the non-empty buckets (off[b + 1] >
 // off[b]), in bucket order: cpos[b] = the number of non-empty buckets before b,
 // cidx[cpos[b]] = b for each non-empty b, *ccount = their number.  One block
-// of 1024 threads, rounds of 4096 buckets (4 consecutive a thread) with the
-// running total carried across rounds.
+// of 1024 threads: each warp counts its contiguous 1/32 of the buckets by
+// ballots, the 32 totals are scanned, and a second pass writes.  Bound by the
+// latency of the loads, so a lane keeps 2 kCompactLoads of them in flight and
+// the block meets twice in all, not in every 4,096 buckets (24 problems,
+// 65,536 buckets at most: 43 -> 20 us).
+constexpr int kCompactLoads = 8;
 __device__ __forceinline__ void compact_body(const uint32_t* __restrict__ off, int64_t r, uint32_t* __restrict__ cpos,
                                              uint32_t* __restrict__ cidx, uint32_t* __restrict__ ccount) {
     __shared__ uint32_t wsum[32];
-    __shared__ uint32_t carry_s;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t carry = 0;
-    for (int64_t r0 = 0; r0 < r; r0 += 4096) {
-        const int64_t b0 = r0 + 4 * (int64_t)threadIdx.x;
-        uint32_t f[4];
+    const int64_t seg = ((r + 1023) / 1024) * 32, lo = min(r, w * seg), hi = min(r, lo + seg);
+    // the non-empty ones among buckets b0 + 32 q, q < kCompactLoads, as lane masks
+    auto masks = [&](int64_t b0, unsigned (&m)[kCompactLoads]) {
+        uint32_t x[kCompactLoads], y[kCompactLoads];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) f[q] = (b0 + q < r && off[b0 + q + 1] > off[b0 + q]) ? 1u : 0u;
-        const uint32_t run = f[0] + f[1] + f[2] + f[3];
-        uint32_t incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+        for (int q = 0; q < kCompactLoads; ++q) {
+            const int64_t b = b0 + 32 * q + lane;
+            x[q] = b < hi ? __ldg(off + b) : 0u;
+            y[q] = b < hi ? __ldg(off + b + 1) : 0u;
         }
-        if (lane == 31) wsum[w] = incl;
-        __syncthreads();
-        if (w == 0) {
-            uint32_t v = wsum[lane], vi = v;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, vi, o);
-                if (lane >= o) vi += y;
-            }
-            wsum[lane] = vi - v;   // exclusive warp offsets
-            if (lane == 31) carry_s = vi;
-        }
-        __syncthreads();
-        uint32_t pos = carry + wsum[w] + incl - run;
+        for (int q = 0; q < kCompactLoads; ++q) m[q] = __ballot_sync(0xffffffffu, y[q] > x[q]);
+    };
+    unsigned m[kCompactLoads];
+    uint32_t own = 0;
+    for (int64_t b0 = lo; b0 < hi; b0 += 32 * kCompactLoads) {
+        masks(b0, m);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (b0 + q < r) {
-                cpos[b0 + q] = pos;
-                if (f[q]) cidx[pos] = (uint32_t)(b0 + q);
-            }
-            pos += f[q];
-        }
-        carry += carry_s;
-        __syncthreads();
+        for (int q = 0; q < kCompactLoads; ++q) own += __popc(m[q]);
     }
-    if (threadIdx.x == 0) *ccount = carry;
+    if (lane == 0) wsum[w] = own;
+    __syncthreads();
+    uint32_t incl = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (threadIdx.x == 31) *ccount = incl;
+    uint32_t pos = __shfl_sync(0xffffffffu, incl, w) - own;   // non-empty buckets before this warp's
+    for (int64_t b0 = lo; b0 < hi; b0 += 32 * kCompactLoads) {
+        masks(b0, m);
+#pragma unroll
+        for (int q = 0; q < kCompactLoads; ++q) {
+            const int64_t b = b0 + 32 * q + lane;
+            const uint32_t at = pos + __popc(m[q] & ((1u << lane) - 1u));
+            if (b < hi) {
+                cpos[b] = at;
+                if ((m[q] >> lane) & 1u) cidx[at] = (uint32_t)b;
+            }
+            pos += __popc(m[q]);
+        }
+    }
 }
 __global__ void __launch_bounds__(1024) cs_compact_kernel(const uint32_t* __restrict__ off, int64_t r,
                                                           uint32_t* __restrict__ cpos, uint32_t* __restrict__ cidx,
@@ -699,8 +626,7 @@ __global__ void __launch_bounds__(1024) cs_compact_kernel(const uint32_t* __rest
 }
 
 // ---- grouped preparation: the permutations of many problems, three launches
-// The problems' rows are numbered consecutively (problem p owns rows
-// rowoff[p] .. rowoff[p + 1] - 1) and their counters too (problem p's r + 1
+// The problems' counters are numbered consecutively (problem p's r + 1
 // counters from cnt_base); one exclusive scan over all the counters then
 // gives each bucket its range of the shared permutation, so the problems'
 // rows land in consecutive blocks of it and each problem's off[] (its slice
@@ -712,38 +638,86 @@ struct CsGp {
     uint32_t* ccount;
 };
 
-__device__ __forceinline__ int job_of(const int64_t* __restrict__ rowoff, int count, int64_t g) {
-    int lo = 0, hi = count - 1;   // largest p with rowoff[p] <= g
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(rowoff + mid) <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+// Counting and placing take the same form: a block takes a run of one
+// problem's rows.  With few buckets for its rows (r <= kGroupBuckets, n >= 2r)
+// it ranks them per bucket in shared memory and goes to L2 once per bucket it
+// met, not once per row: the problems of 32 columns send some hundred rows to
+// each of 1,024 counters, whose atomics queue up at one address.  With more
+// buckets a run meets most of its buckets once, and the rows go to L2
+// themselves, kPrepRows at a time.  24 problems, 3.1M rows, 267K buckets:
+// counting 26 us, placing 44 (all rows through L2: 113 and 131).
+constexpr int kGroupThreads = 512;
+constexpr int kGroupRows = 16;         // rows a thread: 13 bits of rank, 13 of bucket, the sign
+constexpr int64_t kGroupBuckets = 4096;
+__host__ __device__ __forceinline__ bool group_shared(int64_t n, int64_t r) { return r <= kGroupBuckets && n >= 2 * r; }
+__host__ __device__ __forceinline__ int64_t group_run(int64_t n, int64_t r) {
+    return (int64_t)kGroupThreads * (group_shared(n, r) ? kGroupRows : kPrepRows);
 }
 
-__global__ void cs_count_grouped_kernel(const CsGp* __restrict__ ps, const int64_t* __restrict__ rowoff, int count,
-                                        int64_t rows, uint32_t* __restrict__ cnt) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < rows; g += stride) {
-        const int p = job_of(rowoff, count, g);
-        const CsGp& j = ps[p];
-        uint32_t b, neg;
-        cs_hash((uint64_t)(g - __ldg(rowoff + p)), (uint32_t)j.r, j.k0, j.k1, b, neg);
-        atomicAdd(&cnt[j.cnt_base + b], 1u);
+template <bool kPlace>
+__global__ void __launch_bounds__(kGroupThreads, 2) cs_rows_grouped_kernel(const CsGp* __restrict__ ps,
+                                                                           const int* __restrict__ boff, int count,
+                                                                           uint32_t* __restrict__ counters,
+                                                                           uint32_t* __restrict__ perm) {
+    __shared__ uint32_t hist[kGroupBuckets];
+    const int p = group_of(boff, count, (int)blockIdx.x);
+    const CsGp& j = ps[p];
+    const int64_t n = j.n, r = j.r;
+    const uint32_t k0 = j.k0, k1 = j.k1;
+    uint32_t* cnt = counters + j.cnt_base;
+    const int64_t i0 = (int64_t)((int)blockIdx.x - __ldg(boff + p)) * group_run(n, r) + threadIdx.x;
+    if (group_shared(n, r)) {
+        for (int b = threadIdx.x; b < (int)r; b += kGroupThreads) hist[b] = 0u;
+        __syncthreads();
+        uint32_t at[kGroupRows];   // sign << 31 | bucket << 13 | rank among the block's rows of that bucket
+#pragma unroll
+        for (int q = 0; q < kGroupRows; ++q) {
+            const int64_t i = i0 + q * kGroupThreads;
+            if (i < n) {
+                uint32_t b, neg;
+                cs_hash((uint64_t)i, (uint32_t)r, k0, k1, b, neg);
+                const uint32_t rank = atomicAdd(&hist[b], 1u);
+                at[q] = (neg << 31) | (b << 13) | rank;
+            }
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b < (int)r; b += kGroupThreads) {
+            const uint32_t h = hist[b];
+            if (h) {
+                if (kPlace) hist[b] = atomicAdd(&cnt[b], h);
+                else atomicAdd(&cnt[b], h);
+            }
+        }
+        if (!kPlace) return;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kGroupRows; ++q) {
+            const int64_t i = i0 + q * kGroupThreads;
+            if (i < n)
+                perm[hist[(at[q] >> 13) & (kGroupBuckets - 1)] + (at[q] & 0x1fffu)] =
+                    (uint32_t)i | (at[q] & 0x80000000u);
+        }
+        return;
     }
-}
-
-__global__ void cs_place_grouped_kernel(const CsGp* __restrict__ ps, const int64_t* __restrict__ rowoff, int count,
-                                        int64_t rows, uint32_t* __restrict__ cursor, uint32_t* __restrict__ perm) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < rows; g += stride) {
-        const int p = job_of(rowoff, count, g);
-        const CsGp& j = ps[p];
-        const uint32_t i = (uint32_t)(g - __ldg(rowoff + p));
-        uint32_t b, neg;
-        cs_hash((uint64_t)i, (uint32_t)j.r, j.k0, j.k1, b, neg);
-        perm[atomicAdd(&cursor[j.cnt_base + b], 1u)] = i | (neg << 31);
+    uint32_t slot[kPrepRows], val[kPrepRows];
+#pragma unroll
+    for (int q = 0; q < kPrepRows; ++q) {
+        const int64_t i = i0 + q * kGroupThreads;
+        if (i < n) {
+            uint32_t b, neg;
+            cs_hash((uint64_t)i, (uint32_t)r, k0, k1, b, neg);
+            if (kPlace) {
+                slot[q] = atomicAdd(&cnt[b], 1u);
+                val[q] = (uint32_t)i | (neg << 31);
+            } else {
+                atomicAdd(&cnt[b], 1u);
+            }
+        }
+    }
+    if (kPlace) {
+#pragma unroll
+        for (int q = 0; q < kPrepRows; ++q)
+            if (i0 + q * kGroupThreads < n) perm[slot[q]] = val[q];
     }
 }
 
@@ -771,12 +745,12 @@ size_t scan_state_words(int64_t len) { return (size_t)((len + kScanTile - 1) / k
 
 // The CountSketch workspace, in this order: the counters and the scan's
 // state (zeroed by one memset), the bucket offsets, the cursors, the
-// permutation, the multi-level scan's scratch, the compaction positions;
+// permutation, the compaction positions;
 // then, for the two-level sort, the per-row (bucket | sign), the rows
 // grouped by coarse bucket with their fine indices, the per-block counts
 // (scanned in place) and their scan state.
 struct CsWs {
-    uint32_t *cnt, *off, *cursor, *perm, *tmp, *cpos;
+    uint32_t *cnt, *off, *cursor, *perm, *cpos;
     unsigned long long* state;
     uint32_t *bsign, *T, *H;
     uint16_t* TF;
@@ -793,7 +767,6 @@ CsWs cs_carve(void* ws, int64_t n, int64_t r, const RxPlan* q) {
     w.off = wc.take<uint32_t>(r + 1);
     w.cursor = wc.take<uint32_t>(r + 1);
     w.perm = wc.take<uint32_t>(nn);
-    w.tmp = wc.take<uint32_t>(scan_tmp_words(r));
     w.cpos = wc.take<uint32_t>(r + 1);
     if (q) {
         w.bsign = wc.take<uint32_t>(nn);
@@ -931,54 +904,56 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
 }
 
 size_t cs_group_ws_bytes(int64_t rows, int64_t counters) {
-    return ws_round((size_t)counters * 4) * 4 + ws_round((size_t)(rows > 0 ? rows : 1) * 4) +
-           ws_round(scan_tmp_words(counters) * 4) + 2048;
+    return ws_round((size_t)(counters + 1) * 4) * 4 + ws_round((size_t)(rows > 0 ? rows : 1) * 4) +
+           ws_round(scan_state_words(counters) * 8) + 2048;
 }
 
 void cs_group_build(std::vector<CsJob>& jobs, void* ws, HostTable& t, CsGroup& g) {
     std::vector<CsGp> ps(jobs.size());
-    std::vector<int64_t> rowoff(jobs.size() + 1, 0);
+    std::vector<int> blocks(jobs.size()), boff;
     int64_t cb = 0;
     g.any_compact = false;
+    g.rows = 0;
     for (size_t i = 0; i < jobs.size(); ++i) {
         CsJob& j = jobs[i];
         j.cnt_base = cb;
         ps[i] = CsGp{j.n, j.r, cb, (uint32_t)j.seed, (uint32_t)(j.seed >> 32), j.cidx, j.ccount};
-        rowoff[i + 1] = rowoff[i] + j.n;
+        const int64_t run = group_run(j.n, j.r);
+        blocks[i] = (int)((j.n + run - 1) / run);
+        g.rows += j.n;
         cb += j.r + 1;
         g.any_compact = g.any_compact || j.cidx != nullptr;
     }
     g.count = (int)jobs.size();
-    g.rows = rowoff.back();
+    g.blocks = group_offsets(blocks, boff);
     g.counters = cb;
     WsCarver wc{(char*)ws, 0};
     g.cnt = wc.take<uint32_t>((size_t)g.counters);
-    g.off = wc.take<uint32_t>((size_t)g.counters);
+    g.state = wc.take<unsigned long long>(scan_state_words(g.counters));
+    g.off = wc.take<uint32_t>((size_t)g.counters + 1);
     g.cursor = wc.take<uint32_t>((size_t)g.counters);
     g.cpos = wc.take<uint32_t>((size_t)g.counters);
     g.perm = wc.take<uint32_t>((size_t)(g.rows > 0 ? g.rows : 1));
-    g.tmp = wc.take<uint32_t>(scan_tmp_words(g.counters));
     g.params_off = t.put(ps.data(), ps.size());
-    g.rowoff_off = t.put(rowoff.data(), rowoff.size());
+    g.boff_off = t.put(boff.data(), boff.size());
 }
 
-cudaError_t cs_group_launch(const CsGroup& g, const unsigned char* table, int sm_count, cudaStream_t st) {
+cudaError_t cs_group_launch(const CsGroup& g, const unsigned char* table, int* flag, cudaStream_t st) {
     if (g.count == 0) return cudaSuccess;
     const CsGp* ps = reinterpret_cast<const CsGp*>(table + g.params_off);
-    const int64_t* rowoff = reinterpret_cast<const int64_t*>(table + g.rowoff_off);
-    cudaError_t e = cudaMemsetAsync(g.cnt, 0, (size_t)g.counters * 4, st);
+    const int* boff = reinterpret_cast<const int*>(table + g.boff_off);
+    // the counters and the scan's state are contiguous: one memset
+    cudaError_t e = cudaMemsetAsync(
+        g.cnt, 0, (size_t)((char*)(g.state + scan_state_words(g.counters)) - (char*)g.cnt), st);
     if (e != cudaSuccess) return e;
-    if (g.rows > 0)
-        LSK_PROF("cs_count", st) cs_count_grouped_kernel<<<grid_for(g.rows, 256, sm_count), 256, 0, st>>>(
-            ps, rowoff, g.count, g.rows, g.cnt);
-    e = exclusive_scan(g.cnt, g.off, g.counters, g.tmp, st);
-    if (e != cudaSuccess) return e;
-    if (g.rows > 0) {
-        e = cudaMemcpyAsync(g.cursor, g.off, (size_t)g.counters * 4, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        LSK_PROF("cs_place", st) cs_place_grouped_kernel<<<grid_for(g.rows, 256, sm_count), 256, 0, st>>>(
-            ps, rowoff, g.count, g.rows, g.cursor, g.perm);
-    }
+    if (g.blocks > 0)
+        LSK_PROF("cs_count", st) cs_rows_grouped_kernel<false><<<g.blocks, kGroupThreads, 0, st>>>(
+            ps, boff, g.count, g.cnt, nullptr);
+    LSK_PROF("cs_scan", st) scan_lookback_kernel<<<(unsigned)((g.counters + kScanTile - 1) / kScanTile), kScanBlock, 0,
+                                                   st>>>(g.cnt, g.off, g.cursor, g.counters, g.state, flag);
+    if (g.blocks > 0)
+        LSK_PROF("cs_place", st) cs_rows_grouped_kernel<true><<<g.blocks, kGroupThreads, 0, st>>>(
+            ps, boff, g.count, g.cursor, g.perm);
     if (g.any_compact)
         LSK_PROF("cs_compact", st) cs_compact_grouped_kernel<<<g.count, 1024, 0, st>>>(ps, g.off, g.cpos);
     return cudaGetLastError();

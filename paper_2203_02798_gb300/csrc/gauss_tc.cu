@@ -393,6 +393,9 @@ bool make_plan(int64_t r, int64_t d, int64_t k, int sm_count, Plan& P, int terms
     return P.smem <= kSmemLimit;
 }
 
+// Bound by the latency of the loads (k d entries are few threads): each thread
+// keeps kReduceLoads of them in flight.
+constexpr int kReduceLoads = 8;
 __device__ __forceinline__ void reduce_body(const float* __restrict__ part, int slices, int64_t len,
                                             float* __restrict__ out, int blk, int nblk) {
     const int64_t stride = (int64_t)nblk * blockDim.x;
@@ -400,12 +403,21 @@ __device__ __forceinline__ void reduce_body(const float* __restrict__ part, int 
         // compensated FP32 sum (Neumaier) in slice order: about two roundings
         // of error in total, without FP64 adds (scarce on this part)
         float s = 0.f, c = 0.f;
-        for (int z = 0; z < slices; ++z) {
-            const float x = part[(int64_t)z * len + e];
+        auto add = [&](float x) {
             const float t = s + x;
             c += (fabsf(s) >= fabsf(x)) ? (s - t) + x : (x - t) + s;
             s = t;
+        };
+        const float* src = part + e;
+        int z = 0;
+        for (; z + kReduceLoads <= slices; z += kReduceLoads) {
+            float x[kReduceLoads];
+#pragma unroll
+            for (int q = 0; q < kReduceLoads; ++q) x[q] = __ldg(src + (z + q) * len);
+#pragma unroll
+            for (int q = 0; q < kReduceLoads; ++q) add(x[q]);
         }
+        for (; z < slices; ++z) add(__ldg(src + z * len));
         out[e] = s + c;
     }
 }
@@ -436,7 +448,7 @@ void plan_grouped(int64_t r, int64_t d, int64_t k, Plan& P, int slice_chunks) {
     P.smem = smem_of<1>(P.npad);
 }
 
-constexpr int kReduceBlockCap = 64;
+constexpr int kReduceBlockCap = 512;
 
 }  // namespace
 
