@@ -4,15 +4,15 @@
 // own whole rows of SA (Alg. 2, the b_r = r case of Sec. 2.3), so that no two
 // threads write the same output row.  Here S is never stored: (h(i), sigma_i)
 // is recomputed from Philox whenever it is needed, and row ownership is kept
-// at the finest grain -- one warp owns one bucket (one row of SA):
+// at a fine grain:
 //
 //   1. count: cnt[h(i)]++ for every row (fire-and-forget atomics)
 //   2. scan:  off = exclusive prefix sum of cnt        (bucket -> first slot),
 //             and a copy of it as each bucket's fill cursor
 //   3. place: perm[cursor[h(i)]++] = i | sigma_bit << 31
-//   4. gather (dense): the warp owning bucket b streams the rows listed in
-//      perm[off[b] .. off[b+1]) with 16-byte coalesced loads, accumulates them
-//      (with their signs) in registers and writes row b of SA exactly once.
+//   4. gather (dense): teams of 8 to 32 lanes stream the rows listed in
+//      stretches of perm with coalesced loads, accumulate them (with their
+//      signs) in registers and write each bucket's row of SA once.
 //      gather (CSR): same ownership, the row of SA is accumulated in shared
 //      memory because CSR columns are scattered.
 //
@@ -373,17 +373,34 @@ __global__ void __launch_bounds__(kRxThreads) rx_fine_kernel(int64_t n, int64_t 
 }
 
 // ---- dense gather ---------------------------------------------------------
-// One warp per bucket part.  Lanes own VEC consecutive columns in each of U
-// column groups of 32*VEC; the rows are fetched kBatch at a time so that
-// each warp keeps kBatch rows of loads in flight.  With few buckets (small r,
-// long buckets) each bucket's row list is cut into P contiguous parts, one
-// warp each, so that enough warps stream A; their sums are then added into
-// SA (zeroed first) atomically.  With P = 1 each warp stores its bucket.
+// The rows of A in the order of perm, summed bucket by bucket.  A team of L
+// lanes takes a contiguous stretch of perm and walks it, kRows rows of loads in
+// flight, across the ends of its buckets: with a bucket (or a part of one) per
+// warp at a time, each bucket of 5 to 30 rows waited for its own chain of
+// offsets, permutation and rows, and with 20,000 parts on 9,728 warps a third
+// round ran nearly empty.  Lanes own VEC consecutive columns in each of U
+// groups of L VEC; a row of 32 or 64 columns is 8 or 16 lanes wide, and 4 or 2
+// teams share a warp in step (a warp per row left the other lanes without
+// loads).  The ends of the next L buckets stand in the team's lanes.  Bound by
+// DRAM, which random rows of 400 bytes hold at 4.5 TB/s and of 1 KB at 6.2:
+// 1,234,567 x 100 -> 10,000 in 112 us (123 with a warp per bucket part),
+// 1M x 100 -> 256 in 88 (111), 790,706 x 32 -> 1,024 in 25 (54), 500,000 x 200 ->
+// 40,000 in 87 (105), 22,379 x 256 -> 65,536 in 23 (42).
+//
+// Team t of T starts at the point t r / T of the buckets.  own: rounded down to
+// a bucket, so that each bucket is one team's and is stored, empty ones as
+// zeros.  Otherwise the fraction is taken of the bucket's rows, so that few
+// long buckets are shared out evenly; what a team holds of a bucket that it
+// shares is added to SA (zeroed first) atomically.
 template <int VEC>
 struct VecT;
 template <>
 struct VecT<4> {
     using T = float4;
+};
+template <>
+struct VecT<2> {
+    using T = float2;
 };
 template <>
 struct VecT<1> {
@@ -396,12 +413,20 @@ __device__ __forceinline__ void vadd(float4& a, const float4& b, float s) {
     a.z = fmaf(s, b.z, a.z);
     a.w = fmaf(s, b.w, a.w);
 }
+__device__ __forceinline__ void vadd(float2& a, const float2& b, float s) {
+    a.x = fmaf(s, b.x, a.x);
+    a.y = fmaf(s, b.y, a.y);
+}
 __device__ __forceinline__ void vadd(float& a, const float& b, float s) { a = fmaf(s, b, a); }
 __device__ __forceinline__ void vzero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ void vzero(float2& a) { a = make_float2(0.f, 0.f); }
 __device__ __forceinline__ void vzero(float& a) { a = 0.f; }
 __device__ __forceinline__ void vatomic_add(float4* p, const float4& v) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                  : "memory");
+}
+__device__ __forceinline__ void vatomic_add(float2* p, const float2& v) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
 }
 __device__ __forceinline__ void vatomic_add(float* p, const float& v) { atomicAdd(p, v); }
 
@@ -413,6 +438,10 @@ __device__ __forceinline__ typename VecT<VEC>::T ldg_stream(const float* p) {
                      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                      : "l"(p));
         return v;
+    } else if constexpr (VEC == 2) {
+        float2 v;
+        asm("ld.global.nc.L1::no_allocate.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+        return v;
     } else {
         float v;
         asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
@@ -420,74 +449,152 @@ __device__ __forceinline__ typename VecT<VEC>::T ldg_stream(const float* p) {
     }
 }
 
-template <int VEC, int U>
-__global__ void __launch_bounds__(256) cs_dense_gather_kernel(
-    const float* __restrict__ A, int64_t lda, int64_t d, uint32_t r,
-    const uint32_t* __restrict__ off, const uint32_t* __restrict__ perm, float* __restrict__ SA, int P,
-    int accumulate, const uint32_t* __restrict__ cpos) {
+// three blocks an SM keep 32 loads a lane in registers; single floats need fewer
+constexpr int kGatherThreads = 256;
+__host__ __device__ constexpr int gather_per_sm(int vec) { return vec == 1 ? 4 : 3; }
+template <int VEC, int U, int L>
+__global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC)) cs_dense_gather_kernel(
+    const float* __restrict__ A, int64_t lda, int64_t d, uint32_t r, const uint32_t* __restrict__ off,
+    const uint32_t* __restrict__ perm, float* __restrict__ SA, int64_t teams, int own, int accumulate,
+    const uint32_t* __restrict__ cpos) {
     using V = typename VecT<VEC>::T;
-    constexpr int kCols = 32 * VEC * U;  // columns per pass
-    constexpr int kBatch = (VEC * U >= 8) ? 8 : 4;   // rows of loads in flight per warp
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t items = (int64_t)r * P;
-    for (int64_t vb = warp; vb < items; vb += nwarps) {
-        const int64_t b = vb / P;
-        const uint32_t part = (uint32_t)(vb % P);
-        const uint32_t s0 = off[b], len = off[b + 1] - s0;
-        const uint32_t s = s0 + (uint32_t)(((uint64_t)len * part) / P);
-        const uint32_t e = s0 + (uint32_t)(((uint64_t)len * (part + 1)) / P);
-        if ((P > 1 || accumulate || cpos) && s == e) continue;
-        const int64_t orow = cpos ? (int64_t)cpos[b] : b;   // compacted: the bucket's rank among the non-empty
-        for (int64_t c0 = 0; c0 < d; c0 += kCols) {
-            V acc[U];
+    constexpr unsigned kAll = 0xffffffffu, kTeam = L == 32 ? kAll : (1u << (L & 31)) - 1u;
+    constexpr int kCols = L * VEC * U;              // columns per pass
+    constexpr int kRows = VEC * U >= 8 ? 4 : 8;     // rows of loads in flight
+    const int lane = threadIdx.x & 31, tl = lane & (L - 1), sh = lane & ~(L - 1);
+    const int64_t team = ((int64_t)blockIdx.x * kGatherThreads + threadIdx.x) / L;
+    int64_t b0 = 0, b1 = 0;
+    uint32_t s = 0, e = 0;
+    bool shared_start = false;
+    if (team < teams) {
+        const int64_t x0 = team * (int64_t)r, x1 = x0 + r;
+        b0 = x0 / teams;
+        b1 = x1 / teams;
+        s = __ldg(off + b0);
+        e = __ldg(off + b1);
+        if (!own) {
+            const uint64_t f0 = (uint64_t)(x0 - b0 * teams), f1 = (uint64_t)(x1 - b1 * teams);
+            const uint32_t s0 = s;
+            if (f0) s += (uint32_t)((uint64_t)(__ldg(off + b0 + 1) - s) * f0 / (uint64_t)teams);
+            if (f1) e += (uint32_t)((uint64_t)(__ldg(off + b1 + 1) - e) * f1 / (uint64_t)teams);
+            shared_start = s != s0;
+        }
+    }
+    for (int64_t c0 = 0; c0 < d; c0 += kCols) {
+        bool colok[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) vzero(acc[u]);
-            bool colok[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) colok[u] = (c0 + (int64_t)(u * 32 + lane) * VEC) < d;
-            for (uint32_t t0 = s; t0 < e; t0 += 32) {
-                const uint32_t m = min(32u, e - t0);
-                const uint32_t mine = (lane < (int)m) ? perm[t0 + lane] : 0u;
-                uint32_t j = 0;
-                for (; j + kBatch <= m; j += kBatch) {
-                    V v[kBatch][U];
-                    float sg[kBatch];
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q) {
-                        const uint32_t p = __shfl_sync(0xffffffffu, mine, j + q);
-                        sg[q] = (p >> 31) ? -1.0f : 1.0f;
-                        const float* row = A + (int64_t)(p & 0x7fffffffu) * lda + c0;
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            if (colok[u]) v[q][u] = ldg_stream<VEC>(row + (u * 32 + lane) * VEC);
-                            else vzero(v[q][u]);
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < kBatch; ++q)
-#pragma unroll
-                        for (int u = 0; u < U; ++u) vadd(acc[u], v[q][u], sg[q]);
-                }
-                for (; j < m; ++j) {
-                    const uint32_t p = __shfl_sync(0xffffffffu, mine, j);
-                    const float sg = (p >> 31) ? -1.0f : 1.0f;
-                    const float* row = A + (int64_t)(p & 0x7fffffffu) * lda + c0;
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        if (colok[u]) vadd(acc[u], ldg_stream<VEC>(row + (u * 32 + lane) * VEC), sg);
+        for (int u = 0; u < U; ++u) colok[u] = c0 + (int64_t)(u * L + tl) * VEC < d;
+        uint32_t next = s + tl < e ? __ldg(perm + s + tl) : 0u;
+        int64_t bb = b0;                            // lane tl: the end (and the rank) of bucket bb + tl
+        uint32_t ends = __ldg(off + min(bb + 1 + tl, (int64_t)r));
+        uint32_t ranks = cpos ? __ldg(cpos + min(bb + tl, (int64_t)r - 1)) : 0u;
+        uint32_t end = 0;                           // of the bucket that is summed
+        int64_t orow = 0;                           // its row of SA
+        // the bucket that holds position t, for the teams that want it
+        auto find = [&](uint32_t t, bool want) {
+            int at = 0;
+            for (;;) {
+                const unsigned m = (__ballot_sync(kAll, ends > t) >> sh) & kTeam;
+                if (want && m) at = __ffs(m) - 1;
+                const bool more = want && !m;
+                if (!__any_sync(kAll, more)) break;
+                if (more) {
+                    bb += L;
+                    ends = __ldg(off + min(bb + 1 + tl, (int64_t)r));
+                    if (cpos) ranks = __ldg(cpos + min(bb + tl, (int64_t)r - 1));
                 }
             }
-            float* out = SA + orow * d + c0;
-            if (P == 1 && !accumulate) {
+            const uint32_t en = __shfl_sync(kAll, ends, sh + at), rk = __shfl_sync(kAll, ranks, sh + at);
+            if (want) {
+                end = en;
+                orow = cpos ? (int64_t)rk : bb + at;
+            }
+        };
+        find(s, s < e);
+        bool whole = !shared_start;                 // the bucket's first row is this team's
+        V acc[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (colok[u]) *reinterpret_cast<V*>(out + (u * 32 + lane) * VEC) = acc[u];
-            } else {
+        for (int u = 0; u < U; ++u) vzero(acc[u]);
+        for (uint32_t t0 = s; __any_sync(kAll, t0 < e); t0 += L) {
+            const uint32_t mine = next;
+            next = t0 + L + tl < e ? __ldg(perm + t0 + L + tl) : 0u;
+#pragma unroll 1
+            for (int j = 0; j < L; j += kRows) {
+                if (!__any_sync(kAll, t0 + j < e)) break;
+                V v[kRows][U];
+                float sg[kRows];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (colok[u]) vatomic_add(reinterpret_cast<V*>(out + (u * 32 + lane) * VEC), acc[u]);
+                for (int q = 0; q < kRows; ++q) {
+                    const uint32_t p = __shfl_sync(kAll, mine, sh + j + q);
+                    const bool ok = t0 + j + q < e;
+                    sg[q] = (p >> 31) ? -1.0f : 1.0f;
+                    const float* row = A + (int64_t)(p & 0x7fffffffu) * lda + c0;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (ok && colok[u]) v[q][u] = ldg_stream<VEC>(row + (u * L + tl) * VEC);
+                        else vzero(v[q][u]);
+                    }
+                }
+                // no team's bucket ends among these rows: summed in pairs first,
+                // an eighth (a quarter) of the roundings into the running sum
+                const uint32_t t8 = t0 + j + kRows;
+                if (__all_sync(kAll, (t8 < end && t8 < e) || t0 + j >= e)) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        V x[kRows / 2];
+#pragma unroll
+                        for (int q = 0; q < kRows / 2; ++q) {
+                            vzero(x[q]);
+                            vadd(x[q], v[2 * q][u], sg[2 * q]);
+                            vadd(x[q], v[2 * q + 1][u], sg[2 * q + 1]);
+                        }
+#pragma unroll
+                        for (int o = kRows / 4; o; o >>= 1)
+#pragma unroll
+                            for (int q = 0; q < o; ++q) vadd(x[q], x[q + o], 1.0f);
+                        vadd(acc[u], x[0], 1.0f);
+                    }
+                    continue;
+                }
+#pragma unroll
+                for (int q = 0; q < kRows; ++q) {
+                    const uint32_t t = t0 + j + q + 1;   // past this row
+#pragma unroll
+                    for (int u = 0; u < U; ++u) vadd(acc[u], v[q][u], sg[q]);
+                    const bool last = t <= e && (t == end || t == e);
+                    if (!__any_sync(kAll, last)) continue;
+                    if (last) {
+                        float* out = SA + orow * d + c0;
+                        const bool store = whole && end <= e && !accumulate;
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            if (colok[u]) {
+                                V* o = reinterpret_cast<V*>(out + (u * L + tl) * VEC);
+                                if (store) *o = acc[u];
+                                else vatomic_add(o, acc[u]);
+                            }
+                            vzero(acc[u]);
+                        }
+                        whole = true;
+                    }
+                    find(t, last && t < e);
+                }
+            }
+        }
+        if (own && !accumulate && !cpos) {          // empty buckets
+            for (int64_t x0 = b0; __any_sync(kAll, x0 < b1); x0 += L) {
+                const int64_t x = x0 + tl;
+                const bool empty = x < b1 && __ldg(off + x) == __ldg(off + x + 1);
+                unsigned m = (__ballot_sync(kAll, empty) >> sh) & kTeam;
+                while (m) {
+                    float* out = SA + (x0 + __ffs(m) - 1) * d + c0;
+                    m &= m - 1;
+                    V z;
+                    vzero(z);
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (colok[u]) *reinterpret_cast<V*>(out + (u * L + tl) * VEC) = z;
+                }
             }
         }
     }
@@ -859,35 +966,45 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
     const int64_t n = A->n, d = A->d;
     cudaError_t e = cudaSuccess;
     const bool compact = cpos != nullptr;
-    // parts per bucket: enough warps to stream A when there are few buckets,
-    // while each part keeps several rows (one part a bucket when compacting)
-    int P = 1;
-    while (!compact && P < 32 && r * P < 16384 && n >= (int64_t)r * P * 8) P *= 2;
-    if (P > 1 && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
-    const int acc = accumulate ? 1 : 0;   // add into SA (the parts add atomically either way)
-    const int64_t warps_needed = r * P;
+    const int acc = accumulate ? 1 : 0;   // add into SA (shared buckets add atomically either way)
     if (A->kind == LSK_DENSE) {
         const float* Av = (const float*)A->values;
-        const bool vec4 = (d % 4 == 0) && (A->ld % 4 == 0) && (((uintptr_t)Av & 15) == 0) &&
-                          (((uintptr_t)SA & 15) == 0);
-        const unsigned grid = grid_for(warps_needed * 32, 256, sm_count, 8);
-        if (vec4) {
-            if (d <= 128)
-                LSK_PROF("cs_dense_gather", st) cs_dense_gather_kernel<4, 1><<<grid, 256, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, P, acc, cpos);
-            else
-                LSK_PROF("cs_dense_gather", st) cs_dense_gather_kernel<4, 2><<<grid, 256, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, P, acc, cpos);
-        } else {
-            if (d <= 32)
-                LSK_PROF("cs_dense_gather", st) cs_dense_gather_kernel<1, 1><<<grid, 256, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, P, acc, cpos);
-            else
-                LSK_PROF("cs_dense_gather", st) cs_dense_gather_kernel<1, 2><<<grid, 256, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, P, acc, cpos);
-        }
+        const uintptr_t at = (uintptr_t)Av | (uintptr_t)SA | (uintptr_t)(4 * d) | (uintptr_t)(4 * A->ld);
+        const int vec = (at & 15) == 0 ? 4 : (at & 7) == 0 ? 2 : 1;
+        const int L = vec == 4 ? (d <= 32 ? 8 : d <= 64 ? 16 : 32) : 32;
+        // one wave of teams, of 8 rows at least
+        int64_t teams = (int64_t)sm_count * gather_per_sm(vec) * kGatherThreads / L;
+        teams = std::max<int64_t>(1, std::min(teams, (n + 7) / 8));
+        // Whole buckets per team where each has eight of them, or two that are
+        // short: the rows are then shared out to about an eighth, or to a few
+        // dozen rows, and SA need not be zeroed.  A compacted SA holds no rows
+        // for the empty buckets to zero, and its buckets are short.
+        const int own = compact || r >= 8 * teams || (r >= 2 * teams && n <= 32 * r) ? 1 : 0;
+        if (!own && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
+        const unsigned grid = (unsigned)((teams * L + kGatherThreads - 1) / kGatherThreads);
+        auto launch = [&](auto kernel) {
+            LSK_PROF("cs_dense_gather", st) kernel<<<grid, kGatherThreads, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, teams, own, acc, cpos);
+        };
+        if (L == 8) launch(cs_dense_gather_kernel<4, 1, 8>);
+        else if (L == 16) launch(cs_dense_gather_kernel<4, 1, 16>);
+        else if (vec == 4 && d <= 128) launch(cs_dense_gather_kernel<4, 1, 32>);
+        else if (vec == 4) launch(cs_dense_gather_kernel<4, 2, 32>);
+        else if (vec == 2 && d <= 64) launch(cs_dense_gather_kernel<2, 1, 32>);
+        else if (vec == 2) launch(cs_dense_gather_kernel<2, 2, 32>);
+        else if (d <= 32) launch(cs_dense_gather_kernel<1, 1, 32>);
+        else launch(cs_dense_gather_kernel<1, 2, 32>);
     } else {
         // shared-memory row per warp: pick warps per block to fit 200 KB
         int warps = 8;
         while (warps > 1 && (size_t)warps * d * 4 > 200 * 1024) warps >>= 1;
         const size_t smem = (size_t)warps * d * 4;
         if (smem > 200 * 1024) return cudaErrorInvalidValue;
+        // parts per bucket: enough warps to stream A when there are few buckets,
+        // while each part keeps several rows (one part a bucket when compacting)
+        int P = 1;
+        while (!compact && P < 32 && r * P < 16384 && n >= (int64_t)r * P * 8) P *= 2;
+        if (P > 1 && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
+        const int64_t warps_needed = r * P;
         if (smem > 48 * 1024) {
             e = allow_dynamic_smem(cs_csr_gather_kernel);
             if (e != cudaSuccess) return e;
