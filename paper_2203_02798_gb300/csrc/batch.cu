@@ -230,7 +230,9 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
             const lsk_batch_item& it = items[i];
             cudaError_t er = cudaSuccess;
             if (b->grouped[i]) {
-                if (b->wave[i] == w) {
+                if (b->wave[i] == w && cs_scatters(&it.A, it.r, b->cidx[i] != nullptr)) {
+                    er = cs_csr_scatter_launch(&it.A, it.r, it.seed, b->SA[i], ctx->flag, ctx->sm_count, st);
+                } else if (b->wave[i] == w) {
                     if (!prepared && (er = cudaStreamWaitEvent(st, ev_prep(w), 0)) != cudaSuccess) return er;
                     prepared = true;
                     const CsGroup& g = b->cg[w];
@@ -353,6 +355,7 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
                  gauss_group_part_bytes(rs, d, k, wslice[b->wave[i]]) + ws_round(qr_workspace_bytes(k, d)) +
                  ws_round((size_t)d * d * 4) + (compacts(items[i]) ? ws_round((size_t)(rs + 1) * 4) : 0) +
                  ws_round(prepared_bytes(items[i], prec));
+        if (cs_scatters(&items[i].A, items[i].r, compacts(items[i]))) continue;   // no permutation
         wrows[b->wave[i]] += items[i].A.n;
         wcnt[b->wave[i]] += items[i].r + 1;
     }
@@ -401,8 +404,10 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
             gjob.rcount = cidx + rs;
         }
         gj[b->wave[i]].push_back(gjob);
-        cj[b->wave[i]].push_back(CsJob{items[i].A.n, items[i].r, items[i].seed, cidx, cidx ? cidx + rs : nullptr, 0});
-        cj_item[b->wave[i]].push_back(i);
+        if (!cs_scatters(&items[i].A, items[i].r, cidx != nullptr)) {
+            cj[b->wave[i]].push_back(CsJob{items[i].A.n, items[i].r, items[i].seed, cidx, cidx ? cidx + rs : nullptr, 0});
+            cj_item[b->wave[i]].push_back(i);
+        }
         QrJob q{};
         qr_group_job(q, GSA, k, d, qws, nullptr, Ri32, ctx->flag);
         qj[b->wave[i]].push_back(q);

@@ -658,6 +658,58 @@ __global__ void cs_csr_gather_kernel(const float* __restrict__ V, const int32_t*
     }
 }
 
+// ---- CSR scatter ----------------------------------------------------------
+// S A without a permutation: a warp hashes 32 consecutive rows, then deals
+// their nonzeros out to its lanes, each one reduction in L2 on its entry of SA
+// (zeroed first).  The entries of A are read once, in order; L2 takes 176
+// scattered reductions a ns where they spread over 2^20 addresses, 82 over
+// 2^14, so the reductions cost less than finding each bucket's rows and
+// fetching their two or three nonzeros from anywhere in A: the sketch of 1M x
+// 200 at 1% into 40,000 buckets takes 28 us (79 with the permutation), 500,000 x
+// 256 at 2% into 65,536 32 (98), 20,000 x 64 at 5% into 4,096 14 (30).
+__global__ void __launch_bounds__(256) cs_csr_scatter_kernel(const float* __restrict__ V,
+                                                             const int32_t* __restrict__ J,
+                                                             const int64_t* __restrict__ I, int64_t n, int64_t nnz,
+                                                             int64_t d, uint64_t row0, uint32_t r, uint32_t k0,
+                                                             uint32_t k1, float* __restrict__ SA, int* flag) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    bool bad = false;
+    for (int64_t i0 = warp * 32; i0 < n; i0 += nwarps * 32) {
+        RowGroup g;
+        if (!g.load(I, i0 + lane, n, nnz)) bad = true;
+        uint32_t b, neg;
+        cs_hash(row0 + (uint64_t)(i0 + lane), r, k0, k1, b, neg);
+        const uint32_t to = b | (neg << 31);
+        constexpr int kEntries = 2;   // entries a lane at once
+        for (int64_t e0 = 0; e0 < g.total; e0 += 32 * kEntries) {
+            int32_t col[kEntries];
+            float v[kEntries];
+            uint32_t t[kEntries];
+#pragma unroll
+            for (int u = 0; u < kEntries; ++u) {
+                const int64_t e = min(e0 + 32 * u + lane, g.total - 1);
+                const int q = g.lane_of(e);
+                const int64_t at = __shfl_sync(0xffffffffu, g.first, q) + e;
+                t[u] = __shfl_sync(0xffffffffu, to, q);
+                col[u] = __ldg(J + at);
+                v[u] = __ldg(V + at);
+            }
+#pragma unroll
+            for (int u = 0; u < kEntries; ++u) {
+                if (e0 + 32 * u + lane >= g.total) continue;
+                if (col[u] < 0 || col[u] >= d) {
+                    bad = true;
+                    continue;
+                }
+                atomicAdd(SA + (int64_t)(t[u] & 0x7fffffffu) * d + col[u], (t[u] >> 31) ? -v[u] : v[u]);
+            }
+        }
+    }
+    if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
+}
+
 __global__ void cs_hash_debug_kernel(int64_t n, uint32_t r, uint32_t k0, uint32_t k1,
                                      int32_t* bucket, int8_t* sign) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -943,15 +995,39 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
     return cudaGetLastError();
 }
 
+// Every CSR sketch but a compacted one (which needs the buckets' counts), one of
+// so few entries that the reductions queue up at their addresses (2^14), and one
+// that sums more than 16 nonzeros to an entry: there the permutation's form,
+// with partial sums of parts of a bucket, rounds less (r = 64 of 1M x 256 at 5%,
+// 781 to an entry: error 1.4e-7 against 5.0e-7 at 269 and 130 us; with 10 to an
+// entry 5.5e-8 against 6.4e-8 at 147 and 50 us).
+bool cs_scatters(const lsk_mat* A, int64_t r, bool compact) {
+    return A->kind == LSK_CSR && !compact && r * A->d >= (1 << 14) && r < ((int64_t)1 << 31) &&
+           A->nnz / 16 <= r * A->d;
+}
+
+cudaError_t cs_csr_scatter_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, int* flag, int sm_count,
+                                  cudaStream_t st, uint64_t row0, bool accumulate) {
+    cudaError_t e;
+    if (!accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * A->d * 4, st)) != cudaSuccess) return e;
+    if (A->n <= 0) return cudaSuccess;
+    LSK_PROF("cs_csr_scatter", st) cs_csr_scatter_kernel<<<grid_for(A->n, 256, sm_count, 32), 256, 0, st>>>(
+        (const float*)A->values, A->colidx, A->rowptr, A->n, A->nnz, A->d, row0, (uint32_t)r, (uint32_t)seed,
+        (uint32_t)(seed >> 32), SA, flag);
+    return cudaGetLastError();
+}
+
 cudaError_t cs_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, void* ws, int* flag,
                       int sm_count, cudaStream_t st, uint64_t row0, bool accumulate, uint32_t* cidx,
                       uint32_t* ccount, bool rx) {
     const int64_t n = A->n;
+    const bool compact = cidx != nullptr && ccount != nullptr && !accumulate;
+    if (cs_scatters(A, r, compact))
+        return cs_csr_scatter_launch(A, r, seed, SA, flag, sm_count, st, row0, accumulate);
     const uint32_t* off = nullptr;
     const uint32_t* perm = nullptr;
     cudaError_t e = cs_prep_launch(n, r, seed, ws, sm_count, st, &off, &perm, row0, flag, rx);
     if (e != cudaSuccess) return e;
-    const bool compact = cidx != nullptr && ccount != nullptr && !accumulate;
     uint32_t* cpos = nullptr;
     if (compact) {
         cpos = cs_carve(ws, n, r, nullptr).cpos;   // the same place in either form

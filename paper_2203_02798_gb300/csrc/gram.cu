@@ -7,13 +7,17 @@
 //         chunk of rows; FP32 products are accumulated in registers and
 //         folded into FP64 every kFold rows (bounding FP32 chain length), the
 //         FP64 partials of the chunks are added in a fixed order.
-//  CSR:   a block owns a slice of rows of C held in shared memory (the
-//         "private d x d" of Alg. 7, sliced so it fits) and a range of rows
-//         of A; each thread runs Alg. 5 on its rows (the upper-triangle
-//         outer products of the row's nonzeros, shared-memory atomics), the
-//         FP32 slices of all blocks are then summed in FP64 in a fixed order
-//         and mirrored.
+//  CSR:   sparse rows or large d: warps deal 32 rows' nonzeros out to their
+//         lanes and add the products to a partial matrix per block (the
+//         "private d x d" of Alg. 7) by reductions in L2.  Else a block owns a
+//         slice of rows of C held in shared memory and a range of rows of A;
+//         each thread runs Alg. 5 on its rows (the upper-triangle outer
+//         products of the row's nonzeros, shared-memory atomics).  The
+//         partials of all blocks are then summed with compensation and
+//         mirrored.
 #include "lsk_internal.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -188,6 +192,62 @@ __global__ void __launch_bounds__(1024) gram_csr_kernel(const float* __restrict_
     for (int64_t e = threadIdx.x; e < sl * d; e += blockDim.x) P[e] = S[e];
 }
 
+// The same products as reductions in L2.  A warp takes 32 consecutive rows and
+// deals their nonzeros out to its lanes; the lane of entry p adds the products
+// with the entries after it to one of the `copies` partial matrices (zeroed
+// first), a copy per block, or a few blocks to one where d is large, so that
+// no entry's reductions queue up and each copy sums as few products as the
+// shared-memory form's.  The diagonal, which every row hits, is summed in shared
+// memory.  Shared memory has no FP32 add: its loop of compare-and-swap with a
+// row a thread, two nonzeros in most, left lanes and time idle.  1M x 200 with
+// two nonzeros a row: 58 us (86), 1M x 256 79 (194).
+__global__ void __launch_bounds__(1024) gram_csr_red_kernel(const float* __restrict__ V, const int32_t* __restrict__ J,
+                                                           const int64_t* __restrict__ I, int64_t n, int64_t nnz,
+                                                           int64_t d, float* __restrict__ part, int copies,
+                                                           int* flag) {
+    extern __shared__ float D[];
+    float* P = part + (int64_t)(blockIdx.x % copies) * d * d;
+    for (int64_t c = threadIdx.x; c < d; c += blockDim.x) D[c] = 0.f;
+    if (copies == (int)gridDim.x)   // the block's own; else zeroed before the launch
+        for (int64_t c = threadIdx.x; c < d * d; c += blockDim.x) P[c] = 0.f;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    // consecutive groups go to different blocks: few rows still reach every copy
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    bool bad = false;
+    for (int64_t i0 = warp * 32; i0 < n; i0 += nwarps * 32) {
+        RowGroup g;
+        if (!g.load(I, i0 + lane, n, nnz)) bad = true;
+        const int64_t stop = g.first + g.upto;   // past this lane's row
+        for (int64_t e0 = 0; e0 < g.total; e0 += 32) {
+            const int64_t e = min(e0 + lane, g.total - 1);
+            const int q = g.lane_of(e);
+            const int64_t at = __shfl_sync(0xffffffffu, g.first, q) + e, last = __shfl_sync(0xffffffffu, stop, q);
+            if (e0 + lane >= g.total) continue;
+            const int32_t jp = __ldg(J + at);
+            if (jp < 0 || jp >= d) {
+                bad = true;
+                continue;
+            }
+            const float vp = __ldg(V + at);
+            float own = vp * vp;
+            for (int64_t k = at + 1; k < last; ++k) {
+                const int32_t jq = __ldg(J + k);
+                if (jq < 0 || jq >= d) continue;
+                const float w = vp * __ldg(V + k);
+                if (jp == jq) own += 2.f * w;
+                else atomicAdd(P + (int64_t)min(jp, jq) * d + max(jp, jq), w);
+            }
+            atomicAdd(&D[jp], own);
+        }
+    }
+    if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
+    __syncthreads();
+    for (int64_t c = threadIdx.x; c < d; c += blockDim.x)
+        if (D[c] != 0.f) atomicAdd(P + c * d + c, D[c]);
+}
+
 // C[a][b] = C[b][a] = alpha sum_z part[z][a][b] + beta C (a <= b): a block
 // takes 32 consecutive entries; thread (g, x) adds the partials z = g, g + 8,
 // ... of entry x with compensation, then the 8 group sums are added in order
@@ -262,6 +322,14 @@ CsrPlan csr_plan(int64_t n, int64_t d, int sm_count) {
     return p;
 }
 
+// Reductions in L2 where rows hold four nonzeros or fewer on average, or where
+// a partial matrix does not fit in shared memory, whose form then reads A once
+// per slice.  Denser rows make d^2 products each out of few loads: with 6.4
+// nonzeros a row (300,000 x 128) 106 us against 100, with 16 (100,000 x 32) 171
+// against 148; with 3.2 (300,000 x 64) 44 against 52; 50,000 x 256 with 128, two
+// slices, 2.8 ms against 6.7.
+bool gram_csr_reduces(const lsk_mat* A, const CsrPlan& p) { return p.nslices > 1 || A->nnz / 4 <= A->n; }
+
 }  // namespace
 
 size_t gram_workspace_bytes(const lsk_mat* A, int sm_count) {
@@ -294,11 +362,21 @@ cudaError_t gram_launch_t(const lsk_mat* A, double alpha, double beta, OutT* C, 
             <<<(unsigned)((len + 31) / 32), 256, 0, st>>>(part, p.nchunks, d, alpha, beta, C, redo);
     } else {
         const CsrPlan p = csr_plan(n, d, sm_count);
-        if (p.smem > 48 * 1024) {
-            cudaError_t e = allow_dynamic_smem(gram_csr_kernel);
-            if (e != cudaSuccess) return e;
-        }
         float* part = (float*)ws;
+        cudaError_t e;
+        if (gram_csr_reduces(A, p)) {
+            if ((e = allow_dynamic_smem(gram_csr_red_kernel)) != cudaSuccess) return e;
+            const int64_t groups = std::max<int64_t>(1, (n + 31) / 32);
+            const int blocks = (int)std::min<int64_t>(groups, sm_count);
+            const int copies = (int)std::min<int64_t>(blocks, p.nblocks);
+            if (copies < blocks && (e = cudaMemsetAsync(part, 0, (size_t)(copies * len) * 4, st)) != cudaSuccess) return e;
+            LSK_PROF("gram_csr", st) gram_csr_red_kernel<<<blocks, 1024, (size_t)d * 4, st>>>(
+                (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, part, copies, flag);
+            LSK_PROF("gram_reduce", st) gram_csr_reduce_kernel<OutT>
+                <<<(unsigned)((len + 31) / 32), 256, 0, st>>>(part, copies, d, alpha, beta, C);
+            return cudaGetLastError();
+        }
+        if (p.smem > 48 * 1024 && (e = allow_dynamic_smem(gram_csr_kernel)) != cudaSuccess) return e;
         dim3 grid((unsigned)p.nblocks, (unsigned)p.nslices);
         LSK_PROF("gram_csr", st) gram_csr_kernel<<<grid, 1024, p.smem, st>>>((const float*)A->values, A->colidx,
                                                                             A->rowptr, n, A->nnz, d, p.slice_rows,
