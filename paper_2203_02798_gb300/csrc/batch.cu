@@ -238,7 +238,7 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
                     const CsGroup& g = b->cg[w];
                     er = cs_gather_launch(&it.A, it.r, g.off + b->cnt_base[i], g.perm,
                                           b->cidx[i] ? g.cpos + b->cnt_base[i] : nullptr, b->SA[i], ctx->flag,
-                                          ctx->sm_count, st);
+                                          ctx->sm_count, st, false, false);
                 }
             } else if (w == 0) {
                 er = leverage_pipeline(&it.A, it.r, it.k, it.seed, prec, it.ell, nullptr, b->ws[s], ctx->flag,
@@ -313,7 +313,7 @@ bool groupable(const lsk_batch_item& it, int32_t prec) {
 // the schedule's longer slices give that many already: 196 us.  Of 2, 4 and 8
 // blocks an SM the whole call takes 1071, 1078 and 1093 us with 24 problems,
 // 4.37, 4.53 and 4.83 ms with 64, 7.22, 7.25 and 7.55 ms with 160 small ones.
-constexpr int64_t kGaussBlocksPerSm = 2, kGaussMinSlice = 8;
+constexpr int64_t kGaussBlocksPerSm = 2, kGaussMinSlice = 24;
 int group_slice(int64_t chunks, int slice, int sm_count) {
     const int64_t want = (chunks + kGaussBlocksPerSm * sm_count - 1) / (kGaussBlocksPerSm * sm_count);
     return (int)std::min<int64_t>(slice, std::max(want, kGaussMinSlice));

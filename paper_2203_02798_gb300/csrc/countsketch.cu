@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(kScanBlock) scan_lookback_kernel(const uint32_
                                                                    uint32_t* __restrict__ off,
                                                                    uint32_t* __restrict__ cursor, int64_t len,
                                                                    unsigned long long* state, int* flag) {
+    pdl_enter(in, off, cursor, state);
     __shared__ uint32_t warp_tot[kScanBlock / 32];
     __shared__ uint32_t s_tile, s_prefix;
     if (threadIdx.x == 0) s_tile = atomicAdd(reinterpret_cast<unsigned int*>(state), 1u);
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(kRxThreads) rx_count_kernel(int64_t n, uint64_
                                                               uint32_t k1, RxPlan q, uint32_t* __restrict__ bsign,
                                                               uint32_t* __restrict__ H, unsigned long long* hstate,
                                                               int hstate_words) {
+    pdl_enter(bsign, H, hstate);
     extern __shared__ uint32_t hs[];
     if (blockIdx.x == 0)   // the scan's state, zeroed for the next launch
         for (int j = threadIdx.x; j < hstate_words; j += blockDim.x) hstate[j] = 0ull;
@@ -297,6 +299,7 @@ __global__ void __launch_bounds__(kRxThreads) rx_scatter_kernel(int64_t n, RxPla
                                                                 const uint32_t* __restrict__ bsign,
                                                                 const uint32_t* __restrict__ base,
                                                                 uint32_t* __restrict__ T, uint16_t* __restrict__ TF) {
+    pdl_enter(bsign, base, T, TF);
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t wsum[kRxThreads / 32 + 1];
     uint32_t* hb = sm;                 // [B] global start of this block's run in coarse bucket c
@@ -338,6 +341,7 @@ __global__ void __launch_bounds__(kRxThreads) rx_fine_kernel(int64_t n, int64_t 
                                                              const uint32_t* __restrict__ T,
                                                              const uint16_t* __restrict__ TF,
                                                              uint32_t* __restrict__ perm, uint32_t* __restrict__ off) {
+    pdl_enter(base, T, TF, perm, off);
     extern __shared__ uint32_t fc[];   // [F] counts, then starts; then the staged rows
     __shared__ uint32_t wsum[kRxThreads / 32 + 1];
     uint32_t* stage = fc + q.F;
@@ -457,6 +461,7 @@ __global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC)) cs_dense_g
     const float* __restrict__ A, int64_t lda, int64_t d, uint32_t r, const uint32_t* __restrict__ off,
     const uint32_t* __restrict__ perm, float* __restrict__ SA, int64_t teams, int own, int accumulate,
     const uint32_t* __restrict__ cpos) {
+    pdl_enter(A, off, perm, cpos, SA);
     using V = typename VecT<VEC>::T;
     constexpr unsigned kAll = 0xffffffffu, kTeam = L == 32 ? kAll : (1u << (L & 31)) - 1u;
     constexpr int kCols = L * VEC * U;              // columns per pass
@@ -968,15 +973,15 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
     if (two_level) {
         if ((e = allow_dynamic_smem(rx_scatter_kernel)) != cudaSuccess) return e;
         if ((e = allow_dynamic_smem(rx_fine_kernel)) != cudaSuccess) return e;
-        LSK_PROF("cs_count", st) rx_count_kernel<<<q.nct, kRxThreads, (size_t)q.B * 4, st>>>(
-            n, row0, (uint32_t)r, k0, k1, q, w.bsign, w.H, w.hstate, w.hstate_words);
+        LSK_PROF("cs_count", st) launch_pdl(rx_count_kernel, q.nct, kRxThreads, (size_t)q.B * 4, 1, st, n, row0, (uint32_t)r,
+                                             k0, k1, q, w.bsign, w.H, w.hstate, w.hstate_words);
         const int64_t len = q.B * q.nct;
-        LSK_PROF("cs_scan", st) scan_lookback_kernel<<<(unsigned)((len + kScanTile - 1) / kScanTile), kScanBlock, 0,
-                                                       st>>>(w.H, w.H, nullptr, len, w.hstate, flag);
-        LSK_PROF("cs_place", st) rx_scatter_kernel<<<q.nct, kRxThreads, rx_scatter_smem(q), st>>>(n, q, w.bsign, w.H,
-                                                                                                  w.T, w.TF);
-        LSK_PROF("cs_fine", st) rx_fine_kernel<<<(unsigned)q.B, kRxThreads, rx_fine_smem(q), st>>>(n, r, q, w.H, w.T,
-                                                                                                   w.TF, w.perm, w.off);
+        LSK_PROF("cs_scan", st) launch_pdl(scan_lookback_kernel, (unsigned)((len + kScanTile - 1) / kScanTile), kScanBlock, 0, 1,
+                                            st, w.H, w.H, nullptr, len, w.hstate, flag);
+        LSK_PROF("cs_place", st) launch_pdl(rx_scatter_kernel, q.nct, kRxThreads, rx_scatter_smem(q), 1, st, n, q, w.bsign, w.H,
+                                             w.T, w.TF);
+        LSK_PROF("cs_fine", st) launch_pdl(rx_fine_kernel, (unsigned)q.B, kRxThreads, rx_fine_smem(q), 1, st, n, r, q, w.H, w.T,
+                                            w.TF, w.perm, w.off);
         *off_out = w.off;
         *perm_out = w.perm;
         return cudaGetLastError();
@@ -986,7 +991,7 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
     if (e != cudaSuccess) return e;
     if (n > 0) LSK_PROF("cs_count", st) cs_count_kernel<<<grid_for(n, 256, sm_count), 256, 0, st>>>(n, row0, (uint32_t)r, k0, k1, w.cnt);
     const unsigned tiles = (unsigned)((r + kScanTile - 1) / kScanTile);
-    LSK_PROF("cs_scan", st) scan_lookback_kernel<<<tiles, kScanBlock, 0, st>>>(w.cnt, w.off, w.cursor, r, w.state, flag);
+    LSK_PROF("cs_scan", st) launch_pdl(scan_lookback_kernel, tiles, kScanBlock, 0, 1, st, w.cnt, w.off, w.cursor, r, w.state, flag);
     if (n > 0) {
         LSK_PROF("cs_place", st) cs_place_kernel<<<grid_for(n, 256, sm_count), 256, 0, st>>>(n, row0, (uint32_t)r, k0, k1, w.cursor, w.perm);
     }
@@ -1038,7 +1043,7 @@ cudaError_t cs_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, voi
 
 cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, const uint32_t* perm,
                              const uint32_t* cpos, float* SA, int* flag, int sm_count, cudaStream_t st,
-                             bool accumulate) {
+                             bool accumulate, bool early) {
     const int64_t n = A->n, d = A->d;
     cudaError_t e = cudaSuccess;
     const bool compact = cpos != nullptr;
@@ -1059,7 +1064,8 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         if (!own && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
         const unsigned grid = (unsigned)((teams * L + kGatherThreads - 1) / kGatherThreads);
         auto launch = [&](auto kernel) {
-            LSK_PROF("cs_dense_gather", st) kernel<<<grid, kGatherThreads, 0, st>>>(Av, A->ld, d, (uint32_t)r, off, perm, SA, teams, own, acc, cpos);
+            LSK_PROF("cs_dense_gather", st) launch_chained(early, kernel, grid, kGatherThreads, 0, 1, st, Av, A->ld, d,
+                                                           (uint32_t)r, off, perm, SA, teams, own, acc, cpos);
         };
         if (L == 8) launch(cs_dense_gather_kernel<4, 1, 8>);
         else if (L == 16) launch(cs_dense_gather_kernel<4, 1, 16>);
@@ -1142,8 +1148,8 @@ cudaError_t cs_group_launch(const CsGroup& g, const unsigned char* table, int* f
     if (g.blocks > 0)
         LSK_PROF("cs_count", st) cs_rows_grouped_kernel<false><<<g.blocks, kGroupThreads, 0, st>>>(
             ps, boff, g.count, g.cnt, nullptr);
-    LSK_PROF("cs_scan", st) scan_lookback_kernel<<<(unsigned)((g.counters + kScanTile - 1) / kScanTile), kScanBlock, 0,
-                                                   st>>>(g.cnt, g.off, g.cursor, g.counters, g.state, flag);
+    LSK_PROF("cs_scan", st) launch_pdl(scan_lookback_kernel, (unsigned)((g.counters + kScanTile - 1) / kScanTile), kScanBlock,
+                                        0, 1, st, g.cnt, g.off, g.cursor, g.counters, g.state, flag);
     if (g.blocks > 0)
         LSK_PROF("cs_place", st) cs_rows_grouped_kernel<true><<<g.blocks, kGroupThreads, 0, st>>>(
             ps, boff, g.count, g.cursor, g.perm);

@@ -23,6 +23,7 @@ constexpr int BK = 16;    // reduction step
 __global__ void __launch_bounds__(256, 2) gauss_simt_kernel(
     const float* __restrict__ SA, int64_t r, int64_t d, int64_t k, uint32_t k0, uint32_t k1,
     float scale, int bf16, int64_t kc, float* __restrict__ part) {
+    pdl_enter(SA, part);
     __shared__ __align__(16) float Gs[BK][BM];
     __shared__ __align__(16) float Ss[BK][BN];
     const int tid = threadIdx.x;
@@ -112,14 +113,22 @@ __global__ void __launch_bounds__(256, 2) gauss_simt_kernel(
     }
 }
 
-// GSA[e] = sum_z part[z][e] in FP64, in increasing z.
+// GSA[e] = sum_z part[z][e], compensated in FP32, in increasing z, with eight
+// loads in flight (FP64 adds and conversions issue at 1/64 of the FP32 rate).
 __global__ void reduce_partials_kernel(const float* __restrict__ part, int64_t nz, int64_t len,
                                        float* __restrict__ out) {
+    pdl_enter(part, out);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
-        double s = 0.0;
-        for (int64_t z = 0; z < nz; ++z) s += (double)part[z * len + e];
-        out[e] = (float)s;
+        float s = 0.f, c = 0.f;
+        for (int64_t z = 0; z < nz; z += 8) {
+            float v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = z + q < nz ? part[(z + q) * len + e] : 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) comp_add(s, c, v[q]);
+        }
+        out[e] = s + c;
     }
 }
 
@@ -192,12 +201,12 @@ cudaError_t gauss_launch(const float* SA, int64_t r, int64_t d, int64_t k, uint6
     const float scale = (float)(1.0 / sqrt((double)k));
     dim3 grid((unsigned)p.tiles_n, (unsigned)p.tiles_m, (unsigned)p.nz);
     float* part = (float*)ws;
-    LSK_PROF("gauss_simt", st) gauss_simt_kernel<<<grid, 256, 0, st>>>(SA, r, d, k, (uint32_t)seed, (uint32_t)(seed >> 32),
-                                            scale, prec == LSK_PREC_BF16 ? 1 : 0, p.kc, part);
+    LSK_PROF("gauss_simt", st) launch_pdl(gauss_simt_kernel, grid, 256, 0, 1, st, SA, r, d, k, (uint32_t)seed,
+                                           (uint32_t)(seed >> 32), scale, prec == LSK_PREC_BF16 ? 1 : 0, p.kc, part);
     const int64_t len = k * d;
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
-    LSK_PROF("gauss_reduce", st) reduce_partials_kernel<<<(unsigned)g, 256, 0, st>>>(part, p.nz, len, GSA);
+    LSK_PROF("gauss_reduce", st) launch_pdl(reduce_partials_kernel, (unsigned)g, 256, 0, 1, st, part, p.nz, len, GSA);
     return cudaGetLastError();
 }
 

@@ -362,7 +362,11 @@ __device__ __forceinline__ void gauss_tc_body(const GtParams& p, const int blk) 
 }
 
 template <int T>
-__global__ void __launch_bounds__(kThreads, 1) gauss_tc_kernel(const GtParams p) { gauss_tc_body<T>(p, blockIdx.x); }
+__global__ void __launch_bounds__(kThreads, 1) gauss_tc_kernel(const GtParams q) {
+    GtParams p = q;
+    pdl_enter(p.SA, p.part);
+    gauss_tc_body<T>(p, blockIdx.x);
+}
 
 // Grouped: the blocks of many problems in one grid.
 __global__ void __launch_bounds__(kThreads, 1) gauss_tc_grouped_kernel(const GtParams* __restrict__ ps,
@@ -423,6 +427,7 @@ __device__ __forceinline__ void reduce_body(const float* __restrict__ part, int 
 }
 __global__ void gauss_tc_reduce_kernel(const float* __restrict__ part, int slices, int64_t len,
                                        float* __restrict__ out) {
+    pdl_enter(part, out);
     reduce_body(part, slices, len, out, blockIdx.x, gridDim.x);
 }
 __global__ void gauss_tc_reduce_grouped_kernel(const GtParams* __restrict__ ps, const int* __restrict__ roff,
@@ -488,16 +493,16 @@ cudaError_t gauss_tc_launch(const float* SA, int64_t r, int64_t d, int64_t k, ui
     if (terms == 3) {
         e = allow_dynamic_smem(gauss_tc_kernel<3>);
         if (e != cudaSuccess) return e;
-        LSK_PROF("gauss_tc_fp32", st) gauss_tc_kernel<3><<<P.tiles_m * P.slices, kThreads, P.smem, st>>>(p);
+        LSK_PROF("gauss_tc_fp32", st) launch_pdl(gauss_tc_kernel<3>, P.tiles_m * P.slices, kThreads, P.smem, 1, st, p);
     } else {
         e = allow_dynamic_smem(gauss_tc_kernel<1>);
         if (e != cudaSuccess) return e;
-        LSK_PROF("gauss_tc", st) gauss_tc_kernel<1><<<P.tiles_m * P.slices, kThreads, P.smem, st>>>(p);
+        LSK_PROF("gauss_tc", st) launch_pdl(gauss_tc_kernel<1>, P.tiles_m * P.slices, kThreads, P.smem, 1, st, p);
     }
     const int64_t len = k * d;
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
-    LSK_PROF("gauss_reduce", st) gauss_tc_reduce_kernel<<<(unsigned)g, 256, 0, st>>>(p.part, P.slices, len, GSA);
+    LSK_PROF("gauss_reduce", st) launch_pdl(gauss_tc_reduce_kernel, (unsigned)g, 256, 0, 1, st, p.part, P.slices, len, GSA);
     return cudaGetLastError();
 }
 
@@ -508,7 +513,7 @@ cudaError_t gauss_tc_reduce_launch(const float* part, int slices, int64_t len, f
     if (len <= 0) return cudaSuccess;
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
-    LSK_PROF("gauss_reduce", st) gauss_tc_reduce_kernel<<<(unsigned)g, 256, 0, st>>>(part, slices, len, out);
+    LSK_PROF("gauss_reduce", st) launch_pdl(gauss_tc_reduce_kernel, (unsigned)g, 256, 0, 1, st, part, slices, len, out);
     return cudaGetLastError();
 }
 

@@ -39,32 +39,11 @@ struct CgState {
 
 constexpr int kPassThreads = 256;
 
-// Programmatic dependent launch: the passes and the vector step of the inner
-// solve alternate some 130 times, so each lets the next one's blocks start
-// (and load what no kernel of the solve writes) while it finishes; everything
-// the previous kernel writes is read after pdl_wait, with __ldcg (a load the
-// compiler may not take for one of constant memory and move ahead of the wait).  Every kernel launched
-// this way waits before it returns, so completion stays in launch order.
-__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <class F, class... Args>
-cudaError_t launch_pdl(F* kernel, int blocks, int threads, size_t smem, int cluster, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)cluster;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
+// The passes and the vector step of the inner solve alternate some 130 times, so
+// each is launched programmatically: the next one's blocks start (and load what
+// no kernel of the solve writes) while it finishes; everything the previous
+// kernel writes is read after pdl_wait, with __ldcg (a load the compiler may not
+// take for one of constant memory and move ahead of the wait).
 
 // ---- FP32 pairs: x = h + l carries ~48 bits at the FP32 rate (FP64 runs at
 // 1/64 of it here).  Products by FMA, sums by Knuth's TwoSum; a dot product

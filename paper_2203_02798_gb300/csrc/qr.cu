@@ -139,10 +139,12 @@ __device__ __forceinline__ void sketch_gram64_reduce_body(const double* __restri
 
 __global__ void __launch_bounds__(256) sketch_gram64_kernel(const float* __restrict__ B, int64_t k, int64_t d,
                                                             int64_t rows_per, double* __restrict__ part) {
+    pdl_enter(B, part);
     sketch_gram64_body(B, k, d, rows_per, part, blockIdx.x, blockIdx.y);
 }
 __global__ void sketch_gram64_reduce_kernel(const double* __restrict__ part, int64_t nchunks, int64_t d,
                                             double* __restrict__ C, float2* __restrict__ Cp) {
+    pdl_enter(part, C, Cp);
     sketch_gram64_reduce_body(part, nchunks, d, C, blockIdx.x, gridDim.x, Cp);
 }
 // grouped over QrJob tables: local block b of a job = (tile b % ntiles, chunk b / ntiles)
@@ -366,11 +368,11 @@ cudaError_t sketch_gram64_launch(const float* B, int64_t k, int64_t d, double* C
                                  cudaStream_t st, float2* Cp) {
     const QrPlan p = qr_plan(k, d);
     double* part = (double*)ws;
-    LSK_PROF("qr_gram64", st) sketch_gram64_kernel<<<dim3((unsigned)p.ntiles, (unsigned)p.nchunks), 256, 0, st>>>(B, k, d, p.rows_per,
-                                                                                      part);
+    LSK_PROF("qr_gram64", st) launch_pdl(sketch_gram64_kernel, dim3((unsigned)p.ntiles, (unsigned)p.nchunks), 256, 0, 1, st, B,
+                                         k, d, p.rows_per, part);
     int64_t g = (d * d + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
-    LSK_PROF("qr_gram64", st) sketch_gram64_reduce_kernel<<<(unsigned)g, 256, 0, st>>>(part, p.nchunks, d, C, Cp);
+    LSK_PROF("qr_gram64", st) launch_pdl(sketch_gram64_reduce_kernel, (unsigned)g, 256, 0, 1, st, part, p.nchunks, d, C, Cp);
     return cudaGetLastError();
 }
 

@@ -152,6 +152,7 @@ __device__ __forceinline__ void trinv32_body(const float* __restrict__ Lpk, int 
 }
 // X = Rt^-1 as FP32 pairs (the single-sketch chain keeps its matrices in pair form)
 __global__ void __launch_bounds__(512) trinv32_pair_kernel(const float* __restrict__ Lpk, int d, float2* __restrict__ X) {
+    pdl_enter(Lpk, X);
     trinv32_body(Lpk, d, X, blockIdx.x, gridDim.x);
 }
 
@@ -456,6 +457,7 @@ __device__ __forceinline__ void chol_eq_body(const float2* __restrict__ Cp, int 
 
 __global__ void __launch_bounds__(512) chol_eq_kernel(const float2* __restrict__ Cp, int d, int* __restrict__ e_out,
                                                       float2* __restrict__ Rt, float* __restrict__ Lpk, int* flag) {
+    pdl_enter(Cp, e_out, Rt, Lpk);
     chol_eq_body(Cp, d, e_out, Rt, Lpk, flag);
 }
 
@@ -600,7 +602,11 @@ __device__ __forceinline__ void tri_gemm_pair_body(const TriGemmP& g, const int 
     }
 }
 
-__global__ void __launch_bounds__(kTgThreads) tri_gemm_pair_kernel(const TriGemmP g) { tri_gemm_pair_body(g, blockIdx.x); }
+__global__ void __launch_bounds__(kTgThreads) tri_gemm_pair_kernel(const TriGemmP q) {
+    TriGemmP g = q;
+    pdl_enter(g.A, g.B, g.Cin, g.ea, g.e, g.Out);
+    tri_gemm_pair_body(g, blockIdx.x);
+}
 
 // ---- grouped: one grid per stage over many sketches (QrJob table), the
 // same pair chain as one sketch's (R is not formed in a group) -------------
@@ -730,16 +736,16 @@ cudaError_t qr_mixed_launch(const double* C, const float2* Cp, int64_t d64, doub
         Cp = Cq;
     }
     if ((err = allow_dynamic_smem(chol_eq_kernel)) != cudaSuccess) return err;
-    LSK_PROF("qr_chol32", st) chol_eq_kernel<<<1, 512, chol_eq_smem(d), st>>>(Cp, d, e, R ? Rt : nullptr, Lpk, flag);
+    LSK_PROF("qr_chol32", st) launch_pdl(chol_eq_kernel, 1, 512, chol_eq_smem(d), 1, st, Cp, d, e, R ? Rt : nullptr, Lpk, flag);
     const size_t pk = (size_t)d * (d + 1) / 2 * 4;
     if ((err = allow_dynamic_smem(trinv32_pair_kernel)) != cudaSuccess) return err;
-    LSK_PROF("qr_trinv32", st) trinv32_pair_kernel<<<(d * 32 + 127) / 128, 128, pk, st>>>(Lpk, d, X);
+    LSK_PROF("qr_trinv32", st) launch_pdl(trinv32_pair_kernel, (d * 32 + 127) / 128, 128, pk, 1, st, Lpk, d, X);
     if ((err = allow_dynamic_smem(tri_gemm_pair_kernel)) != cudaSuccess) return err;
     const int nt = (d + TT - 1) / TT;
     const unsigned tiles = (unsigned)(nt * (nt + 1) / 2);
     const size_t tsm = tri_gemm_pair_smem(d);
     auto run = [&](const TriGemmP& g) {
-        LSK_PROF("qr_refine64", st) tri_gemm_pair_kernel<<<tiles, kTgThreads, tsm, st>>>(g);
+        LSK_PROF("qr_refine64", st) launch_pdl(tri_gemm_pair_kernel, tiles, kTgThreads, tsm, 1, st, g);
         return cudaGetLastError();
     };
     // W = Ct X on the upper triangle (only k <= j is needed by M); Ct = D^-1 C D^-1 on the fly

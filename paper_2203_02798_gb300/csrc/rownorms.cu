@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ B,
     int64_t c, int upper_tri, float alpha, float beta, float* __restrict__ x, const int* __restrict__ list,
     const int* __restrict__ count) {
+    pdl_enter(A, B, x, list, count);
     __shared__ __align__(16) float As[RK][RMP];
     __shared__ __align__(16) float Bs[RK][RN];
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -125,6 +126,7 @@ __device__ __forceinline__ void bbt_body(const float* __restrict__ B, int64_t d,
 }
 __global__ void __launch_bounds__(256) bbt_kernel(const float* __restrict__ B, int64_t d, int64_t c,
                                                   float* __restrict__ M) {
+    pdl_enter(B, M);
     bbt_body(B, d, c, M, (int64_t)blockIdx.y * 16, (int64_t)blockIdx.x * 16);
 }
 // B B^T of many problems in one launch: problem g's 16 x 16 tiles are blocks
@@ -141,10 +143,11 @@ __global__ void rownorm_csr_kernel(const float* __restrict__ V, const int32_t* _
                                    const int64_t* __restrict__ I, int64_t n, int64_t nnz, int64_t d,
                                    const float* __restrict__ M, float alpha, float beta,
                                    float* __restrict__ x, int* flag) {
+    pdl_enter(V, J, I, M, x);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int64_t k0 = I[i], k1 = I[i + 1];
+        const int64_t k0 = __ldg(I + i), k1 = __ldg(I + i + 1);
         float q = 0.f;
         if (k0 < 0 || k1 < k0 || k1 > nnz) {
             bad = true;
@@ -210,21 +213,20 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         const unsigned tiles = (unsigned)((n + RM - 1) / RM);
         if (tc3) {
             const unsigned grid = std::min(tiles, 4u * (unsigned)sm_count);
-            LSK_PROF("rownorm_dense_simt", st) rownorm_dense_kernel<true><<<grid, 256, 0, st>>>(
+            LSK_PROF("rownorm_dense_simt", st) launch_pdl(rownorm_dense_kernel<true>, grid, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, list, count);
         } else {
-            LSK_PROF("rownorm_dense_simt", st) rownorm_dense_kernel<false><<<tiles, 256, 0, st>>>(
+            LSK_PROF("rownorm_dense_simt", st) launch_pdl(rownorm_dense_kernel<false>, tiles, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, nullptr, nullptr);
         }
     } else {
         float* M = prepared ? (float*)prepared : (float*)ws;   // prepared: built by bbt_group_launch
         const dim3 bg((unsigned)((d + 15) / 16), (unsigned)((d + 15) / 16));
-        if (!prepared) LSK_PROF("rownorm_bbt", st) bbt_kernel<<<bg, 256, 0, st>>>(B, d, c, M);
+        if (!prepared) LSK_PROF("rownorm_bbt", st) launch_pdl(bbt_kernel, bg, 256, 0, 1, st, B, d, c, M);
         int64_t gr = (n + 255) / 256;
         if (gr > 16 * (int64_t)sm_count) gr = 16 * (int64_t)sm_count;
-        LSK_PROF("rownorm_csr", st) rownorm_csr_kernel<<<(unsigned)gr, 256, 0, st>>>((const float*)A->values, A->colidx, A->rowptr,
-                                                         n, A->nnz, d, M, (float)alpha, (float)beta, x,
-                                                         flag);
+        LSK_PROF("rownorm_csr", st) launch_chained(!prepared, rownorm_csr_kernel, (unsigned)gr, 256, 0, 1, st, (const float*)A->values, A->colidx,
+                                              A->rowptr, n, A->nnz, d, M, (float)alpha, (float)beta, x, flag);
     }
     return cudaGetLastError();
 }

@@ -141,6 +141,7 @@ __device__ __forceinline__ void prep_body(const float* __restrict__ B, const RnP
     }
 }
 __global__ void rownorm_tc_prep_kernel(const float* __restrict__ B, const RnParams p, uint8_t* __restrict__ img) {
+    pdl_enter(B, img);
     prep_body(B, p, img, blockIdx.x, gridDim.x);
 }
 // the images of many problems' B in one launch (kPrepBlocks blocks a problem)
@@ -1093,7 +1094,7 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
         int ncl = 0;
         const TmaVariant* tv = nullptr;
         if (!tf32_plan(A, p, ncl, &tv)) return cudaErrorNotSupported;
-        LSK_PROF("rownorm_tc_prep", st) rownorm_tc_prep_kernel<<<64, 256, 0, st>>>(B, p, img);
+        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rownorm_tc_prep_kernel, 64, 256, 0, 1, st, B, p, img);
         CUtensorMap tmA;
         if (!make_tmap(p, &tmA)) return cudaErrorNotSupported;
         const int want2 = (p.ntiles2 + kMinTiles0 - 1) / kMinTiles0;
@@ -1109,7 +1110,7 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
     p.pair = ncl > 0 ? 1 : 0;
     if (!p.pair && p.stages < 2) return cudaErrorNotSupported;
     if (img_ready) img = const_cast<uint8_t*>(img_ready);   // built by rownorms_image_group_launch
-    else LSK_PROF("rownorm_tc_prep", st) rownorm_tc_prep_kernel<<<64, 256, 0, st>>>(B, p, img);
+    else LSK_PROF("rownorm_tc_prep", st) launch_pdl(rownorm_tc_prep_kernel, 64, 256, 0, 1, st, B, p, img);
     cudaError_t e;
     // CTAs (pairs) for at least min_tiles tiles each: a small problem then
     // leaves SMs to the problems on other streams (its per-CTA set-up -- TMEM,
