@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(256) cs_csr_scatter_kernel(const float* __rest
             for (int u = 0; u < kEntries; ++u) {
                 const int64_t e = min(e0 + 32 * u + lane, g.total - 1);
                 const int q = g.lane_of(e);
-                const int64_t at = __shfl_sync(0xffffffffu, g.first, q) + e;
+                const int64_t at = g.first_of(q) + e;
                 t[u] = __shfl_sync(0xffffffffu, to, q);
                 col[u] = __ldg(J + at);
                 v[u] = __ldg(V + at);

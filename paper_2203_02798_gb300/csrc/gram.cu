@@ -219,11 +219,10 @@ __global__ void __launch_bounds__(1024) gram_csr_red_kernel(const float* __restr
     for (int64_t i0 = warp * 32; i0 < n; i0 += nwarps * 32) {
         RowGroup g;
         if (!g.load(I, i0 + lane, n, nnz)) bad = true;
-        const int64_t stop = g.first + g.upto;   // past this lane's row
         for (int64_t e0 = 0; e0 < g.total; e0 += 32) {
             const int64_t e = min(e0 + lane, g.total - 1);
             const int q = g.lane_of(e);
-            const int64_t at = __shfl_sync(0xffffffffu, g.first, q) + e, last = __shfl_sync(0xffffffffu, stop, q);
+            const int64_t first = g.first_of(q), at = first + e, last = first + g.upto_of(q);
             if (e0 + lane >= g.total) continue;
             const int32_t jp = __ldg(J + at);
             if (jp < 0 || jp >= d) {

@@ -87,3 +87,17 @@ def test_bad_csr_is_reported(lsk, spoil):
         with pytest.raises(lsk.LskError) as ei:
             lsk.context().sync()
         assert ei.value.name == "BAD_CSR"
+
+
+@pytest.mark.parametrize("kind", ["sparse", "long", "dense"])
+@pytest.mark.parametrize("n,d", [(1, 5), (31, 40), (33, 64), (5000, 64), (600, 700)])
+def test_csr_row_norms(lsk, kind, n, d):
+    """||a_i B||^2 = a_i (B B^T) a_i^T for whole numbers: every product and sum of
+    the quadratic form is exact in FP32 below 2^24, so the result is."""
+    counts = np.minimum(counts_of(kind, n), 60 if kind == "dense" else 301)
+    V, J, I = integers(counts, d, n + d)
+    V = np.sign(V).astype(np.float32)
+    B = np.random.default_rng(d).integers(-1, 2, size=(d, 3)).astype(np.float32)
+    ref = np.square(dense(V, J, I, n, d) @ B).sum(1)
+    got = lsk.rownorms_prod(csr(lsk, V, J, I, n, d), torch.from_numpy(B).cuda()).cpu().numpy()
+    assert np.array_equal(got, ref)
