@@ -21,10 +21,10 @@
 // One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
 // half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
 // 24 KB stages (128 rows x 32 K, three slices).  Warps: 0-7 epilogue (two per
-// TMEM lane quarter), 8 MMA issue (even CTA), 9-19 converters (64-row pieces:
-// 16-byte loads, scale, split, 64-byte-swizzled stores).  Up to 128 columns
+// TMEM lane quarter), 8 MMA issue (even CTA), 9-19 converters (32- or 64-row
+// pieces: 16-byte loads, scale, split, 64-byte-swizzled stores).  Up to 128 columns
 // the accumulators are double-buffered.  750,001 x 200 times 200 x 200:
-// 0.41 ms against 1.98 on CUDA cores; errors 4.5e-8 (root mean square, relative)
+// 0.38 ms against 1.98 on CUDA cores; errors 4.5e-8 (root mean square, relative)
 // against 6.8e-8, 2e-7 at most against 3.5e-7.
 #include "tc_common.cuh"
 
@@ -40,6 +40,19 @@ constexpr int kEpiWarps = 8, kMmaWarp = 8, kConv0 = 9, kConvWarps = 11;
 constexpr int kThreads = (kConv0 + kConvWarps) * 32;
 constexpr uint32_t kSlice = kRows * kKC * 2;          // one bf16 tile of a stage: 8 KB
 constexpr uint32_t kStage = 3 * kSlice;
+// Pieces a converter warp works in.  64 rows: loads, then waits for its stage,
+// then splits and stores; 16 loads a lane in flight keep A streaming.  Early, 32
+// rows: has the piece split, in registers, before it waits, and the next one's
+// loads on their way.  With B's image beside it the ring has three stages at 200
+// columns, and the time from a stage's release to its refill is what the MMAs wait
+// for (750,001 x 200 times 200 x 200: 390 us early, 431 late; 500,000 x 256
+// triangular, four stages, 246 and 250).  With five stages and more (1M x 128
+// times 128 x 128) it is A: 206 early, 170 late.
+template <bool kEarly>
+struct Piece {
+    static constexpr int kRowsOf = kEarly ? 32 : 64, kQuads = kRowsOf / 4, kParts = kRows / kRowsOf;
+};
+constexpr int kEarlyStages = 4;
 constexpr int kMaxStages = 8, kMinStages = 3;
 constexpr size_t kSmemLimit = 232448;
 constexpr uint32_t kTail = 1024;                      // barriers
@@ -67,13 +80,16 @@ __device__ __forceinline__ int exponent(float v) { return (int)(__float_as_uint(
 // s_j: 2^10 over the power of two below the median, over 64 groups of 8
 // consecutive rows spread over A, of the largest |a_ij| (a few outlying rows
 // do not move it; a column that is mostly zero takes its largest).
-__global__ void __launch_bounds__(256) rn3_units_kernel(const float* __restrict__ A, int64_t lda, int64_t n, int d,
-                                                        float* __restrict__ s, int* __restrict__ count) {
+constexpr int kUnitWarps = 32;
+__global__ void __launch_bounds__(kUnitWarps * 32) rn3_units_kernel(const float* __restrict__ A, int64_t lda, int64_t n, int d,
+                                                                  float* __restrict__ s, int* __restrict__ count) {
+    pdl_enter(A, s, count);
     __shared__ float gm[kSampleGroups][33];
     __shared__ float med[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = (int)blockIdx.x * 32 + lane;
     if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
-    for (int g = w; g < kSampleGroups; g += 8) {
+#pragma unroll
+    for (int g = w; g < kSampleGroups; g += kUnitWarps) {
         const int64_t r0 = (n - kSampleRows) * g / (kSampleGroups - 1);
         float v[kSampleRows], m = 0.f;
 #pragma unroll
@@ -85,7 +101,7 @@ __global__ void __launch_bounds__(256) rn3_units_kernel(const float* __restrict_
     __syncthreads();
     float mx = 0.f;
     for (int g = 0; g < kSampleGroups; ++g) mx = fmaxf(mx, gm[g][lane]);
-    for (int g = w; g < kSampleGroups; g += 8) {
+    for (int g = w; g < kSampleGroups; g += kUnitWarps) {
         const float v = gm[g][lane];
         int rank = 0;
         for (int h = 0; h < kSampleGroups; ++h) rank += gm[h][lane] < v || (gm[h][lane] == v && h < g);
@@ -131,11 +147,13 @@ __device__ __forceinline__ void split3(float2 y, uint32_t& hi, uint32_t& mid, ui
 // c0 + l of B) is scaled so that its largest |b_jl| / s_j is in [128, 256).
 __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict__ B, int ldb, int c0, const Rn3Params p,
                                                         uint8_t* __restrict__ img, float* __restrict__ t) {
+    const float* s = p.s;
+    pdl_enter(B, s, img, t);
     __shared__ float red[32][9];
     const int col = threadIdx.x & 7, part = threadIdx.x >> 3, l = (int)blockIdx.x * 8 + col;
     float m = 0.f;
     if (l < p.c)
-        for (int j = part; j < p.d; j += 32) m = fmaxf(m, fabsf(__ldg(B + (int64_t)j * ldb + c0 + l)) / p.s[j]);
+        for (int j = part; j < p.d; j += 32) m = fmaxf(m, fabsf(__ldg(B + (int64_t)j * ldb + c0 + l)) / s[j]);
     red[part][col] = m;
     __syncthreads();
     for (int k = 0; k < 32; ++k) m = fmaxf(m, red[k][col]);
@@ -146,8 +164,8 @@ __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict_
         const int q = i / (kKC / 2), kl = (i % (kKC / 2)) * 2, r = l - (int)p.n0[q];
         if (r < 0) continue;
         const int k = kKC * q + kl;
-        const float b0 = (k < p.d && l < p.c) ? __ldg(B + (int64_t)k * ldb + c0 + l) / p.s[k] * f : 0.f;
-        const float b1 = (k + 1 < p.d && l < p.c) ? __ldg(B + (int64_t)(k + 1) * ldb + c0 + l) / p.s[k + 1] * f : 0.f;
+        const float b0 = (k < p.d && l < p.c) ? __ldg(B + (int64_t)k * ldb + c0 + l) / s[k] * f : 0.f;
+        const float b1 = (k + 1 < p.d && l < p.c) ? __ldg(B + (int64_t)(k + 1) * ldb + c0 + l) / s[k + 1] * f : 0.f;
         uint32_t w[3];
         split3(make_float2(b0, b1), w[0], w[1], w[2]);
         const int hn = (int)p.nn[q] / 2, h = r / hn;
@@ -157,17 +175,17 @@ __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict_
     }
 }
 
-// Lane l: float4 number l + 32 i of a 64-row x 32-column piece (row l / 8 + 4 i,
-// columns 4 (l % 8) ..).
-template <bool VEC>
-__device__ __forceinline__ void load_piece(const Rn3Params& p, int64_t row0, int q, int lane, float4 (&v)[16]) {
+// Lane l: float4 number l + 32 i of a piece of 4 Q rows x 32 columns (row l / 8 +
+// 4 i, columns 4 (l % 8) ..).
+template <bool VEC, int Q>
+__device__ __forceinline__ void load_piece(const Rn3Params& p, int64_t row0, int q, int lane, float4 (&v)[Q]) {
     const int k = kKC * q + 4 * (lane & 7);
     const int64_t r0 = row0 + (lane >> 3);
-    if (VEC && row0 + 64 <= p.n && kKC * q + kKC <= p.d) {
+    if (VEC && row0 + 4 * Q <= p.n && kKC * q + kKC <= p.d) {
         const float* src = p.A + r0 * p.lda + k;
         const int64_t step = 4 * p.lda;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < Q; ++i) {
             asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
                          : "=f"(v[i].x), "=f"(v[i].y), "=f"(v[i].z), "=f"(v[i].w) : "l"(src));
             src += step;
@@ -175,7 +193,7 @@ __device__ __forceinline__ void load_piece(const Rn3Params& p, int64_t row0, int
         return;
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int i = 0; i < Q; ++i) {
         v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         const int64_t row = r0 + 4 * i;
         if (row >= p.n || k >= p.d) continue;
@@ -191,23 +209,27 @@ __device__ __forceinline__ void load_piece(const Rn3Params& p, int64_t row0, int
     }
 }
 
-// Scale, split and store the piece: rows 64 half + l / 8 + 4 i of the stage's
-// K-major 64-byte-swizzled tiles (two base offsets a lane, as the swizzle phase
-// of a row depends on i's parity alone).
-__device__ __forceinline__ void store_piece(uint8_t* stage, int half, int lane, float4 s, const float4 (&v)[16]) {
+// Scale and split a quad: its three terms.
+__device__ __forceinline__ void split_quad(float4 s, float4 v, uint2 (&w)[3]) {
+    split3(mul2(make_float2(v.x, v.y), make_float2(s.x, s.y)), w[0].x, w[1].x, w[2].x);
+    split3(mul2(make_float2(v.z, v.w), make_float2(s.z, s.w)), w[0].y, w[1].y, w[2].y);
+}
+// Store a piece, quad i's terms by terms(i, w): rows 4 Q part + l / 8 + 4 i of the
+// stage's K-major 64-byte-swizzled tiles (two base offsets a lane, as the swizzle
+// phase of a row depends on i's parity alone).
+template <int Q, class F>
+__device__ __forceinline__ void store_piece(uint8_t* stage, int part, int lane, const F& terms) {
     const uint32_t l8 = (uint32_t)lane >> 3, c4 = (uint32_t)lane & 7u;
-    const uint32_t lane_part = (uint32_t)half * 4096u + l8 * 64u + (c4 & 1u) * 8u;
+    const uint32_t lane_part = (uint32_t)part * (4u * Q * 64u) + l8 * 64u + (c4 & 1u) * 8u;
     uint8_t* const even = stage + lane_part + ((((c4 >> 1) ^ (l8 >> 1)) & 3u) << 4);
     uint8_t* const odd = stage + lane_part + 256u + ((((c4 >> 1) ^ (2u + (l8 >> 1))) & 3u) << 4);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        uint2 hi, mid, lo;
-        split3(mul2(make_float2(v[i].x, v[i].y), make_float2(s.x, s.y)), hi.x, mid.x, lo.x);
-        split3(mul2(make_float2(v[i].z, v[i].w), make_float2(s.z, s.w)), hi.y, mid.y, lo.y);
+    for (int i = 0; i < Q; ++i) {
         uint8_t* const dst = ((i & 1) ? odd : even) + (i >> 1) * 512;
-        *reinterpret_cast<uint2*>(dst) = hi;
-        *reinterpret_cast<uint2*>(dst + kSlice) = mid;
-        *reinterpret_cast<uint2*>(dst + 2 * kSlice) = lo;
+        uint2 w[3];
+        terms(i, w);
+#pragma unroll
+        for (int z = 0; z < 3; ++z) *reinterpret_cast<uint2*>(dst + z * kSlice) = w[z];
     }
 }
 
@@ -217,7 +239,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-template <bool VEC>
+template <bool VEC, bool kEarly>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm_tc3_kernel(const Rn3Params p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -226,7 +248,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     const int cid = (int)tc::cluster_id_x(), ncl = (int)tc::nclusters_x();
     uint8_t* sB = smem + S * kStage;                       // this CTA's half of B: three slices
     uint64_t* bars = reinterpret_cast<uint64_t*>(sB + 3 * p.hb);
-    uint64_t* full = bars;                       // [S] even CTA: stage filled in both CTAs (4 arrivals)
+    uint64_t* full = bars;                       // [S] even CTA: stage filled in both CTAs (2 kParts arrivals)
     uint64_t* empty = bars + kMaxStages;         // [S] stage consumed (multicast commit)
     uint64_t* tfull = bars + 2 * kMaxStages;     // [2] accumulators done (multicast commit)
     uint64_t* tempty = tfull + 2;                // [2] even CTA: accumulators read in both (16 arrivals)
@@ -242,7 +264,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            tc::mbar_init(full + s, 4);
+            tc::mbar_init(full + s, 2 * Piece<kEarly>::kParts);
             tc::mbar_init(empty + s, 1);
             stored[s] = 0;
         }
@@ -255,6 +277,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
         *abort = 0;
         tc::fence_mbar_init();
     }
+    const uint8_t* img = p.img;
+    pdl_enter(img);
     for (int j = threadIdx.x; j < 256; j += kThreads) {
         ss[j] = p.s[j];
         ts[j] = j < p.npad ? p.t[j] : 0.f;
@@ -264,7 +288,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
         tc::tmem_relinquish_pair();
     }
     {   // this CTA's half of B
-        const uint4* src = reinterpret_cast<const uint4*>(p.img + (size_t)rank * 3 * p.hb);
+        const uint4* src = reinterpret_cast<const uint4*>(img + (size_t)rank * 3 * p.hb);
         uint4* dst = reinterpret_cast<uint4*>(sB);
         const uint32_t n16 = (3 * p.hb) >> 4;
         for (uint32_t i = threadIdx.x; i < n16; i += kThreads) dst[i] = __ldg(src + i);
@@ -388,20 +412,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
         __syncwarp();
     } else {
         // ------------------------------------------------------------ converters
-        // piece pc: half pc % 2 of chunk g = pc / 2 = (tile g / nq, K-chunk g % nq);
+        // piece pc: part pc % kParts of chunk g = pc / kParts = (tile g / nq, K-chunk g % nq);
         // the uses of each stage are claimed in piece order (stored[s])
-        const int G = my_tiles * p.nq;
-        float4 v[16];
-        for (int pc = warp - kConv0; pc < 2 * G; pc += kConvWarps) {
-            const int g = pc >> 1, half = pc & 1, t = g / p.nq, q = g - t * p.nq, u = g / S, s = g - u * S;
-            load_piece<VEC>(p, ((int64_t)cid + (int64_t)t * ncl) * (2 * kRows) + rank * kRows + half * 64, q, lane, v);
+        constexpr int kQuads = Piece<kEarly>::kQuads, kParts = Piece<kEarly>::kParts;
+        const int total = my_tiles * p.nq * kParts;
+        float4 v[kQuads];
+        const auto load = [&](int pc) {
+            const int g = pc / kParts, t = g / p.nq, q = g - t * p.nq;
+            load_piece<VEC, kQuads>(p, ((int64_t)cid + (int64_t)t * ncl) * (2 * kRows) + rank * kRows + (pc % kParts) * 4 * kQuads,
+                                    q, lane, v);
+        };
+        if (kEarly && warp - kConv0 < total) load(warp - kConv0);
+        for (int pc = warp - kConv0; pc < total; pc += kConvWarps) {
+            const int g = pc / kParts, q = g % p.nq, u = g / S, s = g - u * S;
             const float4 sc = *reinterpret_cast<const float4*>(ss + kKC * q + 4 * (lane & 7));
+            uint2 early[kEarly ? kQuads : 1][3];
+            if constexpr (kEarly) {
+#pragma unroll
+                for (int i = 0; i < kQuads; ++i) split_quad(sc, v[i], early[i]);
+                if (pc + kConvWarps < total) load(pc + kConvWarps);
+            } else {
+                load(pc);
+            }
             int ok = 1;
             if (lane == 0)
-                ok = tc::counter_wait(reinterpret_cast<volatile int*>(stored + s), 2 * u, abort) &&
+                ok = tc::counter_wait(reinterpret_cast<volatile int*>(stored + s), kParts * u, abort) &&
                      tc::mbar_wait(empty + s, ((uint32_t)u & 1u) ^ 1u, abort);
             if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-            store_piece(smem + (size_t)s * kStage, half, lane, sc, v);
+            store_piece<kQuads>(smem + (size_t)s * kStage, pc % kParts, lane, [&](int i, uint2 (&w)[3]) {
+                if constexpr (kEarly) {
+#pragma unroll
+                    for (int z = 0; z < 3; ++z) w[z] = early[i][z];
+                } else {
+                    split_quad(sc, v[i], w);
+                }
+            });
             tc::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -466,17 +511,22 @@ size_t image_bytes(const lsk_mat* A, int64_t c, int upper_tri) {
     return ws_round(6 * (size_t)p.hb);
 }
 
+using Rn3Kernel = void (*)(const Rn3Params);
+Rn3Kernel kernel_of(bool vec, int stages) {
+    if (!vec) return rownorm_tc3_kernel<false, false>;
+    return stages <= kEarlyStages ? rownorm_tc3_kernel<true, true> : rownorm_tc3_kernel<true, false>;
+}
 // clusters that fit on the device at once (cached per device, kernel and size)
-int pair_clusters(bool vec, size_t smem) {
+int pair_clusters(Rn3Kernel kernel, size_t smem) {
     static std::mutex mu;
-    static std::map<std::tuple<int, bool, size_t>, int> cache;
+    static std::map<std::tuple<int, const void*, size_t>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lock(mu);
-    const auto key = std::make_tuple(dev, vec, smem);
+    const void* fn = (const void*)kernel;
+    const auto key = std::make_tuple(dev, fn, smem);
     const auto it = cache.find(key);
     if (it != cache.end()) return it->second;
-    const void* fn = vec ? (const void*)rownorm_tc3_kernel<true> : (const void*)rownorm_tc3_kernel<false>;
     int n = 0;
     if (allow_dynamic_smem(fn) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
@@ -513,7 +563,8 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
     float* t = wc.take<float>(256);
     int* rows = wc.take<int>((size_t)np * A->n);
     int* cnt = wc.take<int>(1);
-    LSK_PROF("rownorm_tc_prep", st) rn3_units_kernel<<<8, 256, 0, st>>>((const float*)A->values, A->ld, A->n, (int)A->d, s, cnt);
+    LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_units_kernel, 8, kUnitWarps * 32, 0, 1, st, (const float*)A->values, A->ld, A->n,
+                                             (int)A->d, s, cnt);
     for (int k = 0; k < np; ++k) {
         Rn3Params p{};
         const int64_t c0 = k * per, ck = std::min<int64_t>(per, c - c0);
@@ -535,17 +586,15 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
         p.count = cnt;
         p.flag = flag;
         const size_t smem = smem_of(p);
-        const int ncl = std::min(p.ntiles, pair_clusters(vec, smem));
+        const Rn3Kernel kernel = kernel_of(vec, p.stages);
+        const int ncl = std::min(p.ntiles, pair_clusters(kernel, smem));
         if (ncl <= 0) {
             if (k == 0) return false;
             *e = cudaErrorNotSupported;
             return true;
         }
-        LSK_PROF("rownorm_tc_prep", st) rn3_image_kernel<<<p.npad / 8, 256, 0, st>>>(B, (int)c, (int)c0, p, img, t);
-        if (vec)
-            LSK_PROF("rownorm_dense_tc3", st) rownorm_tc3_kernel<true><<<2 * ncl, kThreads, smem, st>>>(p);
-        else
-            LSK_PROF("rownorm_dense_tc3", st) rownorm_tc3_kernel<false><<<2 * ncl, kThreads, smem, st>>>(p);
+        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_image_kernel, p.npad / 8, 256, 0, 1, st, B, (int)c, (int)c0, p, img, t);
+        LSK_PROF("rownorm_dense_tc3", st) launch_pdl(kernel, 2 * ncl, kThreads, smem, 1, st, p);
     }
     *list = rows;
     *count = cnt;
