@@ -78,10 +78,10 @@ typedef struct lsk_mat {
 } lsk_mat;
 
 /* precision of the contractions (Gaussian stage, row-norm GEMM) */
-#define LSK_PREC_FP32 0     /* FP32 accuracy: CUDA cores, or (the Gaussian  */
-                            /* stage of a sketch with r >= 8192) the BF16   */
-                            /* tensor pipe on three-term bf16 splits of G   */
-                            /* and SA with FP32 accumulation                */
+#define LSK_PREC_FP32 0     /* FP32 accuracy: CUDA cores, or the BF16 tensor */
+                            /* pipe on three-term bf16 splits of the        */
+                            /* operands (sketches with r >= 8192, the Gram  */
+                            /* matrix and row norms of large dense A)       */
 #define LSK_PREC_TF32 1     /* LSK_PREC_BF16 with the row-norm GEMM A B in  */
                             /* TF32: one product of A and B each rounded to */
                             /* the nearest TF32 (10 mantissa bits), FP32    */
@@ -166,13 +166,16 @@ int lsk_set_fused_sketch(int mode);
  * row-major, read when beta != 0 and overwritten.  Dense A with d <= 256
  * (d, ld multiples of 4, 16-byte aligned values) runs on the tensor cores as
  * lsk_gram_prec(LSK_PREC_BF16) (about 1e-5 relative Frobenius error: 7e-6 at
- * 4M x 256 with column scales 1e-3 .. 1e3); CSR A and other dense A run in
- * FP32 on the CUDA cores, partial sums folded into FP64 before the final
- * FP32 store (lsk_gram_prec(LSK_PREC_FP32) always takes this path). */
+ * 4M x 256 with column scales 1e-3 .. 1e3); CSR A and other dense A run to
+ * FP32 accuracy (lsk_gram_prec(LSK_PREC_FP32) always does). */
 int lsk_gram(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta,
              float* C);
-/* lsk_gram with a precision: LSK_PREC_FP32 on the CUDA cores in FP32 (as
- * lsk_gram for CSR A); LSK_PREC_BF16 (and LSK_PREC_TF32) forms the products of dense
+/* lsk_gram with a precision: LSK_PREC_FP32 to FP32 accuracy (as lsk_gram for
+ * CSR A): dense A with d <= 256 and n d >= 2^19 on the tensor cores, as eight
+ * products of three-term bf16 splits whose leading one accumulates exactly
+ * (about 2e-8 relative Frobenius error; columns outside the split's range
+ * send the call to the CUDA cores), else FP32 on the CUDA cores with partial
+ * sums folded into FP64; LSK_PREC_BF16 (and LSK_PREC_TF32) forms the products of dense
  * A with d <= 256 on the tensor
  * cores from a bfloat16 split of A (a = hi + lo; hi^T hi + hi^T lo + lo^T hi,
  * about 2^-16 relative per product), accumulating at most 1024 rows in FP32
@@ -187,7 +190,11 @@ int lsk_gram_prec(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta,
  * x: device n floats, read when beta != 0.  A*B is never stored.
  * `upper_triangular` != 0 promises B[i][j] == 0 for i > j (c == d), which
  * lets the dense kernels skip the zero blocks.  prec (dense A):
- * LSK_PREC_FP32 = CUDA-core FP32; LSK_PREC_BF16 = tensor cores with A and B
+ * LSK_PREC_FP32 = FP32 accuracy: for d, c <= 256 and n d c >= 2^30 on the
+ * tensor cores, as six products of scaled three-term bf16 splits whose
+ * leading one accumulates exactly (4.5e-8 relative; rows outside the split's
+ * range are formed on the CUDA cores), else on the CUDA cores (a wide general
+ * B with beta != 0 too); LSK_PREC_BF16 = tensor cores with A and B
  * split into bf16 hi + lo, A B ~ AhBh + AhBl + AlBh, FP32 accumulation, for
  * d, c <= 256 (other shapes run the FP32 kernel); LSK_PREC_TF32 = one TF32
  * product on the tensor cores, A streamed by the copy engine (TMA), which
@@ -340,7 +347,7 @@ int lsk_leverage_scores_hrn(lsk_ctx* ctx, const lsk_mat* A, int64_t r, int64_t k
  * of that construction (column index = row index of A); bfloat16-rounded in
  * the BF16 mode.  A: CSR only (LSK_ERR_UNSUPPORTED otherwise; a dense A is a
  * plain GEMM).  C: device m x d floats, row-major (written).  FP32 partial
- * sums over row ranges of A, summed in FP64 in a fixed order.  Malformed
+ * sums over row ranges of A, added with compensation in a fixed order.  Malformed
  * CSR sets the deferred LSK_ERR_BAD_CSR.  m in [1, 2^20], d <= 1280. */
 int lsk_csrjlt(lsk_ctx* ctx, const lsk_mat* A, int64_t m, uint64_t seed,
                int32_t prec, float* C);
@@ -400,8 +407,8 @@ int lsk_batch_leverage_scores(lsk_ctx* ctx, int32_t count, const lsk_batch_item*
 /* Stream count chosen for this batch signature (0 if none yet). */
 int lsk_batch_streams(lsk_ctx* ctx, int32_t count, const lsk_batch_item* items, int32_t prec);
 /* The schedule of this batch signature, out[4] = {worker streams, most waves
- * of grouped problems, chunks of 32 sketch columns per block of the grouped
- * Gaussian stage, least 128-row tiles per CTA of the dense row norms}.
+ * of grouped problems, chunks of 32 sketch columns, at most, per block of the
+ * grouped Gaussian stage, least 128-row tiles per CTA of the dense row norms}.
  * LSK_BATCH_AUTOTUNE picks it by coordinate descent over waves {2, 4, 8, 16},
  * streams {2, 4, 8, 16}, slice {64, 128, 256} and tiles {8, 16, 32}, each
  * candidate timed on the batch itself.  Returns 1 when a tuned schedule is

@@ -288,9 +288,10 @@ def set_fused_sketch(mode):
 
 def gram(A, alpha=1.0, beta=0.0, C=None, prec="fp32", ctx=None):
     """alpha A^T A + beta C (d x d float32, C updated in place if given).
-    prec: "fp32" (lsk_gram_prec FP32: CUDA-core FP32), "bf16" or "tf32"
-    (lsk_gram_prec BF16: tensor-core products of a bf16 split), None
-    (lsk_gram: the tensor cores for dense d <= 256, else FP32)."""
+    prec: "fp32" (lsk_gram_prec FP32: FP32 accuracy, large dense A on the
+    tensor cores), "bf16" or "tf32" (lsk_gram_prec BF16: tensor-core products
+    of a bf16 split), None (lsk_gram: as "bf16" for dense d <= 256, else
+    "fp32")."""
     m, n, d = _mat(A)
     ctx = ctx or context(_dev(A).index)
     if C is None:
@@ -305,7 +306,8 @@ def gram(A, alpha=1.0, beta=0.0, C=None, prec="fp32", ctx=None):
 
 def rownorms_prod(A, B, alpha=1.0, beta=0.0, x=None, upper_triangular=False, prec="fp32", ctx=None):
     """lsk_rownorms_prod: alpha ||A_i B||^2 + beta x_i (n float32).  prec:
-    "fp32" CUDA cores; "bf16" BF16x3 on the tensor cores; "tf32" one TF32
+    "fp32" FP32 accuracy (large dense A on the tensor cores, three-term
+    splits); "bf16" BF16x3 on the tensor cores; "tf32" one TF32
     product on the tensor cores (dense A with 32 <= d <= 256, rows 16-byte
     aligned, n >= 256; other shapes take the BF16x3 or FP32 form)."""
     m, n, d = _mat(A)

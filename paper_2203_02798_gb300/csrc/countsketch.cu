@@ -94,8 +94,7 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__global__ void __launch_bounds__(kScanBlock) scan_lookback_kernel(const uint32_t* __restrict__ in,
-                                                                   uint32_t* __restrict__ off,
+__global__ void __launch_bounds__(kScanBlock) scan_lookback_kernel(const uint32_t* in, uint32_t* off,
                                                                    uint32_t* __restrict__ cursor, int64_t len,
                                                                    unsigned long long* state, int* flag) {
     pdl_enter(in, off, cursor, state);

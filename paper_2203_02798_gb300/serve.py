@@ -156,6 +156,13 @@ def latency_summary(completions, slots=None):
     return out
 
 
+#: Workspace a slot takes when it first serves a request: the sketch of d = 512
+#: columns with r = d^2 and the permutation of 10 M rows fit in it.  Otherwise
+#: every new largest request maps memory while it waits (0.1 ms and 1 ms a GB;
+#: the slot now pays that once, with its first request).
+SLOT_WORKSPACE = 1 << 30
+
+
 class Server:
     """GPU executor: one library context and CUDA stream per slot."""
 
@@ -169,6 +176,7 @@ class Server:
         self.slots = slots
         self.streams = [torch.cuda.Stream(device=self.device) for _ in range(slots)]
         self.ctxs = [lsk.Context(device) for _ in range(slots)]
+        self.reserved = [False] * slots
 
     @staticmethod
     def footprint(n, d, nnz=None, r=None, k=None):
@@ -181,6 +189,12 @@ class Server:
         """One request on ``slot``'s stream; returns (x on the host, info)."""
         torch = self.torch
         with torch.cuda.stream(self.streams[slot]):
+            if not self.reserved[slot]:   # a slot serves one request at a time
+                self.reserved[slot] = True
+                try:
+                    self.ctxs[slot].reserve(SLOT_WORKSPACE)
+                except self.lsk.LskError:   # no room: the workspace grows with the requests
+                    pass
             x, info = self.lsk.sketch_precondition_lsq(A, b, ctx=self.ctxs[slot], **opts)
             xh = x.cpu()
         return xh.numpy(), info
