@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1) rownorm_tc_kernel(const RnParams 
         tc::tmem_alloc(tmem_slot, kTmemCols);
         tc::tmem_relinquish();
     }
+    pdl_enter(img);
     {   // resident B (hi and lo images), 16-byte copies
         const uint4* src = reinterpret_cast<const uint4*>(img);
         uint4* dst = reinterpret_cast<uint4*>(sB);
@@ -455,6 +456,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tc::tmem_alloc_pair(tmem_slot, kTmemCols);
         tc::tmem_relinquish_pair();
     }
+    pdl_enter(img);
     {   // this CTA's half of B (hi and lo images), 16-byte copies
         const uint4* src = reinterpret_cast<const uint4*>(img + (size_t)rank * 2 * p.hb_bytes);
         uint4* dst = reinterpret_cast<uint4*>(sB);
@@ -686,6 +688,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T::kThreads, 1)
         tc::tmem_relinquish_pair();
     }
     if (warp == kTmaWarp && lane == 0) tc::prefetch_tmap(&tmA);
+    pdl_read(img);
     {   // this CTA's half of B (hi and lo images), 16-byte copies
         const uint4* src = reinterpret_cast<const uint4*>(img + (size_t)rank * 2 * p.hb_bytes);
         uint4* dst = reinterpret_cast<uint4*>(sB);
@@ -937,15 +940,15 @@ const void* pair_kernel(bool vec) {
 struct TmaVariant {
     const void* fn;
     int threads, groups;
-    void (*launch)(int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img,
-                   const CUtensorMap& tmA);
+    cudaError_t (*launch)(bool early, int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img,
+                          const CUtensorMap& tmA);
 };
 template <int G, int W>
 TmaVariant tma_variant_of() {
     using T = TmaShape<G, W>;
     return {(const void*)rownorm_tma2_kernel<T>, T::kThreads, T::kGroups,
-            [](int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img, const CUtensorMap& tmA) {
-                rownorm_tma2_kernel<T><<<grid, T::kThreads, smem, st>>>(p, img, tmA);
+            [](bool early, int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img, const CUtensorMap& tmA) {
+                return launch_chained(early, rownorm_tma2_kernel<T>, grid, T::kThreads, smem, 1, st, p, img, tmA);
             }};
 }
 const TmaVariant& tma_variant() {
@@ -963,8 +966,8 @@ template <int G>
 TmaVariant tf32_variant_of() {
     using T = TmaShape<G, 1>;
     return {(const void*)rownorm_tma2_kernel<T, true>, T::kThreads, T::kGroups,
-            [](int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img, const CUtensorMap& tmA) {
-                rownorm_tma2_kernel<T, true><<<grid, T::kThreads, smem, st>>>(p, img, tmA);
+            [](bool early, int grid, size_t smem, cudaStream_t st, const RnParams& p, const uint8_t* img, const CUtensorMap& tmA) {
+                return launch_chained(early, rownorm_tma2_kernel<T, true>, grid, T::kThreads, smem, 1, st, p, img, tmA);
             }};
 }
 const TmaVariant* tf32_variant(int stages2) {
@@ -1099,7 +1102,7 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
         if (!make_tmap(p, &tmA)) return cudaErrorNotSupported;
         const int want2 = (p.ntiles2 + kMinTiles0 - 1) / kMinTiles0;
         const int grid2 = 2 * (want2 < ncl ? want2 : ncl);
-        LSK_PROF("rownorm_dense_tf32", st) tv->launch(grid2, smem_bytes2(p), st, p, img, tmA);
+        LSK_PROF("rownorm_dense_tf32", st) tv->launch(true, grid2, smem_bytes2(p), st, p, img, tmA);
         return cudaGetLastError();
     }
     const PairChoice pc = choose_form(A, p, vec);
@@ -1109,6 +1112,7 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
     if (use_tma) p.stages2 = pc.stages2;
     p.pair = ncl > 0 ? 1 : 0;
     if (!p.pair && p.stages < 2) return cudaErrorNotSupported;
+    const bool early = !img_ready;   // a batch's other streams have blocks to run meanwhile
     if (img_ready) img = const_cast<uint8_t*>(img_ready);   // built by rownorms_image_group_launch
     else LSK_PROF("rownorm_tc_prep", st) launch_pdl(rownorm_tc_prep_kernel, 64, 256, 0, 1, st, B, p, img);
     cudaError_t e;
@@ -1124,13 +1128,13 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
         if (use_tma) {
             CUtensorMap tmA;
             if (!make_tmap(p, &tmA)) return cudaErrorNotSupported;
-            LSK_PROF("rownorm_dense_tc", st) tv.launch(grid2, smem2, st, p, img, tmA);
+            LSK_PROF("rownorm_dense_tc", st) tv.launch(early, grid2, smem2, st, p, img, tmA);
         } else if (vec) {
             LSK_PROF("rownorm_dense_tc", st)
-                rownorm_tc2_kernel<true, kPieceRows><<<grid2, kThreads, smem2, st>>>(p, img);
+                launch_chained(early, rownorm_tc2_kernel<true, kPieceRows>, grid2, kThreads, smem2, 1, st, p, img);
         } else {
             LSK_PROF("rownorm_dense_tc", st)
-                rownorm_tc2_kernel<false, kPieceRows><<<grid2, kThreads, smem2, st>>>(p, img);
+                launch_chained(early, rownorm_tc2_kernel<false, kPieceRows>, grid2, kThreads, smem2, 1, st, p, img);
         }
         return cudaGetLastError();
     }
@@ -1140,11 +1144,11 @@ cudaError_t rownorms_tc_launch(const lsk_mat* A, const float* B, int64_t c, floa
     if (vec) {
         e = allow_dynamic_smem(rownorm_tc_kernel<true>);
         if (e != cudaSuccess) return e;
-        LSK_PROF("rownorm_dense_tc", st) rownorm_tc_kernel<true><<<grid, kThreads, smem, st>>>(p, img);
+        LSK_PROF("rownorm_dense_tc", st) launch_chained(early, rownorm_tc_kernel<true>, grid, kThreads, smem, 1, st, p, img);
     } else {
         e = allow_dynamic_smem(rownorm_tc_kernel<false>);
         if (e != cudaSuccess) return e;
-        LSK_PROF("rownorm_dense_tc", st) rownorm_tc_kernel<false><<<grid, kThreads, smem, st>>>(p, img);
+        LSK_PROF("rownorm_dense_tc", st) launch_chained(early, rownorm_tc_kernel<false>, grid, kThreads, smem, 1, st, p, img);
     }
     return cudaGetLastError();
 }
