@@ -223,6 +223,19 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
         }
     }
 
+    // the CSR sketches that need no permutation go first: they run while wave w's
+    // permutations are prepared (24 problems: 923 us a call, 941 with the problems in
+    // the order of their cost alone; 64: 3.81 ms, 3.94)
+    auto scatters = [&](int s, int w) -> cudaError_t {
+        for (int i : lanes[s]) {
+            const lsk_batch_item& it = items[i];
+            if (!b->grouped[i] || b->wave[i] != w || !cs_scatters(&it.A, it.r, b->cidx[i] != nullptr)) continue;
+            const cudaError_t er =
+                cs_csr_scatter_launch(&it.A, it.r, it.seed, b->SA[i], ctx->flag, ctx->sm_count, b->streams[s]);
+            if (er != cudaSuccess) return er;
+        }
+        return cudaSuccess;
+    };
     auto phase1 = [&](int s, int w) -> cudaError_t {
         cudaStream_t st = b->streams[s];
         bool prepared = false;   // this stream waits for wave w's permutations before its first gather
@@ -230,9 +243,7 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
             const lsk_batch_item& it = items[i];
             cudaError_t er = cudaSuccess;
             if (b->grouped[i]) {
-                if (b->wave[i] == w && cs_scatters(&it.A, it.r, b->cidx[i] != nullptr)) {
-                    er = cs_csr_scatter_launch(&it.A, it.r, it.seed, b->SA[i], ctx->flag, ctx->sm_count, st);
-                } else if (b->wave[i] == w) {
+                if (b->wave[i] == w && !cs_scatters(&it.A, it.r, b->cidx[i] != nullptr)) {
                     if (!prepared && (er = cudaStreamWaitEvent(st, ev_prep(w), 0)) != cudaSuccess) return er;
                     prepared = true;
                     const CsGroup& g = b->cg[w];
@@ -276,9 +287,12 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
     // stream: phase 2 of each wave once its gathers are in; phase 3 on a
     // stream pool of its own (its operands are in the arena), so no gather
     // waits behind a row norm that waits for a grouped stage
-    for (int s = 0; s < S; ++s)
-        for (int w = 0; w < std::max(W, 1); ++w)
+    for (int w = 0; w < std::max(W, 1); ++w) {
+        for (int s = 0; s < S; ++s)
+            if ((e = scatters(s, w)) != cudaSuccess) return e;
+        for (int s = 0; s < S; ++s)
             if ((e = phase1(s, w)) != cudaSuccess) return e;
+    }
     for (int w = 0; w < W; ++w)
         if ((e = phase2(w)) != cudaSuccess) return e;
     for (int s = 0; s < S; ++s) {
