@@ -322,9 +322,10 @@ bool groupable(const lsk_batch_item& it, int32_t prec) {
 // Chunks per block of one wave's Gaussian stage.  A block draws 256 x 32 entries
 // a chunk, 3.5 us, and has an SM to itself: blocks of 128 chunks left most SMs
 // without one when the wave holds a few dozen problems (24 problems, 52 blocks:
-// 457 us).  A wave is cut into kGaussBlocksPerSm blocks an SM, down to 8 chunks
-// (below, writing the k x d partials costs more than it shares out), unless
-// the schedule's longer slices give that many already: 196 us.  Of 2, 4 and 8
+// 457 us).  A wave is cut into kGaussBlocksPerSm blocks an SM, down to 24 chunks
+// (below, the k x d partials cost what the shares give: 8 problems take 942 us with
+// 8 chunks, 906 with 16 and 890 with 24; 24 take 963, 965 and 968), unless the
+// schedule's longer slices give that many already: 196 us.  Of 2, 4 and 8
 // blocks an SM the whole call takes 1071, 1078 and 1093 us with 24 problems,
 // 4.37, 4.53 and 4.83 ms with 64, 7.22, 7.25 and 7.55 ms with 160 small ones.
 constexpr int64_t kGaussBlocksPerSm = 2, kGaussMinSlice = 24;
