@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <new>
 #include <string.h>
+#include <utility>
 
 namespace cg = cooperative_groups;
 
@@ -729,7 +730,11 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
                                                            double* __restrict__ z, float* __restrict__ p) {
     using T = typename std::conditional<kStart, double, float>::type;
     const T* part = reinterpret_cast<const T*>(part_);
+    // Another CTA's shared memory may be written once that CTA is known to run:
+    // every CTA arrives here, the wait before the first such store finds them
+    // all there.
     cg::cluster_group cl = cg::this_cluster();
+    auto started = cl.barrier_arrive();
     __shared__ double qv[1024], sv[1024], pv[1024];
     __shared__ float2 v2[256];      // the vector being multiplied, as pairs (d <= 256)
     __shared__ T red[kVecThreads];
@@ -749,6 +754,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     }
     pdl_wait();
     pdl_launch_next();
+    cl.barrier_wait(std::move(started));
     // everything the pass and the previous step left is loaded at once
     const int done = kStart ? 0 : __ldcg(&st->done);
     const double rho = kStart ? 0.0 : __ldcg(&st->rho);
