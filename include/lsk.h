@@ -467,6 +467,10 @@ int lsk_debug_gauss(lsk_ctx* ctx, int64_t k, int64_t r, uint64_t seed,
  * the kernel returns; the next lsk_sync reports LSK_ERR_TIMEOUT and the
  * context stays usable.  Asynchronous on the context stream. */
 int lsk_debug_wait_timeout(lsk_ctx* ctx, int64_t limit_us);
+/* Later least-squares solves on this context run their CG step in a cluster of
+ * at most `ctas` CTAs (2, 4, 8 or 16; 0: the largest that the device can
+ * place, the default), as they would on a device that places no larger one. */
+int lsk_debug_lsq_ctas(lsk_ctx* ctx, int32_t ctas);
 
 /* ---- fixed-capacity CountSketch (no device allocation) ------------------ */
 /* The paper has no counterpart to this call: it is an interface for callers

@@ -110,6 +110,7 @@ _SIGS = {
     "lsk_debug_hash": (ctypes.c_int, [_P, _I64, _I64, _U64, _P, _P]),
     "lsk_debug_gauss": (ctypes.c_int, [_P, _I64, _I64, _U64, _I32, _P]),
     "lsk_debug_wait_timeout": (ctypes.c_int, [_P, _I64]),
+    "lsk_debug_lsq_ctas": (ctypes.c_int, [_P, _I32]),
     "lsk_batch_leverage_scores": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32, _I32]),
     "lsk_batch_streams": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32]),
     "lsk_batch_schedule": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32, _P]),
@@ -597,6 +598,11 @@ def debug_wait_timeout(limit_us, device=None, ctx=None):
     next ctx.sync() raises LskError TIMEOUT."""
     ctx = ctx or context(device)
     ctx._call("lsk_debug_wait_timeout", int(limit_us))
+
+
+def debug_lsq_ctas(ctas, ctx):
+    """lsk_debug_lsq_ctas: the most CTAs of the CG step's cluster (0: the default)."""
+    ctx._call("lsk_debug_lsq_ctas", int(ctas))
 
 
 def debug_gauss(k, r, seed, prec="fp32", device=None, ctx=None):

@@ -890,6 +890,13 @@ int lsk_debug_wait_timeout(lsk_ctx* ctx, int64_t limit_us) {
     return finish(ctx, "lsk_debug_wait_timeout");
 }
 
+int lsk_debug_lsq_ctas(lsk_ctx* ctx, int32_t ctas) {
+    if (!ctx) return LSK_ERR_INVALID_ARG;
+    if (ctas != 0 && (ctas < 2 || ctas > 16 || (ctas & (ctas - 1)))) return fail(ctx, LSK_ERR_INVALID_ARG, "ctas must be 0, 2, 4, 8 or 16");
+    ctx->lsq_ctas = ctas;
+    return LSK_OK;
+}
+
 int lsk_debug_gauss(lsk_ctx* ctx, int64_t k, int64_t r, uint64_t seed, int32_t prec, float* G) {
     if (!ctx) return LSK_ERR_INVALID_ARG;
     if (k < 1 || r < 1 || !G) return fail(ctx, LSK_ERR_INVALID_ARG, "bad k / r / G");

@@ -695,15 +695,16 @@ __global__ void __launch_bounds__(kPassThreads) cg_pass_dense_kernel(
 // z += a p_cg, s -= a w, p_cg = s + b p_cg, p = N p_cg -- is a chain of two
 // d x d products and two dot products.  One block took 84 us for it at d = 128
 // (FP64 issues at 2 lanes a cycle per SM, and its reads of N were serial),
-// twice the pass itself.  Here a cluster of 16 CTAs runs it in one launch:
+// twice the pass itself.  Here a cluster of 16 CTAs (or the largest one that the
+// device can place, cg_vec_ctas) runs it in one launch:
 // for d <= 256 every warp owns one row of N^T and one of N, as FP32 pairs
 // in registers before anything is waited for (with FP64 products each of the
 // two took 4,800 of the step's 25,000 cycles at d = 256), one more warp a CTA
 // does the scalars, and the two vectors that each step needs whole are
-// exchanged through distributed shared memory: 9 us a step.  d > 256 reads N
-// from L2 in FP64.
+// exchanged through distributed shared memory: 9 us a step.  Where d is more
+// than the warps of the cluster, N is read from L2 in FP64.
 // kStart: the residual pass's FP64 partials, eta and the start of a solve.
-constexpr int kVecCtas = 16, kVecThreads = 512, kVecWarps = kVecCtas * kVecThreads / 32;
+constexpr int kVecCtas = 16, kVecThreads = 512;   // CTAs at most (2 at least)
 constexpr int kVecBlock = kVecThreads + 32;   // one more warp for the scalars
 
 // the lane's eight entries of a row of N (or N^T) times v, summed over the warp
@@ -740,9 +741,10 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     __shared__ T red[kVecThreads];
     __shared__ double gv[kVecCtas]; // the CTAs' shares of ||u||^2
     __shared__ double sc[4];        // step length, ||s||^2, beta
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, cta = (int)cl.block_rank();
-    const bool scalar_warp = tid >= kVecThreads, small = d <= kVecWarps;
-    const int gw = scalar_warp ? d : w * kVecCtas + cta;   // rows gw, gw + 256, ... of N^T and N
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, cta = (int)cl.block_rank(), ctas = (int)gridDim.x;
+    const int warps = ctas * (kVecThreads / 32);
+    const bool scalar_warp = tid >= kVecThreads, small = N2 != nullptr;   // a row a warp
+    const int gw = scalar_warp ? d : w * ctas + cta;   // rows gw, gw + warps, ... of N^T and N
     float2 nt[8], nn[8];
     if (small && gw < d) {
 #pragma unroll
@@ -759,7 +761,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     const int done = kStart ? 0 : __ldcg(&st->done);
     const double rho = kStart ? 0.0 : __ldcg(&st->rho);
     // the partials of this CTA's columns: ng threads a column, then a tree
-    const int cpc = (d + kVecCtas - 1) / kVecCtas, j0 = cta * cpc, nc = max(0, min(cpc, d - j0));
+    const int cpc = (d + ctas - 1) / ctas, j0 = cta * cpc, nc = max(0, min(cpc, d - j0));
     int ng = 1;
     while (2 * ng * cpc <= kVecThreads) ng *= 2;
     const int col = tid % cpc, grp = tid / cpc;
@@ -787,16 +789,16 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         }
         red[tid] = acc;
     } else if (!kStart) {
-        for (int q = cta + kVecCtas * lane; q < nblocks; q += kVecCtas * 32) g += __ldcg(sspart + q);
+        for (int q = cta + ctas * lane; q < nblocks; q += ctas * 32) g += __ldcg(sspart + q);
         g = warp_sum(g);
-        if (lane < kVecCtas) cl.map_shared_rank(gv, lane)[cta] = g;
+        if (lane < ctas) cl.map_shared_rank(gv, lane)[cta] = g;
     }
     __syncthreads();
     for (int m = ng >> 1; m; m >>= 1) {
         if (grp < m) red[tid] += red[tid + m * cpc];
         __syncthreads();
     }
-    for (int e = tid; e < nc * kVecCtas; e += kVecBlock)
+    for (int e = tid; e < nc * ctas; e += kVecBlock)
         cl.map_shared_rank(qv, e / nc)[j0 + e % nc] = (double)red[e % nc];
     cl.sync();   // qv = A^T u (or A^T r) and gv in every CTA
     if (done) return;   // the same in every CTA: written only after the second cluster barrier
@@ -807,7 +809,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     double t = 0.0;
     if (scalar_warp) {
         if (!kStart) {
-            double G = lane < kVecCtas ? gv[lane] : 0.0;
+            double G = lane < ctas ? gv[lane] : 0.0;
             G = warp_sum(G);
             if (lane == 0) sc[0] = G > 0.0 ? rho / G : 0.0;
         } else if (cta == 0) {   // eta = ||A^T r|| / ||A^T b||
@@ -826,7 +828,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     __syncthreads();
     const double a = kStart ? 0.0 : sc[0];
     if (!scalar_warp)
-        for (int j = gw; j < d; j += kVecWarps) {
+        for (int j = gw; j < d; j += warps) {
             if (!small) {
                 t = 0.0;
                 for (int i = lane; i <= j; i += 32) t = fma(Nt[(int64_t)j * d + i], qv[i], t);
@@ -842,7 +844,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
                 s[j] = snew;
                 z[j] = kStart ? 0.0 : fma(a, pj, zj);
             }
-            if (lane < kVecCtas) cl.map_shared_rank(sv, lane)[j] = snew;
+            if (lane < ctas) cl.map_shared_rank(sv, lane)[j] = snew;
         }
     cl.sync();   // sv = the new s in every CTA
     if (scalar_warp) {
@@ -874,7 +876,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     }
     __syncthreads();
     if (scalar_warp) return;
-    for (int i = gw; i < d; i += kVecWarps) {   // p = N p_cg
+    for (int i = gw; i < d; i += warps) {   // p = N p_cg
         if (small) {
             t = row_dot(nn, v2, d, lane, gw >> 5, (d - 1) >> 5);
         } else {
@@ -920,13 +922,36 @@ __global__ void __launch_bounds__(256) update_x_kernel(const double* __restrict_
 }
 
 template <bool kStart>
-cudaError_t launch_vec(const void* part, const double* sspart, int nblocks, int64_t d, const double* N, const double* Nt,
+bool cg_vec_places(int ctas) {
+    // more than 8 CTAs a cluster are above the portable size: opt in (idempotent, the same value always)
+    if (cudaFuncSetAttribute(cg_vec_kernel<kStart>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+    cfg.blockDim = dim3(kVecBlock, 1, 1);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, cg_vec_kernel<kStart>, &cfg) == cudaSuccess && n > 0;
+}
+// CTAs of the step's cluster: the most that the current device can place (a
+// device or a partition of one may have no processing cluster of 16 free SMs).
+int cg_vec_ctas() {
+    int ctas = kVecCtas;
+    while (ctas > 2 && !(cg_vec_places<true>(ctas) && cg_vec_places<false>(ctas))) ctas >>= 1;
+    cudaGetLastError();
+    return ctas;
+}
+
+template <bool kStart>
+cudaError_t launch_vec(int ctas, const void* part, const double* sspart, int nblocks, int64_t d, const double* N, const double* Nt,
                        const float2* N2, const float2* Nt2, int first, double inner_tol, CgState* S, double* s, double* pc, double* z, float* p,
                        cudaStream_t st) {
-    // 16 CTAs a cluster is above the portable 8: opt in (idempotent, the same value always)
-    cudaError_t e = cudaFuncSetAttribute(cg_vec_kernel<kStart>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    LSK_PROF("lsq_small", st) e = launch_pdl(cg_vec_kernel<kStart>, kVecCtas, kVecBlock, 0, kVecCtas, st, part, sspart,
+    cudaError_t e = cudaSuccess;
+    LSK_PROF("lsq_small", st) e = launch_pdl(cg_vec_kernel<kStart>, ctas, kVecBlock, 0, ctas, st, part, sspart,
                                              nblocks, (int)d, N, Nt, N2, Nt2, first, inner_tol, S, s, pc, z, p);
     return e;
 }
@@ -1077,6 +1102,7 @@ cudaError_t atr64_launch(const lsk_mat* A, const double* b, const double* x, dou
 struct LsqHost {
     CgState* state;       // two, pinned
     cudaEvent_t ev[2];
+    int ctas;             // of the step's cluster
     cudaError_t read(int slot, const CgState* S, cudaStream_t st) {
         const cudaError_t e = cudaMemcpyAsync(state + slot, S, sizeof(CgState), cudaMemcpyDeviceToHost, st);
         return e != cudaSuccess ? e : cudaEventRecord(ev[slot], st);
@@ -1106,6 +1132,7 @@ LsqHost* lsq_host(lsk_ctx* ctx) {
         lsq_host_free(ctx);
         return nullptr;
     }
+    h->ctas = cg_vec_ctas();
     return h;
 }
 }  // namespace
@@ -1124,13 +1151,16 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
     const int64_t d = A->d;
     const bool dense = A->kind == LSK_DENSE;
     WsCarver wc{(char*)ws, 0};
+    LsqHost* host = lsq_host(ctx);
+    if (!host) return LSK_ERR_CUDA;
+    const int ctas = ctx->lsq_ctas > 0 ? std::min(ctx->lsq_ctas, host->ctas) : host->ctas;
     CgState* S = wc.take<CgState>(1);
     double* y = wc.take<double>(d);
     double* cg_s = wc.take<double>(d);
     double* cg_p = wc.take<double>(d);
     double* Nt = wc.take<double>((size_t)d * d);
     float2 *N2 = nullptr, *Nt2 = nullptr;
-    if (d <= kVecWarps) {
+    if (d <= 256 && d <= ctas * (kVecThreads / 32)) {   // a row a warp
         N2 = wc.take<float2>((size_t)d * d);
         Nt2 = reinterpret_cast<float2*>(Nt);
     }
@@ -1140,8 +1170,6 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
     float* qpart32 = reinterpret_cast<float*>(qpart64);   // reused by the FP32 pass
 
     CgState h{};
-    LsqHost* host = lsq_host(ctx);
-    if (!host) return LSK_ERR_CUDA;
     cudaError_t e = cudaMemsetAsync(x, 0, (size_t)d * 8, st);
     if (e != cudaSuccess) return LSK_ERR_CUDA;
     const dim3 tg((unsigned)((d + 31) / 32), (unsigned)((d + 31) / 32));
@@ -1171,7 +1199,7 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
         } else {
             LSK_PROF("lsq_resid64", st) tile_pass_kernel<float2><<<nb, kPassThreads, sh64, st>>>(t, nullptr, x, b, S, qpart64, sspart);
         }
-        if (launch_vec<true>(qpart64, sspart, nb, d, Rinv64, Nt, N2, Nt2, step == 0 ? 1 : 0, 0.0, S, cg_s, cg_p, y, p, st) != cudaSuccess)
+        if (launch_vec<true>(ctas, qpart64, sspart, nb, d, Rinv64, Nt, N2, Nt2, step == 0 ? 1 : 0, 0.0, S, cg_s, cg_p, y, p, st) != cudaSuccess)
             return LSK_ERR_CUDA;
         e = cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1205,7 +1233,7 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
                     LSK_PROF("lsq_pass", st) launch_pdl(tile_pass_kernel<float>, nb, kPassThreads, sh32, 1, st, t, (const float*)p,
                                                         (const double*)nullptr, (const double*)nullptr, (const CgState*)S,
                                                         (void*)qpart32, sspart);
-                if (launch_vec<false>(qpart32, sspart, nb, d, Rinv64, Nt, N2, Nt2, 0, stop_rel, S, cg_s, cg_p, y, p, st) != cudaSuccess)
+                if (launch_vec<false>(ctas, qpart32, sspart, nb, d, Rinv64, Nt, N2, Nt2, 0, stop_rel, S, cg_s, cg_p, y, p, st) != cudaSuccess)
                     return LSK_ERR_CUDA;
             }
             if ((e = host->read(batch & 1, S, st)) != cudaSuccess) return LSK_ERR_CUDA;
