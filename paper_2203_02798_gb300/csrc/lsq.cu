@@ -36,6 +36,7 @@ struct CgState {
     double atb_norm, eta;
     double rho, rho0;   // ||s||^2 now and at the start of the inner solve
     int done, it;
+    int pe;             // p holds 2^-pe N p_cg
 };
 
 constexpr int kPassThreads = 256;
@@ -703,9 +704,17 @@ __global__ void __launch_bounds__(kPassThreads) cg_pass_dense_kernel(
 // does the scalars, and the two vectors that each step needs whole are
 // exchanged through distributed shared memory: 9 us a step.  Where d is more
 // than the warps of the cluster, N is read from L2 in FP64.
+//
+// p is handed to the pass scaled by a power of two that brings ||A p|| near one,
+// taken from ||s||: the pass squares u = A p in FP32, and ||u|| follows the scale
+// of b and falls by ten orders during a solve, so that without it u^2 left FP32's
+// range for b of 1e-13 and less or 1e18 and more.  The scaling is exact and undone
+// in the step length.
 // kStart: the residual pass's FP64 partials, eta and the start of a solve.
 constexpr int kVecCtas = 16, kVecThreads = 512;   // CTAs at most (2 at least)
 constexpr int kVecBlock = kVecThreads + 32;   // one more warp for the scalars
+
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }   // |e| < 1023
 
 // the lane's eight entries of a row of N (or N^T) times v, summed over the warp
 __device__ __forceinline__ double row_dot(const float2 (&n)[8], const float2* v, int d, int lane, int c_lo, int c_hi) {
@@ -740,7 +749,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     __shared__ float2 v2[256];      // the vector being multiplied, as pairs (d <= 256)
     __shared__ T red[kVecThreads];
     __shared__ double gv[kVecCtas]; // the CTAs' shares of ||u||^2
-    __shared__ double sc[4];        // step length, ||s||^2, beta
+    __shared__ double sc[3];        // step length, beta, the scale of p
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, cta = (int)cl.block_rank(), ctas = (int)gridDim.x;
     const int warps = ctas * (kVecThreads / 32);
     const bool scalar_warp = tid >= kVecThreads, small = N2 != nullptr;   // a row a warp
@@ -760,6 +769,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
     // everything the pass and the previous step left is loaded at once
     const int done = kStart ? 0 : __ldcg(&st->done);
     const double rho = kStart ? 0.0 : __ldcg(&st->rho);
+    const int pe = kStart ? 0 : __ldcg(&st->pe);
     // the partials of this CTA's columns: ng threads a column, then a tree
     const int cpc = (d + ctas - 1) / ctas, j0 = cta * cpc, nc = max(0, min(cpc, d - j0));
     int ng = 1;
@@ -811,7 +821,8 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         if (!kStart) {
             double G = lane < ctas ? gv[lane] : 0.0;
             G = warp_sum(G);
-            if (lane == 0) sc[0] = G > 0.0 ? rho / G : 0.0;
+            const double m = pow2d(-pe);
+            if (lane == 0) sc[0] = G > 0.0 ? rho * m * m / G : 0.0;
         } else if (cta == 0) {   // eta = ||A^T r|| / ||A^T b||
             double a2 = 0.0;
             for (int j = lane; j < d; j += 32) a2 = fma(qv[j], qv[j], a2);
@@ -826,7 +837,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         t = row_dot(nt, v2, d, lane, 0, gw >> 5);   // (N^T q)_gw
     }
     __syncthreads();
-    const double a = kStart ? 0.0 : sc[0];
+    const double a = kStart ? 0.0 : sc[0], as = kStart ? 0.0 : a * pow2d(pe);   // as: for the scaled A^T u
     if (!scalar_warp)
         for (int j = gw; j < d; j += warps) {
             if (!small) {
@@ -839,7 +850,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
                     pj = pv[j];
                 }
             }
-            const double snew = kStart ? t : fma(-a, t, sj);
+            const double snew = kStart ? t : fma(-as, t, sj);
             if (lane == 0) {
                 s[j] = snew;
                 z[j] = kStart ? 0.0 : fma(a, pj, zj);
@@ -852,9 +863,13 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         for (int j = lane; j < d; j += 32) r2 = fma(sv[j], sv[j], r2);
         r2 = warp_sum(r2);
         if (lane == 0) {
-            sc[2] = (!kStart && rho > 0.0) ? r2 / rho : 0.0;
+            sc[1] = (!kStart && rho > 0.0) ? r2 / rho : 0.0;
+            // 2^e: ||s|| rounded down to a power of two, e half the exponent of ||s||^2
+            const int e = ((__double2hiint(r2) >> 20) - 1023) >> 1;   // [-512, 512]
+            sc[2] = pow2d(-e);
             if (cta == 0) {
                 st->rho = r2;
+                st->pe = e;
                 if (kStart) {
                     st->rho0 = r2;
                     st->it = 0;
@@ -867,11 +882,11 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         }
     }
     __syncthreads();
-    const double bta = sc[2];
+    const double bta = sc[1], ps = sc[2];
     for (int j = tid; j < d; j += kVecBlock) {
         const double v = kStart ? sv[j] : fma(bta, pv[j], sv[j]);
         pv[j] = v;
-        if (small) v2[j] = to_pair(v);
+        if (small) v2[j] = to_pair(v * ps);
         if (cta == 0) pc[j] = v;
     }
     __syncthreads();
@@ -882,7 +897,7 @@ __global__ void __launch_bounds__(kVecBlock, 1) cg_vec_kernel(const void* __rest
         } else {
             t = 0.0;
             for (int j = i + lane; j < d; j += 32) t = fma(N[(int64_t)i * d + j], pv[j], t);
-            t = warp_sum(t);
+            t = warp_sum(t) * ps;
         }
         if (lane == 0) p[i] = (float)t;
     }
