@@ -72,6 +72,17 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2)
     h = s;
 }
 
+// (double)a by integer instructions: the conversion instruction issues on the FP64
+// pipe, which the residual passes keep full with their products.
+__device__ __forceinline__ double to_double(float a) {
+    const uint32_t mag = __float_as_uint(a) & 0x7fffffffu;
+    const bool small = mag < 0x00800000u;                                  // zero or subnormal: scaled up first
+    const uint32_t bits = __float_as_uint(small ? a * 16777216.f : a);     // 2^24
+    const uint32_t bias = mag >= 0x7f800000u ? 0x70000000u : small ? (896u - 24u) << 20 : 896u << 20;
+    const uint32_t hi = (((uint32_t)((int32_t)bits >> 3)) & 0x8fffffffu) + (mag ? bias : 0u);
+    return __hiloint2double((int)hi, (int)(bits << 29));
+}
+
 // Sum each of RB per-lane values over groups of L lanes: at every step a lane
 // keeps half of its values and hands over the other half, so the RB sums cost
 // about RB + 3 exchanges instead of 5 RB.  On return the sum of value r is in
@@ -91,42 +102,23 @@ __device__ __forceinline__ int sum_index(int lane) {
     for (int b = 0; (1 << b) < RB; ++b) r |= (lane & (L >> (b + 1))) ? 1 << b : 0;
     return r;
 }
-template <int RB, int L>
-__device__ __forceinline__ float warp_sum_rows(float (&v)[RB], int lane) {
+template <int RB, int L, class T>
+__device__ __forceinline__ T warp_sum_rows(T (&v)[RB], int lane) {
     int o = L / 2;
 #pragma unroll
     for (int m = RB; m > 1; m >>= 1, o >>= 1) {
         const bool up = lane & o;
 #pragma unroll
         for (int r = 0; r < m / 2; ++r) {   // even values stay in the lower lanes
-            const float keep = up ? v[2 * r + 1] : v[2 * r];
-            const float give = up ? v[2 * r] : v[2 * r + 1];
+            const T keep = up ? v[2 * r + 1] : v[2 * r];
+            const T give = up ? v[2 * r] : v[2 * r + 1];
             v[r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
     }
-    float t = v[0];
+    T t = v[0];
     for (; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     return t;
 }
-template <int RB, int L>
-__device__ __forceinline__ float2 warp_sum_rows(float (&h)[RB], float (&l)[RB], int lane) {
-    int o = L / 2;
-#pragma unroll
-    for (int m = RB; m > 1; m >>= 1, o >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int r = 0; r < m / 2; ++r) {
-            float kh = up ? h[2 * r + 1] : h[2 * r], kl = up ? l[2 * r + 1] : l[2 * r];
-            const float gh = up ? h[2 * r] : h[2 * r + 1], gl = up ? l[2 * r] : l[2 * r + 1];
-            pair_add(kh, kl, __shfl_xor_sync(0xffffffffu, gh, o), __shfl_xor_sync(0xffffffffu, gl, o));
-            h[r] = kh;
-            l[r] = kl;
-        }
-    }
-    for (; o; o >>= 1) pair_add(h[0], l[0], __shfl_xor_sync(0xffffffffu, h[0], o), __shfl_xor_sync(0xffffffffu, l[0], o));
-    return make_float2(h[0], l[0]);
-}
-
 // ---- dense passes, d <= 256 --------------------------------------------------
 // A warp takes RB x (32 / L) rows at a time: L lanes own a row, each E entries
 // of it -- kVec: E / 4 runs of four columns (16-byte loads; d, lda multiples
@@ -173,10 +165,11 @@ struct DenseRows {
     }
 };
 
-// r = b - A x and partial sums of A^T r in one read of A.  The dots and the
-// sums over rows are FP32 pairs, r itself FP64; FP64 arithmetic throughout (two
-// FMAs, two conversions an entry at 1/64 rate) took 471 us at 316,227 x 128,
-// where reading A takes 24; this takes 57.
+// r = b - A x and partial sums of A^T r in one read of A, in FP64 (x == nullptr:
+// r = b).  Two FMAs an entry at 2 lanes a cycle and SM bound it: 140 us for
+// 316,227 x 128, and half of that for the first pass, whose x is zero; the three
+// passes of a solve take 390.  With a conversion instruction an entry on the same
+// pipe a pass took 471; FP32 pairs took 57 but hold 48 bits, and FP32's range.
 template <int L, int E, int RB, bool kVec>
 __global__ void __launch_bounds__(kPassThreads, 2) resid_dense_rows_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int d, const double* __restrict__ b,
@@ -184,14 +177,12 @@ __global__ void __launch_bounds__(kPassThreads, 2) resid_dense_rows_kernel(
     using Rows = DenseRows<L, E, RB, kVec>;
     __shared__ double qs[(kPassThreads / 32) * Rows::kRpl][L * E];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane / L, li = lane % L;
-    float xh[E], xl[E], qh[E], ql[E];
+    double xr[E], q[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int j = Rows::col(li, e);
-        const float2 v = to_pair(j < d ? x[j] : 0.0);
-        xh[e] = v.x;
-        xl[e] = v.y;
-        qh[e] = ql[e] = 0.f;
+        xr[e] = x && j < d ? x[j] : 0.0;
+        q[e] = 0.0;
     }
     const int mine = sum_index<RB, L>(lane) * Rows::kRpl + sub;   // the row whose sum this lane receives
     const int64_t step = (int64_t)gridDim.x * (kPassThreads / 32) * Rows::kRows;
@@ -203,32 +194,31 @@ __global__ void __launch_bounds__(kPassThreads, 2) resid_dense_rows_kernel(
         if (i0 + mine < n) bn = b[i0 + mine];
     }
     for (; i0 < n; i0 += step) {
-        const double bi = bn;
+        double ri = bn;   // rows past n: zero
         if (i0 + step < n) {
             nxt.load(A, lda, n, d, i0 + step, lane);
             bn = i0 + step + mine < n ? b[i0 + step + mine] : 0.0;
         }
-        float h[RB], l[RB];
+        if (x) {
+            double dot[RB];
 #pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            h[r] = l[r] = 0.f;
+            for (int r = 0; r < RB; ++r) {
+                dot[r] = 0.0;
 #pragma unroll
-            for (int e = 0; e < E; ++e) pair_fma(h[r], l[r], cur.a[r][e], xh[e], xl[e]);
+                for (int e = 0; e < E; ++e) dot[r] = fma(to_double(cur.a[r][e]), xr[e], dot[r]);
+            }
+            ri -= warp_sum_rows<RB, L>(dot, lane);
         }
-        const float2 dot = warp_sum_rows<RB, L>(h, l, lane);
-        const float2 ri = to_pair(i0 + mine < n ? (bi - (double)dot.x) - (double)dot.y : 0.0);
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
-            const int src = sub * L + sum_lane<RB, L>(r);
-            const float rh = __shfl_sync(0xffffffffu, ri.x, src);
-            const float rl = __shfl_sync(0xffffffffu, ri.y, src);
+            const double rr = __shfl_sync(0xffffffffu, ri, sub * L + sum_lane<RB, L>(r));
 #pragma unroll
-            for (int e = 0; e < E; ++e) pair_fma(qh[e], ql[e], cur.a[r][e], rh, rl);
+            for (int e = 0; e < E; ++e) q[e] = fma(to_double(cur.a[r][e]), rr, q[e]);
         }
         cur.take(nxt);
     }
 #pragma unroll
-    for (int e = 0; e < E; ++e) qs[w * Rows::kRpl + sub][Rows::col(li, e)] = (double)qh[e] + (double)ql[e];
+    for (int e = 0; e < E; ++e) qs[w * Rows::kRpl + sub][Rows::col(li, e)] = q[e];
     __syncthreads();
     for (int j = threadIdx.x; j < d; j += blockDim.x) {
         double t = 0.0;
@@ -387,20 +377,9 @@ __global__ void __launch_bounds__(kPassThreads) csr_tiles_kernel(CsrTiles t, int
 // out[s] += sum over the entries e of segment s of val[e] vec[idx[e]], for the
 // segments [ptr[s], ptr[s + 1]) of a run of entries.  The run starts at a
 // multiple of four (`shift` entries before the first segment); 2^lg lanes a
-// segment.  Values are float, or pairs (float2) for the residual pass.
+// segment.  Sums are float, or double in the residual pass.
 __device__ __forceinline__ float seg_mul(float v, float x) { return v * x; }
-__device__ __forceinline__ float2 seg_mul(float v, float2 x) {
-    const float p = v * x.x;
-    return make_float2(p, fmaf(v, x.y, fmaf(v, x.x, -p)));
-}
-__device__ __forceinline__ void seg_add(float& s, float v) { s += v; }
-__device__ __forceinline__ void seg_add(float2& s, float2 v) { pair_add(s.x, s.y, v.x, v.y); }
-__device__ __forceinline__ float seg_shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ float2 seg_shfl(float2 v, int o) {
-    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
-}
-__device__ __forceinline__ float seg_zero(float) { return 0.f; }
-__device__ __forceinline__ float2 seg_zero(float2) { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ double seg_mul(float v, double x) { return to_double(v) * x; }
 
 __device__ __forceinline__ int4 idx_quad(const int32_t* p) { return __ldg(reinterpret_cast<const int4*>(p)); }
 __device__ __forceinline__ int4 idx_quad(const uint16_t* p) {
@@ -448,8 +427,8 @@ __device__ __forceinline__ void mul_quads(const EntryQuads& r, const T* vec, int
         if constexpr (sizeof(T) == sizeof(float)) {
             *reinterpret_cast<float4*>(prod + e) = make_float4(a, b, c, f);
         } else {
-            *reinterpret_cast<float4*>(prod + e) = make_float4(a.x, a.y, b.x, b.y);
-            *reinterpret_cast<float4*>(prod + e + 2) = make_float4(c.x, c.y, f.x, f.y);
+            *reinterpret_cast<double2*>(prod + e) = make_double2(a, b);
+            *reinterpret_cast<double2*>(prod + e + 2) = make_double2(c, f);
         }
     }
 }
@@ -460,15 +439,15 @@ __device__ __forceinline__ void sum_segments(const T* prod, int c0, int m, int s
     const int G = 1 << lg, sub = threadIdx.x & (G - 1);
     for (int s0 = 0; s0 < nseg; s0 += kPassThreads >> lg) {
         const int s = s0 + (threadIdx.x >> lg);
-        T t = seg_zero(T{});
+        T t = 0;
         int k0 = 0, k1 = 0;
         if (s < nseg) {
             k0 = max(ptr[s] + shift, c0);
             k1 = min(ptr[s + 1] + shift, c0 + m);
-            for (int k = k0 + sub; k < k1; k += G) seg_add(t, prod[k - c0]);
+            for (int k = k0 + sub; k < k1; k += G) t += prod[k - c0];
         }
-        for (int o = G >> 1; o; o >>= 1) seg_add(t, seg_shfl(t, o));
-        if (k1 > k0 && sub == 0) seg_add(out[s], t);
+        for (int o = G >> 1; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (k1 > k0 && sub == 0) out[s] += t;
     }
 }
 
@@ -479,14 +458,14 @@ __device__ __forceinline__ int seg_lanes(int nseg) {   // log2 of the lanes a se
 }
 
 // T = float: u = A p and partial sums of A^T u, ||u||^2.
-// T = float2: r = b - A x and partial sums of A^T r (FP64 partials).
+// T = double: r = b - A x and partial sums of A^T r.
 template <class T>
 __global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(CsrTiles t, const float* __restrict__ p,
                                                                  const double* __restrict__ x,
                                                                  const double* __restrict__ b,
                                                                  const CgState* __restrict__ st,
                                                                  void* __restrict__ qpart, double* __restrict__ sspart) {
-    constexpr bool kResid = sizeof(T) == sizeof(float2);
+    constexpr bool kResid = sizeof(T) == sizeof(double);
     extern __shared__ __align__(16) unsigned char tile_sh[];
     __shared__ double ssw[kPassThreads / 32];
     const int d = (int)t.d;
@@ -511,9 +490,9 @@ __global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(Cs
     pdl_launch_next();
     if (!kResid && __ldcg(&st->done)) return;
     for (int j = threadIdx.x; j < d; j += kPassThreads) {
-        if constexpr (kResid) vec[j] = to_pair(x[j]);
+        if constexpr (kResid) vec[j] = x[j];
         else vec[j] = __ldcg(p + j);
-        q[j] = seg_zero(T{});
+        q[j] = 0;
     }
     float sh = 0.f, sl = 0.f;
     for (int64_t tile = blockIdx.x; tile < t.ntiles; tile += gridDim.x) {
@@ -529,7 +508,7 @@ __global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(Cs
         __syncthreads();   // the last tile's readers of rptr, cptr, u
         for (int i = threadIdx.x; i <= rows; i += kPassThreads) {
             rptr[i] = (int32_t)(t.I[r0 + i] - base);
-            if (i < rows) u[i] = seg_zero(T{});
+            if (i < rows) u[i] = 0;
         }
         for (int j = threadIdx.x; j <= d; j += kPassThreads) cptr[j] = t.cptr[tile * (d + 1) + j];
         __syncthreads();
@@ -544,7 +523,7 @@ __global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(Cs
             __syncthreads();
         }
         for (int i = threadIdx.x; i < rows; i += kPassThreads) {
-            if constexpr (kResid) u[i] = to_pair((b[r0 + i] - (double)u[i].x) - (double)u[i].y);
+            if constexpr (kResid) u[i] = b[r0 + i] - u[i];
             else pair_fma(sh, sl, u[i], u[i], 0.f);
         }
         __syncthreads();
@@ -559,8 +538,7 @@ __global__ void __launch_bounds__(kPassThreads, kTilesPerSm) tile_pass_kernel(Cs
     }
     __syncthreads();
     for (int j = threadIdx.x; j < d; j += kPassThreads) {
-        if constexpr (kResid) reinterpret_cast<double*>(qpart)[(int64_t)blockIdx.x * d + j] = (double)q[j].x + (double)q[j].y;
-        else reinterpret_cast<float*>(qpart)[(int64_t)blockIdx.x * d + j] = q[j];
+        reinterpret_cast<T*>(qpart)[(int64_t)blockIdx.x * d + j] = q[j];
     }
     if constexpr (!kResid) {
         const double ss = warp_sum((double)sh + (double)sl);
@@ -710,7 +688,8 @@ __global__ void __launch_bounds__(kPassThreads) cg_pass_dense_kernel(
 // of b and falls by ten orders during a solve, so that without it u^2 left FP32's
 // range for b of 1e-13 and less or 1e18 and more.  The scaling is exact and undone
 // in the step length.
-// kStart: the residual pass's FP64 partials, eta and the start of a solve.
+// kStart: the residual pass's FP64 partials, eta and the start of a solve, three
+// or four times in all, with N in FP64.
 constexpr int kVecCtas = 16, kVecThreads = 512;   // CTAs at most (2 at least)
 constexpr int kVecBlock = kVecThreads + 32;   // one more warp for the scalars
 
@@ -919,8 +898,8 @@ __global__ void __launch_bounds__(256) factor_forms_kernel(const double* __restr
     for (int k = y; k < 32; k += 8)
         if (j0 + k < d && i0 + x < d) {
             const double v = tile[x][k];
+            Nt[(int64_t)(j0 + k) * d + i0 + x] = v;
             if (Nt2) Nt2[(j0 + k) * d + i0 + x] = to_pair(v);
-            else Nt[(int64_t)(j0 + k) * d + i0 + x] = v;
         }
 }
 
@@ -1024,6 +1003,7 @@ void launch_resid(const lsk_mat* A, int nb, const double* b, const double* x, do
 }
 
 // dense b - A x and the blocks' partial sums of A^T (b - A x)
+// (x == nullptr: x = 0, d <= 256 only)
 cudaError_t resid_dense(const lsk_mat* A, int nb, const double* b, const double* x, double* qpart, cudaStream_t st) {
     const int64_t d = A->d;
     if (d > 256) {
@@ -1036,8 +1016,8 @@ cudaError_t resid_dense(const lsk_mat* A, int nb, const double* b, const double*
                                                                                        A->n, d, b, x, qpart);
     } else if (rows_vec4(A)) {
         if (d <= 32) launch_resid<8, 4, 4, true>(A, nb, b, x, qpart, st);
-        else if (d <= 64) launch_resid<16, 4, 4, true>(A, nb, b, x, qpart, st);
-        else if (d <= 128) launch_resid<32, 4, 8, true>(A, nb, b, x, qpart, st);
+        else if (d <= 64) launch_resid<8, 8, 4, true>(A, nb, b, x, qpart, st);
+        else if (d <= 128) launch_resid<16, 8, 4, true>(A, nb, b, x, qpart, st);
         else launch_resid<32, 8, 4, true>(A, nb, b, x, qpart, st);
     } else {
         if (d <= 32) launch_resid<32, 1, 8, false>(A, nb, b, x, qpart, st);
@@ -1097,7 +1077,7 @@ cudaError_t atr64_launch(const lsk_mat* A, const double* b, const double* x, dou
     double* qpart = wc.take<double>((size_t)nb * d);
     double* zero = wc.take<double>(d);
     cudaError_t e = cudaSuccess;
-    if (!x) {
+    if (!x && !(A->kind == LSK_DENSE && d <= 256)) {
         if ((e = cudaMemsetAsync(zero, 0, (size_t)d * 8, st)) != cudaSuccess) return e;
         x = zero;
     }
@@ -1155,7 +1135,7 @@ LsqHost* lsq_host(lsk_ctx* ctx) {
 size_t lsq_workspace_bytes(const lsk_mat* A, int sm_count) {
     const int64_t d = A->d;
     const int nb = kMaxPassBlocks;
-    return ws_round(sizeof(CgState)) + 4 * ws_round((size_t)d * 8) + 2 * ws_round((size_t)d * d * 8) +
+    return ws_round(sizeof(CgState)) + 4 * ws_round((size_t)d * 8) + 3 * ws_round((size_t)d * d * 8) +
            ws_round((size_t)nb * d * 8) + ws_round((size_t)nb * 8) + ws_round((size_t)d * 4) +
            (A->kind == LSK_CSR ? tiles_bytes(A, sm_count) : 0) + 4096;
 }
@@ -1173,11 +1153,11 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
     double* y = wc.take<double>(d);
     double* cg_s = wc.take<double>(d);
     double* cg_p = wc.take<double>(d);
-    double* Nt = wc.take<double>((size_t)d * d);
+    double* Nt = wc.take<double>((size_t)d * d);   // N^T
     float2 *N2 = nullptr, *Nt2 = nullptr;
     if (d <= 256 && d <= ctas * (kVecThreads / 32)) {   // a row a warp
         N2 = wc.take<float2>((size_t)d * d);
-        Nt2 = reinterpret_cast<float2*>(Nt);
+        Nt2 = wc.take<float2>((size_t)d * d);
     }
     double* qpart64 = wc.take<double>((size_t)kMaxPassBlocks * d);
     double* sspart = wc.take<double>(kMaxPassBlocks);
@@ -1198,9 +1178,9 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
         t.tval = wc.take<float>((size_t)A->nnz);
         t.trow = wc.take<uint16_t>((size_t)A->nnz);
         sh32 = tiles_smem(t, sizeof(float));
-        sh64 = tiles_smem(t, sizeof(float2));
+        sh64 = tiles_smem(t, sizeof(double));
         if (allow_dynamic_smem(tile_pass_kernel<float>) != cudaSuccess ||
-            allow_dynamic_smem(tile_pass_kernel<float2>) != cudaSuccess)
+            allow_dynamic_smem(tile_pass_kernel<double>) != cudaSuccess)
             return LSK_ERR_CUDA;
         nb = (int)std::max<int64_t>(1, std::min<int64_t>(t.ntiles, kTilesPerSm * (int64_t)ctx->sm_count));
         if (t.ntiles > 0)
@@ -1210,11 +1190,11 @@ int lsq_run(lsk_ctx* ctx, const lsk_mat* A, const double* b, double* x, const ls
     double eta = INFINITY;
     for (int step = 0; step <= o->max_refine; ++step) {
         if (dense) {
-            if (resid_dense(A, nb, b, x, qpart64, st) != cudaSuccess) return LSK_ERR_CUDA;
+            if (resid_dense(A, nb, b, step == 0 && d <= 256 ? nullptr : x, qpart64, st) != cudaSuccess) return LSK_ERR_CUDA;
         } else {
-            LSK_PROF("lsq_resid64", st) tile_pass_kernel<float2><<<nb, kPassThreads, sh64, st>>>(t, nullptr, x, b, S, qpart64, sspart);
+            LSK_PROF("lsq_resid64", st) tile_pass_kernel<double><<<nb, kPassThreads, sh64, st>>>(t, nullptr, x, b, S, qpart64, sspart);
         }
-        if (launch_vec<true>(ctas, qpart64, sspart, nb, d, Rinv64, Nt, N2, Nt2, step == 0 ? 1 : 0, 0.0, S, cg_s, cg_p, y, p, st) != cudaSuccess)
+        if (launch_vec<true>(ctas, qpart64, sspart, nb, d, Rinv64, Nt, nullptr, nullptr, step == 0 ? 1 : 0, 0.0, S, cg_s, cg_p, y, p, st) != cudaSuccess)
             return LSK_ERR_CUDA;
         e = cudaMemcpyAsync(&h, S, sizeof(h), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);

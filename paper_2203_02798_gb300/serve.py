@@ -183,7 +183,7 @@ class Server:
         """Device bytes one solve holds beyond its inputs: sketch, factors, vectors."""
         r = r if r is not None else max(d * d, 4 * d)
         k = k if k is not None else 2 * d
-        return int(4 * r * d + 4 * k * d + 56 * d * d + 20 * n + 8 * (nnz or 0) + (6 << 20))
+        return int(4 * r * d + 4 * k * d + 64 * d * d + 20 * n + 8 * (nnz or 0) + (6 << 20))
 
     def solve(self, slot, A, b, **opts):
         """One request on ``slot``'s stream; returns (x on the host, info)."""
