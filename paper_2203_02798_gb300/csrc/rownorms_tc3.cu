@@ -14,9 +14,12 @@
 // epilogue.  (Ozaki, Ogita, Oishi & Rump, Numer. Algorithms 59, 2012, with the
 // first slice on a fixed grid.)
 //
-// That holds for rows within a factor of about 30 of the typical row: a row whose
-// acc1 is not small against acc0, whose acc0 reaches 2^24 or whose sum is not
-// finite is put on a list, and the CUDA-core kernel does the listed rows.
+// That holds for rows within a factor of about 30 of the typical row.  A row is put
+// on a list, and the CUDA-core kernel does the listed rows, where acc1 t_l is more
+// than 2^-5 of the whole in the norm (every column counts, by its share of the
+// result: at 2^-5 the terms left out are as large as FP32's roundings), where an
+// accumulator reaches 2^24, and where the sum is not finite or so small that the
+// squares of acc1 t_l could underflow.
 //
 // One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
 // half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
@@ -311,7 +314,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
             if (!warp_wait(tfull + b, par, abort)) break;
             tc::fence_after_sync();
             const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + 256u * (uint32_t)b;
-            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s0 = 0.f, s1 = 0.f, mx = 0.f;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s1[2] = {0.f, 0.f}, mx = 0.f;
             for (int col = 32 * half; col < p.npad; col += 64) {
                 uint32_t v0[32], v1[32];
                 tc::tmem_ld_32x32b_x32(taddr + (uint32_t)col, v0);
@@ -319,14 +322,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
                 tc::tmem_ld_wait();
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
-                    const float a0 = __uint_as_float(v0[e]), a1 = __uint_as_float(v1[e]);
-                    const float y = (a0 + a1) * ts[col + e];
+                    const float a1 = __uint_as_float(v1[e]), a = __uint_as_float(v0[e]) + a1, t = ts[col + e];
+                    const float y = a * t, y1 = a1 * t;
                     sum[e & 3] = fmaf(y, y, sum[e & 3]);
-                    mx = fmaxf(mx, fabsf(a0));
-                    if (e & 1) {
-                        s0 = fmaf(a0, a0, s0);
-                        s1 = fmaf(a1, a1, s1);
-                    }
+                    s1[e & 1] = fmaf(y1, y1, s1[e & 1]);
+                    mx = fmaxf(mx, fabsf(a));
                 }
             }
             tc::fence_before_sync();
@@ -336,8 +336,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
                 else tc::mbar_arrive_cluster(tempty + b, 0);
             }
             float tot = (sum[0] + sum[1]) + (sum[2] + sum[3]);
-            // outside the split's range: NaN, which no sum within it is
-            if (!(s1 <= 9.765625e-4f * s0 && mx < 16777216.f)) tot = __uint_as_float(0x7FC00000u);
+            // outside the split's range: NaN, which no sum within it is (2^-10; 2^-110, or all zero)
+            if (!(s1[0] + s1[1] <= 9.765625e-4f * tot && mx < 16777216.f && (tot >= 7.703719778e-34f || mx == 0.f)))
+                tot = __uint_as_float(0x7FC00000u);
             // The second half's sum goes to the first through shared memory.
             // Four cells a row: the second half is at most two tiles ahead (the
             // MMAs of a tile wait for both halves of the one two before).

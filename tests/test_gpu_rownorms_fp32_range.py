@@ -1,0 +1,53 @@
+"""FP32 row norms of large dense A: rows outside the range of the tensor-core form
+go to the CUDA cores, whatever columns of B their result comes from.  Compared
+with the CUDA-core form on the same rows (a call on few rows takes it)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+KINDS = ["general", "odd_zero", "even_zero", "one", "two", "dominant"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_rows_outside_the_range(kind):
+    import paper_2203_02798_gb300 as lsk
+    d, c = 256, {"one": 1, "two": 2}.get(kind, 256)
+    n = (1 << 30) // (d * c) + 37          # the smallest that takes the tensor-core form
+    g = torch.Generator(device="cuda").manual_seed(7)
+    k = torch.arange(n, device="cuda") % 21
+    A = torch.randn((n, d), generator=g, device="cuda")
+    # one row in 21 each is scaled by 2^0 .. 2^-20 in the first 8,400 rows; the others stand for the typical row
+    A[:8400] *= torch.pow(2.0, -k[:8400].float()).view(-1, 1)
+    B = torch.randn((d, c), generator=g, device="cuda")
+    if kind == "odd_zero":
+        B[:, 1::2] = 0.0
+    if kind == "even_zero":
+        B[:, 0::2] = 0.0
+    if kind == "dominant":                 # one column makes the norm, its largest entry meets only zeros
+        B[:, 6] *= 1e3
+        B[0, 6] = 1e6
+        A[:, 0] = 0.0
+    x = lsk.rownorms_prod(A, B, prec="fp32")[:8400].double()
+    few = lsk.rownorms_prod(A[:2100].contiguous(), B, prec="fp32")
+    few = torch.cat([few] + [lsk.rownorms_prod(A[i:i + 2100].contiguous(), B, prec="fp32") for i in (2100, 4200, 6300)]).double()
+    want = (A[:8400].double() @ B.double()).square().sum(1)
+    rms = lambda v, i: ((v / want - 1.0)[k[:8400] == i]).square().mean().sqrt().item()
+    for i in range(21):
+        # no more than twice the CUDA-core form's error (a result's rounding, 2^-24, at least)
+        assert rms(x, i) <= 2.0 * max(rms(few, i), 2.0 ** -24), (i, rms(x, i), rms(few, i))
+
+
+def test_zero_and_tiny_rows():
+    import paper_2203_02798_gb300 as lsk
+    d = c = 256
+    n = (1 << 30) // (d * c) + 5
+    g = torch.Generator(device="cuda").manual_seed(8)
+    A = torch.randn((n, d), generator=g, device="cuda")
+    A[::3] = 0.0
+    A[1::9] *= 1e-18                       # squares near and below FP32's bottom
+    B = torch.randn((d, c), generator=g, device="cuda") / 16.0
+    x = lsk.rownorms_prod(A, B, prec="fp32")
+    few = torch.cat([lsk.rownorms_prod(A[i:i + 4000].contiguous(), B, prec="fp32") for i in range(0, n, 4000)])
+    assert torch.equal(x[::3], torch.zeros_like(x[::3]))
+    assert torch.allclose(x, few, rtol=2e-6, atol=0.0)
