@@ -15,11 +15,14 @@
 // first slice on a fixed grid.)
 //
 // That holds for rows within a factor of about 30 of the typical row.  A row is put
-// on a list, and the CUDA-core kernel does the listed rows, where acc1 t_l is more
-// than 2^-5 of the whole in the norm (every column counts, by its share of the
-// result: at 2^-5 the terms left out are as large as FP32's roundings), where an
-// accumulator reaches 2^24, and where the sum is not finite or so small that the
-// squares of acc1 t_l could underflow.
+// on a list, and the CUDA-core kernel does the listed rows, where the second
+// accumulator may hold more than 2^-5 of the norm (there the terms left out are as
+// large as FP32's roundings), where an accumulator reaches 2^24, and where the sum
+// is not finite or near FP32's bottom.  What acc1 holds is not taken from acc1, which
+// may cancel where few columns make the norm, but from what the remainders after
+// hi add to it on average: those of A's entries, 1/12 each, squared, times B, and
+// those of B's columns times the row's entries, of the size that the sum of its
+// unscaled y_l^2 says; every column counts by its share t_l of the result.
 //
 // One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
 // half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
@@ -58,7 +61,7 @@ struct Piece {
 constexpr int kEarlyStages = 4;
 constexpr int kMaxStages = 8, kMinStages = 3;
 constexpr size_t kSmemLimit = 232448;
-constexpr uint32_t kTail = 1024;                      // barriers
+constexpr uint32_t kTail = 1024;                      // barriers, and four floats at its end
 constexpr uint32_t kXchg = 4 * kRows * 4;             // the epilogue halves' exchange
 constexpr size_t kExtra = 1024 + kTail + 2 * 256 * 4 + kXchg;
 constexpr int kSampleGroups = 64, kSampleRows = 8;
@@ -73,6 +76,7 @@ struct Rn3Params {
     uint32_t hb;              // bytes of one slice of a CTA's half of B
     const uint8_t* img;       // [half][slice][hb]
     const float *s, *t;       // column scales of A, result scales of B's columns
+    const float *norm, *rest; // of B's scaled columns: sum of squares, and of the remainders after hi
     int *list, *count;        // rows left to the CUDA-core kernel
     int* flag;
 };
@@ -149,10 +153,11 @@ __device__ __forceinline__ void split3(float2 y, uint32_t& hi, uint32_t& mid, ui
 // The image of B: 8 columns a block.  Column l (0-based in this pass, column
 // c0 + l of B) is scaled so that its largest |b_jl| / s_j is in [128, 256).
 __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict__ B, int ldb, int c0, const Rn3Params p,
-                                                        uint8_t* __restrict__ img, float* __restrict__ t) {
+                                                        uint8_t* __restrict__ img, float* __restrict__ t,
+                                                        float* __restrict__ norm, float* __restrict__ rest) {
     const float* s = p.s;
-    pdl_enter(B, s, img, t);
-    __shared__ float red[32][9];
+    pdl_enter(B, s, img, t, norm, rest);
+    __shared__ float red[32][9], red1[32][9];
     const int col = threadIdx.x & 7, part = threadIdx.x >> 3, l = (int)blockIdx.x * 8 + col;
     float m = 0.f;
     if (l < p.c)
@@ -163,6 +168,7 @@ __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict_
     const int e = (m > 0.f && m <= 3.402823466e38f) ? exponent(m) : 0;
     const float f = pow2f(7 - e);
     if (part == 0) t[l] = pow2f(e - 7);
+    float nb = 0.f, rb = 0.f;
     for (int i = part; i < p.nq * (kKC / 2); i += 32) {
         const int q = i / (kKC / 2), kl = (i % (kKC / 2)) * 2, r = l - (int)p.n0[q];
         if (r < 0) continue;
@@ -171,10 +177,25 @@ __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict_
         const float b1 = (k + 1 < p.d && l < p.c) ? __ldg(B + (int64_t)(k + 1) * ldb + c0 + l) / s[k + 1] * f : 0.f;
         uint32_t w[3];
         split3(make_float2(b0, b1), w[0], w[1], w[2]);
+        const float2 rem = add2(make_float2(b0, b1), neg_bf16x2(w[0]));
+        nb += b0 * b0 + b1 * b1;
+        rb += rem.x * rem.x + rem.y * rem.y;
         const int hn = (int)p.nn[q] / 2, h = r / hn;
         const uint32_t off = (uint32_t)h * 3 * p.hb + p.hoff[q] + tc::sw64_offset((uint32_t)(r - h * hn), (uint32_t)kl);
 #pragma unroll
         for (int z = 0; z < 3; ++z) *reinterpret_cast<uint32_t*>(img + off + (uint32_t)z * p.hb) = w[z];
+    }
+    __syncthreads();
+    red[part][col] = nb;
+    red1[part][col] = rb;
+    __syncthreads();
+    if (part == 0) {
+        for (int k = 1; k < 32; ++k) {
+            nb += red[k][col];
+            rb += red1[k][col];
+        }
+        norm[l] = nb;
+        rest[l] = rb;
     }
 }
 
@@ -263,6 +284,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     float* ss = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTail);   // [256] column scales of A
     float* ts = ss + 256;                                                              // [256] result scales
     float* xchg = ts + 256;                                                            // [4][128]
+    float* need = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTail) - 4;   // [2] halves of the columns:
+    float* rests = need + 2;                                                                // [2] what a row needs (below)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -285,6 +308,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     for (int j = threadIdx.x; j < 256; j += kThreads) {
         ss[j] = p.s[j];
         ts[j] = j < p.npad ? p.t[j] : 0.f;
+    }
+    if (warp < 2) {
+        // A row's sum of squares t_l^2 y_l^2 is at least 2^10 / 12 of what unit
+        // entries of the scaled A would give, and 2^10 times what B's remainders
+        // would, with entries as large as its sum of the unscaled y_l^2 says.
+        float unit = 0.f, rest = 0.f, norm = 0.f;
+        for (int l = 32 * warp + lane; l < p.npad; l += 64) {
+            const float t = p.t[l], f = p.norm[l];
+            unit += t * t * f;
+            rest += t * t * p.rest[l];
+            norm += f;
+        }
+        unit = warp_sum(unit);
+        rest = warp_sum(rest);
+        norm = warp_sum(norm);
+        if (lane == 0) {
+            need[warp] = unit * (1024.f / 12.f);
+            rests[warp] = norm > 0.f ? rest / norm : 0.f;
+        }
     }
     if (warp == kMmaWarp) {
         tc::tmem_alloc_pair(tmem_slot, 512u);
@@ -314,19 +356,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
             if (!warp_wait(tfull + b, par, abort)) break;
             tc::fence_after_sync();
             const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + 256u * (uint32_t)b;
-            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s1[2] = {0.f, 0.f}, mx = 0.f;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s0[2] = {0.f, 0.f}, mx = 0.f;
             for (int col = 32 * half; col < p.npad; col += 64) {
                 uint32_t v0[32], v1[32];
                 tc::tmem_ld_32x32b_x32(taddr + (uint32_t)col, v0);
                 tc::tmem_ld_32x32b_x32(taddr + acc1 + (uint32_t)col, v1);
                 tc::tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float a1 = __uint_as_float(v1[e]), a = __uint_as_float(v0[e]) + a1, t = ts[col + e];
-                    const float y = a * t, y1 = a1 * t;
-                    sum[e & 3] = fmaf(y, y, sum[e & 3]);
-                    s1[e & 1] = fmaf(y1, y1, s1[e & 1]);
-                    mx = fmaxf(mx, fabsf(a));
+                for (int e = 0; e < 32; e += 4) {   // (four squares at a time: fewer roundings into the running sums)
+                    float q = 0.f;
+#pragma unroll
+                    for (int k = e; k < e + 4; ++k) {
+                        const float a = __uint_as_float(v0[k]) + __uint_as_float(v1[k]), y = a * ts[col + k];
+                        q = k == e ? y * y : fmaf(y, y, q);
+                        mx = fmaxf(mx, fabsf(a));
+                        s0[k & 1] = fmaf(a, a, s0[k & 1]);
+                    }
+                    sum[(e >> 2) & 3] += q;
                 }
             }
             tc::fence_before_sync();
@@ -335,9 +381,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
                 if (rank == 0) tc::mbar_arrive(tempty + b);
                 else tc::mbar_arrive_cluster(tempty + b, 0);
             }
-            float tot = (sum[0] + sum[1]) + (sum[2] + sum[3]);
-            // outside the split's range: NaN, which no sum within it is (2^-10; 2^-110, or all zero)
-            if (!(s1[0] + s1[1] <= 9.765625e-4f * tot && mx < 16777216.f && (tot >= 7.703719778e-34f || mx == 0.f)))
+            float tot = sum[0], low = 0.f;   // the last sums with compensation: one rounding, not three
+#pragma unroll
+            for (int k = 1; k < 4; ++k) comp_add(tot, low, sum[k]);
+            if (half == 1) tot += low;
+            // outside the split's range: NaN, which no sum within it is (2^-10; 2^-110 unless all zero)
+            if (!((s0[0] + s0[1]) * rests[half] <= 9.765625e-4f * tot && mx < 16777216.f &&
+                  (tot >= fmaxf(need[half], 7.703719778e-34f) || mx == 0.f)))
                 tot = __uint_as_float(0x7FC00000u);
             // The second half's sum goes to the first through shared memory.
             // Four cells a row: the second half is at most two tiles ahead (the
@@ -350,7 +400,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
                 if (lane == 0) tc::mbar_arrive(xbar);
             } else {
                 if (!warp_wait(xbar, (uint32_t)(i >> 2) & 1u, abort)) break;
-                tot += *cell;
+                comp_add(tot, low, *cell);
+                tot += low;   // (NaN where a sum was not finite)
                 const int64_t row = ((int64_t)cid + (int64_t)i * ncl) * (2 * kRows) + rank * kRows + lr;
                 if (row < p.n) {
                     if (tot <= 3.402823466e38f) p.x[row] = (p.beta != 0.f) ? fmaf(p.alpha, tot, p.beta * p.x[row]) : p.alpha * tot;
@@ -547,7 +598,7 @@ size_t rownorms_tc3_workspace_bytes(const lsk_mat* A, int64_t c, int upper_tri) 
     int64_t per = 0;
     const int np = passes_of(A, c, upper_tri, 0.0, &per);
     if (!np) return 0;
-    return image_bytes(A, per, upper_tri) + 2 * ws_round(256 * 4) + ws_round((size_t)np * A->n * 4) + ws_round(4);
+    return image_bytes(A, per, upper_tri) + 4 * ws_round(256 * 4) + ws_round((size_t)np * A->n * 4) + ws_round(4);
 }
 
 // False: not this kernel's shape.  True: launched (*e its status); rows
@@ -562,6 +613,8 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
     uint8_t* img = wc.take<uint8_t>(image_bytes(A, per, upper_tri));
     float* s = wc.take<float>(256);
     float* t = wc.take<float>(256);
+    float* norm = wc.take<float>(256);
+    float* rest = wc.take<float>(256);
     int* rows = wc.take<int>((size_t)np * A->n);
     int* cnt = wc.take<int>(1);
     LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_units_kernel, 8, kUnitWarps * 32, 0, 1, st, (const float*)A->values, A->ld, A->n,
@@ -583,6 +636,8 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
         p.img = img;
         p.s = s;
         p.t = t;
+        p.norm = norm;
+        p.rest = rest;
         p.list = rows;
         p.count = cnt;
         p.flag = flag;
@@ -594,7 +649,7 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
             *e = cudaErrorNotSupported;
             return true;
         }
-        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_image_kernel, p.npad / 8, 256, 0, 1, st, B, (int)c, (int)c0, p, img, t);
+        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_image_kernel, p.npad / 8, 256, 0, 1, st, B, (int)c, (int)c0, p, img, t, norm, rest);
         LSK_PROF("rownorm_dense_tc3", st) launch_pdl(kernel, 2 * ncl, kThreads, smem, 1, st, p);
     }
     *list = rows;

@@ -51,3 +51,22 @@ def test_zero_and_tiny_rows():
     few = torch.cat([lsk.rownorms_prod(A[i:i + 4000].contiguous(), B, prec="fp32") for i in range(0, n, 4000)])
     assert torch.equal(x[::3], torch.zeros_like(x[::3]))
     assert torch.allclose(x, few, rtol=2e-6, atol=0.0)
+
+
+
+@pytest.mark.parametrize("n,d", [(70_000, 128), (262_144, 64), (20_000, 256), (33_000, 200)])
+def test_error_of_inverse_factors(n, d):
+    """x = ||A_i R^-1||^2 with A's own R, as the leverage scores form them: no
+    further off than on the CUDA cores (3% for the spread of the mean over n rows)."""
+    import paper_2203_02798_gb300 as lsk
+    g = torch.Generator(device="cuda").manual_seed(10)
+    A = torch.randn((n, d), generator=g, device="cuda")
+    R = torch.linalg.qr(A.double(), mode="r")[1]
+    B = torch.linalg.solve_triangular(R, torch.eye(d, dtype=torch.float64, device="cuda"), upper=True).float().contiguous()
+    step = (1 << 30) // (d * d) - 1        # rows of a call that takes the CUDA cores
+    x = lsk.rownorms_prod(A, B, upper_triangular=True, prec="fp32").double()
+    few = torch.cat([lsk.rownorms_prod(A[i:i + step].contiguous(), B, upper_triangular=True, prec="fp32")
+                     for i in range(0, n, step)]).double()
+    want = (A.double() @ B.double()).square().sum(1)
+    rms = lambda v: (v / want - 1.0).square().mean().sqrt().item()
+    assert rms(x) <= 1.03 * rms(few)
