@@ -18,11 +18,10 @@
 // on a list, and the CUDA-core kernel does the listed rows, where the second
 // accumulator may hold more than 2^-5 of the norm (there the terms left out are as
 // large as FP32's roundings), where an accumulator reaches 2^24, and where the sum
-// is not finite or near FP32's bottom.  What acc1 holds is not taken from acc1, which
-// may cancel where few columns make the norm, but from what the remainders after
-// hi add to it on average: those of A's entries, 1/12 each, squared, times B, and
-// those of B's columns times the row's entries, of the size that the sum of its
-// unscaled y_l^2 says; every column counts by its share t_l of the result.
+// is not finite or near FP32's bottom.  A column's own acc1 may cancel, so that its
+// share is taken from all columns: the sum of the acc1^2 times the weight that
+// columns with such remainders have in the norm (by their t_l^2); and the norm is at
+// least 2^10 of what remainders of 1/12 each, squared, in A's entries would give.
 //
 // One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
 // half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
@@ -285,7 +284,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     float* ts = ss + 256;                                                              // [256] result scales
     float* xchg = ts + 256;                                                            // [4][128]
     float* need = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTail) - 4;   // [2] halves of the columns:
-    float* rests = need + 2;                                                                // [2] what a row needs (below)
+    float* weigh = need + 2;                                                                // [2] what a row needs (below)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -310,22 +309,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
         ts[j] = j < p.npad ? p.t[j] : 0.f;
     }
     if (warp < 2) {
-        // A row's sum of squares t_l^2 y_l^2 is at least 2^10 / 12 of what unit
-        // entries of the scaled A would give, and 2^10 times what B's remainders
-        // would, with entries as large as its sum of the unscaled y_l^2 says.
-        float unit = 0.f, rest = 0.f, norm = 0.f;
+        // need: 2^10 / 12 of what unit entries of the scaled A give; weigh: the
+        // mean of t_l^2 over the columns, by their remainders or by their size
+        float unit = 0.f, rest = 0.f, norm = 0.f, rest1 = 0.f;
         for (int l = 32 * warp + lane; l < p.npad; l += 64) {
             const float t = p.t[l], f = p.norm[l];
             unit += t * t * f;
             rest += t * t * p.rest[l];
+            rest1 += p.rest[l];
             norm += f;
         }
         unit = warp_sum(unit);
         rest = warp_sum(rest);
+        rest1 = warp_sum(rest1);
         norm = warp_sum(norm);
         if (lane == 0) {
             need[warp] = unit * (1024.f / 12.f);
-            rests[warp] = norm > 0.f ? rest / norm : 0.f;
+            weigh[warp] = fmaxf(norm > 0.f ? unit / norm : 0.f, rest1 > 0.f ? rest / rest1 : 0.f);
         }
     }
     if (warp == kMmaWarp) {
@@ -356,7 +356,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
             if (!warp_wait(tfull + b, par, abort)) break;
             tc::fence_after_sync();
             const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + 256u * (uint32_t)b;
-            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s0[2] = {0.f, 0.f}, mx = 0.f;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f}, s1[2] = {0.f, 0.f}, mx = 0.f;
             for (int col = 32 * half; col < p.npad; col += 64) {
                 uint32_t v0[32], v1[32];
                 tc::tmem_ld_32x32b_x32(taddr + (uint32_t)col, v0);
@@ -367,10 +367,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
                     float q = 0.f;
 #pragma unroll
                     for (int k = e; k < e + 4; ++k) {
-                        const float a = __uint_as_float(v0[k]) + __uint_as_float(v1[k]), y = a * ts[col + k];
+                        const float a1 = __uint_as_float(v1[k]), a = __uint_as_float(v0[k]) + a1, y = a * ts[col + k];
                         q = k == e ? y * y : fmaf(y, y, q);
                         mx = fmaxf(mx, fabsf(a));
-                        s0[k & 1] = fmaf(a, a, s0[k & 1]);
+                        s1[k & 1] = fmaf(a1, a1, s1[k & 1]);
                     }
                     sum[(e >> 2) & 3] += q;
                 }
@@ -386,7 +386,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
             for (int k = 1; k < 4; ++k) comp_add(tot, low, sum[k]);
             if (half == 1) tot += low;
             // outside the split's range: NaN, which no sum within it is (2^-10; 2^-110 unless all zero)
-            if (!((s0[0] + s0[1]) * rests[half] <= 9.765625e-4f * tot && mx < 16777216.f &&
+            if (!((s1[0] + s1[1]) * weigh[half] <= 9.765625e-4f * tot && mx < 16777216.f &&
                   (tot >= fmaxf(need[half], 7.703719778e-34f) || mx == 0.f)))
                 tot = __uint_as_float(0x7FC00000u);
             // The second half's sum goes to the first through shared memory.

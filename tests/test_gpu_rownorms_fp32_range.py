@@ -6,7 +6,7 @@ import torch
 
 pytestmark = pytest.mark.gpu
 
-KINDS = ["general", "odd_zero", "even_zero", "one", "two", "dominant"]
+KINDS = ["general", "odd_zero", "even_zero", "one", "two", "dominant", "dominant_row"]
 
 
 @pytest.mark.parametrize("kind", KINDS)
@@ -28,6 +28,10 @@ def test_rows_outside_the_range(kind):
         B[:, 6] *= 1e3
         B[0, 6] = 1e6
         A[:, 0] = 0.0
+    if kind == "dominant_row":             # one row of B makes every column but for the (larger) rows with a zero there
+        B[0] *= 1e4
+        A[:8400] *= torch.pow(4.0, k[:8400].float()).view(-1, 1)
+        A[:8400, 0] = 0.0
     x = lsk.rownorms_prod(A, B, prec="fp32")[:8400].double()
     few = lsk.rownorms_prod(A[:2100].contiguous(), B, prec="fp32")
     few = torch.cat([few] + [lsk.rownorms_prod(A[i:i + 2100].contiguous(), B, prec="fp32") for i in (2100, 4200, 6300)]).double()
