@@ -22,7 +22,8 @@ constexpr int RK = 16;    // reduction step
 constexpr int RMP = RM + 4;
 
 // thread (ty, tx) = (tid / 16, tid % 16): rows 8*ty..8*ty+7, cols 4*tx..4*tx+3.
-// kList: the rows list[0 .. *count) of A and x only, a persistent grid.
+// kList: the rows list[0 .. *count) of A and x only (all where *count < 0), a
+// persistent grid.
 template <bool kList>
 __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ B,
@@ -32,12 +33,22 @@ __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     __shared__ __align__(16) float As[RK][RMP];
     __shared__ __align__(16) float Bs[RK][RN];
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const int64_t rows = kList ? (int64_t)*count : n;
-    const auto row_of = [&](int64_t i) { return kList ? (int64_t)__ldg(list + i) : i; };
+    const bool all = !kList || *count < 0;
+    const int64_t rows = all ? n : (int64_t)*count;
+    const auto row_of = [&](int64_t i) { return all ? i : (int64_t)__ldg(list + i); };
     for (int64_t i0 = (int64_t)blockIdx.x * RM; i0 < rows; i0 += (int64_t)gridDim.x * RM) {
         float rowsum[8];
 #pragma unroll
         for (int a = 0; a < 8; ++a) rowsum[a] = 0.f;
+        // a thread loads the same eight rows of every chunk
+        int64_t at[kList ? 8 : 1];
+        if constexpr (kList) {
+#pragma unroll
+            for (int t = 0; t < (RM * RK) / 256; ++t) {
+                const int64_t i = i0 + tid / RK + (256 / RK) * t;
+                at[t] = i < rows ? row_of(i) * lda : 0;
+            }
+        }
 
         for (int64_t c0 = 0; c0 < c; c0 += RN) {
             const int64_t kmax = upper_tri ? min(d, c0 + RN) : d;
@@ -52,7 +63,8 @@ __global__ void __launch_bounds__(256) rownorm_dense_kernel(
                     const int idx = tid + 256 * t;
                     const int row = idx / RK, kk = idx % RK;
                     const int64_t i = i0 + row, kx = k0 + kk;
-                    As[kk][row] = (i < rows && kx < kmax) ? __ldg(A + row_of(i) * lda + kx) : 0.f;
+                    const int64_t row_at = kList ? at[kList ? t : 0] : i * lda;
+                    As[kk][row] = (i < rows && kx < kmax) ? __ldg(A + row_at + kx) : 0.f;
                 }
 #pragma unroll
                 for (int t = 0; t < (RK * RN) / 256; ++t) {

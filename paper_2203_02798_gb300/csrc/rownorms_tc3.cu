@@ -19,9 +19,9 @@
 // accumulator may hold more than 2^-5 of the norm (there the terms left out are as
 // large as FP32's roundings), where an accumulator reaches 2^24, and where the sum
 // is not finite or near FP32's bottom.  A column's own acc1 may cancel, so that its
-// share is taken from all columns: the sum of the acc1^2 times the weight that
-// columns with such remainders have in the norm (by their t_l^2); and the norm is at
-// least 2^10 of what remainders of 1/12 each, squared, in A's entries would give.
+// share is taken from all columns.  The norm has to be 2^10 times what remainders
+// of 1/12 each, squared, in A's entries would give on average, and 2^10 times the sum
+// of the acc1^2 with the weight (t_l^2) that B's remainders have on average.
 //
 // One persistent CTA pair per two SMs (cta_group::2, M = 256): each CTA keeps
 // half of every K-chunk's B tile, three bf16 slices of it, beside a ring of
@@ -76,7 +76,7 @@ struct Rn3Params {
     const uint8_t* img;       // [half][slice][hb]
     const float *s, *t;       // column scales of A, result scales of B's columns
     const float *norm, *rest; // of B's scaled columns: sum of squares, and of the remainders after hi
-    int *list, *count;        // rows left to the CUDA-core kernel
+    int *list, *count;        // rows left to the CUDA-core kernel (*count < 0: all)
     int* flag;
 };
 
@@ -85,23 +85,32 @@ __device__ __forceinline__ int exponent(float v) { return (int)(__float_as_uint(
 
 // s_j: 2^10 over the power of two below the median, over 64 groups of 8
 // consecutive rows spread over A, of the largest |a_ij| (a few outlying rows
-// do not move it; a column that is mostly zero takes its largest).
+// do not move it; a column that is mostly zero takes its largest, one with no
+// nonzero in the sample is left at 0: scale_of()).  *count: 0, or -1 where more than
+// two thirds of the sampled rows are so far from the typical one, by their first 32
+// columns, that their norms would be left to the CUDA cores (rows 2^-6 of it or
+// 2^6 times): these then do all rows at once (750,001 x 200 times 200 x 200 with 85%
+// of the rows scaled by 1e-4: 2,487 us with the tensor-core pass before them).
 constexpr int kUnitWarps = 32;
 __global__ void __launch_bounds__(kUnitWarps * 32) rn3_units_kernel(const float* __restrict__ A, int64_t lda, int64_t n, int d,
                                                                   float* __restrict__ s, int* __restrict__ count) {
     pdl_enter(A, s, count);
     __shared__ float gm[kSampleGroups][33];
     __shared__ float med[32];
+    __shared__ int far;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = (int)blockIdx.x * 32 + lane;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *count = 0;
+    constexpr int kGroups = kSampleGroups / kUnitWarps;   // of a warp
+    float v[kGroups][kSampleRows];
+    if (threadIdx.x == 0) far = 0;
 #pragma unroll
-    for (int g = w; g < kSampleGroups; g += kUnitWarps) {
+    for (int k = 0; k < kGroups; ++k) {
+        const int g = w + k * kUnitWarps;
         const int64_t r0 = (n - kSampleRows) * g / (kSampleGroups - 1);
-        float v[kSampleRows], m = 0.f;
+        float m = 0.f;
 #pragma unroll
-        for (int i = 0; i < kSampleRows; ++i) v[i] = j < d ? __ldg(A + (r0 + i) * lda + j) : 0.f;
+        for (int i = 0; i < kSampleRows; ++i) v[k][i] = j < d ? fabsf(__ldg(A + (r0 + i) * lda + j)) : 0.f;
 #pragma unroll
-        for (int i = 0; i < kSampleRows; ++i) m = fmaxf(m, fabsf(v[i]));
+        for (int i = 0; i < kSampleRows; ++i) m = fmaxf(m, v[k][i]);
         gm[g][lane] = m;
     }
     __syncthreads();
@@ -114,11 +123,32 @@ __global__ void __launch_bounds__(kUnitWarps * 32) rn3_units_kernel(const float*
         if (rank == kSampleGroups / 2) med[lane] = v;
     }
     __syncthreads();
-    if (w == 0 && j < 256) {
-        const float m = med[lane] > 0.f ? med[lane] : mx;
-        s[j] = (m > 0.f && m <= 3.402823466e38f) ? pow2f(10 - exponent(m)) : 1.f;
-    }
+    const float m = med[lane] > 0.f ? med[lane] : mx;
+    const float sj = m > 0.f ? (m <= 3.402823466e38f ? pow2f(10 - exponent(m)) : 1.f) : 0.f;
+    if (w == 0 && j < 256) s[j] = sj;
+    if (blockIdx.x != 0) return;
+    // the sampled rows' largest scaled entries: 2^10 .. 2^12 in a typical row
+    int out = 0;
+#pragma unroll
+    for (int k = 0; k < kGroups; ++k)
+#pragma unroll
+        for (int i = 0; i < kSampleRows; ++i) {
+            float r = v[k][i] * sj;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+            out += r > 0.f && (r < 16.f || r > 262144.f);
+        }
+    if (lane == 0) atomicAdd(&far, out);
+    __syncthreads();
+    if (threadIdx.x == 0) *count = 3 * far > 2 * kSampleGroups * kSampleRows ? -1 : 0;
 }
+
+// The scale of a column: its own, or the largest of all where the sample had no
+// nonzero, which leaves its row of B, scaled by 1 / s_j, the least weight.  (At
+// scale 1 it had the most: B's columns were then scaled by an entry that next to
+// no row uses, and every row was left to the CUDA cores, 2,752 us at 750,001 x 200
+// times 200 x 200.)
+__device__ __forceinline__ float scale_of(float sj, float smax) { return sj > 0.f ? sj : smax > 0.f ? smax : 1.f; }
 
 // scaled value y (an integer part below 2^24) as hi + mid + lo
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
@@ -152,11 +182,23 @@ __device__ __forceinline__ void split3(float2 y, uint32_t& hi, uint32_t& mid, ui
 // The image of B: 8 columns a block.  Column l (0-based in this pass, column
 // c0 + l of B) is scaled so that its largest |b_jl| / s_j is in [128, 256).
 __global__ void __launch_bounds__(256) rn3_image_kernel(const float* __restrict__ B, int ldb, int c0, const Rn3Params p,
+                                                        const float* __restrict__ sample, float* __restrict__ scale,
                                                         uint8_t* __restrict__ img, float* __restrict__ t,
                                                         float* __restrict__ norm, float* __restrict__ rest) {
-    const float* s = p.s;
-    pdl_enter(B, s, img, t, norm, rest);
-    __shared__ float red[32][9], red1[32][9];
+    pdl_enter(B, sample, scale, img, t, norm, rest);
+    __shared__ float red[32][9], red1[32][9], s[256], wmax[8];
+    {
+        const float own = sample[threadIdx.x];
+        float m = own;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+        __syncthreads();
+        for (int w = 0; w < 8; ++w) m = fmaxf(m, wmax[w]);
+        s[threadIdx.x] = scale_of(own, m);
+        if (blockIdx.x == 0) scale[threadIdx.x] = s[threadIdx.x];
+        __syncthreads();
+    }
     const int col = threadIdx.x & 7, part = threadIdx.x >> 3, l = (int)blockIdx.x * 8 + col;
     float m = 0.f;
     if (l < p.c)
@@ -304,28 +346,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) rownorm
     }
     const uint8_t* img = p.img;
     pdl_enter(img);
+    if (*(volatile const int*)p.count < 0) return;   // (both CTAs of every pair) the CUDA cores do all rows
     for (int j = threadIdx.x; j < 256; j += kThreads) {
         ss[j] = p.s[j];
         ts[j] = j < p.npad ? p.t[j] : 0.f;
     }
     if (warp < 2) {
         // need: 2^10 / 12 of what unit entries of the scaled A give; weigh: the
-        // mean of t_l^2 over the columns, by their remainders or by their size
-        float unit = 0.f, rest = 0.f, norm = 0.f, rest1 = 0.f;
+        // mean of t_l^2 over B's columns by their remainders
+        float unit = 0.f, rest = 0.f, rest1 = 0.f;
         for (int l = 32 * warp + lane; l < p.npad; l += 64) {
-            const float t = p.t[l], f = p.norm[l];
-            unit += t * t * f;
+            const float t = p.t[l];
+            unit += t * t * p.norm[l];
             rest += t * t * p.rest[l];
             rest1 += p.rest[l];
-            norm += f;
         }
         unit = warp_sum(unit);
         rest = warp_sum(rest);
         rest1 = warp_sum(rest1);
-        norm = warp_sum(norm);
         if (lane == 0) {
             need[warp] = unit * (1024.f / 12.f);
-            weigh[warp] = fmaxf(norm > 0.f ? unit / norm : 0.f, rest1 > 0.f ? rest / rest1 : 0.f);
+            weigh[warp] = rest1 > 0.f ? rest / rest1 : 0.f;
         }
     }
     if (warp == kMmaWarp) {
@@ -598,11 +639,12 @@ size_t rownorms_tc3_workspace_bytes(const lsk_mat* A, int64_t c, int upper_tri) 
     int64_t per = 0;
     const int np = passes_of(A, c, upper_tri, 0.0, &per);
     if (!np) return 0;
-    return image_bytes(A, per, upper_tri) + 4 * ws_round(256 * 4) + ws_round((size_t)np * A->n * 4) + ws_round(4);
+    return image_bytes(A, per, upper_tri) + 5 * ws_round(256 * 4) + ws_round((size_t)np * A->n * 4) + ws_round(4);
 }
 
 // False: not this kernel's shape.  True: launched (*e its status); rows
-// list[0 .. *count) of x are then left to the caller.
+// list[0 .. *count) of x, or all of them where *count < 0, are then left to the
+// caller.
 bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alpha, float beta, int upper_tri, float* x,
                          void* ws, int* flag, cudaStream_t st, const int** list, const int** count, cudaError_t* e) {
     int64_t per = 0;
@@ -611,6 +653,7 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
     const bool vec = (A->d % 4 == 0) && (A->ld % 4 == 0) && (((uintptr_t)A->values & 15) == 0);
     WsCarver wc{(char*)ws, 0};
     uint8_t* img = wc.take<uint8_t>(image_bytes(A, per, upper_tri));
+    float* sample = wc.take<float>(256);
     float* s = wc.take<float>(256);
     float* t = wc.take<float>(256);
     float* norm = wc.take<float>(256);
@@ -618,7 +661,7 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
     int* rows = wc.take<int>((size_t)np * A->n);
     int* cnt = wc.take<int>(1);
     LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_units_kernel, 8, kUnitWarps * 32, 0, 1, st, (const float*)A->values, A->ld, A->n,
-                                             (int)A->d, s, cnt);
+                                             (int)A->d, sample, cnt);
     for (int k = 0; k < np; ++k) {
         Rn3Params p{};
         const int64_t c0 = k * per, ck = std::min<int64_t>(per, c - c0);
@@ -649,7 +692,7 @@ bool rownorms_tc3_launch(const lsk_mat* A, const float* B, int64_t c, float alph
             *e = cudaErrorNotSupported;
             return true;
         }
-        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_image_kernel, p.npad / 8, 256, 0, 1, st, B, (int)c, (int)c0, p, img, t, norm, rest);
+        LSK_PROF("rownorm_tc_prep", st) launch_pdl(rn3_image_kernel, p.npad / 8, 256, 0, 1, st, B, (int)c, (int)c0, p, sample, s, img, t, norm, rest);
         LSK_PROF("rownorm_dense_tc3", st) launch_pdl(kernel, 2 * ncl, kThreads, smem, 1, st, p);
     }
     *list = rows;

@@ -74,3 +74,45 @@ def test_error_of_inverse_factors(n, d):
     want = (A.double() @ B.double()).square().sum(1)
     rms = lambda v: (v / want - 1.0).square().mean().sqrt().item()
     assert rms(x) <= 1.03 * rms(few)
+
+
+def stage_times(lsk, A, B):
+    """x, and the time of the tensor-core pass and of the CUDA-core pass behind it (ms)."""
+    lsk.rownorms_prod(A, B, prec="fp32")
+    ctx = lsk.context()
+    ctx.profile_reset()
+    ctx.profile(True)
+    x = lsk.rownorms_prod(A, B, prec="fp32")
+    ctx.sync()
+    times = ctx.profile_totals()
+    ctx.profile(False)
+    return x, times["rownorm_dense_tc3"][1], times["rownorm_dense_simt"][1]
+
+
+@pytest.mark.parametrize("c", [96, 256])
+@pytest.mark.parametrize("kind", ["zero_column", "rare_column", "first_columns_zero", "mostly_small_rows", "mostly_zero_rows"])
+def test_work_shared_by_the_sample(kind, c):
+    """Columns that the sampled rows do not show leave the rows on the tensor
+    cores; where most rows are outside the range, the CUDA cores do all of them
+    and the tensor-core pass ends at once."""
+    import paper_2203_02798_gb300 as lsk
+    n, d = 300_000, 96
+    g = torch.Generator(device="cuda").manual_seed(9)
+    A = torch.randn((n, d), generator=g, device="cuda") * torch.logspace(-2, 2, d, device="cuda")
+    B = torch.randn((d, c), generator=g, device="cuda")
+    if kind == "zero_column":
+        A[:, 50] = 0.0
+    if kind == "rare_column":
+        A[:, 3] = 0.0
+        A[1234::100_000, 3] = 1.0
+    if kind == "first_columns_zero":
+        A[:, :40] = 0.0
+    if kind == "mostly_small_rows":
+        A[torch.arange(n, device="cuda") % 8 != 3] *= 1e-5
+    if kind == "mostly_zero_rows":
+        A[torch.arange(n, device="cuda") % 8 != 3] = 0.0
+    x, tc, simt = stage_times(lsk, A, B)
+    want = (A.double() @ B.double()).square().sum(1)
+    bound = (2 * (d + 2) + c + 4) * 2.0 ** -24 * ((A.double().abs() @ B.double().abs()).square().sum(1))
+    assert torch.all((x.double() - want).abs() <= bound)
+    assert (tc < 0.3 * simt) if kind == "mostly_small_rows" else (simt < tc)
