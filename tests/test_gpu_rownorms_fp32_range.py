@@ -116,3 +116,31 @@ def test_work_shared_by_the_sample(kind, c):
     bound = (2 * (d + 2) + c + 4) * 2.0 ** -24 * ((A.double().abs() @ B.double().abs()).square().sum(1))
     assert torch.all((x.double() - want).abs() <= bound)
     assert (tc < 0.3 * simt) if kind == "mostly_small_rows" else (simt < tc)
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+@pytest.mark.parametrize("listed", [1, 5, 156, 158, 627, 629, 1500])
+def test_few_listed_rows(listed, beta):
+    """The CUDA cores' forms for few listed rows (up to four a block of the 157
+    tiles here) and for more: the rows that a call on them alone gives."""
+    import paper_2203_02798_gb300 as lsk
+    n, d = 20_001, 256
+    g = torch.Generator(device="cuda").manual_seed(11)
+    A = torch.randn((n, d), generator=g, device="cuda")
+    at = torch.arange(listed, device="cuda") * (n // listed)
+    A[at] *= 2.0 ** -14
+    B = torch.triu(torch.randn((d, d), generator=g, device="cuda"))
+    x0 = torch.rand(n, generator=g, device="cuda")
+    x = lsk.rownorms_prod(A, B, alpha=2.0, beta=beta, x=x0.clone(), upper_triangular=True, prec="fp32").double()
+    want = 2.0 * (A.double() @ B.double()).square().sum(1) + beta * x0.double()
+    size = 2.0 * (A.double().abs() @ B.double().abs()).square().sum(1) + beta * x0.double()
+    assert torch.all((x - want).abs() <= 2 * (d + 4) * 2.0 ** -24 * size)
+
+
+def test_few_listed_rows_cost_little():
+    import paper_2203_02798_gb300 as lsk
+    n, d = 33_000, 256
+    A = torch.randn((n, d), generator=torch.Generator(device="cuda").manual_seed(12), device="cuda")
+    A[::10_000] *= 2.0 ** -14
+    x, tc, simt = stage_times(lsk, A, torch.eye(d, device="cuda"))
+    assert simt < 0.5 * tc
