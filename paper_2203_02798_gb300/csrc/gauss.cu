@@ -128,6 +128,12 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, int64_t n
 #pragma unroll
             for (int q = 0; q < 8; ++q) comp_add(s, c, v[q]);
         }
+        if (!comp_ok(s, c)) {
+            double t = 0.0;
+            for (int64_t z = 0; z < nz; ++z) t += (double)part[z * len + e];
+            s = (float)t;
+            c = 0.f;
+        }
         out[e] = s + c;
     }
 }

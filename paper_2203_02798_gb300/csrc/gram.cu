@@ -271,6 +271,11 @@ __global__ void __launch_bounds__(256) gram_csr_reduce_kernel(const float* __res
             for (int i = 0; i < 8; ++i) comp_add(s, c, v[i]);
         }
     acc[g][x] = (double)s + (double)c;
+    if (!comp_ok(s, c)) {
+        double t = 0.0;
+        for (int64_t z = g; z < nblocks; z += 8) t += (double)part[z * len + e];
+        acc[g][x] = t;
+    }
     __syncthreads();
     if (g == 0 && upper) {
         double t = 0.0;

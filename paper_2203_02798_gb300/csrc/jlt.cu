@@ -217,6 +217,11 @@ __global__ void __launch_bounds__(256) csrjlt_reduce_kernel(const float* __restr
             for (int k = 0; k < 8; ++k) comp_add(s, c, v[k]);
         }
     acc[g][threadIdx.x & 63] = (double)s + (double)c;
+    if (!comp_ok(s, c)) {
+        double t = 0.0;
+        for (int b = g; b < nsplit; b += 4) t += (double)part[(int64_t)b * total + x];
+        acc[g][threadIdx.x & 63] = t;
+    }
     __syncthreads();
     if (g == 0 && x < total) {
         const int i = threadIdx.x;
