@@ -484,8 +484,8 @@ namespace {
 // summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
 // (2.9e-8 for the CUDA-core kernel; storing C in FP32 alone costs 1.85e-8),
 // 4.5e-8 against 2.5e-7 with five rows scaled x100.  A column below 2^-48 (its
-// small products would leave FP32's range) or a diagonal that is not finite
-// sets *redo, and the CUDA-core kernel forms C.
+// small products would leave FP32's range) or a diagonal whose sum might leave it
+// sets *redo, and the CUDA-core kernel, which adds up in FP64, forms C.
 //
 // Work: a job is a 128-column panel of C's rows against the columns from the
 // panel's first on (d > 128: two jobs, N = npad and npad - 128; the SMs are
@@ -723,6 +723,7 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
         constexpr uint32_t idesc = tc::idesc_bf16_f32_mn(128, (uint32_t)NPAD);
         const uint32_t acc0 = tmem, acc1 = tmem + (uint32_t)NPAD;
         const int quarter = warp & 3, row = quarter * 32 + lane;
+        float diag = 0.f;   // of this CTA's rows so far
         bool okm = true;
         int s = 0;
         uint32_t ph = 0;
@@ -773,12 +774,13 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
                 tc::tmem_ld_32x32b_x32(ta, va);
                 tc::tmem_ld_32x32b_x32(ta + (uint32_t)NPAD, vb);
                 tc::tmem_ld_wait();
-                if (col == quarter * 32) {   // the diagonal: an entry outside FP32's range shows here first
-                    float dg = 0.f;
+                if (col == quarter * 32) {
+                    // the diagonal, which bounds every sum of its row and column: the
+                    // CTAs' (some 300 at most) stay within FP32's range below 2^117 each
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
-                        if (i == lane) dg = __uint_as_float(va[i]) + __uint_as_float(vb[i]);
-                    if (!(fabsf(dg) <= 3.402823466e38f)) atomicOr(q.redo, 1);
+                        if (i == lane) diag += __uint_as_float(va[i]) + __uint_as_float(vb[i]);
+                    if (!(diag <= 1.66153499e35f)) atomicOr(q.redo, 1);
                 }
                 if (col + 32 >= NPAD) {
                     tc::fence_before_sync();

@@ -86,3 +86,15 @@ def test_large_sums_and_alpha():
     C = lsk.gram(lsk.csr_from_numpy(V, J, I, d), alpha=1e-20).cpu().numpy()
     want = np.eye(d) * (n / d) * float(V[0]) ** 2 * 1e-20
     assert np.allclose(C, want, rtol=1e-5, atol=0.0)
+
+
+@pytest.mark.parametrize("n,d", [(300_000, 32), (200_000, 130)])
+def test_large_sums_of_dense_products(n, d):
+    """Products of 1e35: a few thousand rows' sums leave FP32's range, no thousand's
+    do.  The CUDA cores, which form them, add up 1,024 equal products in FP32 at a
+    time, each addition rounding the same way: within 1,024 x 2^-24."""
+    import paper_2203_02798_gb300 as lsk
+    A = 3e17 * torch.sign(torch.randn((n, d), generator=torch.Generator(device="cuda").manual_seed(3), device="cuda"))
+    C = lsk.gram(A, alpha=1e-20, prec="fp32").double()
+    want = 1e-20 * (A.double().T @ A.double())
+    assert torch.all((C - want).abs() <= 1024 * 2.0 ** -24 * want.diagonal().max())
