@@ -480,8 +480,10 @@ namespace {
 // first, where that rounding no longer matters.  The unit is only a choice of
 // rounding: an entry above the maximum seen (the first rows of the CTA, then a
 // quarter of each segment and of the one before) costs exactness in its
-// segment, no more.  The CTAs' partials keep the two accumulators apart and are
-// summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
+// segment, no more.  A CTA adds up to kChain segments in FP32, the two accumulators
+// apart, and starts another partial for the next ones, so that the error does not
+// grow with its rows (offset entries, 16M x 64, 103 segments: 2.2e-8 in one chain,
+// 1.8e-8 in five; CUDA cores 1.8e-8); all partials are summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
 // (2.9e-8 for the CUDA-core kernel; storing C in FP32 alone costs 1.85e-8),
 // 4.5e-8 against 2.5e-7 with five rows scaled x100.  A column below 2^-48 (its
 // small products would leave FP32's range) or a diagonal whose sum might leave it
@@ -505,11 +507,13 @@ namespace {
 // roundings of lo over); more rows the longer segments, since every flush of
 // the accumulators costs L2 reductions (1.5 GB of them at 1M x 256 with 256-row
 // segments: 0.13 ms).
+constexpr int kChain = 24, kMaxSlabs = 64;   // (2.5 GB of partials at most)
 struct Gr3Params {
     GrParams a;          // A, lda, n, d, vec, part, flag
     int chunks;          // 32-row chunks of A
     int ctas[2];         // CTAs of the two jobs (ctas[1] = 0 for d <= 128)
     int seg_chunks;
+    int slabs, chain;    // partials a CTA, and the segments of each
     uint32_t magic_add;  // exponent of 1.5 * 2^23 units above the column maximum's, and the 1.5
     int* redo;
 };
@@ -519,7 +523,7 @@ __host__ __device__ constexpr int stages3_of(int npad) {
     return (int)((232448 - 6144) / stage3_bytes(npad)) < kMaxStages ? (int)((232448 - 6144) / stage3_bytes(npad)) : kMaxStages;
 }
 __host__ __device__ constexpr uint32_t tmem3_cols(int npad) { return npad <= 32 ? 64u : npad <= 64 ? 128u : npad <= 128 ? 256u : 512u; }
-// FP32 words of one CTA's partial: two planes of 128 x N
+// FP32 words of one partial: two planes of 128 x N
 __host__ __device__ constexpr size_t part3_floats(int npad) { return 2u * kMT * (size_t)npad; }
 
 // two FP32 additions in one instruction (the low word is the first of the pair)
@@ -768,6 +772,8 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
             if (lane == 0 && okm) okw = tc::mbar_wait(done, (uint32_t)z & 1u, abort) ? 1 : 0;
             if (!__shfl_sync(0xffffffffu, okw, 0)) break;
             tc::fence_after_sync();
+            const int slab = z / q.chain;
+            const bool first = slab * q.chain == z;
             for (int col = 0; col < NPAD; col += 32) {
                 uint32_t va[32], vb[32];
                 const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col;
@@ -790,10 +796,10 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
                 // the partial is stored by columns: a warp's 32 rows are one
                 // 128-byte line (row-major v4 reductions, a line a lane, took
                 // 7,700 cycles a flush at N = 128)
-                float* dst = part + (size_t)col * kMT + row;
+                float* dst = part + (size_t)slab * part3_floats(NPAD) + (size_t)col * kMT + row;
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    if (z == 0) {   // (one thread an address: the first segment stores, later ones add)
+                    if (first) {   // (one thread an address: the first segment stores, later ones add)
                         dst[i * kMT] = __uint_as_float(va[i]);
                         dst[(NPAD + i) * kMT] = __uint_as_float(vb[i]);
                     } else {
@@ -803,6 +809,8 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
                 }
             }
         }
+        for (int y = (nseg + q.chain - 1) / q.chain; y < q.slabs; ++y)   // (a CTA of fewer segments than others)
+            for (int i = 0; i < 2 * NPAD; ++i) part[(size_t)y * part3_floats(NPAD) + (size_t)i * kMT + row] = 0.f;
         if (warp == kMmaWarp) {   // also when a wait gave up: every MMA issued is complete before TMEM goes
             if (tc::elect_one()) tc::mma_commit(fin);
             __syncwarp();
@@ -833,7 +841,7 @@ __global__ void __launch_bounds__(Shape3::kThreads, 1) gram_tc3_kernel(const Gr3
     const int job = (int)blockIdx.x >= p.ctas[0];
     const int64_t c = (int)blockIdx.x - (job ? p.ctas[0] : 0), nc = job ? p.ctas[1] : p.ctas[0];
     const int g0 = (int)(p.chunks * c / nc), g1 = (int)(p.chunks * (c + 1) / nc);
-    float* part = p.a.part + (job ? p.ctas[0] * part3_floats(NPAD) + c * part3_floats(NPAD - kMT) : c * part3_floats(NPAD));
+    float* part = p.a.part + p.slabs * (job ? p.ctas[0] * part3_floats(NPAD) + c * part3_floats(NPAD - kMT) : c * part3_floats(NPAD));
     if constexpr (NPAD > kMT) {
         if (job) {
             GrParams b = p.a;
@@ -861,7 +869,7 @@ __global__ void __launch_bounds__(256) gram_tc3_reduce_kernel(const float* __res
     const bool upper = e < d * d && a <= b;
     float s = 0.f, c = 0.f;
     if (upper) {
-        const int job = a >= kMT, w = job ? npad - kMT : npad, n = job ? ctas1 : ctas0;
+        const int job = a >= kMT, w = job ? npad - kMT : npad, n = job ? ctas1 : ctas0;   // (partials of all CTAs)
         const size_t one = part3_floats(w), plane = (size_t)kMT * w;
         const float* src = part + (job ? ctas0 * part3_floats(npad) : 0) + (size_t)(b - job * kMT) * kMT + (a - job * kMT);
         for (int z = g; z < n; z += 32) {   // eight loads in flight
@@ -888,7 +896,7 @@ __global__ void __launch_bounds__(256) gram_tc3_reduce_kernel(const float* __res
 }
 
 struct Gr3Plan {
-    int npad, chunks, ctas[2];
+    int npad, chunks, ctas[2], seg_chunks, slabs, chain;
     size_t part_bytes;
 };
 // The SMs are shared out between the two jobs by a chunk's cost: 6 N cycles of
@@ -905,7 +913,12 @@ Gr3Plan gram_tc3_plan(const lsk_mat* A, int sm_count) {
         q.ctas[0] = sm_count;
     }
     for (int j = 0; j < 2; ++j) q.ctas[j] = std::min(q.ctas[j], q.chunks);
-    q.part_bytes = q.ctas[0] * part3_floats(q.npad) * 4 + (q.npad > kMT ? q.ctas[1] * part3_floats(q.npad - kMT) * 4 : 0);
+    q.seg_chunks = q.chunks <= 32 * q.ctas[0] ? 8 : 32;   // (at most 1,024 rows a CTA: the finer unit)
+    const int fewest = q.npad > kMT ? std::min(q.ctas[0], q.ctas[1]) : q.ctas[0];   // CTAs of a job
+    const int64_t most = ((q.chunks + fewest - 1) / fewest + q.seg_chunks - 1) / q.seg_chunks;   // segments of a CTA
+    q.slabs = (int)std::max<int64_t>(1, std::min<int64_t>((most + kChain - 1) / kChain, kMaxSlabs));
+    q.chain = (int)((most + q.slabs - 1) / q.slabs);
+    q.part_bytes = q.slabs * (q.ctas[0] * part3_floats(q.npad) * 4 + (q.npad > kMT ? q.ctas[1] * part3_floats(q.npad - kMT) * 4 : 0));
     return q;
 }
 
@@ -955,9 +968,10 @@ cudaError_t gram_tc3_launch(const lsk_mat* A, double alpha, double beta, OutT* C
     p.chunks = q.chunks;
     p.ctas[0] = q.ctas[0];
     p.ctas[1] = q.ctas[1];
-    const bool few = q.chunks <= 32 * q.ctas[0];   // at most 1,024 rows a CTA
-    p.seg_chunks = few ? 8 : 32;
-    p.magic_add = ((few ? 16u : 17u) << 23) + 0x400000u;
+    p.seg_chunks = q.seg_chunks;
+    p.slabs = q.slabs;
+    p.chain = q.chain;
+    p.magic_add = ((q.seg_chunks == 8 ? 16u : 17u) << 23) + 0x400000u;
     cudaError_t e = cudaMemsetAsync(p.redo, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
     switch (q.npad) {
@@ -972,7 +986,7 @@ cudaError_t gram_tc3_launch(const lsk_mat* A, double alpha, double beta, OutT* C
     }
     if (e != cudaSuccess) return e;
     LSK_PROF("gram_reduce", st) gram_tc3_reduce_kernel<OutT><<<(unsigned)((A->d * A->d + 31) / 32), 256, 0, st>>>(
-        p.a.part, q.ctas[0], q.ctas[1], (int)A->d, q.npad, p.redo, alpha, beta, C);
+        p.a.part, q.slabs * q.ctas[0], q.slabs * q.ctas[1], (int)A->d, q.npad, p.redo, alpha, beta, C);
     return cudaGetLastError();
 }
 template cudaError_t gram_tc3_launch<float>(const lsk_mat*, double, double, float*, void*, int*, int, cudaStream_t, const int**);
