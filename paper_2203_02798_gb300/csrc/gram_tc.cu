@@ -105,29 +105,29 @@ __device__ __forceinline__ void load_row(const GrParams& p, int64_t row, int64_t
         }
     }
 }
-// The eight rows from row0 on; rows of whole 16-byte quads that are all in
-// range go without per-row checks (the registers of lanes past d, zero before,
-// are left as they are).
+// The eight rows from row0 on, v[r] the row r + turn, modulo 8; rows of whole
+// 16-byte quads that are all in range go without per-row checks (the registers of
+// lanes past d, zero before, are left as they are).
 template <int NPAD>
-__device__ __forceinline__ void load_piece_quads(const GrParams& p, int64_t row0, int64_t r_end, int lane,
+__device__ __forceinline__ void load_piece_quads(const GrParams& p, int64_t row0, int64_t r_end, int lane, int turn,
                                                  float4 (&v)[8][(NPAD + kMT - 1) / kMT]) {
     constexpr int H = (NPAD + kMT - 1) / kMT;
     if (p.vec && (p.d & 3) == 0 && row0 + 8 <= r_end) {
-        const char* src = reinterpret_cast<const char*>(p.A + row0 * p.lda + 4 * lane);
+        const char* const src0 = reinterpret_cast<const char*>(p.A + row0 * p.lda + 4 * lane);
         const int64_t step = p.lda * 4;
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
+            const char* const src = src0 + ((r + turn) & 7) * step;
 #pragma unroll
             for (int h = 0; h < H; ++h)
                 if (4 * lane + kMT * h < p.d)
                     asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
                                  : "=f"(v[r][h].x), "=f"(v[r][h].y), "=f"(v[r][h].z), "=f"(v[r][h].w)
                                  : "l"(src + 4 * kMT * h));
-            src += step;
         }
     } else {
 #pragma unroll
-        for (int r = 0; r < 8; ++r) load_row<NPAD>(p, row0 + r, r_end, lane, v[r]);
+        for (int r = 0; r < 8; ++r) load_row<NPAD>(p, row0 + ((r + turn) & 7), r_end, lane, v[r]);
     }
 }
 template <int NPAD, int PR>
@@ -479,8 +479,11 @@ namespace {
 // ways round, and mid mid) go to a second accumulator, a small part of the
 // first, where that rounding no longer matters.  The unit is only a choice of
 // rounding: an entry above the maximum seen (the first rows of the CTA, then a
-// quarter of each segment and of the one before) costs exactness in its
-// segment, no more.  A CTA adds up to kChain segments in FP32, the two accumulators
+// quarter of each segment and of the one before, or, where these show none, the
+// largest ever) costs exactness in its segment, no more.  Warps note what they see
+// while others split, so that equal calls may differ in the last bits.  Entries below
+// 2^-8 of their column's unit keep 16 bits: the error is small against the norms
+// of the two columns, but not entry by entry against sum |a_ij a_ik|.  A CTA adds up to kChain segments in FP32, the two accumulators
 // apart, and starts another partial for the next ones, so that the error does not
 // grow with its rows (offset entries, 16M x 64, 103 segments: 2.2e-8 in one chain,
 // 1.8e-8 in five; CUDA cores 1.8e-8); all partials are summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
@@ -561,6 +564,10 @@ __device__ __forceinline__ uint4 ld_shared4(const uint32_t* p) {
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(tc::smem_u32(p)));
     return v;
 }
+// where the rows of chunk c's pieces begin in a lane's registers: the two rows that
+// are looked at (store_piece3) are other ones from chunk to chunk, so that no
+// pattern of rows hides from them
+__device__ __forceinline__ int turn_of(int c) { return (int)(((uint32_t)c * 0x9E3779B1u) >> 30) * 2; }
 __device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t h) {   // per half: max(m, |h|), m >= 0
     const __nv_bfloat162 r = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&m), __habs2(*reinterpret_cast<__nv_bfloat162*>(&h)));
     return *reinterpret_cast<const uint32_t*>(&r);
@@ -650,7 +657,7 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
             for (int r = 0; r < 8; ++r)
 #pragma unroll
                 for (int h = 0; h < H; ++h) v[b][r][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-            load_piece_quads<NPAD>(p, row_base + (int64_t)(c0 + 4 * b) * kKC, r_end, lane, v[b]);
+            load_piece_quads<NPAD>(p, row_base + (int64_t)(c0 + 4 * b) * kKC, r_end, lane, turn_of(c0 + 4 * b), v[b]);
         }
 #pragma unroll
         for (int h = 0; h < H; ++h) {   // the first rows give the columns' units
@@ -689,8 +696,13 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
 #pragma unroll
             for (int i = 0; i < H; ++i) {
                 const uint4 b = ld_shared4(cur + kMT * i), d = ld_shared4(last + kMT * i);   // other warps may be raising these
-                mg[i] = make_float4(unit_magic(max(b.x, d.x), q.magic_add), unit_magic(max(b.y, d.y), q.magic_add),
-                                    unit_magic(max(b.z, d.z), q.magic_add), unit_magic(max(b.w, d.w), q.magic_add));
+                uint4 u = make_uint4(max(b.x, d.x), max(b.y, d.y), max(b.z, d.z), max(b.w, d.w));
+                if (!u.x || !u.y || !u.z || !u.w) {
+                    const uint4 o = ld_shared4(cm + 2 * kCols + kMT * i);
+                    u = make_uint4(u.x ? u.x : o.x, u.y ? u.y : o.y, u.z ? u.z : o.z, u.w ? u.w : o.w);
+                }
+                mg[i] = make_float4(unit_magic(u.x, q.magic_add), unit_magic(u.y, q.magic_add), unit_magic(u.z, q.magic_add),
+                                    unit_magic(u.w, q.magic_add));
             }
             const int s = c % kStages;
             int okl = 1;
@@ -713,10 +725,10 @@ __device__ __forceinline__ void gram_tc3_body(const GrParams& p, const Gr3Params
         };
         for (int c = c0; c < nchunks; c += 4 * NB) {
             if (!put(c, v[0])) break;
-            load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 4 * NB) * kKC, r_end, lane, v[0]);
+            load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 4 * NB) * kKC, r_end, lane, turn_of(c + 4 * NB), v[0]);
             if constexpr (NB == 2) {
                 if (c + 4 >= nchunks || !put(c + 4, v[1])) break;
-                load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 12) * kKC, r_end, lane, v[1]);
+                load_piece_quads<NPAD>(p, row_base + (int64_t)(c + 12) * kKC, r_end, lane, turn_of(c + 12), v[1]);
             }
         }
     } else {
