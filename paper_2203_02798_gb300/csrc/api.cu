@@ -163,7 +163,7 @@ int lsk_cs_sketch(lsk_ctx* ctx, const lsk_mat* A, int64_t r, uint64_t seed, floa
     if (r < 1 || r >= ((int64_t)1 << 31)) return fail(ctx, LSK_ERR_INVALID_ARG, "r must be in [1, 2^31)");
     if (!SA) return fail(ctx, LSK_ERR_INVALID_ARG, "SA is NULL");
     if (A->kind == LSK_CSR && A->d > 51200) return fail(ctx, LSK_ERR_UNSUPPORTED, "CSR sketch needs d <= 51200");
-    rc = ws_ensure(ctx, cs_workspace_bytes(A->n, r));
+    rc = ws_ensure(ctx, cs_workspace_bytes(A, r));
     if (rc) return rc;
     cudaError_t e = cs_launch(A, r, seed, SA, ctx->ws, ctx->flag, ctx->sm_count, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lsk_cs_sketch");
@@ -295,7 +295,7 @@ struct SketchBufs {
 };
 
 size_t stage_scratch(const lsk_mat* A, int64_t r, int64_t k, int32_t prec, int sm) {
-    size_t s = cs_workspace_bytes(A->n, r);
+    size_t s = cs_workspace_bytes(A, r);
     if (k > 0) {
         const size_t g = gauss_workspace_bytes(r, A->d, k, prec, sm);
         if (g > s) s = g;
@@ -441,7 +441,7 @@ int lsk_sketch_rows(lsk_ctx* ctx, const lsk_mat* A, int64_t r, int64_t k, uint64
     prec = sketch_prec(prec);
     cudaError_t e;
     if (k == 0) {   // S A straight into out (the gather adds into it when accumulating)
-        rc = ws_ensure(ctx, cs_workspace_bytes(A->n, r));
+        rc = ws_ensure(ctx, cs_workspace_bytes(A, r));
         if (rc) return rc;
         e = cs_launch(A, r, seed, out, ctx->ws, ctx->flag, ctx->sm_count, ctx->stream, (uint64_t)row0, accumulate != 0);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "lsk_sketch_rows");

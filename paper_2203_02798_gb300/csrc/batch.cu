@@ -75,6 +75,7 @@ struct LskBatch {
     std::vector<char> grouped;       // per item: takes the grouped path
     std::vector<int> wave;           // per grouped item: its wave
     std::vector<float*> SA, Rinv32;  // per grouped item: its sketch and FP32 R^-1 in the arena
+    std::vector<float*> SA2;         // and the second copy that its CSR sketch is formed in (or null)
     std::vector<uint32_t*> cidx;     // per compacted item: the buckets of its sketch's rows, then their count
     std::vector<CsGroup> cg;         // per wave: the grouped CountSketch preparation
     std::vector<RnImageGroup> ig;    // per wave: the row norms' B images (dense) ...
@@ -231,7 +232,7 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
             const lsk_batch_item& it = items[i];
             if (!b->grouped[i] || b->wave[i] != w || !cs_scatters(&it.A, it.r, b->cidx[i] != nullptr)) continue;
             const cudaError_t er =
-                cs_csr_scatter_launch(&it.A, it.r, it.seed, b->SA[i], ctx->flag, ctx->sm_count, b->streams[s]);
+                cs_csr_scatter_launch(&it.A, it.r, it.seed, b->SA[i], b->SA2[i], ctx->flag, ctx->sm_count, b->streams[s]);
             if (er != cudaSuccess) return er;
         }
         return cudaSuccess;
@@ -342,6 +343,7 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
     LskBatch* b = ctx->batch;
     b->grouped.assign(count, 0);
     b->SA.assign(count, nullptr);
+    b->SA2.assign(count, nullptr);
     b->Rinv32.assign(count, nullptr);
     b->cidx.assign(count, nullptr);
     b->cnt_base.assign(count, 0);
@@ -370,6 +372,7 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
                  gauss_group_part_bytes(rs, d, k, wslice[b->wave[i]]) + ws_round(qr_workspace_bytes(k, d)) +
                  ws_round((size_t)d * d * 4) + (compacts(items[i]) ? ws_round((size_t)(rs + 1) * 4) : 0) +
                  ws_round(prepared_bytes(items[i], prec));
+        bytes += cs_scatter_copy_bytes(&items[i].A, items[i].r, compacts(items[i]));
         if (cs_scatters(&items[i].A, items[i].r, compacts(items[i]))) continue;   // no permutation
         wrows[b->wave[i]] += items[i].A.n;
         wcnt[b->wave[i]] += items[i].r + 1;
@@ -410,6 +413,8 @@ int prepare_groups(lsk_ctx* ctx, const lsk_batch_item* items, int count, int32_t
             imj[b->wave[i]].push_back(RnImageJob{items[i].A, Ri32, d, 1, (uint8_t*)prep});
         else if (prep)
             bbj[b->wave[i]].push_back(BbtJob{Ri32, d, d, (float*)prep});
+        const size_t cb = cs_scatter_copy_bytes(&items[i].A, items[i].r, cidx != nullptr);
+        b->SA2[i] = cb ? (float*)wc.take<char>(cb) : nullptr;
         b->SA[i] = SA;
         b->Rinv32[i] = Ri32;
         b->cidx[i] = cidx;

@@ -675,7 +675,8 @@ __global__ void __launch_bounds__(256) cs_csr_scatter_kernel(const float* __rest
                                                              const int32_t* __restrict__ J,
                                                              const int64_t* __restrict__ I, int64_t n, int64_t nnz,
                                                              int64_t d, uint64_t row0, uint32_t r, uint32_t k0,
-                                                             uint32_t k1, float* __restrict__ SA, int* flag) {
+                                                             uint32_t k1, float* SA, float* copy, int64_t stride,
+                                                             int more, int* flag) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -686,6 +687,8 @@ __global__ void __launch_bounds__(256) cs_csr_scatter_kernel(const float* __rest
         uint32_t b, neg;
         cs_hash(row0 + (uint64_t)(i0 + lane), r, k0, k1, b, neg);
         const uint32_t to = b | (neg << 31);
+        const int at_copy = (int)(i0 >> 5) & more;   // groups of rows take turns (more: copies - 1)
+        float* const out = at_copy ? copy + (at_copy - 1) * stride : SA;
         constexpr int kEntries = 2;   // entries a lane at once
         for (int64_t e0 = 0; e0 < g.total; e0 += 32 * kEntries) {
             int32_t col[kEntries];
@@ -707,11 +710,21 @@ __global__ void __launch_bounds__(256) cs_csr_scatter_kernel(const float* __rest
                     bad = true;
                     continue;
                 }
-                atomicAdd(SA + (int64_t)(t[u] & 0x7fffffffu) * d + col[u], (t[u] >> 31) ? -v[u] : v[u]);
+                atomicAdd(out + (int64_t)(t[u] & 0x7fffffffu) * d + col[u], (t[u] >> 31) ? -v[u] : v[u]);
             }
         }
     }
     if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
+}
+
+// SA += the copies of a CSR scatter, in pairs
+__global__ void cs_add_copies_kernel(float* __restrict__ SA, const float* __restrict__ copy, int64_t stride, int more,
+                                     int64_t entries) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < entries; i += (int64_t)gridDim.x * blockDim.x) {
+        float s = SA[i] + __ldg(copy + i);
+        if (more == 3) s += __ldg(copy + stride + i) + __ldg(copy + 2 * stride + i);
+        SA[i] = s;
+    }
 }
 
 __global__ void cs_hash_debug_kernel(int64_t n, uint32_t r, uint32_t k0, uint32_t k1,
@@ -947,6 +960,9 @@ size_t cs_workspace_bytes(int64_t n, int64_t r) {
     RxPlan q;
     return cs_carve(nullptr, n, r, rx_plan(n, r, q) ? &q : nullptr).bytes;
 }
+size_t cs_workspace_bytes(const lsk_mat* A, int64_t r) {
+    return std::max(cs_workspace_bytes(A->n, r), cs_scatter_copy_bytes(A, r, false));
+}
 size_t cs_workspace_bytes_atomic(int64_t n, int64_t r) { return cs_carve(nullptr, n, r, nullptr).bytes; }
 
 cudaError_t cs_hash_launch(int64_t n, int64_t r, uint64_t seed, int32_t* bucket, int8_t* sign,
@@ -999,25 +1015,56 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
     return cudaGetLastError();
 }
 
-// Every CSR sketch but a compacted one (which needs the buckets' counts), one of
-// so few entries that the reductions queue up at their addresses (2^14), and one
-// that sums more than 16 nonzeros to an entry: there the permutation's form,
-// with partial sums of parts of a bucket, rounds less (r = 64 of 1M x 256 at 5%,
-// 781 to an entry: error 1.4e-7 against 5.0e-7 at 269 and 130 us; with 10 to an
-// entry 5.5e-8 against 6.4e-8 at 147 and 50 us).
-bool cs_scatters(const lsk_mat* A, int64_t r, bool compact) {
-    return A->kind == LSK_CSR && !compact && r * A->d >= (1 << 14) && r < ((int64_t)1 << 31) &&
-           A->nnz / 16 <= r * A->d;
+// Parts of a bucket in the permutation's form: enough warps to stream A when there
+// are few buckets, while each part keeps several rows (one part a bucket when
+// compacting).
+static int csr_parts(int64_t n, int64_t r, bool compact) {
+    int P = 1;
+    while (!compact && P < 32 && r * P < 16384 && n >= r * P * 8) P *= 2;
+    return P;
 }
 
-cudaError_t cs_csr_scatter_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, int* flag, int sm_count,
-                                  cudaStream_t st, uint64_t row0, bool accumulate) {
+// Matrices that the reductions of a CSR sketch are added to: one where the
+// permutation's form sums an entry in one chain too, or where an entry has half a
+// nonzero or fewer.  Of split buckets the partial sums are shorter chains, and two
+// or four (all but the first in the workspace, added to it at the end) keep theirs as
+// short: 200,000 x 64 -> 4,096 with 4 nonzeros to an entry is 4.5e-8 off with one,
+// 4.2e-8 with two and by the permutation, 15 to an entry 7.7e-8, 5.8e-8 with four and
+// 5.9e-8 (21 us, 14 with one, 45 by the permutation; 33, 25 and 70).
+static int scatter_copies(const lsk_mat* A, int64_t r) {
+    const int64_t entries = r * A->d;
+    if (csr_parts(A->n, r, false) == 1 || 2 * A->nnz <= entries) return 1;
+    return A->nnz / 4 <= entries ? 2 : 4;
+}
+size_t cs_scatter_copy_bytes(const lsk_mat* A, int64_t r, bool compact) {
+    return cs_scatters(A, r, compact) ? (scatter_copies(A, r) - 1) * ws_round((size_t)r * A->d * 4) : 0;
+}
+
+// Every CSR sketch but a compacted one (which needs the buckets' counts), one of
+// so few entries that the reductions queue up at their addresses (2^14), one
+// that sums more than 16 nonzeros to an entry (there the permutation's form rounds
+// less: r = 64 of 1M x 256 at 5%, 781 to an entry, 1.4e-7 against 5.0e-7 at 269 and 130
+// us), and one whose copies would be large (16 MB each).
+bool cs_scatters(const lsk_mat* A, int64_t r, bool compact) {
+    const int64_t entries = r * A->d;
+    return A->kind == LSK_CSR && !compact && entries >= (1 << 14) && r < ((int64_t)1 << 31) && A->nnz / 16 <= entries &&
+           (scatter_copies(A, r) == 1 || entries <= (1 << 22));
+}
+
+cudaError_t cs_csr_scatter_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, float* copy, int* flag,
+                                  int sm_count, cudaStream_t st, uint64_t row0, bool accumulate) {
     cudaError_t e;
     if (!accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * A->d * 4, st)) != cudaSuccess) return e;
     if (A->n <= 0) return cudaSuccess;
+    const int64_t entries = r * A->d, stride = (int64_t)ws_round((size_t)entries * 4) / 4;
+    const int copies = scatter_copies(A, r);
+    if (copies > 1 && (e = cudaMemsetAsync(copy, 0, (size_t)stride * 4 * (copies - 1), st)) != cudaSuccess) return e;
     LSK_PROF("cs_csr_scatter", st) cs_csr_scatter_kernel<<<grid_for(A->n, 256, sm_count, 32), 256, 0, st>>>(
         (const float*)A->values, A->colidx, A->rowptr, A->n, A->nnz, A->d, row0, (uint32_t)r, (uint32_t)seed,
-        (uint32_t)(seed >> 32), SA, flag);
+        (uint32_t)(seed >> 32), SA, copy, stride, copies - 1, flag);
+    if (copies > 1)
+        LSK_PROF("cs_csr_scatter", st) cs_add_copies_kernel<<<grid_for(entries, 256, sm_count), 256, 0, st>>>(SA, copy, stride,
+                                                                                                           copies - 1, entries);
     return cudaGetLastError();
 }
 
@@ -1026,8 +1073,10 @@ cudaError_t cs_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, voi
                       uint32_t* ccount, bool rx) {
     const int64_t n = A->n;
     const bool compact = cidx != nullptr && ccount != nullptr && !accumulate;
-    if (cs_scatters(A, r, compact))
-        return cs_csr_scatter_launch(A, r, seed, SA, flag, sm_count, st, row0, accumulate);
+    // (without rx: a workspace of fixed size, which has no room for a second copy beyond its own)
+    const size_t copy = cs_scatter_copy_bytes(A, r, compact);
+    if (cs_scatters(A, r, compact) && (rx || copy <= cs_workspace_bytes_atomic(n, r)))
+        return cs_csr_scatter_launch(A, r, seed, SA, (float*)ws, flag, sm_count, st, row0, accumulate);
     const uint32_t* off = nullptr;
     const uint32_t* perm = nullptr;
     cudaError_t e = cs_prep_launch(n, r, seed, ws, sm_count, st, &off, &perm, row0, flag, rx);
@@ -1080,10 +1129,7 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         while (warps > 1 && (size_t)warps * d * 4 > 200 * 1024) warps >>= 1;
         const size_t smem = (size_t)warps * d * 4;
         if (smem > 200 * 1024) return cudaErrorInvalidValue;
-        // parts per bucket: enough warps to stream A when there are few buckets,
-        // while each part keeps several rows (one part a bucket when compacting)
-        int P = 1;
-        while (!compact && P < 32 && r * P < 16384 && n >= (int64_t)r * P * 8) P *= 2;
+        const int P = csr_parts(n, r, compact);
         if (P > 1 && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
         const int64_t warps_needed = r * P;
         if (smem > 48 * 1024) {
