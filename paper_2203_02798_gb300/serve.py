@@ -51,19 +51,25 @@ class Scheduler:
 
     ``admit(now)`` returns the requests that may start now; ``release`` returns
     a finished request's slot and bytes.  A request larger than the whole
-    budget is rejected (it could never be admitted).
+    budget is rejected (it could never be admitted).  ``slot_bytes``: what every
+    slot holds whether it works or not; it is off the budget from the start, and a
+    request counts with what it needs beyond it.
     """
 
-    def __init__(self, slots, hbm_budget):
+    def __init__(self, slots, hbm_budget, slot_bytes=0):
         self.slots = int(slots)
-        self.budget = int(hbm_budget)
+        self.slot_bytes = int(slot_bytes)
+        self.budget = int(hbm_budget) - self.slots * self.slot_bytes
         self.free_slots = int(slots)
         self.used = 0
         self.waiting = collections.deque()
         self.rejected = []
 
+    def cost(self, req):
+        return max(0, req.footprint - self.slot_bytes)
+
     def arrive(self, req):
-        if req.footprint > self.budget:
+        if self.cost(req) > self.budget:
             self.rejected.append(req)
             return False
         self.waiting.append(req)
@@ -71,20 +77,20 @@ class Scheduler:
 
     def admit(self):
         started = []
-        while self.waiting and self.free_slots > 0 and self.used + self.waiting[0].footprint <= self.budget:
+        while self.waiting and self.free_slots > 0 and self.used + self.cost(self.waiting[0]) <= self.budget:
             req = self.waiting.popleft()
             self.free_slots -= 1
-            self.used += req.footprint
+            self.used += self.cost(req)
             started.append(req)
         return started
 
     def release(self, req):
         self.free_slots += 1
-        self.used -= req.footprint
+        self.used -= self.cost(req)
         assert self.free_slots <= self.slots and self.used >= 0
 
 
-def run_trace(requests, execute, slots, hbm_budget, time_scale=1.0, clock=time.perf_counter):
+def run_trace(requests, execute, slots, hbm_budget, time_scale=1.0, clock=time.perf_counter, slot_bytes=0):
     """Replay ``requests`` (sorted by arrival) against ``execute(slot, req)``.
 
     ``execute`` runs on one of ``slots`` worker threads and returns the
@@ -92,7 +98,7 @@ def run_trace(requests, execute, slots, hbm_budget, time_scale=1.0, clock=time.p
     ``time_scale``); admission follows :class:`Scheduler`.  Returns the
     completions in finish order and the rejected requests.
     """
-    sched = Scheduler(slots, hbm_budget)
+    sched = Scheduler(slots, hbm_budget, slot_bytes)
     lock = threading.Condition()
     done = []
     free_slot_ids = list(range(slots))
@@ -163,6 +169,14 @@ def latency_summary(completions, slots=None):
 SLOT_WORKSPACE = 1 << 30
 
 
+def slot_workspace(requests, slots, hbm_budget):
+    """What each slot reserves for a trace: SLOT_WORKSPACE, or nothing where the
+    budget has no room for that and the trace's largest admissible request beside
+    it (which would then be rejected)."""
+    largest = max((r.footprint for r in requests if r.footprint <= hbm_budget), default=0)
+    return SLOT_WORKSPACE if slots * SLOT_WORKSPACE + max(0, largest - SLOT_WORKSPACE) <= hbm_budget else 0
+
+
 class Server:
     """GPU executor: one library context and CUDA stream per slot."""
 
@@ -177,22 +191,24 @@ class Server:
         self.streams = [torch.cuda.Stream(device=self.device) for _ in range(slots)]
         self.ctxs = [lsk.Context(device) for _ in range(slots)]
         self.reserved = [False] * slots
+        self.slot_bytes = SLOT_WORKSPACE
 
     @staticmethod
     def footprint(n, d, nnz=None, r=None, k=None):
         """Device bytes one solve holds beyond its inputs: sketch, factors, vectors."""
         r = r if r is not None else max(d * d, 4 * d)
         k = k if k is not None else 2 * d
-        return int(4 * r * d + 4 * k * d + 64 * d * d + 20 * n + 8 * (nnz or 0) + (6 << 20))
+        copies = 12 * r * d if nnz and r < 16_384 else 0   # a CSR sketch of few buckets: four matrices, not one
+        return int(4 * r * d + 4 * k * d + 64 * d * d + 20 * n + 8 * (nnz or 0) + copies + (6 << 20))
 
     def solve(self, slot, A, b, **opts):
         """One request on ``slot``'s stream; returns (x on the host, info)."""
         torch = self.torch
         with torch.cuda.stream(self.streams[slot]):
-            if not self.reserved[slot]:   # a slot serves one request at a time
+            if self.slot_bytes and not self.reserved[slot]:   # a slot serves one request at a time
                 self.reserved[slot] = True
                 try:
-                    self.ctxs[slot].reserve(SLOT_WORKSPACE)
+                    self.ctxs[slot].reserve(self.slot_bytes)
                 except self.lsk.LskError:   # no room: the workspace grows with the requests
                     pass
             x, info = self.lsk.sketch_precondition_lsq(A, b, ctx=self.ctxs[slot], **opts)
@@ -200,11 +216,21 @@ class Server:
         return xh.numpy(), info
 
     def run(self, requests, hbm_budget=150 * 10**9, time_scale=1.0):
-        """Replay a trace whose payloads are dicts with A, b and options."""
+        """Replay a trace whose payloads are dicts with A, b and options.  The
+        slots' reserved workspaces count against the budget."""
+        requests = list(requests)
+        self.slot_bytes = slot_workspace(requests, self.slots, hbm_budget)
+        if not self.slot_bytes:
+            for s in range(self.slots):   # what an earlier trace reserved
+                if self.reserved[s]:
+                    self.ctxs[s].close()
+                    self.ctxs[s] = self.lsk.Context(self.device.index)
+                    self.reserved[s] = False
+
         def execute(slot, req):
             p = req.payload
             return self.solve(slot, p["A"], p["b"], **p.get("opts", {}))
-        return run_trace(requests, execute, self.slots, hbm_budget, time_scale)
+        return run_trace(requests, execute, self.slots, hbm_budget, time_scale, slot_bytes=self.slot_bytes)
 
     def close(self):
         for c in self.ctxs:
