@@ -467,6 +467,10 @@ int lsk_debug_gauss(lsk_ctx* ctx, int64_t k, int64_t r, uint64_t seed,
  * the kernel returns; the next lsk_sync reports LSK_ERR_TIMEOUT and the
  * context stays usable.  Asynchronous on the context stream. */
 int lsk_debug_wait_timeout(lsk_ctx* ctx, int64_t limit_us);
+/* The radius of the Gaussian draws, sqrt(-2 ln u), is formed without a branch;
+ * *mismatches (host) = for how many of the 2^24 values of u it differs from
+ * sqrtf's in any bit (0).  Synchronises the stream. */
+int lsk_debug_radius(lsk_ctx* ctx, int32_t* mismatches);
 /* Later least-squares solves on this context run their CG step in a cluster of
  * at most `ctas` CTAs (2, 4, 8 or 16; 0: the largest that the device can
  * place, the default), as they would on a device that places no larger one. */

@@ -111,6 +111,7 @@ _SIGS = {
     "lsk_debug_gauss": (ctypes.c_int, [_P, _I64, _I64, _U64, _I32, _P]),
     "lsk_debug_wait_timeout": (ctypes.c_int, [_P, _I64]),
     "lsk_debug_lsq_ctas": (ctypes.c_int, [_P, _I32]),
+    "lsk_debug_radius": (ctypes.c_int, [_P, ctypes.POINTER(_I32)]),
     "lsk_batch_leverage_scores": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32, _I32]),
     "lsk_batch_streams": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32]),
     "lsk_batch_schedule": (ctypes.c_int, [_P, _I32, ctypes.POINTER(_BatchItem), _I32, _P]),
@@ -598,6 +599,14 @@ def debug_wait_timeout(limit_us, device=None, ctx=None):
     next ctx.sync() raises LskError TIMEOUT."""
     ctx = ctx or context(device)
     ctx._call("lsk_debug_wait_timeout", int(limit_us))
+
+
+def debug_radius(device=None, ctx=None):
+    """lsk_debug_radius: the values of the draws' first uniform whose radius is not sqrtf's."""
+    ctx = ctx or context(device)
+    n = ctypes.c_int32(-1)
+    ctx._call("lsk_debug_radius", ctypes.byref(n))
+    return n.value
 
 
 def debug_lsq_ctas(ctas, ctx):

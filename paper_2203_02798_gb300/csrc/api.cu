@@ -890,6 +890,19 @@ int lsk_debug_wait_timeout(lsk_ctx* ctx, int64_t limit_us) {
     return finish(ctx, "lsk_debug_wait_timeout");
 }
 
+int lsk_debug_radius(lsk_ctx* ctx, int32_t* mismatches) {
+    if (!ctx) return LSK_ERR_INVALID_ARG;
+    if (!mismatches) return fail(ctx, LSK_ERR_INVALID_ARG, "mismatches is NULL");
+    const int rc = ws_ensure(ctx, sizeof(int));
+    if (rc) return rc;
+    cudaError_t e = cudaMemsetAsync(ctx->ws, 0, sizeof(int), ctx->stream);
+    if (e == cudaSuccess) e = radius_debug_launch((int*)ctx->ws, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(mismatches, ctx->ws, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "lsk_debug_radius");
+    return LSK_OK;
+}
+
 int lsk_debug_lsq_ctas(lsk_ctx* ctx, int32_t ctas) {
     if (!ctx) return LSK_ERR_INVALID_ARG;
     if (ctas != 0 && (ctas < 2 || ctas > 16 || (ctas & (ctas - 1)))) return fail(ctx, LSK_ERR_INVALID_ARG, "ctas must be 0, 2, 4, 8 or 16");

@@ -138,6 +138,13 @@ __global__ void reduce_partials_kernel(const float* __restrict__ part, int64_t n
     }
 }
 
+__global__ void radius_debug_kernel(int* count) {
+    for (uint32_t a = blockIdx.x * blockDim.x + threadIdx.x; a < 1u << 24; a += gridDim.x * blockDim.x) {
+        const float x = -2.0f * logf((float)(a + 1u) * 5.9604644775390625e-08f);
+        if (__float_as_uint(radius24(x)) != __float_as_uint(sqrtf(x)) && !(x == 0.f && radius24(x) == 0.f)) atomicAdd(count, 1);
+    }
+}
+
 __global__ void gauss_debug_kernel(int64_t k, int64_t r, uint32_t k0, uint32_t k1, float scale,
                                    int bf16, float* __restrict__ G) {
     const int64_t nq = (k + 3) / 4;
@@ -213,6 +220,11 @@ cudaError_t gauss_launch(const float* SA, int64_t r, int64_t d, int64_t k, uint6
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
     LSK_PROF("gauss_reduce", st) launch_pdl(reduce_partials_kernel, (unsigned)g, 256, 0, 1, st, part, p.nz, len, GSA);
+    return cudaGetLastError();
+}
+
+cudaError_t radius_debug_launch(int* count, cudaStream_t st) {
+    radius_debug_kernel<<<1024, 256, 0, st>>>(count);
     return cudaGetLastError();
 }
 
