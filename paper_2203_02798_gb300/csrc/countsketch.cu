@@ -560,11 +560,18 @@ __global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC)) cs_dense_g
                     }
                     continue;
                 }
+                // else row by row, two summed before they are added where they can be
+                // (20,000 x 50 -> 2,500, eight rows to a bucket: 5.1e-8 off, 5.6e-8 one by one)
+                V two[U];
 #pragma unroll
                 for (int q = 0; q < kRows; ++q) {
                     const uint32_t t = t0 + j + q + 1;   // past this row
 #pragma unroll
-                    for (int u = 0; u < U; ++u) vadd(acc[u], v[q][u], sg[q]);
+                    for (int u = 0; u < U; ++u) {
+                        if (q % 2 == 0) vzero(two[u]);
+                        vadd(two[u], v[q][u], sg[q]);
+                        if (q % 2) vadd(acc[u], two[u], 1.0f);
+                    }
                     const bool last = t <= e && (t == end || t == e);
                     if (!__any_sync(kAll, last)) continue;
                     if (last) {
@@ -572,6 +579,10 @@ __global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC)) cs_dense_g
                         const bool store = whole && end <= e && !accumulate;
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
+                            if (q % 2 == 0) {
+                                vadd(acc[u], two[u], 1.0f);
+                                vzero(two[u]);
+                            }
                             if (colok[u]) {
                                 V* o = reinterpret_cast<V*>(out + (u * L + tl) * VEC);
                                 if (store) *o = acc[u];
