@@ -1122,6 +1122,12 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         const int own = compact || r >= 8 * teams || (r >= 2 * teams && n <= 32 * r) ? 1 : 0;
         if (!own && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
         const unsigned grid = (unsigned)((teams * L + kGatherThreads - 1) / kGatherThreads);
+        // A long gather's blocks are not sent out while the permutation's last kernel
+        // runs (without a memset of SA between the two): waiting beside that kernel's
+        // blocks they cost more than they save.  1M x 200 -> 65,536 233 us against 190,
+        // 300,000 x 100 -> 10,000 54 against 49, 100,000 x 256 -> 8,192 40 against 39;
+        // 50,000 x 100 -> 10,000 26 against 29, 33,333 x 256 -> 65,536 33 against 36.
+        if (own && n * d >= (1 << 24)) early = false;
         auto launch = [&](auto kernel) {
             LSK_PROF("cs_dense_gather", st) launch_chained(early, kernel, grid, kGatherThreads, 0, 1, st, Av, A->ld, d,
                                                            (uint32_t)r, off, perm, SA, teams, own, acc, cpos);
