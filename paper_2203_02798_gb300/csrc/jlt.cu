@@ -323,7 +323,8 @@ cudaError_t jlt_launch(const lsk_mat* A, int64_t m, uint64_t seed, int32_t prec,
     p.part = (float*)ws;
     p.flag = flag;
     cudaError_t e;
-    if (q.smem > 48 * 1024 && (e = allow_dynamic_smem(csrjlt_kernel)) != cudaSuccess) return e;
+    // (at any size: the default limit, 48 KB, counts the kernel's static arrays too)
+    if ((e = allow_dynamic_smem(csrjlt_kernel)) != cudaSuccess) return e;
     LSK_PROF("csrjlt", st) csrjlt_kernel<<<dim3((unsigned)q.jblocks, (unsigned)q.nsplit), kThreads, q.smem, st>>>(p);
     const int64_t total = d * m;
     const bool many = q.nsplit * q.parts > 256;   // (128 loads in flight an entry, or 32)

@@ -1,4 +1,9 @@
-"""csrjlt (Alg. 4) in FP32: the error of long sums against 64 bits."""
+"""csrjlt (Alg. 4) in FP32: the error of long sums against 64 bits, and slices of
+every size."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -32,3 +37,25 @@ def test_error_of_long_sums(n, d, nz, m):
             want[j] += np.bincount(J[blk], weights=V[blk] * G[j, rows[blk] - i], minlength=d)
     L = n * nz / (d * min(n // 1024, 152 * (160 << 10) // (d * m * 4)))
     assert np.linalg.norm(C - want) <= 2.0 ** -24 * np.sqrt(2.25 + 0.11 * L) * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d,m", [(120, 60), (128, 221), (256, 73), (1100, 8)])
+def test_first_call_of_a_process(d, m):
+    """Slices of C just below 48 KB, as the first call of a process (a larger one
+    before it would have raised the kernel's limit)."""
+    code = f"""
+import numpy as np, paper_2203_02798_gb300 as lsk
+from oracle import gaussian as oga
+n, d, m = 3000, {d}, {m}
+rng = np.random.default_rng(d)
+J = rng.integers(0, d, size=n).astype(np.int32)
+V = rng.standard_normal(n).astype(np.float32)
+C = lsk.csrjlt(lsk.csr_from_numpy(V, J, np.arange(n + 1, dtype=np.int64), d), m, 3, "fp32").cpu().numpy()
+G = oga.gaussian_columns(m, 0, n, 3, oga.PREC_FP32, oga.STREAM_JLT)
+A = np.zeros((n, d))
+A[np.arange(n), J] = V
+assert np.linalg.norm(C - G @ A) <= 1e-6 * np.linalg.norm(G @ A)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert p.returncode == 0, p.stderr[-2000:]
