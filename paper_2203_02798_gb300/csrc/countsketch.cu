@@ -1112,9 +1112,11 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         const uintptr_t at = (uintptr_t)Av | (uintptr_t)SA | (uintptr_t)(4 * d) | (uintptr_t)(4 * A->ld);
         const int vec = (at & 15) == 0 ? 4 : (at & 7) == 0 ? 2 : 1;
         const int L = vec == 4 ? (d <= 32 ? 8 : d <= 64 ? 16 : 32) : 32;
-        // one wave of teams, of 8 rows at least
+        // one wave of teams, of 8 rows or 16 buckets (to store, empty ones too) at least
         int64_t teams = (int64_t)sm_count * gather_per_sm(vec) * kGatherThreads / L;
-        teams = std::max<int64_t>(1, std::min(teams, (n + 7) / 8));
+        teams = std::max<int64_t>(1, std::min(teams, std::max((n + 7) / 8, (r + 15) / 16)));
+        // two buckets a team where that makes them 16 rows at most: whole ones need no zeroed SA
+        if (!compact && r >= 2 && r < 2 * teams && n <= 8 * r) teams = r / 2;
         // Whole buckets per team where each has eight of them, or two that are
         // short: the rows are then shared out to about an eighth, or to a few
         // dozen rows, and SA need not be zeroed.  A compacted SA holds no rows
