@@ -200,11 +200,13 @@ __global__ void __launch_bounds__(1024) gram_csr_kernel(const float* __restrict_
 // shared-memory form's.  The diagonal, which every row hits, is summed in shared
 // memory.  Shared memory has no FP32 add: its loop of compare-and-swap with a
 // row a thread, two nonzeros in most, left lanes and time idle.  1M x 200 with
-// two nonzeros a row: 58 us (86), 1M x 256 79 (194).
+// two nonzeros a row: 58 us (86), 1M x 256 79 (194).  2^lg warps share a group of
+// rows where there are few of them for the GPU's warps (10,000 x 256 with 50 nonzeros
+// a row: 684 us with a warp a group, 165 now, 273 by the shared-memory form).
 __global__ void __launch_bounds__(1024) gram_csr_red_kernel(const float* __restrict__ V, const int32_t* __restrict__ J,
                                                            const int64_t* __restrict__ I, int64_t n, int64_t nnz,
                                                            int64_t d, float* __restrict__ part, int copies,
-                                                           int* flag) {
+                                                           int lg, int* flag) {
     extern __shared__ float D[];
     float* P = part + (int64_t)(blockIdx.x % copies) * d * d;
     for (int64_t c = threadIdx.x; c < d; c += blockDim.x) D[c] = 0.f;
@@ -216,10 +218,11 @@ __global__ void __launch_bounds__(1024) gram_csr_red_kernel(const float* __restr
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     bool bad = false;
-    for (int64_t i0 = warp * 32; i0 < n; i0 += nwarps * 32) {
+    const int64_t tasks = ((n + 31) / 32) << lg;
+    for (int64_t t = warp; t < tasks; t += nwarps) {
         RowGroup g;
-        if (!g.load(I, i0 + lane, n, nnz)) bad = true;
-        for (int64_t e0 = 0; e0 < g.total; e0 += 32) {
+        if (!g.load(I, (t >> lg) * 32 + lane, n, nnz)) bad = true;
+        for (int64_t e0 = (t & ((1 << lg) - 1)) * 32; e0 < g.total; e0 += (int64_t)32 << lg) {
             const int64_t e = min(e0 + lane, g.total - 1);
             const int q = g.lane_of(e);
             const int64_t first = g.first_of(q), at = first + e, last = first + g.upto_of(q);
@@ -328,10 +331,12 @@ CsrPlan csr_plan(int64_t n, int64_t d, int sm_count) {
 
 // Reductions in L2 where rows hold four nonzeros or fewer on average, or where
 // a partial matrix does not fit in shared memory, whose form then reads A once
-// per slice.  Denser rows make d^2 products each out of few loads: with 6.4
-// nonzeros a row (300,000 x 128) 106 us against 100, with 16 (100,000 x 32) 171
-// against 148; with 3.2 (300,000 x 64) 44 against 52; 50,000 x 256 with 128, two
-// slices, 2.8 ms against 6.7.
+// per slice: of d = 230 .. 512, 5 .. 100 nonzeros a row and 10,000 .. 200,000 rows
+// they are the faster everywhere (200,000 x 256 with 5: 42 us against 43, 10,000 x 256
+// with 23: 63 against 84, 50,000 x 512 with 100: 1.5 ms against 11).  For smaller d the
+// shared-memory form keeps denser rows: with 6.4 nonzeros a row (300,000 x 128) 106 us
+// against 100, with 16 (100,000 x 32) 171 against 148; with 3.2 (300,000 x 64) 44 against
+// 52.
 bool gram_csr_reduces(const lsk_mat* A, const CsrPlan& p) { return p.nslices > 1 || A->nnz / 4 <= A->n; }
 
 }  // namespace
@@ -371,11 +376,16 @@ cudaError_t gram_launch_t(const lsk_mat* A, double alpha, double beta, OutT* C, 
         if (gram_csr_reduces(A, p)) {
             if ((e = allow_dynamic_smem(gram_csr_red_kernel)) != cudaSuccess) return e;
             const int64_t groups = std::max<int64_t>(1, (n + 31) / 32);
-            const int blocks = (int)std::min<int64_t>(groups, sm_count);
+            // a task for every warp, of 32 nonzeros or more; four of 96 or more
+            int lg = 0;
+            const int64_t warps = 32 * (int64_t)sm_count;
+            while ((groups << lg) < warps && A->nnz >> (lg + 1) >= n) ++lg;
+            while ((groups << lg) < 4 * warps && (A->nnz >> (lg + 1)) / 3 >= n) ++lg;
+            const int blocks = (int)std::min<int64_t>(groups << lg, sm_count);
             const int copies = (int)std::min<int64_t>(blocks, p.nblocks);
             if (copies < blocks && (e = cudaMemsetAsync(part, 0, (size_t)(copies * len) * 4, st)) != cudaSuccess) return e;
             LSK_PROF("gram_csr", st) gram_csr_red_kernel<<<blocks, 1024, (size_t)d * 4, st>>>(
-                (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, part, copies, flag);
+                (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, part, copies, lg, flag);
             LSK_PROF("gram_reduce", st) gram_csr_reduce_kernel<OutT>
                 <<<(unsigned)((len + 31) / 32), 256, 0, st>>>(part, copies, d, alpha, beta, C);
             return cudaGetLastError();
