@@ -67,12 +67,12 @@ __device__ __noinline__ void short_list(const float* __restrict__ A, int64_t lda
 // thread (ty, tx) = (tid / 16, tid % 16): rows 8*ty..8*ty+7, cols 4*tx..4*tx+3.
 // kList: the rows list[0 .. *count) of A and x only (all where *count < 0), a
 // persistent grid.
-template <bool kList>
+template <bool kList, bool kPdl = true>
 __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     const float* __restrict__ A, int64_t lda, int64_t n, int64_t d, const float* __restrict__ B,
     int64_t c, int upper_tri, float alpha, float beta, float* __restrict__ x, const int* __restrict__ list,
     const int* __restrict__ count) {
-    pdl_enter(A, B, x, list, count);
+    if constexpr (kPdl) pdl_enter(A, B, x, list, count);
     __shared__ __align__(16) float As[RK][RMP];
     __shared__ __align__(16) float Bs[RK][RN];
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(256) rownorm_dense_kernel(
     const int64_t rows = all ? n : (int64_t)*count;
     const auto row_of = [&](int64_t i) { return all ? i : (int64_t)__ldg(list + i); };
     const bool brief = kList && !all && rows <= (int64_t)kShort * gridDim.x && c <= 256 && d <= 256;
-    for (int64_t i0 = (int64_t)blockIdx.x * RM; i0 < rows && !brief; i0 += (int64_t)gridDim.x * RM) {
+    int64_t i0 = (int64_t)blockIdx.x * RM;
+    if (!kList || (i0 < rows && !brief)) do {
         float rowsum[8];
 #pragma unroll
         for (int a = 0; a < 8; ++a) rowsum[a] = 0.f;
@@ -156,7 +157,8 @@ __global__ void __launch_bounds__(256) rownorm_dense_kernel(
             }
         }
         if (!kList) return;   // one tile a block
-    }
+        i0 += (int64_t)gridDim.x * RM;
+    } while (i0 < rows);
     if (brief) short_list(A, lda, (int)rows, (int)d, B, (int)c, alpha, beta, x, list, &As[0][0], &Bs[0][0]);
 }
 
@@ -335,7 +337,11 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
             LSK_PROF("rownorm_dense_simt", st) launch_pdl(rownorm_dense_kernel<true>, grid, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, list, count);
         } else {
-            LSK_PROF("rownorm_dense_simt", st) launch_pdl(rownorm_dense_kernel<false>, tiles, 256, 0, 1, st,
+            // chained only where it is short: 4,014 x 32 times 32 x 64 15.7 us (18 plainly), but
+            // 496,154 x 300 times 300 x 64 546 (535 plainly)
+            const bool early = tiles <= 4u * (unsigned)sm_count;
+            LSK_PROF("rownorm_dense_simt", st) launch_chained(
+                early, early ? rownorm_dense_kernel<false> : rownorm_dense_kernel<false, false>, tiles, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, nullptr, nullptr);
         }
     } else {
