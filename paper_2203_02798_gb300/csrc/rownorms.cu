@@ -238,26 +238,26 @@ __global__ void rownorm_csr_kernel(const float* __restrict__ V, const int32_t* _
     if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
 }
 
-// The same with the nonzeros of 32 consecutive rows dealt out to the lanes of a
-// warp: the lane of entry p forms v_p (v_p M_pp + 2 sum_{t > p} v_t M_pt), a
-// segmented sum over the lanes adds up each row's entries, and the lane of the
-// row keeps the sum.  For denser rows, whose pairs would otherwise follow one
-// another in one thread: 50,000 x 256 with 128 nonzeros a row 1.0 ms (2.1),
-// 200,000 x 256 with 12.8 71 us (98), 300,000 x 128 with 6.4 36 (42); with two a
-// row (1M x 200) finding the entries costs more than it shares out, 39 against 36.
+// The same with the nonzeros of `rows` (32 or fewer) consecutive rows dealt out to
+// the lanes of a warp: the lane of entry p forms v_p (v_p M_pp + 2 sum_{t > p} v_t
+// M_pt), a segmented sum over the lanes adds up each row's entries, and the lane of
+// the row keeps the sum.  For denser rows, whose pairs would otherwise follow one
+// another in one thread: 50,000 x 256 with 128 nonzeros a row 1.0 ms (2.1), 200,000
+// x 256 with eight 45 us (59), 300,000 x 128 with 6.4 36 (42); with two a row (1M x
+// 200) finding the entries costs more than it shares out, 39 against 36.
 __global__ void __launch_bounds__(256, 8) rownorm_csr_flat_kernel(const float* __restrict__ V, const int32_t* __restrict__ J,
                                                                   const int64_t* __restrict__ I, int64_t n, int64_t nnz,
                                                                   int64_t d, const float* __restrict__ M, float alpha,
-                                                                  float beta, float* __restrict__ x, int* flag) {
+                                                                  float beta, float* __restrict__ x, int rows, int* flag) {
     pdl_read(V, J, I, M, x);
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     bool bad = false;
-    for (int64_t i0 = warp * 32; i0 < n; i0 += nwarps * 32) {
-        const int64_t i = i0 + lane;
+    for (int64_t i0 = warp * rows; i0 < n; i0 += nwarps * rows) {
+        const int64_t i = i0 + lane, i1 = min(n, i0 + rows);
         RowGroup g;
-        if (!g.load(I, i, n, nnz)) bad = true;
+        if (!g.load(I, i, i1, nnz)) bad = true;
         int64_t before = __shfl_up_sync(0xffffffffu, g.upto, 1);   // entries of the rows before it
         if (lane == 0) before = 0;
         float sum = 0.f;
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(256, 8) rownorm_csr_flat_kernel(const float* _
             const float part = __shfl_sync(0xffffffffu, q, (int)(end - 1 - e0) & 31);
             if (end > e0 && end > before) sum += part;
         }
-        if (i < n) x[i] = (beta != 0.f) ? fmaf(alpha, sum, beta * x[i]) : alpha * sum;
+        if (i < i1) x[i] = (beta != 0.f) ? fmaf(alpha, sum, beta * x[i]) : alpha * sum;
     }
     if (bad) set_flag(flag, LSK_FLAG_BAD_CSR);
 }
@@ -352,12 +352,17 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         float* M = prepared ? (float*)prepared : (float*)ws;   // prepared: built by bbt_group_launch
         const dim3 bg((unsigned)((d + 15) / 16), (unsigned)((d + 15) / 16));
         if (!prepared) LSK_PROF("rownorm_bbt", st) launch_pdl(bbt_kernel, bg, 256, 0, 1, st, B, d, c, M);
-        int64_t gr = (n + 255) / 256;
+        const bool flat = A->nnz / 3 > n;
+        int rows = 32;   // of a warp of the flat form: fewer where warps are few, 64 nonzeros or more
+        while (flat && rows > 4 && n / rows < 32 * (int64_t)sm_count && A->nnz * (rows / 2) >= 64 * n) rows /= 2;
+        int64_t gr = flat ? (n + 8 * rows - 1) / (8 * rows) : (n + 255) / 256;
         if (gr > 16 * (int64_t)sm_count) gr = 16 * (int64_t)sm_count;
-        LSK_PROF("rownorm_csr", st)
-            launch_chained(!prepared, A->nnz / 3 > n ? rownorm_csr_flat_kernel : rownorm_csr_kernel, (unsigned)gr, 256, 0,
-                           1, st, (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, M, (float)alpha,
-                           (float)beta, x, flag);
+        if (flat)
+            LSK_PROF("rownorm_csr", st) launch_chained(!prepared, rownorm_csr_flat_kernel, (unsigned)gr, 256, 0, 1, st,
+                (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, M, (float)alpha, (float)beta, x, rows, flag);
+        else
+            LSK_PROF("rownorm_csr", st) launch_chained(!prepared, rownorm_csr_kernel, (unsigned)gr, 256, 0, 1, st,
+                (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, M, (float)alpha, (float)beta, x, flag);
     }
     return cudaGetLastError();
 }
