@@ -341,9 +341,10 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
             LSK_PROF("rownorm_dense_simt", st) launch_pdl(rownorm_dense_kernel<true>, grid, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, list, count);
         } else {
-            // chained only where it is short: 4,014 x 32 times 32 x 64 15.7 us (18 plainly), but
-            // 496,154 x 300 times 300 x 64 546 (535 plainly)
-            const bool early = tiles <= 4u * (unsigned)sm_count;
+            // chained only where every block finds an SM of its own: sent out early, more than
+            // that pile up on those that are free first (19,000 x 400 times 400 x 64 31.0 us
+            // chained, 33.3 plainly; 50,000 x 400 102 and 79; 496,154 x 300 546 and 535)
+            const bool early = tiles <= (unsigned)sm_count;
             LSK_PROF("rownorm_dense_simt", st) launch_chained(
                 early, early ? rownorm_dense_kernel<false> : rownorm_dense_kernel<false, false>, tiles, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, nullptr, nullptr);
