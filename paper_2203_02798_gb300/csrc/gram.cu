@@ -381,7 +381,9 @@ cudaError_t gram_launch_t(const lsk_mat* A, double alpha, double beta, OutT* C, 
             const int64_t warps = 32 * (int64_t)sm_count;
             while ((groups << lg) < warps && A->nnz >> (lg + 1) >= n) ++lg;
             while ((groups << lg) < 4 * warps && (A->nnz >> (lg + 1)) / 3 >= n) ++lg;
-            const int blocks = (int)std::min<int64_t>(groups << lg, sm_count);
+            // with one slice a copy for every block, which then needs no zeroing: its rows_per
+            // may make a few blocks fewer than the SMs (15,964 x 50, 151 of 152)
+            const int blocks = (int)std::min<int64_t>(groups << lg, p.nslices > 1 ? (int64_t)sm_count : std::min<int64_t>(sm_count, p.nblocks));
             const int copies = (int)std::min<int64_t>(blocks, p.nblocks);
             if (copies < blocks && (e = cudaMemsetAsync(part, 0, (size_t)(copies * len) * 4, st)) != cudaSuccess) return e;
             LSK_PROF("gram_csr", st) gram_csr_red_kernel<<<blocks, 1024, (size_t)d * 4, st>>>(
