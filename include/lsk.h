@@ -116,7 +116,11 @@ int lsk_reserve(lsk_ctx* ctx, size_t bytes);
  * m = 0, Sec. 5).  S is r x n with one +-1 per column (hash and signs from
  * `seed`, see the header comment).  A: dense or CSR, n x d.  SA: device,
  * r*d floats, row-major, fully overwritten (rows no row of A hashes to are
- * zero).  Requires 1 <= r < 2^31, n < 2^31. */
+ * zero).  Requires 1 <= r < 2^31, n < 2^31.  The order of a bucket's rows (of
+ * an entry's nonzeros for CSR A) is not fixed: equal calls agree to FP32
+ * rounding, not bit for bit, except on data whose sums are exact.  For CSR A
+ * most sketches are summed by reductions in L2, which flush sums below 2^-126
+ * to zero. */
 int lsk_cs_sketch(lsk_ctx* ctx, const lsk_mat* A, int64_t r, uint64_t seed,
                   float* SA);
 
@@ -173,15 +177,25 @@ int lsk_gram(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta,
 /* lsk_gram with a precision: LSK_PREC_FP32 to FP32 accuracy (as lsk_gram for
  * CSR A): dense A with d <= 256 and n d >= 2^19 on the tensor cores, as eight
  * products of three-term bf16 splits whose leading one accumulates exactly
- * (about 2e-8 relative Frobenius error; columns outside the split's range
- * send the call to the CUDA cores), else FP32 on the CUDA cores with partial
- * sums folded into FP64; LSK_PREC_BF16 (and LSK_PREC_TF32) forms the products of dense
+ * (2e-8 to 3e-8 relative Frobenius error, 4.5e-8 with a few rows scaled x100).
+ * An entry below 2^-8 of the largest that its column showed of late keeps 16 of
+ * its 24 bits, so that C_jl is off by a multiple of FP32's rounding of
+ * ||A_j|| ||A_l||, not of the sum of |a_ij a_il|, and as the largest is found
+ * while it runs, equal calls may differ in the last bits.  Columns outside the
+ * split's range, sums near the end of FP32's, infinities and NaN send the call
+ * to the CUDA cores.  Other dense A: FP32 on the CUDA cores with partial
+ * sums folded into FP64 (equal calls agree bit for bit).  CSR A: products
+ * summed in FP32, where rows hold four nonzeros or fewer (or d > 221) by
+ * reductions in L2 in no fixed order, which flush sums below 2^-126 to zero.
+ * LSK_PREC_BF16 (and LSK_PREC_TF32) forms the products of dense
  * A with d <= 256 on the tensor
  * cores from a bfloat16 split of A (a = hi + lo; hi^T hi + hi^T lo + lo^T hi,
  * about 2^-16 relative per product), accumulating at most 1024 rows in FP32
  * before the slices are added (compensated FP32, alpha and beta in FP64).
- * CSR A or d > 256 take the FP32 path.  Workspace: ceil(n / 1024) d*d
- * floats for the BF16 path. */
+ * CSR A or d > 256 take the FP32 path.  Workspace: one d*d matrix of floats
+ * for each block of the BF16 path (a block an SM at most), and one for every 24
+ * segments of 1024 rows of a block in the FP32 tensor-core path, beside the
+ * CUDA-core path's. */
 int lsk_gram_prec(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta,
                   int32_t prec, float* C);
 
@@ -192,8 +206,9 @@ int lsk_gram_prec(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta,
  * lets the dense kernels skip the zero blocks.  prec (dense A):
  * LSK_PREC_FP32 = FP32 accuracy: for d, c <= 256 and n d c >= 2^30 on the
  * tensor cores, as six products of scaled three-term bf16 splits whose
- * leading one accumulates exactly (4.5e-8 relative; rows outside the split's
- * range are formed on the CUDA cores), else on the CUDA cores (a wide general
+ * leading one accumulates exactly (3.2e-8 relative, rms over the rows; up to
+ * 3.8e-8 with B = R^-1 of A; rows outside the split's range are formed on the
+ * CUDA cores, all rows where most are), else on the CUDA cores (a wide general
  * B with beta != 0 too); LSK_PREC_BF16 = tensor cores with A and B
  * split into bf16 hi + lo, A B ~ AhBh + AhBl + AlBh, FP32 accumulation, for
  * d, c <= 256 (other shapes run the FP32 kernel); LSK_PREC_TF32 = one TF32
@@ -284,11 +299,13 @@ int lsk_leverage_scores_jl(lsk_ctx* ctx, const lsk_mat* A, int64_t r, int64_t k,
                            int64_t m, uint64_t seed, int32_t prec, float* ell,
                            double* R_out);
 
-/* Exact leverage scores (Alg. 13): B = A^T A in FP64 (FP32 partial sums
- * over row blocks, folded in FP64), R from B (FP64 accurate; Cholesky in
- * place of the SVD of step 2 at full rank), theta_i = ||A_i R^-1||^2
- * (Alg. 8).  theta: device n floats; R_out: NULL or device d*d doubles.
- * Rank deficiency is the deferred LSK_ERR_RANK_DEFICIENT; d <= 1024. */
+/* Exact leverage scores (Alg. 13): B = A^T A as lsk_gram_prec(LSK_PREC_FP32)
+ * forms it (FP32 partial sums over row blocks, added in FP64 or, from the
+ * tensor cores and for CSR A, with compensation), stored in FP64, R from B
+ * (FP64 accurate; Cholesky in place of the SVD of step 2 at full rank),
+ * theta_i = ||A_i R^-1||^2 (Alg. 8).  theta: device n floats; R_out: NULL or
+ * device d*d doubles.  Rank deficiency is the deferred
+ * LSK_ERR_RANK_DEFICIENT; d <= 1024. */
 int lsk_leverage_scores_exact(lsk_ctx* ctx, const lsk_mat* A, int32_t prec,
                               float* theta, double* R_out);
 
@@ -347,7 +364,9 @@ int lsk_leverage_scores_hrn(lsk_ctx* ctx, const lsk_mat* A, int64_t r, int64_t k
  * of that construction (column index = row index of A); bfloat16-rounded in
  * the BF16 mode.  A: CSR only (LSK_ERR_UNSUPPORTED otherwise; a dense A is a
  * plain GEMM).  C: device m x d floats, row-major (written).  FP32 partial
- * sums over row ranges of A, added with compensation in a fixed order.  Malformed
+ * sums over row ranges of A of a thousand rows or so (longer ones where their
+ * partials would take more than 160 KB an SM), added with compensation in a fixed
+ * order.  Malformed
  * CSR sets the deferred LSK_ERR_BAD_CSR.  m in [1, 2^20], d <= 1280. */
 int lsk_csrjlt(lsk_ctx* ctx, const lsk_mat* A, int64_t m, uint64_t seed,
                int32_t prec, float* C);
@@ -446,7 +465,8 @@ void lsk_lsq_default_opts(lsk_lsq_opts* opts, int64_t d);
  * eta = ||A^T r|| / ||A^T b|| <= opts->tol.  b: device n doubles; x: device
  * d doubles (output).  info may be NULL.  Synchronises the stream (it reads
  * scalars back); LSK_ERR_NOT_CONVERGED when max_refine steps do not reach
- * tol. */
+ * tol.  The scale of b does not matter (1e-100 to 1e100 are solved alike).
+ * Workspace beside the sketch's: for CSR A its tiles, 6 bytes a nonzero. */
 int lsk_sketch_precondition_lsq(lsk_ctx* ctx, const lsk_mat* A,
                                 const double* b, double* x,
                                 const lsk_lsq_opts* opts, lsk_lsq_info* info);

@@ -209,7 +209,8 @@ int lsk_set_fused_sketch(int mode) { return g_fused_sketch.exchange(mode < 0 ? 0
 
 }  // extern "C"
 namespace {
-// A^T A on the CUDA cores in FP32 (partials folded in FP64); CSR: Alg. 7
+// A^T A to FP32 accuracy: large dense A on the tensor cores, other dense A on the
+// CUDA cores (partials folded in FP64); CSR: Alg. 7
 int gram_fp32(lsk_ctx* ctx, const lsk_mat* A, double alpha, double beta, float* C) {
     ProfGuard pg(ctx);
     int rc = check_mat(ctx, A);

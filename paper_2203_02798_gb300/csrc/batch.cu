@@ -225,8 +225,8 @@ cudaError_t record(lsk_ctx* ctx, cudaStream_t main, const std::vector<std::vecto
     }
 
     // the CSR sketches that need no permutation go first: they run while wave w's
-    // permutations are prepared (24 problems: 923 us a call, 941 with the problems in
-    // the order of their cost alone; 64: 3.81 ms, 3.94)
+    // permutations are prepared (in the order of their cost alone a call takes 2% longer
+    // with 24 problems and 3% with 64)
     auto scatters = [&](int s, int w) -> cudaError_t {
         for (int i : lanes[s]) {
             const lsk_batch_item& it = items[i];
@@ -324,11 +324,10 @@ bool groupable(const lsk_batch_item& it, int32_t prec) {
 // a chunk, 3.5 us, and has an SM to itself: blocks of 128 chunks left most SMs
 // without one when the wave holds a few dozen problems (24 problems, 52 blocks:
 // 457 us).  A wave is cut into kGaussBlocksPerSm blocks an SM, down to 24 chunks
-// (below, the k x d partials cost what the shares give: 8 problems take 942 us with
-// 8 chunks, 906 with 16 and 890 with 24; 24 take 963, 965 and 968), unless the
-// schedule's longer slices give that many already: 196 us.  Of 2, 4 and 8
-// blocks an SM the whole call takes 1071, 1078 and 1093 us with 24 problems,
-// 4.37, 4.53 and 4.83 ms with 64, 7.22, 7.25 and 7.55 ms with 160 small ones.
+// (below, the k x d partials take a multiple of the memory and cost about what the
+// shares give: 24 problems take 930 us a call, 924 with 8 chunks, 64 3.60 ms with
+// both), unless the schedule's longer slices give that many already: 196 us.  With
+// four blocks an SM 24 problems take as long, 64 3% longer; with eight 2% and 11%.
 constexpr int64_t kGaussBlocksPerSm = 2, kGaussMinSlice = 24;
 int group_slice(int64_t chunks, int slice, int sm_count) {
     const int64_t want = (chunks + kGaussBlocksPerSm * sm_count - 1) / (kGaussBlocksPerSm * sm_count);

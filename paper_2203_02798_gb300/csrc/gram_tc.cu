@@ -483,11 +483,12 @@ namespace {
 // largest ever) costs exactness in its segment, no more.  Warps note what they see
 // while others split, so that equal calls may differ in the last bits.  Entries below
 // 2^-8 of their column's unit keep 16 bits: the error is small against the norms
-// of the two columns, but not entry by entry against sum |a_ij a_ik|.  A CTA adds up to kChain segments in FP32, the two accumulators
-// apart, and starts another partial for the next ones, so that the error does not
-// grow with its rows (offset entries, 16M x 64, 103 segments: 2.2e-8 in one chain,
-// 1.8e-8 in five; CUDA cores 1.8e-8); all partials are summed with compensation.  Frobenius errors against FP64: 1.9e-8 at 1M x 256
-// (2.9e-8 for the CUDA-core kernel; storing C in FP32 alone costs 1.85e-8),
+// of the two columns, but not entry by entry against sum |a_ij a_ik|.  A CTA adds up
+// to kChain segments in FP32, the two accumulators apart, and starts another partial
+// for the next ones, so that the error does not grow with its rows (offset entries,
+// 16M x 64, 103 segments: 2.2e-8 in one chain, 1.8e-8 in five; CUDA cores 1.8e-8); all
+// partials are summed with compensation.  Frobenius errors against FP64: 1.9e-8 at
+// 1M x 256 (2.9e-8 for the CUDA-core kernel; storing C in FP32 alone costs 1.85e-8),
 // 4.5e-8 against 2.5e-7 with five rows scaled x100.  A column below 2^-48 (its
 // small products would leave FP32's range) or a diagonal whose sum might leave it
 // sets *redo, and the CUDA-core kernel, which adds up in FP64, forms C.
@@ -497,8 +498,8 @@ namespace {
 // shared out by N), so each CTA's two accumulators (2 N <= 512 columns) fill
 // its TMEM.  Each CTA takes a contiguous range of rows.  At 1M x 256
 // the eight products over the block triangle are 0.41 ms of the tensor pipe's
-// measured rate; this takes 0.55 ms (CUDA cores: 4.20), bound by shared-memory
-// bandwidth (the MMAs' operands and the workers' stores keep its data pipe
+// measured rate; the call takes 0.57 to 0.60 ms, this kernel 0.55 of it (CUDA cores:
+// 4.20), bound by shared-memory bandwidth (the MMAs' operands and the workers' stores keep its data pipe
 // full).  What it took: MMAs issued by an elected lane of a warp that runs
 // along, so that the descriptors stay in uniform registers (else issue takes 120
 // cycles an MMA), few flushes, and partials stored by columns.

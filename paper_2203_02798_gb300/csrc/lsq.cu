@@ -298,7 +298,8 @@ __global__ void __launch_bounds__(kPassThreads, 2) cg_pass_dense_rows_kernel(
 // tiles of `rows_per` rows once and each tile's entries also stored sorted by
 // column (local row, value).  A pass then forms u = A p on a tile from the CSR
 // entries (segments: rows) and A^T u from the sorted ones (segments:
-// columns; the CSR arrays were checked by the sketch): in both, the block multiplies a coalesced run of entries by the
+// columns; the CSR arrays were checked by the sketch): in both, the block multiplies a
+// coalesced run of entries by the
 // vector's values in shared memory and sums the segments from there.  With
 // one thread per row and shared-memory float atomics (compare-and-swap loops)
 // for A^T u, a pass took 35 us at 500,000 x 256 and 2.6 M entries; this takes 15,
@@ -306,8 +307,11 @@ __global__ void __launch_bounds__(kPassThreads, 2) cg_pass_dense_rows_kernel(
 constexpr int kTileRowsMax = 4096;
 constexpr int kTilesPerSm = 3;
 // Entries are taken six quads a thread at a time (16-byte loads, all in flight
-// before any product): 6,144 to a run, so that a tile of 500,000 sparse rows is
-// one run; 80 registers a thread, three blocks an SM, one wave of tiles.
+// before any product), 6,144 to a run: what 80 registers a thread, and with them
+// three blocks an SM, leave room for.  A tile with more takes its entries run by run,
+// each of them another round of loads and barriers: at 500,000 x 256 (456 tiles, one
+// wave) a pass takes 14.8 us with 2,200 entries a tile, 18.4 with 5,500, 21.7 with
+// 6,800 (two runs), 26.0 with 11,500 and 34.1 with 13,200 (three).
 constexpr int kQuads = 6;
 constexpr int kTileEntries = kQuads * 4 * kPassThreads;
 

@@ -5,10 +5,12 @@
 //   squared and summed into per-row partials, so A*B never exists outside
 //   registers (the memory-efficient form of Alg. 8 for dense A).  When B is
 //   upper triangular (B = R^-1) the k-loop of column tile [c0, c0+64) stops
-//   at c0+64, skipping the zero blocks.  This is the CUDA-core (SIMT) path
-//   (LSK_PREC_FP32); the tensor-core path lives in rownorms_tc.cu.
+//   at c0+64, skipping the zero blocks.  This is the CUDA-core (SIMT) path of
+//   LSK_PREC_FP32: A that is small, wide or unaligned, and the rows that the
+//   tensor-core path (rownorms_tc3.cu) leaves; BF16 and TF32 are in rownorms_tc.cu.
 // CSR (csrsqn, Alg. 8): Btilde = B B^T is formed once (FP32, 16 x 16 output
-//   tiles); then one thread per row evaluates
+//   tiles); then one thread per row, or with more than three nonzeros a row one
+//   lane per nonzero, evaluates
 //   sum_{p,q in row} v_p v_q Btilde[J_p, J_q] using the symmetry of Btilde.
 #include "lsk_internal.cuh"
 

@@ -29,8 +29,8 @@
 // TMEM lane quarter), 8 MMA issue (even CTA), 9-19 converters (32- or 64-row
 // pieces: 16-byte loads, scale, split, 64-byte-swizzled stores).  Up to 128 columns
 // the accumulators are double-buffered.  750,001 x 200 times 200 x 200:
-// 0.38 ms against 1.98 on CUDA cores; errors 4.5e-8 (root mean square, relative)
-// against 6.8e-8, 2e-7 at most against 3.5e-7.
+// 0.37 ms against 1.98 on CUDA cores; errors 3.2e-8 (root mean square, relative)
+// against 6.7e-8.
 #include "tc_common.cuh"
 
 #include <algorithm>
@@ -50,9 +50,9 @@ constexpr uint32_t kStage = 3 * kSlice;
 // rows: has the piece split, in registers, before it waits, and the next one's
 // loads on their way.  With B's image beside it the ring has three stages at 200
 // columns, and the time from a stage's release to its refill is what the MMAs wait
-// for (750,001 x 200 times 200 x 200: 390 us early, 431 late; 500,000 x 256
-// triangular, four stages, 246 and 250).  With five stages and more (1M x 128
-// times 128 x 128) it is A: 206 early, 170 late.
+// for (750,001 x 200 times 200 x 200: 372 us early, 439 late; 500,000 x 256
+// triangular, four stages, 235 and 256).  With five stages and more (1M x 128
+// times 128 x 128) it is A: 203 early, 166 late.
 template <bool kEarly>
 struct Piece {
     static constexpr int kRowsOf = kEarly ? 32 : 64, kQuads = kRowsOf / 4, kParts = kRows / kRowsOf;
