@@ -454,9 +454,9 @@ __device__ __forceinline__ typename VecT<VEC>::T ldg_stream(const float* p) {
 
 // three blocks an SM keep 32 loads a lane in registers; single floats need fewer
 constexpr int kGatherThreads = 256;
-__host__ __device__ constexpr int gather_per_sm(int vec) { return vec == 1 ? 4 : 3; }
+__host__ __device__ constexpr int gather_per_sm(int vec, int u) { return vec == 1 && u < 4 ? 4 : 3; }
 template <int VEC, int U, int L>
-__global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC)) cs_dense_gather_kernel(
+__global__ void __launch_bounds__(kGatherThreads, gather_per_sm(VEC, U)) cs_dense_gather_kernel(
     const float* __restrict__ A, int64_t lda, int64_t d, uint32_t r, const uint32_t* __restrict__ off,
     const uint32_t* __restrict__ perm, float* __restrict__ SA, int64_t teams, int own, int accumulate,
     const uint32_t* __restrict__ cpos) {
@@ -1112,9 +1112,13 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         const uintptr_t at = (uintptr_t)Av | (uintptr_t)SA | (uintptr_t)(4 * d) | (uintptr_t)(4 * A->ld);
         const int vec = (at & 15) == 0 ? 4 : (at & 7) == 0 ? 2 : 1;
         const int L = vec == 4 ? (d <= 32 ? 8 : d <= 64 ? 16 : 32) : 32;
+        // Odd widths above 64 in one pass of four floats a lane: two passes follow every
+        // chain of permutation and rows twice (1M x 101 -> 10,201 136 us, 113 in one; 30,000
+        // x 127 -> 16,384 28.3 and 26.3).
+        const int U = L < 32 ? 1 : vec == 4 ? (d <= 128 ? 1 : 2) : vec == 2 ? (d <= 64 ? 1 : 2) : d <= 32 ? 1 : d <= 64 ? 2 : 4;
         // one wave of teams, of 8 rows or 16 buckets (to store, empty ones too) at least
-        int64_t teams = (int64_t)sm_count * gather_per_sm(vec) * kGatherThreads / L;
-        teams = std::max<int64_t>(1, std::min(teams, std::max((n + 7) / 8, (r + 15) / 16)));
+        const int64_t wave = (int64_t)sm_count * gather_per_sm(vec, U) * kGatherThreads / L;
+        int64_t teams = std::max<int64_t>(1, std::min(wave, std::max((n + 7) / 8, (r + 15) / 16)));
         // two buckets a team where that makes them 16 rows at most: whole ones need no zeroed SA
         if (!compact && r >= 2 && r < 2 * teams && n <= 8 * r) teams = r / 2;
         // Whole buckets per team where each has eight of them, or two that are
@@ -1136,12 +1140,13 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         };
         if (L == 8) launch(cs_dense_gather_kernel<4, 1, 8>);
         else if (L == 16) launch(cs_dense_gather_kernel<4, 1, 16>);
-        else if (vec == 4 && d <= 128) launch(cs_dense_gather_kernel<4, 1, 32>);
+        else if (vec == 4 && U == 1) launch(cs_dense_gather_kernel<4, 1, 32>);
         else if (vec == 4) launch(cs_dense_gather_kernel<4, 2, 32>);
-        else if (vec == 2 && d <= 64) launch(cs_dense_gather_kernel<2, 1, 32>);
+        else if (vec == 2 && U == 1) launch(cs_dense_gather_kernel<2, 1, 32>);
         else if (vec == 2) launch(cs_dense_gather_kernel<2, 2, 32>);
-        else if (d <= 32) launch(cs_dense_gather_kernel<1, 1, 32>);
-        else launch(cs_dense_gather_kernel<1, 2, 32>);
+        else if (U == 1) launch(cs_dense_gather_kernel<1, 1, 32>);
+        else if (U == 2) launch(cs_dense_gather_kernel<1, 2, 32>);
+        else launch(cs_dense_gather_kernel<1, 4, 32>);
     } else {
         // shared-memory row per warp: pick warps per block to fit 200 KB
         int warps = 8;
