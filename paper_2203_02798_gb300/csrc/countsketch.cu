@@ -1116,16 +1116,18 @@ cudaError_t cs_gather_launch(const lsk_mat* A, int64_t r, const uint32_t* off, c
         // chain of permutation and rows twice (1M x 101 -> 10,201 136 us, 113 in one; 30,000
         // x 127 -> 16,384 28.3 and 26.3).
         const int U = L < 32 ? 1 : vec == 4 ? (d <= 128 ? 1 : 2) : vec == 2 ? (d <= 64 ? 1 : 2) : d <= 32 ? 1 : d <= 64 ? 2 : 4;
-        // one wave of teams, of 8 rows or 16 buckets (to store, empty ones too) at least
+        // one wave of teams, of four rows or four buckets (to store, empty ones too) at
+        // least: with eight and sixteen 1,000 x 101 -> 3,000 took 19.8 us, 15.5 now
         const int64_t wave = (int64_t)sm_count * gather_per_sm(vec, U) * kGatherThreads / L;
-        int64_t teams = std::max<int64_t>(1, std::min(wave, std::max((n + 7) / 8, (r + 15) / 16)));
-        // two buckets a team where that makes them 16 rows at most: whole ones need no zeroed SA
-        if (!compact && r >= 2 && r < 2 * teams && n <= 8 * r) teams = r / 2;
-        // Whole buckets per team where each has eight of them, or two that are
-        // short: the rows are then shared out to about an eighth, or to a few
+        int64_t teams = std::max<int64_t>(1, std::min(wave, std::max((n + 3) / 4, (r + 3) / 4)));
+        // one or two buckets a team where that makes them 16 rows at most: whole ones need
+        // no zeroed SA
+        if (!compact && r >= 2 && r < 2 * teams && n <= 8 * r) teams = r <= wave ? r : r / 2;
+        // Whole buckets per team where each has eight of them, two that are short, or
+        // one: the rows are then shared out to about an eighth, or to a few
         // dozen rows, and SA need not be zeroed.  A compacted SA holds no rows
         // for the empty buckets to zero, and its buckets are short.
-        const int own = compact || r >= 8 * teams || (r >= 2 * teams && n <= 32 * r) ? 1 : 0;
+        const int own = compact || r >= 8 * teams || (r >= 2 * teams && n <= 32 * r) || teams == r ? 1 : 0;
         if (!own && !accumulate && (e = cudaMemsetAsync(SA, 0, (size_t)r * d * 4, st)) != cudaSuccess) return e;
         const unsigned grid = (unsigned)((teams * L + kGatherThreads - 1) / kGatherThreads);
         // A long gather's blocks are not sent out while the permutation's last kernel
