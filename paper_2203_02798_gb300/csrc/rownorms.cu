@@ -200,16 +200,16 @@ __global__ void __launch_bounds__(256) bbt_grouped_kernel(const BbtJob* __restri
     bbt_body(j.B, j.d, j.c, j.M, (t / tiles) * 16, (t % tiles) * 16);
 }
 
-// x_i = alpha a_i M a_i^T + beta x_i, a row a thread.  M's rows are read again and
-// again through L1, so the kernel after this one, which may be the next call's
-// B B^T with its shared memory, is not let in beside it: with it 1M x 256 with two
-// nonzeros a row took 47.8 us a call, 200,000 x 400 with eight 85; without 40.6
-// and 64.5.
+// x_i = alpha a_i M a_i^T + beta x_i, a row a thread.  Launched plainly, as is the
+// form below: blocks sent out beside B B^T pile up on some SMs and read through
+// pointers that the compiler knows nothing of any more (53,322 x 256 with three
+// nonzeros a row 18.3 us on the GPU against 13.5), and the next call's B B^T, let in
+// early with its shared memory, takes the L1 that M's rows are read through (1M x 256
+// with two a row 47.8 us a call against 40.8).
 __global__ void rownorm_csr_kernel(const float* __restrict__ V, const int32_t* __restrict__ J,
                                    const int64_t* __restrict__ I, int64_t n, int64_t nnz, int64_t d,
                                    const float* __restrict__ M, float alpha, float beta,
                                    float* __restrict__ x, int* flag) {
-    pdl_read(V, J, I, M, x);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     bool bad = false;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -251,7 +251,6 @@ __global__ void __launch_bounds__(256, 8) rownorm_csr_flat_kernel(const float* _
                                                                   const int64_t* __restrict__ I, int64_t n, int64_t nnz,
                                                                   int64_t d, const float* __restrict__ M, float alpha,
                                                                   float beta, float* __restrict__ x, int rows, int* flag) {
-    pdl_read(V, J, I, M, x);
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -361,10 +360,10 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         int64_t gr = flat ? (n + 8 * rows - 1) / (8 * rows) : (n + 255) / 256;
         if (gr > 16 * (int64_t)sm_count) gr = 16 * (int64_t)sm_count;
         if (flat)
-            LSK_PROF("rownorm_csr", st) launch_chained(!prepared, rownorm_csr_flat_kernel, (unsigned)gr, 256, 0, 1, st,
+            LSK_PROF("rownorm_csr", st) rownorm_csr_flat_kernel<<<(unsigned)gr, 256, 0, st>>>(
                 (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, M, (float)alpha, (float)beta, x, rows, flag);
         else
-            LSK_PROF("rownorm_csr", st) launch_chained(!prepared, rownorm_csr_kernel, (unsigned)gr, 256, 0, 1, st,
+            LSK_PROF("rownorm_csr", st) rownorm_csr_kernel<<<(unsigned)gr, 256, 0, st>>>(
                 (const float*)A->values, A->colidx, A->rowptr, n, A->nnz, d, M, (float)alpha, (float)beta, x, flag);
     }
     return cudaGetLastError();
