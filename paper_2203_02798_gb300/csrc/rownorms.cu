@@ -354,7 +354,15 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         float* M = prepared ? (float*)prepared : (float*)ws;   // prepared: built by bbt_group_launch
         const dim3 bg((unsigned)((d + 15) / 16), (unsigned)((d + 15) / 16));
         if (!prepared) LSK_PROF("rownorm_bbt", st) launch_pdl(bbt_kernel, bg, 256, 0, 1, st, B, d, c, M);
-        const bool flat = A->nnz / 3 > n;
+        // A lane a nonzero where rows are dense enough: of 3, 4 or 5 nonzeros on, the wider
+        // A the fewer, as the pairs' loads from M then miss L1 (200,000 rows: d = 32 with 4.5
+        // 18.3 us against 17.4 with a lane a row, 5.5 21.1 against 22.2; d = 128 with 3.4 15.0
+        // and 14.2, 4.5 17.8 and 18.5; d = 256 with 3.4 16.7 and 17.6).  While rows are few,
+        // earlier, since there the lanes are too (60,000 x 17 with 4.5 9.3 and 10.7, 200,000 x
+        // 17 18.5 and 18.0); of 9 columns never (60,000 with 8 12.0 and 8.4).
+        const bool few = n < 1024 * (int64_t)sm_count;
+        const int64_t dense = d < 64 ? (few ? 4 : 5) : d < (few ? 128 : 256) ? 4 : 3;
+        const bool flat = d >= (few ? 17 : 32) && A->nnz / dense > n;
         int rows = 32;   // of a warp of the flat form: fewer where warps are few, 64 nonzeros or more
         while (flat && rows > 4 && n / rows < 32 * (int64_t)sm_count && A->nnz * (rows / 2) >= 64 * n) rows /= 2;
         int64_t gr = flat ? (n + 8 * rows - 1) / (8 * rows) : (n + 255) / 256;
