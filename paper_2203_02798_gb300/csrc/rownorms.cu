@@ -344,8 +344,10 @@ cudaError_t rownorms_launch(const lsk_mat* A, const float* B, int64_t c, double 
         } else {
             // chained only where every block finds an SM of its own: sent out early, more than
             // that pile up on those that are free first (19,000 x 400 times 400 x 64 31.0 us
-            // chained, 33.3 plainly; 50,000 x 400 102 and 79; 496,154 x 300 546 and 535)
-            const bool early = tiles <= (unsigned)sm_count;
+            // chained, 33.3 plainly; 50,000 x 400 102 and 79; 496,154 x 300 546 and 535), and
+            // where the tile is short: handed through the wait, the pointers cost the loop 2%
+            // (1,729 x 256 times 256 x 256 75.1 us on the GPU, 73.7 plainly)
+            const bool early = tiles <= (unsigned)sm_count && d * c < (1 << 15);
             LSK_PROF("rownorm_dense_simt", st) launch_chained(
                 early, early ? rownorm_dense_kernel<false> : rownorm_dense_kernel<false, false>, tiles, 256, 0, 1, st,
                 (const float*)A->values, A->ld, n, d, B, c, upper_tri ? 1 : 0, (float)alpha, (float)beta, x, nullptr, nullptr);
