@@ -23,7 +23,7 @@ constexpr int BK = 16;    // reduction step
 __global__ void __launch_bounds__(256, 2) gauss_simt_kernel(
     const float* __restrict__ SA, int64_t r, int64_t d, int64_t k, uint32_t k0, uint32_t k1,
     float scale, int bf16, int64_t kc, float* __restrict__ part) {
-    pdl_enter(SA, part);
+    pdl_launch_next();
     __shared__ __align__(16) float Gs[BK][BM];
     __shared__ __align__(16) float Ss[BK][BN];
     const int tid = threadIdx.x;
@@ -214,8 +214,11 @@ cudaError_t gauss_launch(const float* SA, int64_t r, int64_t d, int64_t k, uint6
     const float scale = (float)(1.0 / sqrt((double)k));
     dim3 grid((unsigned)p.tiles_n, (unsigned)p.tiles_m, (unsigned)p.nz);
     float* part = (float*)ws;
-    LSK_PROF("gauss_simt", st) launch_pdl(gauss_simt_kernel, grid, 256, 0, 1, st, SA, r, d, k, (uint32_t)seed,
-                                           (uint32_t)(seed >> 32), scale, prec == LSK_PREC_BF16 ? 1 : 0, p.kc, part);
+    // Not sent out early: its blocks would pile up on the SMs that the kernel before has
+    // left (504 x 300 to 600 rows 24.5 us on the GPU, 16.3 plainly; scores of 20,000 x 50
+    // through 2,500 to 100 rows 77 and 70).
+    LSK_PROF("gauss_simt", st) gauss_simt_kernel<<<grid, 256, 0, st>>>(SA, r, d, k, (uint32_t)seed, (uint32_t)(seed >> 32),
+                                                                      scale, prec == LSK_PREC_BF16 ? 1 : 0, p.kc, part);
     const int64_t len = k * d;
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
