@@ -990,7 +990,8 @@ cudaError_t cs_hash_launch(int64_t n, int64_t r, uint64_t seed, int32_t* bucket,
 // cs_workspace_bytes (the two-level sort where its plan applies), else
 // cs_workspace_bytes_atomic (count / scan / place with L2 atomics).
 cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm_count, cudaStream_t st,
-                           const uint32_t** off_out, const uint32_t** perm_out, uint64_t row0, int* flag, bool rx {
+                           const uint32_t** off_out, const uint32_t** perm_out, uint64_t row0, int* flag, bool rx,
+                           bool scan_early) {
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     RxPlan q;
     const bool two_level = rx && rx_plan(n, r, q);
@@ -1002,8 +1003,8 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
         LSK_PROF("cs_count", st) launch_pdl(rx_count_kernel, q.nct, kRxThreads, (size_t)q.B * 4, 1, st, n, row0, (uint32_t)r,
                                              k0, k1, q, w.bsign, w.H, w.hstate, w.hstate_words);
         const int64_t len = q.B * q.nct;
-        LSK_PROF("cs_scan", st) launch_pdl(scan_lookback_kernel, (unsigned)((len + kScanTile - 1) / kScanTile), kScanBlock, 0, 1,
-                                            st, w.H, w.H, nullptr, len, w.hstate, flag);
+        LSK_PROF("cs_scan", st) launch_chained(scan_early, scan_lookback_kernel, (unsigned)((len + kScanTile - 1) / kScanTile),
+                                                kScanBlock, 0, 1, st, w.H, w.H, nullptr, len, w.hstate, flag);
         LSK_PROF("cs_place", st) launch_pdl(rx_scatter_kernel, q.nct, kRxThreads, rx_scatter_smem(q), 1, st, n, q, w.bsign, w.H,
                                              w.T, w.TF);
         // Not early: its blocks would wait where the scatter's leave room, several on an SM
@@ -1020,7 +1021,7 @@ cudaError_t cs_prep_launch(int64_t n, int64_t r, uint64_t seed, void* ws, int sm
     if (e != cudaSuccess) return e;
     if (n > 0) LSK_PROF("cs_count", st) cs_count_kernel<<<grid_for(n, 256, sm_count), 256, 0, st>>>(n, row0, (uint32_t)r, k0, k1, w.cnt);
     const unsigned tiles = (unsigned)((r + kScanTile - 1) / kScanTile);
-    LSK_PROF("cs_scan", st) launch_pdl(scan_lookback_kernel, tiles, kScanBlock, 0, 1, st, w.cnt, w.off, w.cursor, r, w.state, flag);
+    LSK_PROF("cs_scan", st) launch_chained(scan_early, scan_lookback_kernel, tiles, kScanBlock, 0, 1, st, w.cnt, w.off, w.cursor, r, w.state, flag);
     if (n > 0) {
         LSK_PROF("cs_place", st) cs_place_kernel<<<grid_for(n, 256, sm_count), 256, 0, st>>>(n, row0, (uint32_t)r, k0, k1, w.cursor, w.perm);
     }
@@ -1093,7 +1094,11 @@ cudaError_t cs_launch(const lsk_mat* A, int64_t r, uint64_t seed, float* SA, voi
         return cs_csr_scatter_launch(A, r, seed, SA, (float*)ws, flag, sm_count, st, row0, accumulate);
     const uint32_t* off = nullptr;
     const uint32_t* perm = nullptr;
-    cudaError_t e = cs_prep_launch(n, r, seed, ws, sm_count, st, &off, &perm, row0, flag, rx);
+    // (the scan of many rows of CSR A plainly: 237,676 x 300 with 30 nonzeros a row -> 464 87.9
+    // us on the GPU early, 82.3 plainly, 500,000 x 100 with ten -> 1,000 79.5 and 73.0; a call of
+    // 44,670 x 32 -> 349 30.5 and 32.7)
+    cudaError_t e = cs_prep_launch(n, r, seed, ws, sm_count, st, &off, &perm, row0, flag, rx,
+                                   A->kind == LSK_DENSE || n < (1 << 17));
     if (e != cudaSuccess) return e;
     uint32_t* cpos = nullptr;
     if (compact) {
