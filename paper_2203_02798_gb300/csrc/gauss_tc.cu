@@ -503,9 +503,10 @@ cudaError_t gauss_tc_launch(const float* SA, int64_t r, int64_t d, int64_t k, ui
     int64_t g = (len + 255) / 256;
     if (g > 8 * (int64_t)sm_count) g = 8 * (int64_t)sm_count;
     // Blocks that come early find a place only on the SMs that the stage leaves free, and
-    // stay there: up to six on each (16,384 x 128 to 256 rows, 128 blocks on 24 SMs, scores in
-    // all 147 us, 151 plainly; 66,475 x 50 to 100, 20 on three, 145 and 137).
-    const bool early = g <= 6 * ((int64_t)sm_count - (int64_t)P.tiles_m * P.slices);
+    // stay there: on 16 or more, up to six on each (16,384 x 128 to 256 rows, 128 blocks on 24
+    // SMs, scores in all 147 us, 151 plainly; 66,475 x 50 to 100, 20 on three, 145 and 137).
+    const int64_t spare = (int64_t)sm_count - (int64_t)P.tiles_m * P.slices;
+    const bool early = spare >= 16 && g <= 6 * spare;
     LSK_PROF("gauss_reduce", st) launch_chained(early, gauss_tc_reduce_kernel, (unsigned)g, 256, 0, 1, st, p.part, P.slices, len,
                                                 GSA);
     return cudaGetLastError();
